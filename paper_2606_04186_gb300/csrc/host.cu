@@ -613,7 +613,7 @@ cudaError_t enqueue_solve_cls(qflow_ctx* c, SolveArgs* cls, int persistent, int 
     for (int k = 1; k <= 3 && e == cudaSuccess; ++k) {
       if (cls[k].nspaces == 0) continue;
       e = qf::launch_solve(k, c->opt.precision, cls[k], c->stream);
-      ++*launches;
+      *launches += qf::solve_launch_count(c->opt.precision, cls[k]);
     }
     return e;
   }

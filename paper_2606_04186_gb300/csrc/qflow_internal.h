@@ -21,6 +21,8 @@ inline int cuda_status(cudaError_t e) {
 
 // Per-space solver status codes written by the solve kernels.
 enum SpaceStatus : int32_t { kSpaceOk = 0, kSpaceNoConv = 1, kSpaceRoot = 2, kSpaceNonFinite = 3, kSpaceInvalid = 4 };
+// Between the two launches of an FP64 solve only: left by solve_fixed.cu for solve.cu's kernel.
+constexpr int32_t kSpaceDefer = 5;
 
 struct SolveArgs {
   int32_t n, nocc, nvir;
@@ -51,12 +53,18 @@ struct SolveArgs {
                            // internal part from the gathered G block and replaces owned amplitudes
   const void* guess;  // nullable start vectors: double (FP64 path) or float (mixed path)
   void* root_out;     // nullable: receives converged roots (Phi coefficient 1), same type/layout
+  int32_t deferred_only;  // nonzero (solve.cu's FP64 kernel): solve only spaces of status kSpaceDefer
   int32_t max_iter;
   double tol;
 };
 
 // Launch the batched solver for spaces of size class k (1, 2 or 3) in the given precision.
 cudaError_t launch_solve(int k, int precision, const SolveArgs& a, cudaStream_t st);
+// The FP64 solver on fixed-point products (solve_fixed.cu): spaces started from Phi in the SES-CC
+// form; leaves status kSpaceDefer where solve.cu's kernel has to decide.
+cudaError_t launch_solve_fixed(int k, const SolveArgs& a, cudaStream_t st);
+// Kernels launch_solve issues for one size class.
+int solve_launch_count(int precision, const SolveArgs& a);
 // Warp-per-space mixed-precision solvers (solve_warp.cu).  W32: optional FP32 copy of W (same
 // layout); NULL reads and converts the FP64 W.
 // Iteration cap of the warp solver's pass in the mixed path: spaces still unconverged after it

@@ -580,14 +580,27 @@ __global__ void __launch_bounds__(Cas<K>::NT) solve_kernel(SolveArgs a) {
   Smem<K, T>& sm = *reinterpret_cast<Smem<K, T>*>(smem_raw);
   constexpr size_t kDuccOff = (sizeof(Smem<K, T>) + 15) / 16 * 16;
   const int tid = threadIdx.x;
+  const int64_t nitems = a.count_dev ? (int64_t)*a.count_dev : a.nspaces;
+  auto deferred = [&](int64_t item) {
+    const int64_t s = a.items ? a.items[item] : item;
+    return a.status[a.sorted_index ? a.sorted_index[s] : s] == kSpaceDefer;
+  };
+  if (a.deferred_only) {  // most blocks have nothing left to do
+    int any = 0;
+    for (int64_t i = blockIdx.x + (int64_t)gridDim.x * tid; i < nitems; i += (int64_t)gridDim.x * C::NT) any |= deferred(i);
+    if (!__syncthreads_or(any)) return;
+  }
   build_tables<K, T>(sm);
   const int n = a.n;
   const size_t n1 = (size_t)n, n2 = n1 * n1, n3 = n2 * n1;
   const T tol = (T)a.tol;
 
-  const int64_t nitems = a.count_dev ? (int64_t)*a.count_dev : a.nspaces;
   for (int64_t item = blockIdx.x; item < nitems; item += gridDim.x) {
     const int64_t s = a.items ? a.items[item] : item;
+    if (a.deferred_only) {  // the block's own item: its threads agree before one of them writes the status
+      const int mine = tid == 0 ? deferred(item) : 0;
+      if (!__syncthreads_or(mine)) continue;
+    }
     // ---- gather + fold ---------------------------------------------------------------
     if (tid == 0) {
       const qflow_space& q = a.spaces[s];
@@ -994,12 +1007,30 @@ cudaError_t launch_solve_rescue(int k, const SolveArgs& a, int64_t* items, unsig
   return launch_fp64(k, b, st);
 }
 
+// The fixed-point form of the FP64 solver takes SES-CC spaces started from Phi.  Its rounding is
+// that of FP64 on O(1) quantities (about 1e-15), far below any tolerance it is used for; a
+// requested residual below 1e-12 stays with solve_kernel.
+static bool fixed_form(const SolveArgs& a) {
+  return !a.guess && !a.ducc_eri && !a.count_dev && a.tol >= 1e-12;
+}
+
+int solve_launch_count(int precision, const SolveArgs& a) {
+  return precision != QFLOW_PREC_MIXED && fixed_form(a) ? 2 : 1;
+}
+
 cudaError_t launch_solve(int k, int precision, const SolveArgs& a, cudaStream_t st) {
   if (precision == QFLOW_PREC_MIXED) {
     SolveArgs w = a;
     if (w.max_iter > kWarpIterCap) w.max_iter = kWarpIterCap;
     return launch_solve_warp(k, w, a.W32, static_cast<const float*>(a.guess), static_cast<float*>(a.root_out), 0,
                              st);
+  }
+  if (fixed_form(a)) {
+    const cudaError_t e = launch_solve_fixed(k, a, st);
+    if (e != cudaSuccess) return e;
+    SolveArgs b = a;
+    b.deferred_only = 1;
+    return launch_fp64(k, b, st);
   }
   return launch_fp64(k, a, st);
 }
