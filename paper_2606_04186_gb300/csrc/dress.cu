@@ -20,6 +20,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "fix_gemm.cuh"
 #include "qflow_internal.h"
 #include "tc_gemm.cuh"
 
@@ -349,7 +350,6 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 //   Foo[m][i] = f~_mi + sum_nef g~_menf u_in^ef           (blocks 0 .. o^2-1)
 //   Fvv[a][e] = f~_ae - sum_mnf g~_menf u_mn^af           (next v^2 blocks)
 //   R1[a][i]  = f~_ai + sum_me f~_me u_im^ae + sum_mef g~_aemf u_im^ef - sum_mne g~_mine u_mn^ae
-//   Woooo[k][i][l][j] = g~_kilj + sum_ef g~_kelf t_ij^ef
 // u[i j a b] = 2 t_ij^ab - t_ij^ba once per dressing (the small blocks read it many times)
 __global__ void k_make_u(const double* __restrict__ t2, double* __restrict__ U, Dims d) {
   const size_t m = (size_t)d.o * d.o * d.v * d.v;
@@ -385,8 +385,8 @@ struct Walk3 {
 };
 
 __global__ void k_small_blocks(const double* __restrict__ F, const double* __restrict__ W,
-                               const double* __restrict__ U, const double* __restrict__ t2, double* __restrict__ foo, double* __restrict__ fvv,
-                               double* __restrict__ r1, double* __restrict__ wo, Dims d) {
+                               const double* __restrict__ U, double* __restrict__ foo, double* __restrict__ fvv,
+                               double* __restrict__ r1, Dims d) {
   __shared__ double red[TPB];
   const int o = d.o, v = d.v;
   const size_t n1 = d.n, n2 = n1 * n1, n3 = n2 * n1;
@@ -412,7 +412,7 @@ __global__ void k_small_blocks(const double* __restrict__ F, const double* __res
     }
     acc = block_sum(acc, red);
     if (threadIdx.x == 0) fvv[y] = F[(o + a) * d.n + o + e] + acc;
-  } else if (x < o * o + v * v + v * o) {
+  } else {
     const int y = x - o * o - v * v, a = y / o, i = y % o;
     // t = (m, e, f): W[o+a, o+e, m, o+f] U[i, m, e, f]
     for (Walk3 w(threadIdx.x, TPB, v, v); w.x0 < o; w.next()) {
@@ -432,195 +432,7 @@ __global__ void k_small_blocks(const double* __restrict__ F, const double* __res
     }
     acc = block_sum(acc, red);
     if (threadIdx.x == 0) r1[y] = F[(o + a) * d.n + i] + acc;
-  } else {
-    const int y = x - o * o - v * v - v * o;
-    const int k = y / (o * o * o), i = (y / (o * o)) % o, l = (y / o) % o, j = y % o;
-    // t = (e, f): W[k, o+e, l, o+f] t2[i, j, e, f]
-    for (Walk3 w(threadIdx.x, TPB, v, v); w.x0 < 1; w.next()) {
-      const int e = w.x1, f = w.x2;
-      acc += W[(size_t)k * n3 + (size_t)(o + e) * n2 + (size_t)l * n1 + (o + f)] * t2[((i * o + j) * v + e) * v + f];
-    }
-    acc = block_sum(acc, red);
-    if (threadIdx.x == 0) wo[y] = W[gi(d, k, i, l, j)] + acc;
   }
-}
-
-// Ring intermediates for the quadratic doubles terms, each [i][a][n][f] (o v o v), precision T:
-//   A = sum_me u_im^ae g~_menf,  B = sum_me u_im^ae g~_mfne,  Cq = sum_me t_im^ae g~_mfne,
-//   D[j][a][n][f] = sum_me t_jm^ea g~_mfne
-template <typename T>
-__global__ void k_rings(const T* __restrict__ G, const T* __restrict__ t2, T* __restrict__ A, T* __restrict__ B,
-                        T* __restrict__ Cq, T* __restrict__ D, Dims d) {
-  const size_t m_all = (size_t)d.o * d.v * d.o * d.v;
-  const size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (x >= m_all) return;
-  const int i = (int)(x / ((size_t)d.v * d.o * d.v)), a = (int)((x / ((size_t)d.o * d.v)) % d.v);
-  const int nn = (int)((x / d.v) % d.o), f = (int)(x % d.v);
-  T sa = 0, sb = 0, sc = 0, sd = 0;
-  for (int m = 0; m < d.o; ++m)
-    for (int e = 0; e < d.v; ++e) {
-      const T g1 = G[gi(d, m, d.o + e, nn, d.o + f)];
-      const T g2 = G[gi(d, m, d.o + f, nn, d.o + e)];
-      const T t = t2[ti(d, i, m, a, e)];
-      const T tx = t2[ti(d, i, m, e, a)];
-      const T u = (T)2 * t - tx;
-      sa += u * g1;
-      sb += u * g2;
-      sc += t * g2;
-      sd += tx * g2;
-    }
-  A[x] = sa;
-  B[x] = sb;
-  Cq[x] = sc;
-  D[x] = sd;
-}
-
-// R2[i][j][a][b] = <Phi_{ij}^{ab}|H-bar|Phi> (alpha-beta): bare g~ vo|vo (FP64, from W) plus the
-// T2 terms in precision T (G: g~ in precision T; W is only read at untouched bare blocks).
-template <typename T>
-__global__ void k_r2(const double* __restrict__ W, const T* __restrict__ G, const T* __restrict__ t2,
-                     const double* __restrict__ foo, const double* __restrict__ fvv, const double* __restrict__ wo,
-                     const T* __restrict__ A, const T* __restrict__ B, const T* __restrict__ Cq,
-                     const T* __restrict__ D, double* __restrict__ r2, Dims d) {
-  const size_t m_all = (size_t)d.o * d.o * d.v * d.v;
-  const size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (x >= m_all) return;
-  const int i = (int)(x / ((size_t)d.o * d.v * d.v)), j = (int)((x / ((size_t)d.v * d.v)) % d.o);
-  const int a = (int)((x / d.v) % d.v), b = (int)(x % d.v);
-  const int A_ = d.o + a, B_ = d.o + b;
-  T v = 0;
-  for (int e = 0; e < d.v; ++e)
-    v += (T)fvv[b * d.v + e] * t2[ti(d, i, j, a, e)] + (T)fvv[a * d.v + e] * t2[ti(d, i, j, e, b)];
-  for (int m = 0; m < d.o; ++m)
-    v -= (T)foo[m * d.o + j] * t2[ti(d, i, m, a, b)] + (T)foo[m * d.o + i] * t2[ti(d, m, j, a, b)];
-  for (int m = 0; m < d.o; ++m)
-    for (int nn = 0; nn < d.o; ++nn) v += (T)wo[((m * d.o + i) * d.o + nn) * d.o + j] * t2[ti(d, m, nn, a, b)];
-  // particle-particle ladder
-  for (int e = 0; e < d.v; ++e)
-    for (int f = 0; f < d.v; ++f) v += G[gi(d, A_, d.o + e, B_, d.o + f)] * t2[ti(d, i, j, e, f)];
-  // linear rings
-  for (int m = 0; m < d.o; ++m)
-    for (int e = 0; e < d.v; ++e) {
-      const int E_ = d.o + e;
-      v += G[gi(d, m, E_, B_, j)] * Ut(t2, d, i, m, a, e);
-      v -= G[gi(d, m, j, B_, E_)] * t2[ti(d, i, m, a, e)];
-      v -= G[gi(d, m, i, B_, E_)] * t2[ti(d, j, m, e, a)];
-      v -= G[gi(d, m, j, A_, E_)] * t2[ti(d, i, m, e, b)];
-      v += G[gi(d, m, E_, A_, i)] * Ut(t2, d, j, m, b, e);
-      v -= G[gi(d, m, i, A_, E_)] * t2[ti(d, j, m, b, e)];
-    }
-  // quadratic rings through the intermediates
-  const size_t ovov_i = (size_t)d.v * d.o * d.v, ovov_a = (size_t)d.o * d.v;
-  for (int nn = 0; nn < d.o; ++nn)
-    for (int f = 0; f < d.v; ++f) {
-      const size_t ia = i * ovov_i + a * ovov_a + (size_t)nn * d.v + f;
-      const size_t ja = j * ovov_i + a * ovov_a + (size_t)nn * d.v + f;
-      v += A[ia] * Ut(t2, d, j, nn, b, f) - B[ia] * t2[ti(d, j, nn, b, f)] + Cq[ia] * t2[ti(d, j, nn, f, b)] +
-           D[ja] * t2[ti(d, i, nn, f, b)];
-    }
-  r2[x] = W[gi(d, A_, i, B_, j)] + (double)v;
-}
-
-// W[a,e,b,f] += sum_mn g~_menf t_mn^ab  (vvvv block; G reads only the ovov block)
-template <typename T>
-__global__ void k_vvvv(double* __restrict__ W, const T* __restrict__ G, const T* __restrict__ t2, Dims d) {
-  const size_t m_all = (size_t)d.v * d.v * d.v * d.v;
-  const size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (x >= m_all) return;
-  const int a = (int)(x / ((size_t)d.v * d.v * d.v)), e = (int)((x / ((size_t)d.v * d.v)) % d.v);
-  const int b = (int)((x / d.v) % d.v), f = (int)(x % d.v);
-  T v = 0;
-  for (int m = 0; m < d.o; ++m)
-    for (int nn = 0; nn < d.o; ++nn) v += G[gi(d, m, d.o + e, nn, d.o + f)] * t2[ti(d, m, nn, a, b)];
-  W[gi(d, d.o + a, d.o + e, d.o + b, d.o + f)] += (double)v;
-}
-
-// (ov|vo) and its pair partner (vo|ov):
-//   W[m,e,b,j] = g~_mebj + sum_nf g~_menf u_jn^bf - sum_nf g~_mfne t_jn^bf
-template <typename T>
-__global__ void k_ovvo(double* __restrict__ W, const T* __restrict__ G, const T* __restrict__ t2, Dims d) {
-  const size_t m_all = (size_t)d.o * d.v * d.v * d.o;
-  const size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (x >= m_all) return;
-  const int m = (int)(x / ((size_t)d.v * d.v * d.o)), e = (int)((x / ((size_t)d.v * d.o)) % d.v);
-  const int b = (int)((x / d.o) % d.v), j = (int)(x % d.o);
-  T v = 0;
-  for (int nn = 0; nn < d.o; ++nn)
-    for (int f = 0; f < d.v; ++f)
-      v += G[gi(d, m, d.o + e, nn, d.o + f)] * Ut(t2, d, j, nn, b, f) -
-           G[gi(d, m, d.o + f, nn, d.o + e)] * t2[ti(d, j, nn, b, f)];
-  const double w = W[gi(d, m, d.o + e, d.o + b, j)] + (double)v;
-  W[gi(d, m, d.o + e, d.o + b, j)] = w;
-  W[gi(d, d.o + b, j, m, d.o + e)] = w;
-}
-
-// (oo|vv) and (vv|oo):  W[i,j,a,b] = g~_ijab - sum_nf g~_ifnb t_jn^fa
-template <typename T>
-__global__ void k_oovv(double* __restrict__ W, const T* __restrict__ G, const T* __restrict__ t2, Dims d) {
-  const size_t m_all = (size_t)d.o * d.o * d.v * d.v;
-  const size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (x >= m_all) return;
-  const int i = (int)(x / ((size_t)d.o * d.v * d.v)), j = (int)((x / ((size_t)d.v * d.v)) % d.o);
-  const int a = (int)((x / d.v) % d.v), b = (int)(x % d.v);
-  T v = 0;
-  for (int nn = 0; nn < d.o; ++nn)
-    for (int f = 0; f < d.v; ++f) v -= G[gi(d, i, d.o + f, nn, d.o + b)] * t2[ti(d, j, nn, f, a)];
-  const double w = W[gi(d, i, j, d.o + a, d.o + b)] + (double)v;
-  W[gi(d, i, j, d.o + a, d.o + b)] = w;
-  W[gi(d, d.o + a, d.o + b, i, j)] = w;
-}
-
-// (oo|vo) and (vo|oo):
-//   W[m,i,b,j] = g~_mibj + sum_e f~_me t_ij^eb + sum_ef g~_mebf t_ij^ef
-//              + sum_ne [g~_mine u_jn^be - g~_meni t_jn^be - g~_menj t_in^eb]
-template <typename T>
-__global__ void k_oovo(double* __restrict__ W, const T* __restrict__ G, const double* __restrict__ F,
-                       const T* __restrict__ t2, Dims d) {
-  const size_t m_all = (size_t)d.o * d.o * d.v * d.o;
-  const size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (x >= m_all) return;
-  const int m = (int)(x / ((size_t)d.o * d.v * d.o)), i = (int)((x / ((size_t)d.v * d.o)) % d.o);
-  const int b = (int)((x / d.o) % d.v), j = (int)(x % d.o);
-  const int B_ = d.o + b;
-  T v = 0;
-  for (int e = 0; e < d.v; ++e) {
-    const int E_ = d.o + e;
-    v += (T)F[m * d.n + E_] * t2[ti(d, i, j, e, b)];
-    for (int f = 0; f < d.v; ++f) v += G[gi(d, m, E_, B_, d.o + f)] * t2[ti(d, i, j, e, f)];
-    for (int nn = 0; nn < d.o; ++nn)
-      v += G[gi(d, m, i, nn, E_)] * Ut(t2, d, j, nn, b, e) - G[gi(d, m, E_, nn, i)] * t2[ti(d, j, nn, b, e)] -
-           G[gi(d, m, E_, nn, j)] * t2[ti(d, i, nn, e, b)];
-  }
-  const double w = W[gi(d, m, i, B_, j)] + (double)v;
-  W[gi(d, m, i, B_, j)] = w;
-  W[gi(d, B_, j, m, i)] = w;
-}
-
-// (vv|vo) and (vo|vv):
-//   W[a,e,b,i] = g~_aebi - sum_m f~_me t_mi^ab + sum_mn g~_meni t_mn^ab
-//              + sum_mf [g~_mfae u_mi^fb - g~_mebf t_mi^af - g~_meaf t_mi^fb]
-template <typename T>
-__global__ void k_vvvo(double* __restrict__ W, const T* __restrict__ G, const double* __restrict__ F,
-                       const T* __restrict__ t2, Dims d) {
-  const size_t m_all = (size_t)d.v * d.v * d.v * d.o;
-  const size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (x >= m_all) return;
-  const int a = (int)(x / ((size_t)d.v * d.v * d.o)), e = (int)((x / ((size_t)d.v * d.o)) % d.v);
-  const int b = (int)((x / d.o) % d.v), i = (int)(x % d.o);
-  const int A_ = d.o + a, E_ = d.o + e, B_ = d.o + b;
-  T v = 0;
-  for (int m = 0; m < d.o; ++m) {
-    v -= (T)F[m * d.n + E_] * t2[ti(d, m, i, a, b)];
-    for (int nn = 0; nn < d.o; ++nn) v += G[gi(d, m, E_, nn, i)] * t2[ti(d, m, nn, a, b)];
-    for (int f = 0; f < d.v; ++f) {
-      const int F_ = d.o + f;
-      v += G[gi(d, m, F_, A_, E_)] * Ut(t2, d, m, i, f, b) - G[gi(d, m, E_, B_, F_)] * t2[ti(d, m, i, a, f)] -
-           G[gi(d, m, E_, A_, F_)] * t2[ti(d, m, i, f, b)];
-    }
-  }
-  const double w = W[gi(d, A_, E_, B_, i)] + (double)v;
-  W[gi(d, A_, E_, B_, i)] = w;
-  W[gi(d, B_, i, A_, E_)] = w;
 }
 
 // Write the dressed oooo, vo|vo blocks and the oo / vv / vo Fock blocks.
@@ -651,7 +463,10 @@ __global__ void k_finalize(double* __restrict__ W, double* __restrict__ F, const
 }
 
 struct Work {
-  double *ht, *foo, *fvv, *wo, *r1, *r2, *A, *B, *Cq, *D, *t2f;  // A..D, t2f hold T values
+  // FP64: A..D products of t2_terms_fixed, t2f = u, r2 its sum Z; mixed: A..D and t2f hold floats,
+  // r2 = u until the residual is formed there
+  double *ht, *foo, *fvv, *wo, *r1, *r2, *A, *B, *Cq, *D, *t2f;
+  int* scales;    // FP64 path: scale exponents of the products' operand rows
   double* epart;  // energy partials
   float* acc;     // mixed path: FP32 GEMM results (v^3 o floats)
   float* f32;     // mixed path: FP32 copies of f~ (n^2), Foo (o^2), Fvv (v^2) for the FP32 finishing sums
@@ -660,6 +475,7 @@ struct Work {
 };
 
 size_t tc_arena_floats(int n, int nocc);
+size_t fix_scale_ints(int o, int v);
 
 size_t carve(void* base, int n, int o, Work* w, bool mixed = false) {
   const int v = n - o;
@@ -672,6 +488,11 @@ size_t carve(void* base, int n, int o, Work* w, bool mixed = false) {
   for (int k = 0; k < 12; ++k) {
     if (base) *ptrs[k] = reinterpret_cast<double*>(static_cast<char*>(base) + off);
     off += ((sizes[k] * sizeof(double) + 255) / 256) * 256;
+  }
+  w->scales = nullptr;
+  if (!mixed) {
+    if (base) w->scales = reinterpret_cast<int*>(static_cast<char*>(base) + off);
+    off += ((fix_scale_ints(o, v) * sizeof(int) + 255) / 256) * 256;
   }
   w->acc = nullptr;
   w->f32 = nullptr;
@@ -716,33 +537,240 @@ size_t dress_workspace_bytes_mixed(int n, int nocc) {
 
 int dress_launch_count(int n, int nocc, bool mixed) {
   // 4 T1 passes (the first one copies; for nocc > kT1Omax a separate copy + 4), h~, f~, 2 energy,
-  // u, small blocks, finalize; T2 terms: 7 SIMT kernels (FP64) or 2 FP32 copies + 33 operand
+  // u, small blocks, finalize; T2 terms: 2 row scales + 3 product launches (FP64) or 2 FP32 copies + 33 operand
   // packs + 9 GEMM launches + the vvvv pack and two product kernels + FP32 Fock copies + 4 finalize
   // kernels + error check (mixed)
   if (!(n - nocc > 0 && nocc > 0)) return 5;
   const int front = (nocc <= kT1Omax ? 4 : 5) + 7;
-  return front + (mixed ? 53 : 7);
+  return front + (mixed ? 53 : 5);
 }
 
 namespace {
 
-template <typename T>
-void t2_terms(const Dims& d, double* W, const T* G, const double* F, const T* t2, const Work& w, cudaStream_t st) {
-  const size_t o = d.o, v = d.v;
-  T* A = reinterpret_cast<T*>(w.A);
-  T* B = reinterpret_cast<T*>(w.B);
-  T* Cq = reinterpret_cast<T*>(w.Cq);
-  T* D = reinterpret_cast<T*>(w.D);
-  k_rings<T><<<blocks_for(o * v * o * v), TPB, 0, st>>>(G, t2, A, B, Cq, D, d);
-  k_r2<T><<<blocks_for(o * o * v * v), TPB, 0, st>>>(W, G, t2, w.foo, w.fvv, w.wo, A, B, Cq, D, w.r2, d);
-  // blocks that read only unmodified bare blocks (through G) may now be overwritten in W
-  k_vvvv<T><<<blocks_for(v * v * v * v), TPB, 0, st>>>(W, G, t2, d);
-  k_ovvo<T><<<blocks_for(o * v * v * o), TPB, 0, st>>>(W, G, t2, d);
-  k_oovv<T><<<blocks_for(o * o * v * v), TPB, 0, st>>>(W, G, t2, d);
-  k_oovo<T><<<blocks_for(o * o * v * o), TPB, 0, st>>>(W, G, F, t2, d);
-  k_vvvo<T><<<blocks_for(v * v * v * o), TPB, 0, st>>>(W, G, F, t2, d);
+// ---- FP64: the T2 contractions on fixed-point products (fix_gemm.cuh) --------------------------
+//
+// Every contraction is a product over index pairs, D(r, c) = sum_k A(r, k) B(c, k), whose operands
+// are strided views of g~ (W after the T1 passes), t2, u = 2 t2 - t2^T and earlier products.  The
+// doubles residual is summed as X + X^T (pair transpose (ia) <-> (jb)), which halves its rings:
+//   X = (ia|jb) sum_me u_im^ae g~_mebj - t_im^ae g~_mjbe  + E u + C t
+//     + (ja|ib) -sum_me t_jm^ea g~_mibe + 1/2 sum_nf D_janf t_in^fb,
+//   E = 1/2 u g~_menf - t g~_mfne,  C = t g~_mfne,  D_janf = sum_me t_jm^ea g~_mfne
+// (the quadratic rings A u - B t + C t^T + D t with A = u g~_menf, B = u g~_mfne: A u, C t and D t are
+// their own pair transposes).  Three launches, so that a block is overwritten after its last use as
+// an operand and no element has two writers: 64-bit sums are exact, so results do not depend on the
+// tiling.  Before: one thread per output element (FP64 FMA chains), 60.3 ms of the 65.5 ms dressing
+// at 82 orbitals.
+using fg::Job;
+using fg::Operand;
+using fg::Out;
+using fg::Seg;
+
+// rows of scale exponents of all operands below
+size_t fix_scale_ints(int o, int v) {
+  return 5 * (size_t)o * o + 6 * (size_t)v * v + 20 * (size_t)o * v + 2 * (size_t)o * o * v + v;
 }
 
+Seg seg(const double* p, int rd, int rs1, int rs2, int kd, int ks1, int ks2, int K, int neg = 0, int shift = 0) {
+  return Seg{p, rd, rs1, rs2, kd, ks1, ks2, K, neg, shift};
+}
+Out out(double* p, int rd, int rs1, int rs2, int cd, int cs1, int cs2, int add) {
+  return Out{p, rd, rs1, rs2, cd, cs1, cs2, add, nullptr, 0, 0, 0, 0};
+}
+
+cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const double* U, const Work& w, cudaStream_t st) {
+  const int o = d.o, v = d.v, n1 = d.n, n2 = n1 * n1, n3 = n2 * n1;
+  const int oo = o * o, vv = v * v, ov = o * v, ovv = o * vv;
+  // start of a block of W: V(mask) has bit 8, 4, 2, 1 set where the first .. fourth index is virtual
+  auto V = [&](int mask) {
+    return W + (size_t)o * ((mask & 8 ? n3 : 0) + (mask & 4 ? n2 : 0) + (mask & 2 ? n1 : 0) + (mask & 1));
+  };
+  double *E = w.A, *C = w.B, *D = w.Cq, *X = w.D, *Y = w.Cq, *Z = w.r2;
+  int* next = w.scales;
+  auto operand = [&](int rows, Seg a) {
+    Operand x{};
+    x.seg[0] = a;
+    x.nseg = 1;
+    x.rows = rows;
+    x.e = next;
+    next += rows;
+    return x;
+  };
+  auto operand2 = [&](int rows, Seg a, Seg b) {
+    Operand x = operand(rows, a);
+    x.seg[1] = b;
+    x.nseg = 2;
+    return x;
+  };
+  // views of t2 / u: rows and k named by their indices
+  auto t_ia_me = [&](const double* t, int neg, int sh) { return seg(t, v, ovv, v, v, vv, 1, ov, neg, sh); };  // t(i m a e)
+  auto t_ja_me = [&](int neg) { return seg(t2, v, ovv, 1, v, vv, v, ov, neg); };                              // t(j m e a)
+  auto g_nf_me = [&](int swap) { return seg(V(5), v, n1, swap ? n2 : 1, v, n3, swap ? 1 : n2, ov); };           // g(m E n F) / g(m F n E)
+  const Operand wA = operand(oo, seg(V(5), o, n3, n1, v, n2, 1, vv));                    // (k l): g(k E l F)
+  const Operand tij = operand(oo, seg(t2, 1, vv, 0, v, v, 1, vv));                       // (i j): t(i j e f)
+  const Operand gab = operand(vv, seg(V(15), v, n3, n1, v, n2, 1, vv));                  // (a b): g(A E B F)
+  const Operand eA = operand2(ov, t_ia_me(U, 0, -1), t_ia_me(t2, 1, 0));
+  const Operand eB = operand2(ov, g_nf_me(0), g_nf_me(1));
+  const Operand cA = operand(ov, t_ia_me(t2, 0, 0));
+  const Operand gx = operand(ov, g_nf_me(1));
+  const Operand dA = operand(ov, t_ja_me(0));
+  const Operand xA = operand2(ov, t_ia_me(U, 0, 0), t_ia_me(t2, 1, 0));
+  const Operand xB = operand2(ov, seg(V(6), v, 1, n1, v, n3, n2, ov),                    // (j b): g(m E B j)
+                              seg(V(3), v, n2, n1, v, n3, 1, ov));                       //        g(m j B E)
+  const Operand v1A = operand2(vv, seg(V(7), v, n1, 1, v, n3, n2, ov),                   // (a e): g(m F A E)
+                               seg(V(7), v, n1, n2, v, n3, 1, ov, 1));                   //       -g(m E A F)
+  const Operand v1B = operand2(ov, seg(U, o, 1, vv, v, ovv, v, ov), seg(t2, o, 1, vv, v, ovv, v, ov));  // (b i): u, t(m i f b)
+  const Operand o1A = operand(ov, seg(V(7), v, n3, n1, v, n2, 1, vv));                   // (m b): g(m E B F)
+  const Operand x2A = operand2(ov, t_ja_me(0), seg(D, 1, ov, 0, ov, 0, 1, ov, 0, -1));   // (j a): t(j m e a), D/2
+  const Operand x2B = operand2(ov, seg(V(3), v, n2, n1, v, n3, 1, ov, 1),                // (i b): -g(m i B E)
+                               seg(t2, v, ovv, 1, v, vv, v, ov));                        //        t(i n f b)
+  const Operand r2A = operand2(oo, seg(W, o, n2, 1, o, n3, n1, oo), seg(w.wo, o, oo, 1, o, oo * o, o, oo));  // (i j): g, wo(m i n j)
+  const Operand r2B = operand2(vv, seg(t2, vv, 0, 1, oo, 0, vv, oo), seg(t2, vv, 0, 1, oo, 0, vv, oo));  // (a b): t(m n a b)
+  const Operand tab = operand(vv, seg(t2, vv, 0, 1, oo, 0, vv, oo));                     // (a b): t(m n a b)
+  const Operand v2B = operand(ov, seg(V(4), o, n2, 1, o, n3, n1, oo));                   // (e i): g(m E n i)
+  const Operand v4B = operand(vv, seg(V(5), v, n2, 1, o, n3, n1, oo));                   // (e f): g(m E n F)
+  const Operand o2A = operand2(oo, seg(V(1), o, n3, n2, v, n1, 1, ov),                   // (m i): g(m i n E)
+                               seg(V(4), o, n3, 1, v, n1, n2, ov, 1));                   //       -g(m E n i)
+  const Operand o2B = operand2(ov, seg(U, o, v, ovv, v, vv, 1, ov), seg(t2, o, v, ovv, v, vv, 1, ov));  // (b j): u, t(j n b e)
+  const Operand x3A = operand2(ov, seg(E, 1, ov, 0, ov, 0, 1, ov), seg(C, 1, ov, 0, ov, 0, 1, ov));     // (i a): E, C
+  const Operand x3B = operand2(ov, t_ia_me(U, 0, 0), t_ia_me(t2, 0, 0));                 // (j b): u, t(j n b f)
+  const Operand ovA = operand2(ov, seg(V(5), v, n3, n2, v, n1, 1, ov),                   // (m e): g(m E n F)
+                               seg(V(5), v, n3, 1, v, n1, n2, ov, 1));                   //       -g(m F n E)
+  const Operand ooA = operand(ov, seg(V(5), v, n3, 1, v, n1, n2, ov));                   // (i b): g(i F n B)
+  Operand ooB = dA;                                                                      // (j a): -t(j n f a)
+  ooB.seg[0].neg = 1;
+  const Operand v3A = operand(vv, seg(V(7), v, n2, n1, v, n3, 1, ov, 1));                // (e b): -g(m E B F)
+  const Operand v3B = operand(ov, seg(t2, o, v, vv, v, ovv, 1, ov));                     // (a i): t(m i a f)
+  const Operand o3A = operand(oo, seg(V(4), o, n3, 1, v, n1, n2, ov, 1));                // (m j): -g(m E n j)
+  const Operand o3B = operand(ov, seg(t2, o, 1, ovv, v, vv, v, ov));                     // (b i): t(i n e b)
+  const Operand yA = operand(oo * v, seg(t2, 1, v, 0, v, 0, 1, v));                      // (i j a): t(i j a e)
+  const Operand y2A = operand(oo * v, seg(t2, v, vv, 1, v, 0, v, v));                    // (i j b): t(i j e b)
+  const Operand yB = operand(v, seg(w.fvv, 1, v, 0, v, 0, 1, v));                        // b: Fvv(b e)
+
+  fg::Ops ops{};
+  for (const Operand* p : {&wA, &tij, &gab, &eA, &eB, &cA, &gx, &dA, &xA, &xB, &v1A, &v1B, &o1A, &x2B, &r2B, &tab, &v2B,
+                           &v4B, &o2A, &o2B, &x3B, &ovA, &ooA, &v3A, &v3B, &o3A, &o3B, &yA, &y2A, &yB})
+    ops.o[ops.count++] = *p;
+  cudaError_t e = fg::row_scales(ops, st);
+  if (e != cudaSuccess) return e;
+
+  fg::Jobs js{};
+  auto add = [&](const Operand& a, const Operand& b, const Out& to) {
+    Job& j = js.j[js.count++];
+    j.a = a;
+    j.b = b;
+    j.out = to;
+  };
+  const Out vvvo_ae = out(V(14), v, n3, n2, o, n1, 1, 1);  // rows (a e), cols (b i) of W[A E B i]
+  add(wA, tij, out(w.wo, o, oo * o, o, o, oo, 1, 0));      // wo[k i l j], without its bare part
+  add(tij, gab, out(Z, 1, vv, 0, vv, 0, 1, 0));            // ladder
+  add(eA, eB, out(E, 1, ov, 0, ov, 0, 1, 0));
+  add(cA, gx, out(C, 1, ov, 0, ov, 0, 1, 0));
+  add(dA, gx, out(D, 1, ov, 0, ov, 0, 1, 0));
+  add(xA, xB, out(X, v, ovv, v, v, vv, 1, 0));             // (i a)(j b)
+  add(v1A, v1B, vvvo_ae);
+  add(o1A, tij, out(V(2), v, n3, n1, o, n2, 1, 1));        // W[m i B j]: (m b)(i j)
+  e = fg::run(js, st);
+  if (e != cudaSuccess) return e;
+
+  ops.count = 0;
+  for (const Operand* p : {&x2A, &r2A, &x3A}) ops.o[ops.count++] = *p;
+  e = fg::row_scales(ops, st);
+  if (e != cudaSuccess) return e;
+  js.count = 0;
+  add(x2A, x2B, out(X, v, vv, v, v, ovv, 1, 1));           // (j a)(i b)
+  add(r2A, r2B, out(Z, 1, vv, 0, vv, 0, 1, 1));
+  add(tab, v2B, out(V(14), v, n3, n1, o, n2, 1, 1));       // W[A E B i]: (a b)(e i)
+  add(tab, v4B, out(V(15), v, n3, n1, v, n2, 1, 1));       // W[A E B F]: (a b)(e f)
+  add(o2A, o2B, out(V(2), o, n3, n2, o, n1, 1, 1));        // W[m i B j]: (m i)(b j)
+  e = fg::run(js, st);
+  if (e != cudaSuccess) return e;
+
+  js.count = 0;
+  add(x3A, x3B, out(X, v, ovv, v, v, vv, 1, 1));
+  Out to = out(V(6), v, n3, n2, v, 1, n1, 1);              // W[m E B j]: (m e)(j b), and W[B j m E]
+  to.q = V(9);
+  to.qr1 = n1, to.qr2 = 1, to.qc1 = n2, to.qc2 = n3;
+  add(ovA, x3B, to);
+  to = out(V(3), v, n3, 1, v, n2, n1, 1);                  // W[i j A B]: (i b)(j a), and W[A B i j]
+  to.q = V(12);
+  to.qr1 = n1, to.qr2 = n2, to.qc1 = 1, to.qc2 = n3;
+  add(ooA, ooB, to);
+  add(v3A, v3B, out(V(14), v, n2, n1, o, n3, 1, 1));       // W[A E B i]: (e b)(a i)
+  add(o3A, o3B, out(V(2), o, n3, 1, o, n1, n2, 1));        // W[m i B j]: (m j)(b i)
+  add(yA, yB, out(Y, 1, v, 0, v, 0, 1, 0));                // into D's place, read by the second launch
+  add(y2A, yB, out(Z, v, vv, 1, v, 0, v, 1));              // (i j b)(a)
+  return fg::run(js, st);
+}
+
+// FP64: the blocks' last terms (the O(o) and O(v) Fock sums), the residual's pair transpose and the
+// mirrored blocks.
+__global__ void k_fin_fixed(double* __restrict__ W, double* __restrict__ F, const double* __restrict__ t2, const double* __restrict__ foo,
+                            const double* __restrict__ fvv, const double* __restrict__ r1, const double* __restrict__ wo,
+                            const double* __restrict__ X, const double* __restrict__ Y, const double* __restrict__ Z,
+                            Dims d) {
+  const int o = d.o, v = d.v, vv = v * v, oo = o * o;
+  const size_t n_r2 = (size_t)oo * vv, n_vvvo = (size_t)vv * v * o, n_oovo = (size_t)oo * v * o, n_wo = (size_t)oo * oo;
+  size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (x < n_vvvo) {  // W[A E B i] -= sum_m f~_me t_mi^ab, and W[B i A E]
+    const int i = (int)(x % o), b = (int)((x / o) % v), e = (int)((x / ((size_t)v * o)) % v), a = (int)(x / ((size_t)vv * o));
+    double s0 = 0.0, s1 = 0.0;
+    int m = 0;
+    for (; m + 1 < o; m += 2) {
+      s0 += F[m * d.n + o + e] * t2[ti(d, m, i, a, b)];
+      s1 += F[(m + 1) * d.n + o + e] * t2[ti(d, m + 1, i, a, b)];
+    }
+    if (m < o) s0 += F[m * d.n + o + e] * t2[ti(d, m, i, a, b)];
+    const size_t p = gi(d, o + a, o + e, o + b, i);
+    const double w = W[p] - (s0 + s1);
+    W[p] = w;
+    W[gi(d, o + b, i, o + a, o + e)] = w;
+    return;
+  }
+  x -= n_vvvo;
+  if (x < n_r2) {
+    const int b = (int)(x % v), a = (int)((x / v) % v), j = (int)((x / vv) % o), i = (int)(x / ((size_t)vv * o));
+    const size_t xt = ti(d, j, i, b, a);
+    double s0 = X[x] + X[xt], s1 = Y[x];
+    for (int m = 0; m < o; ++m) {
+      s0 -= foo[m * o + j] * t2[ti(d, i, m, a, b)];
+      s1 -= foo[m * o + i] * t2[ti(d, m, j, a, b)];
+    }
+    W[gi(d, o + a, i, o + b, j)] += (s0 + s1) + Z[x];
+    return;
+  }
+  x -= n_r2;
+  if (x < n_oovo) {  // W[m i B j] += sum_e f~_me t_ij^eb, and W[B j m i]
+    const int j = (int)(x % o), b = (int)((x / o) % v), i = (int)((x / ((size_t)v * o)) % o), m = (int)(x / ((size_t)v * oo));
+    double s0 = 0.0, s1 = 0.0;
+    int e = 0;
+    for (; e + 1 < v; e += 2) {
+      s0 += F[m * d.n + o + e] * t2[ti(d, i, j, e, b)];
+      s1 += F[m * d.n + o + e + 1] * t2[ti(d, i, j, e + 1, b)];
+    }
+    if (e < v) s0 += F[m * d.n + o + e] * t2[ti(d, i, j, e, b)];
+    const size_t p = gi(d, m, i, o + b, j);
+    const double w = W[p] + (s0 + s1);
+    W[p] = w;
+    W[gi(d, o + b, j, m, i)] = w;
+    return;
+  }
+  x -= n_oovo;
+  if (x < n_wo) {
+    const int y = (int)x, k = y / (oo * o), i = (y / oo) % o, l = (y / o) % o, j = y % o;
+    W[gi(d, k, i, l, j)] += wo[y];
+    return;
+  }
+  x -= n_wo;
+  if (x < (size_t)oo) {
+    F[(x / o) * d.n + x % o] = foo[x];
+  } else if (x < (size_t)oo + vv) {
+    const int y = (int)x - oo;
+    F[(o + y / v) * d.n + o + y % v] = fvv[y];
+  } else if (x < (size_t)oo + vv + v * o) {
+    const int y = (int)x - oo - vv;
+    F[(o + y / o) * d.n + y % o] = r1[y];
+  }
+}
 
 // ---- mixed precision: the T2 contractions as tensor-core GEMMs ----------------------------
 // Every contraction below is a GEMM over index pairs, D[(r1 r2)][(c1 c2)] = sum_k A(r, k) B(c, k),
@@ -1642,12 +1670,12 @@ cudaError_t launch_dress(const double* h, const double* eri, const double* t1, c
   k_energy_part<<<EGRID, TPB, 0, st>>>(w.ht, W, t2, w.epart, d);
   k_energy_sum<<<1, EGRID, 0, st>>>(w.epart, e0);
   if (v > 0 && o > 0) {
-    // U lives in the r2 slot until the doubles residual is written there
-    k_make_u<<<blocks_for(o * o * v * v), TPB, 0, st>>>(t2, w.r2, d);
-    // the mixed path forms Woooo (a W block) on the tensor cores with its other T2 terms; the
-    // Fock-like blocks stay FP64 sums
-    const unsigned nsb = (unsigned)(o * o + v * v + v * o + (g32 ? 0 : o * o * o * o));
-    k_small_blocks<<<nsb, TPB, 0, st>>>(F, W, w.r2, t2, w.foo, w.fvv, w.r1, w.wo, d);
+    // mixed: u lives in the r2 slot until the doubles residual is written there
+    double* U = mixed ? w.r2 : w.t2f;
+    k_make_u<<<blocks_for(o * o * v * v), TPB, 0, st>>>(t2, U, d);
+    // the Fock-like blocks are FP64 sums in both paths
+    const unsigned nsb = (unsigned)(o * o + v * v + v * o);
+    k_small_blocks<<<nsb, TPB, 0, st>>>(F, W, U, w.foo, w.fvv, w.r1, d);
     if (g32) {  // contractions of the T2 terms in FP32 (mixed precision), bases kept in FP64
       float* t2f = reinterpret_cast<float*>(w.t2f);
       const unsigned gg = blocks_for(n4) > 152u * 64u ? 152u * 64u : blocks_for(n4);
@@ -1656,11 +1684,14 @@ cudaError_t launch_dress(const double* h, const double* eri, const double* t1, c
       Arena ar{w.arena};
       cudaError_t e = t2_terms_tc(d, W, g32, F, t2f, w, e0, ar, st, ladder_bn > 0 ? ladder_bn : kLadderDefault);
       if (e != cudaSuccess) return e;
+      const size_t nf = o * o * v * v + o * o * o * o + o * o + v * v + v * o;
+      k_finalize<<<blocks_for(nf), TPB, 0, st>>>(W, F, w.foo, w.fvv, w.r1, w.wo, w.r2, d);
     } else {
-      t2_terms<double>(d, W, W, F, t2, w, st);
+      const cudaError_t e = t2_terms_fixed(d, W, t2, U, w, st);
+      if (e != cudaSuccess) return e;
+      const size_t nf = v * v * v * o + o * o * v * v + o * o * v * o + o * o * o * o + o * o + v * v + v * o;
+      k_fin_fixed<<<blocks_for(nf), TPB, 0, st>>>(W, F, t2, w.foo, w.fvv, w.r1, w.wo, w.D, w.Cq, w.r2, d);
     }
-    const size_t nf = o * o * v * v + o * o * o * o + o * o + v * v + v * o;
-    k_finalize<<<blocks_for(nf), TPB, 0, st>>>(W, F, w.foo, w.fvv, w.r1, w.wo, w.r2, d);
   }
   return cudaGetLastError();
 }

@@ -1,0 +1,46 @@
+// Fixed-point arithmetic with FP64 accuracy on the integer pipe (GB300: 64 mad.wide per clock and
+// SM against 2 FP64 FMAs).  A number is an integer t times a power of two common to the sums it
+// takes part in, held in two limbs t = hi 2^27 + lo, |lo| <= 2^26.  A product of two numbers is
+// hi hi 2^54 + (hi lo + lo hi) 2^27, two exact 64-bit sums; lo lo is left out (at most 2^52).
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace qf {
+namespace {
+
+constexpr int kLimb = 27;  // bits of a low limb
+
+// round(v 2^(bits - sx)): v in units of 2^(sx - bits); |v| < 2^(sx + 62 - bits).  Subnormal v count
+// as zero.
+__device__ __forceinline__ long long to_fix(double v, int sx, int bits) {
+  const long long b = __double_as_longlong(v);
+  const int e = (int)((b >> 52) & 0x7ff);
+  if (e == 0) return 0;
+  const long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;
+  const int sh = e - 1075 + bits - sx;
+  long long t;
+  if (sh >= 0) {
+    t = m << (sh > 9 ? 9 : sh);
+  } else {
+    const int r = -sh;
+    t = r > 60 ? 0 : (m + (1ll << (r - 1))) >> r;
+  }
+  return b < 0 ? -t : t;
+}
+__device__ __forceinline__ int2 limbs(long long t) {
+  const long long hi = (t + (1ll << (kLimb - 1))) >> kLimb;
+  return make_int2((int)hi, (int)(t - (hi << kLimb)));
+}
+__device__ __forceinline__ long long unlimb(int2 w) { return ((long long)w.x << kLimb) + w.y; }
+__device__ __forceinline__ void madw(long long& s, int a, int b) { s += (long long)a * b; }
+// (high sum, cross sum) -> one sum in units of 2^54 products
+__device__ __forceinline__ long long join(long long hh, long long xx) {
+  return hh + ((xx + (1ll << (kLimb - 1))) >> kLimb);
+}
+// 2^e as a double, |e| < 1022
+__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+
+}  // namespace
+}  // namespace qf

@@ -33,6 +33,7 @@
 
 #include <utility>
 
+#include "fixed.cuh"
 #include "qflow_internal.h"
 
 namespace qf {
@@ -171,39 +172,7 @@ __device__ __forceinline__ const FTab<K>& ftab() {
   else return g_ftab3;
 }
 
-// ---- fixed-point numbers ------------------------------------------------------------------------
-
-constexpr int kLimb = 27;             // bits of a low limb
-constexpr int kFix = 2 * kLimb;       // a number is t 2^-54 of its scale
-
-// round(v 2^(54 - sx)) for |v| < 2^(sx + 2); subnormal v count as zero
-__device__ __forceinline__ long long to_fix(double v, int sx) {
-  const long long bits = __double_as_longlong(v);
-  const int e = (int)((bits >> 52) & 0x7ff);
-  if (e == 0) return 0;
-  const long long m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
-  const int sh = e - 1075 + kFix - sx;
-  long long t;
-  if (sh >= 0) {
-    t = m << (sh > 9 ? 9 : sh);
-  } else {
-    const int r = -sh;
-    t = r > 60 ? 0 : (m + (1ll << (r - 1))) >> r;
-  }
-  return bits < 0 ? -t : t;
-}
-__device__ __forceinline__ int2 limbs(long long t) {
-  const long long hi = (t + (1ll << (kLimb - 1))) >> kLimb;
-  return make_int2((int)hi, (int)(t - (hi << kLimb)));
-}
-__device__ __forceinline__ long long unlimb(int2 w) { return ((long long)w.x << kLimb) + w.y; }
-__device__ __forceinline__ void madw(long long& s, int a, int b) { s += (long long)a * b; }
-// (high sum, cross sum) -> t of the scale's 2^-54
-__device__ __forceinline__ long long join(long long hh, long long xx) {
-  return hh + ((xx + (1ll << (kLimb - 1))) >> kLimb);
-}
-// 2^e as a double, |e| < 1022
-__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+constexpr int kFix = 54;  // a number is t 2^-54 of its scale
 
 // 1 / x to about 2^-46: FP32 reciprocal and one Newton step (|x| within the FP32 range)
 __device__ __forceinline__ double recip(double x) {
@@ -665,7 +634,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
       if (x < C::NW) {
         const int pq = x / NF, rs = x % NF;
         const bool dd = (pq % (NORB + 1)) == 0 && (rs % (NORB + 1)) == 0;
-        sm.W[x] = dd ? make_int2(0, 0) : limbs(to_fix(w[i], sx));
+        sm.W[x] = dd ? make_int2(0, 0) : limbs(to_fix(w[i], sx, kFix));
       }
     }
     __syncthreads();
@@ -686,7 +655,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
       const int p = x / NORB, q = x % NORB;
       if (p != q) {
         if (!(fabs(sm.J[x] - sm.J[q * NORB + p]) <= 1e-13 * (fabs(sm.J[x]) + fabs(sm.J[q * NORB + p])) + 1e-300)) sm.flag[1] = 1;
-        long long v = to_fix(sm.F[x], sx);
+        long long v = to_fix(sm.F[x], sx, kFix);
 #pragma unroll
         for (int k = 0; k < K; ++k)
           v -= 2 * unlimb(sm.W[x * NF + k * NORB + k]) - unlimb(sm.W[(p * NORB + k) * NF + k * NORB + q]);
@@ -890,7 +859,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
       for (int r = 0; r < PER; ++r)
         if (pin[r]) {
           sm.V[k][tid + r * NT] = vk[r];
-          const int2 c = limbs(to_fix(vk[r], 0));
+          const int2 c = limbs(to_fix(vk[r], 0, kFix));
           sm.Cv[pia[r] * NS + pib[r]] = c;
           sm.Cv[pib[r] * NS + pia[r]] = c;
         }
