@@ -1007,11 +1007,11 @@ cudaError_t launch_solve_rescue(int k, const SolveArgs& a, int64_t* items, unsig
   return launch_fp64(k, b, st);
 }
 
-// The fixed-point form of the FP64 solver takes SES-CC spaces started from Phi.  Its rounding is
+// The fixed-point form of the FP64 solver takes spaces started from Phi (both forms).  Its rounding is
 // that of FP64 on O(1) quantities (about 1e-15), far below any tolerance it is used for; a
 // requested residual below 1e-12 stays with solve_kernel.
 static bool fixed_form(const SolveArgs& a) {
-  return !a.guess && !a.ducc_eri && !a.count_dev && a.tol >= 1e-12;
+  return !a.guess && !a.count_dev && a.tol >= 1e-12;
 }
 
 int solve_launch_count(int precision, const SolveArgs& a) {

@@ -31,6 +31,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <type_traits>
 #include <utility>
 
 #include "fixed.cuh"
@@ -187,11 +188,32 @@ __device__ __forceinline__ double rsqrt_nr(double x) {
   return fma(y, fma(-h * y, y, 0.5), y);
 }
 
+// DUCC form: integrals and amplitudes of the space while its internal part is formed.
 template <int K>
+struct DuccFix {
+  using C = FD<K>;
+  static constexpr int K2 = K * K, K4 = K2 * K2;
+  long long W[C::NW];    // G|_A, the internal part taken off
+  int2 g[C::NW];         // two-body elements of the operator (H_A, then B_A)
+  long long F[C::NF], f0[C::NF], Fx[C::NF];
+  int2 f[C::NF], h[C::NF];
+  int2 t1[K2], t2[K4], u[K4];
+  long long part[C::NWARP];
+};
+template <int K>
+struct DavVectors {
+  double V[FD<K>::KM][FD<K>::NP];   // subspace basis (orthonormal), pair values
+  double S[FD<K>::KM][FD<K>::NP];   // H applied to it
+};
+struct NoScratch {};
+
+template <int K, bool DUCC>
 struct FSmem {
   using C = FD<K>;
-  double V[C::KM][C::NP];   // subspace basis (orthonormal), pair values
-  double S[C::KM][C::NP];   // H applied to it
+  union {
+    DavVectors<K> v;
+    std::conditional_t<DUCC, DuccFix<K>, NoScratch> d;  // only before the first vector
+  };
   int2 W[C::NW];            // couplings W[pq][rs] in limbs, (pp|rr) zero
   int2 Hs[C::NDET];         // same-spin couplings, diagonal zero
   int2 Cv[C::NDET];         // the vector sigma is applied to
@@ -207,15 +229,15 @@ struct FSmem {
   double out[C::NWARP][16];
   double theta;
   unsigned off2[2][C::NF];
-  unsigned imax[C::NWARP];
+  unsigned imax[2][C::NWARP];
   int orb[8];
   int flag[2];
 };
 
 // sums of v[0..m) (M = 8 or 16 padded) over the block; every thread reads out[warp][j].
 // In the warp: halves are exchanged, so a value costs about two additions instead of five.
-template <int K, int M>
-__device__ __forceinline__ const double* sum_many(FSmem<K>& sm, double (&v)[M], int m, int& buf) {
+template <int K, bool DUCC, int M>
+__device__ __forceinline__ const double* sum_many(FSmem<K, DUCC>& sm, double (&v)[M], int m, int& buf) {
   using C = FD<K>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int len = M;
@@ -307,8 +329,8 @@ __device__ __forceinline__ void apply_row(long long (&hh)[FD<K>::NS], long long 
 }
 
 // Off-diagonal part of H C in fixed point: B[I][J] + A[I][J] + A[J][I].
-template <int K>
-__device__ __noinline__ void sigma_fixed(FSmem<K>& sm, const unsigned (&rep)[FD<K>::UPT], int row, int part, int mrow) {
+template <int K, bool DUCC>
+__device__ __noinline__ void sigma_fixed(FSmem<K, DUCC>& sm, const unsigned (&rep)[FD<K>::UPT], int row, int part, int mrow) {
   using C = FD<K>;
   constexpr int NS = C::NS;
   {
@@ -390,8 +412,12 @@ __device__ __noinline__ void sigma_fixed(FSmem<K>& sm, const unsigned (&rep)[FD<
 // with the FP32 inverse of (G22 - theta0) corrected to first order in theta - theta0; f and w in
 // FP64.  solve.cu takes the eigenvalue nearest to theta0 - 1e-2: returns false (then that solver
 // decides) unless the rest of the spectrum is clearly farther from it than the found root, the root
-// is dominated by its first coefficient and the iteration settled.
-__device__ __forceinline__ bool newton_root(const double* G, int ld, int kk, double theta0, double* y, double* theta) {
+// is dominated by its first coefficient and the iteration settled.  SYM (DUCC form): of the
+// symmetrised matrix, the eigenvector with the largest Phi weight, which a vector with more than
+// half of the weight is (v0: the basis vectors' Phi coefficients, ld0 apart).
+template <bool SYM>
+__device__ __forceinline__ bool newton_root(const double* G, int ld, int kk, double theta0, double* y, double* theta,
+                                            const double* v0, int ld0) {
   const unsigned full = 0xffffffffu;
   const int r = threadIdx.x & 31, rr = r & 7;
   const bool in = rr < kk;
@@ -399,8 +425,8 @@ __device__ __forceinline__ bool newton_root(const double* G, int ld, int kk, dou
   float gf[8], a[8], g0[8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    g[c] = (in && c < kk) ? G[rr * ld + c] : 0.0;
-    g0[c] = (c < kk) ? (float)G[c] : 0.f;
+    g[c] = (in && c < kk) ? (SYM ? 0.5 * (G[rr * ld + c] + G[c * ld + rr]) : G[rr * ld + c]) : 0.0;
+    g0[c] = (c < kk) ? (SYM ? (float)(0.5 * (G[c] + G[c * ld])) : (float)G[c]) : 0.f;
     gf[c] = (float)g[c];
     a[c] = (in && c < kk) ? gf[c] : 0.f;
     if (c == rr) a[c] = in ? (float)(g[c] - theta0) : 1.f;
@@ -506,21 +532,480 @@ __device__ __forceinline__ bool newton_root(const double* G, int ld, int kk, dou
     if (c < kk) row = fma(g[c], wc, row);
   }
   th = __shfl_sync(full, row, 0);
-  const float gap = nrm * fabsf((float)(th - theta0 + 1e-2));
-  ok = ok && settled && gap < 0.35f && n2 < 1.5 && y0 > 0.5;
-  ok = __all_sync(full, ok);
+  ok = ok && settled && n2 < 1.5 && y0 > 0.5;
   const double inv = rsqrt_nr(n2);
+  if constexpr (SYM) {
+    const double v = in ? v0[rr * ld0] : 0.0;
+    double c = w * inv * v, q = v * v;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      c += __shfl_xor_sync(full, c, o);
+      q += __shfl_xor_sync(full, q, o);
+    }
+    ok = ok && c * c > 0.55 * q;
+  } else {
+    ok = ok && nrm * fabsf((float)(th - theta0 + 1e-2)) < 0.35f;
+  }
+  ok = __all_sync(full, ok);
   if (r < kk) y[r] = w * inv;
   *theta = th;
   return ok;
 }
 
+// ---- the space's integrals ------------------------------------------------------------------------
+
+__device__ __forceinline__ unsigned mag_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+
+// block maximum of the high words of magnitudes (one barrier; slot alternates between calls)
+template <int K, bool DUCC>
+__device__ __forceinline__ unsigned block_max(FSmem<K, DUCC>& sm, unsigned mx, int slot) {
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0) sm.imax[slot][threadIdx.x >> 5] = mx;
+  __syncthreads();
+#pragma unroll
+  for (int v = 0; v < FD<K>::NWARP; ++v) mx = max(mx, sm.imax[slot][v]);
+  return mx;
+}
+// exponent s with |x| < 2^s for the largest magnitude's high word (0 where there is none)
+__device__ __forceinline__ int scale_of(unsigned mx) {
+  const int e = (int)(mx >> 20);
+  return e > 0 ? e - 1022 : 0;
+}
+constexpr unsigned kInfHi = 0x7ff00000u;
+
+// SES-CC: W limbs (relative to the largest element that is not (pp|rr)), J, X and the F block.
+// False (in some thread): an element is not finite or the scale is out of range.
 template <int K>
+__device__ __forceinline__ bool gather_block(FSmem<K, false>& sm, const SolveArgs& a, int& sx) {
+  using C = FD<K>;
+  constexpr int NF = C::NF, NORB = C::NORB, NT = C::NT;
+  const int tid = threadIdx.x;
+  double w[C::NG];
+  unsigned mx = 0, all = 0;
+#pragma unroll
+  for (int i = 0; i < C::NG; ++i) {
+    const int x = tid + i * NT;
+    w[i] = 0.0;
+    if (x < C::NW) w[i] = a.W[sm.off2[0][x / NF] + sm.off2[1][x % NF]];
+  }
+  for (int x = tid; x < NF; x += NT) {
+    const double f = a.F[(unsigned)sm.orb[x / NORB] * (unsigned)a.n + (unsigned)sm.orb[x % NORB]];
+    sm.F[x] = f;
+    all = max(all, mag_hi(f));
+    if (x / NORB != x % NORB) mx = max(mx, mag_hi(f));
+  }
+#pragma unroll
+  for (int i = 0; i < C::NG; ++i) {
+    const int x = tid + i * NT;
+    if (x < C::NW) {
+      const int pq = x / NF, rs = x % NF;
+      const int p = pq / NORB, q = pq % NORB, r = rs / NORB, t = rs % NORB;
+      const unsigned hi = mag_hi(w[i]);
+      all = max(all, hi);
+      if (p == q && r == t) sm.J[p * NORB + r] = w[i];
+      else mx = max(mx, hi);
+      if (p == t && q == r) sm.X[p * NORB + q] = w[i];
+    }
+  }
+  sx = scale_of(block_max(sm, mx, 0));
+#pragma unroll
+  for (int i = 0; i < C::NG; ++i) {
+    const int x = tid + i * NT;
+    if (x < C::NW) {
+      const int pq = x / NF, rs = x % NF;
+      const bool dd = (pq % (NORB + 1)) == 0 && (rs % (NORB + 1)) == 0;
+      sm.W[x] = dd ? make_int2(0, 0) : limbs(to_fix(w[i], sx, kFix));
+    }
+  }
+  return all < kInfHi && sx > -900 && sx < 900;
+}
+
+// Sum of products of limbs.
+struct Acc {
+  long long hh = 0, xx = 0;
+  __device__ __forceinline__ void add(int2 a, int2 b) {
+    madw(hh, a.x, b.x);
+    madw(xx, a.x, b.y);
+    madw(xx, a.y, b.x);
+  }
+  __device__ __forceinline__ void sub(int2 a, int2 b) { add(make_int2(-a.x, -a.y), b); }
+  __device__ __forceinline__ long long value() const { return join(hh, xx); }
+};
+// t 2^-s, rounded (s > 0), or t 2^|s|, which has to fit
+__device__ __forceinline__ long long shift_fix(long long t, int s) {
+  if (s <= 0) return t << -s;
+  return s > 62 ? 0 : (t + (1ll << (s - 1))) >> s;
+}
+
+// DUCC form, [O, T]_(<=2) on the space's orbitals (solve.cu, LinDress: the same terms): T1
+// linearisation (creators by -K, annihilators by +K) plus the connected T2-linear terms.  In units
+// of O's times t's.  Local orbitals: 0..K-1 occupied, K..2K-1 virtual.
+template <int K>
+struct LinFix {
+  static constexpr int NO = 2 * K;
+  const DuccFix<K>& d;
+  __device__ __forceinline__ int2 g(int p, int q, int r, int s) const { return d.g[((p * NO + q) * NO + r) * NO + s]; }
+  __device__ __forceinline__ int2 t(int i, int j, int a, int b) const { return d.t2[((i * K + j) * K + a) * K + b]; }
+  __device__ __forceinline__ int2 u(int i, int j, int a, int b) const { return d.u[((i * K + j) * K + a) * K + b]; }
+  __device__ __forceinline__ int2 f(int p, int q) const { return d.f[p * NO + q]; }
+  __device__ __forceinline__ void dg(Acc& v, int p, int q, int r, int s) const {
+#pragma unroll
+    for (int x = 0; x < K; ++x) {
+      if (p >= K) v.sub(d.t1[x * K + p - K], g(x, q, r, s));
+      if (q < K) v.add(g(p, K + x, r, s), d.t1[q * K + x]);
+      if (r >= K) v.sub(d.t1[x * K + r - K], g(p, q, x, s));
+      if (s < K) v.add(g(p, q, r, K + x), d.t1[s * K + x]);
+    }
+  }
+  __device__ __forceinline__ void dh(Acc& v, int p, int q) const {
+#pragma unroll
+    for (int x = 0; x < K; ++x) {
+      if (q < K) v.add(d.h[p * NO + K + x], d.t1[q * K + x]);
+      if (p >= K) v.sub(d.t1[x * K + p - K], d.h[x * NO + q]);
+    }
+  }
+  // blk: bit 8, 4, 2, 1 set where p, q, r, s is virtual (uniform over most warps)
+  __device__ __forceinline__ void w2(Acc& v, int blk, int p, int q, int r, int s) const {
+    switch (blk) {
+      case 0x0:
+        for (int e = 0; e < K; ++e)
+#pragma unroll
+          for (int ff = 0; ff < K; ++ff) v.add(g(p, K + e, r, K + ff), t(q, s, e, ff));
+        break;
+      case 0xF:
+        for (int m = 0; m < K; ++m)
+#pragma unroll
+          for (int nn = 0; nn < K; ++nn) v.add(g(m, q, nn, s), t(m, nn, p - K, r - K));
+        break;
+      case 0x6:
+      case 0x9: {
+        const int m = (blk == 0x6) ? p : r, e = (blk == 0x6) ? q : s, b = (blk == 0x6) ? r : p, j = (blk == 0x6) ? s : q;
+        for (int nn = 0; nn < K; ++nn)
+#pragma unroll
+          for (int ff = 0; ff < K; ++ff) {
+            v.add(g(m, e, nn, K + ff), u(j, nn, b - K, ff));
+            v.sub(g(m, K + ff, nn, e), t(j, nn, b - K, ff));
+          }
+        break;
+      }
+      case 0x3:
+      case 0xC: {
+        const int i = (blk == 0x3) ? p : r, j = (blk == 0x3) ? q : s, a = (blk == 0x3) ? r : p, b = (blk == 0x3) ? s : q;
+        for (int ff = 0; ff < K; ++ff)
+#pragma unroll
+          for (int nn = 0; nn < K; ++nn) v.sub(g(i, K + ff, nn, b), t(j, nn, ff, a - K));
+        break;
+      }
+      case 0x2:
+      case 0x8: {
+        const int m = (blk == 0x2) ? p : r, i = (blk == 0x2) ? q : s, b = (blk == 0x2) ? r : p, j = (blk == 0x2) ? s : q;
+        for (int e = 0; e < K; ++e) {
+          v.add(f(m, K + e), t(i, j, e, b - K));
+#pragma unroll
+          for (int ff = 0; ff < K; ++ff) v.add(g(m, K + e, b, K + ff), t(i, j, e, ff));
+#pragma unroll
+          for (int nn = 0; nn < K; ++nn) {
+            v.add(g(m, i, nn, K + e), u(j, nn, b - K, e));
+            v.sub(g(m, K + e, nn, i), t(j, nn, b - K, e));
+            v.sub(g(m, K + e, nn, j), t(i, nn, e, b - K));
+          }
+        }
+        break;
+      }
+      case 0xE:
+      case 0xB: {
+        const int a = (blk == 0xE) ? p : r, e = (blk == 0xE) ? q : s, b = (blk == 0xE) ? r : p, i = (blk == 0xE) ? s : q;
+        for (int m = 0; m < K; ++m) {
+          v.sub(f(m, e), t(m, i, a - K, b - K));
+#pragma unroll
+          for (int nn = 0; nn < K; ++nn) v.add(g(m, e, nn, i), t(m, nn, a - K, b - K));
+#pragma unroll
+          for (int ff = 0; ff < K; ++ff) {
+            v.add(g(m, K + ff, a, e), u(m, i, ff, b - K));
+            v.sub(g(m, e, b, K + ff), t(m, i, a - K, ff));
+            v.sub(g(m, e, a, K + ff), t(m, i, ff, b - K));
+          }
+        }
+        break;
+      }
+      case 0xA: {
+        const int a = p - K, i = q, b = r - K, j = s;
+        for (int e = 0; e < K; ++e) {
+          v.add(f(K + b, K + e), t(i, j, a, e));
+          v.add(f(K + a, K + e), t(i, j, e, b));
+#pragma unroll
+          for (int ff = 0; ff < K; ++ff) v.add(g(K + a, K + e, K + b, K + ff), t(i, j, e, ff));
+        }
+        for (int m = 0; m < K; ++m) {
+          v.sub(f(m, j), t(i, m, a, b));
+          v.sub(f(m, i), t(m, j, a, b));
+#pragma unroll
+          for (int nn = 0; nn < K; ++nn) v.add(g(m, i, nn, j), t(m, nn, a, b));
+#pragma unroll
+          for (int e = 0; e < K; ++e) {
+            v.add(g(m, K + e, K + b, j), u(i, m, a, e));
+            v.sub(g(m, j, K + b, K + e), t(i, m, a, e));
+            v.sub(g(m, i, K + b, K + e), t(j, m, e, a));
+            v.sub(g(m, j, K + a, K + e), t(i, m, e, b));
+            v.add(g(m, K + e, K + a, i), u(j, m, b, e));
+            v.sub(g(m, i, K + a, K + e), t(j, m, b, e));
+          }
+        }
+        break;
+      }
+      default:
+        break;  // ooov, ovoo, ovov, ovvv, vvov: no T2-linear term
+    }
+  }
+  __device__ __forceinline__ void f2(Acc& v, int p, int q) const {
+    if (p < K && q < K) {
+      for (int nn = 0; nn < K; ++nn)
+        for (int e = 0; e < K; ++e)
+#pragma unroll
+          for (int ff = 0; ff < K; ++ff) v.add(g(p, K + e, nn, K + ff), u(q, nn, e, ff));
+    } else if (p >= K && q >= K) {
+      for (int m = 0; m < K; ++m)
+        for (int nn = 0; nn < K; ++nn)
+#pragma unroll
+          for (int ff = 0; ff < K; ++ff) v.sub(g(m, q, nn, K + ff), u(m, nn, p - K, ff));
+    } else if (p >= K && q < K) {
+      const int a = p - K, i = q;
+      for (int m = 0; m < K; ++m)
+        for (int e = 0; e < K; ++e) {
+          v.add(f(m, K + e), u(i, m, a, e));
+#pragma unroll
+          for (int ff = 0; ff < K; ++ff) v.add(g(p, K + e, m, K + ff), u(i, m, e, ff));
+#pragma unroll
+          for (int nn = 0; nn < K; ++nn) v.sub(g(m, i, nn, K + e), u(m, nn, a, e));
+        }
+    }
+  }
+};
+
+// Takes c ([O, T] + its transpose) off W and F and 2 c [O, T]'s scalar off e0, O in d.g, d.h, d.f in
+// units of 2^(so - 54), t in units of 2^(st - 54), W and F in units of 2^(S - 54); half: c = 1/2.
+template <int K>
+__device__ __forceinline__ void lin_fixed(FSmem<K, true>& sm, int so, int st, int S, int half, double& e0) {
+  using C = FD<K>;
+  constexpr int NO = C::NORB, NT = C::NT, K4 = DuccFix<K>::K4;
+  DuccFix<K>& d = sm.d;
+  const LinFix<K> L{d};
+  long long* Wx = reinterpret_cast<long long*>(sm.W);
+  const int tid = threadIdx.x;
+  // elements block by block (16 o / v blocks of K^4), so that a warp takes one branch of w2
+  for (int x = tid; x < C::NW; x += NT) {
+    const int blk = x / K4, y = x % K4;
+    const int p = y / (K * K * K) + (blk & 8 ? K : 0), q = (y / (K * K)) % K + (blk & 4 ? K : 0);
+    const int r = (y / K) % K + (blk & 2 ? K : 0), s = y % K + (blk & 1 ? K : 0);
+    Acc v;
+    L.dg(v, p, q, r, s);
+    L.w2(v, blk, p, q, r, s);
+    Wx[((p * NO + q) * NO + r) * NO + s] = v.value();
+  }
+  for (int x = tid; x < C::NF; x += NT) {
+    const int p = x / NO, q = x % NO;
+    Acc v, w;
+    L.dh(v, p, q);
+    L.f2(v, p, q);
+    for (int k = 0; k < K; ++k) {
+      L.dg(w, p, q, k, k);
+      L.dg(w, p, q, k, k);
+      Acc x2;
+      L.dg(x2, p, k, k, q);
+      w.hh -= x2.hh;
+      w.xx -= x2.xx;
+    }
+    d.Fx[x] = v.value() + w.value();
+  }
+  Acc e;
+  for (int x = tid; x < K4; x += NT) {
+    const int i = x / (K * K * K), j = (x / K) % K, aa = (x / (K * K)) % K, b = x % K;  // (i a j b)
+    e.add(L.g(i, K + aa, j, K + b), L.u(i, j, aa, b));
+  }
+  for (int x = tid; x < K * K; x += NT) {
+    const int k = x / K, l = x % K;
+    Acc y, z;
+    L.dg(y, k, k, l, l);
+    L.dg(z, k, l, l, k);
+    if (k == l) L.dh(y, k, k);
+    e.hh += 2 * y.hh - z.hh;
+    e.xx += 2 * y.xx - z.xx;
+  }
+  long long ex = e.value();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ex += __shfl_xor_sync(0xffffffffu, ex, o);
+  if ((tid & 31) == 0) d.part[tid >> 5] = ex;
+  __syncthreads();
+  ex = 0;
+#pragma unroll
+  for (int v = 0; v < C::NWARP; ++v) ex += d.part[v];
+  e0 -= (half ? 1.0 : 2.0) * ((double)ex * pow2(so + st - kFix));
+  const int sh = S - so - st + half;
+  for (int x = tid; x < C::NW; x += NT) {
+    const int p = x / (NO * NO * NO), q = (x / (NO * NO)) % NO, r = (x / NO) % NO, s = x % NO;
+    d.W[x] -= shift_fix(Wx[x] + Wx[((q * NO + p) * NO + s) * NO + r], sh);
+  }
+  for (int x = tid; x < C::NF; x += NT) d.F[x] -= shift_fix(d.Fx[x] + d.Fx[(x % NO) * NO + x / NO], sh);
+  __syncthreads();
+}
+
+// DUCC form: G|_A minus the space's internal part L_A = X_A + X_A^+ + 1/2 (Y_A + Y_A^+) (solve.cu,
+// ducc_local), all in fixed point: W limbs, J, X, F block as gather_block leaves them, and e0.
+template <int K>
+__device__ __noinline__ bool ducc_block(FSmem<K, true>& sm, const SolveArgs& a, double& e0, int& sx) {
+  using C = FD<K>;
+  constexpr int NF = C::NF, NO = C::NORB, NT = C::NT, K2 = K * K, K4 = K2 * K2;
+  DuccFix<K>& d = sm.d;
+  const int tid = threadIdx.x;
+  const unsigned n1 = (unsigned)a.n;
+  unsigned mx = 0, mt = 0;
+  {
+    double w[C::NG], g[C::NG];
+#pragma unroll
+    for (int i = 0; i < C::NG; ++i) {
+      const int x = tid + i * NT;
+      w[i] = g[i] = 0.0;
+      if (x < C::NW) {
+        const unsigned at = sm.off2[0][x / NF] + sm.off2[1][x % NF];
+        w[i] = a.W[at];
+        g[i] = a.ducc_eri[at];
+      }
+    }
+    double f[(NF + NT - 1) / NT], f0[(NF + NT - 1) / NT], t2[(K4 + NT - 1) / NT], t1 = 0.0;
+#pragma unroll
+    for (int i = 0; i < (NF + NT - 1) / NT; ++i) {
+      const int x = tid + i * NT;
+      f[i] = f0[i] = 0.0;
+      if (x < NF) {
+        const unsigned at = (unsigned)sm.orb[x / NO] * n1 + (unsigned)sm.orb[x % NO];
+        f[i] = a.F[at];
+        f0[i] = a.ducc_F0[at];
+      }
+      mx = max(mx, max(mag_hi(f[i]), mag_hi(f0[i])));
+    }
+#pragma unroll
+    for (int i = 0; i < (K4 + NT - 1) / NT; ++i) {
+      const int x = tid + i * NT;
+      t2[i] = 0.0;
+      if (x < K4) {
+        const int ii = x / (K * K2), j = (x / K2) % K, aa = (x / K) % K, b = x % K;
+        t2[i] = a.t2_old[(((size_t)sm.orb[ii] * a.nocc + sm.orb[j]) * a.nvir + (sm.orb[K + aa] - a.nocc)) * a.nvir +
+                         (sm.orb[K + b] - a.nocc)];
+      }
+      mt = max(mt, mag_hi(t2[i]));
+    }
+    if (tid < K2) t1 = a.t1_old[(size_t)sm.orb[tid / K] * a.nvir + (sm.orb[K + tid % K] - a.nocc)];
+    mt = max(mt, mag_hi(t1));
+#pragma unroll
+    for (int i = 0; i < C::NG; ++i) mx = max(mx, max(mag_hi(w[i]), mag_hi(g[i])));
+    mx = block_max(sm, mx, 0);
+    mt = block_max(sm, mt, 1);
+    const int S = scale_of(mx), st = scale_of(mt);
+#pragma unroll
+    for (int i = 0; i < C::NG; ++i) {
+      const int x = tid + i * NT;
+      if (x < C::NW) {
+        d.W[x] = to_fix(w[i], S, kFix);
+        d.g[x] = limbs(to_fix(g[i], S, kFix));
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < (NF + NT - 1) / NT; ++i) {
+      const int x = tid + i * NT;
+      if (x < NF) {
+        d.F[x] = to_fix(f[i], S, kFix);
+        d.f0[x] = to_fix(f0[i], S, kFix);
+        d.f[x] = limbs(d.f0[x]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < (K4 + NT - 1) / NT; ++i) {
+      const int x = tid + i * NT;
+      if (x < K4) d.t2[x] = limbs(to_fix(t2[i], st, kFix));
+    }
+    if (tid < K2) d.t1[tid] = limbs(to_fix(t1, st, kFix));
+  }
+  // uniform: both maxima are the block's.  An amplitude of 1 or more leaves the range in which the
+  // sums below cannot overflow (up to 100 products of 2^54, with t below 1)
+  const int S = scale_of(mx), st = scale_of(mt);
+  if (mx >= kInfHi || mt >= kInfHi || S < -400 || S > 400 || st > 0 || st < -400) return false;
+  __syncthreads();
+  for (int x = tid; x < K4; x += NT) {
+    const int i = x / (K * K2), j = (x / K2) % K, aa = (x / K) % K, b = x % K;
+    const int2 p = d.t2[x], q = d.t2[((i * K + j) * K + b) * K + aa];
+    d.u[x] = make_int2(2 * p.x - q.x, 2 * p.y - q.y);
+  }
+  // X_A: H_A in vacuum order on the space
+  for (int x = tid; x < NF; x += NT) {
+    const int p = x / NO, q = x % NO;
+    long long v = d.f0[x];
+    for (int k = 0; k < K; ++k)
+      v -= 2 * unlimb(d.g[((p * NO + q) * NO + k) * NO + k]) - unlimb(d.g[((p * NO + k) * NO + k) * NO + q]);
+    d.h[x] = limbs(v);
+  }
+  __syncthreads();
+  lin_fixed(sm, S, st, S, 0, e0);
+  // Y_A: B_A = D.T_A + (D.T_A)^+, D from the Fock diagonal; in units of 2^(S + st + 4 - 54), which
+  // leaves the four orbital energies of D their room
+  auto eps = [&](int p) { return d.f0[p * NO + p]; };
+  for (int x = tid; x < C::NW; x += NT) {
+    const int p = x / (NO * NO * NO), q = (x / (NO * NO)) % NO, r = (x / NO) % NO, s = x % NO;
+    Acc v;
+    if (p >= K && q < K && r >= K && s < K)
+      v.add(limbs(eps(p) + eps(r) - eps(q) - eps(s)), d.t2[((q * K + s) * K + (p - K)) * K + (r - K)]);
+    else if (p < K && q >= K && r < K && s >= K)
+      v.add(limbs(eps(q) + eps(s) - eps(p) - eps(r)), d.t2[((p * K + r) * K + (q - K)) * K + (s - K)]);
+    d.g[x] = limbs(shift_fix(v.value(), 4));
+  }
+  for (int x = tid; x < NF; x += NT) {
+    const int p = x / NO, q = x % NO;
+    Acc v;
+    if (p >= K && q < K) v.add(limbs(eps(p) - eps(q)), d.t1[q * K + (p - K)]);
+    if (p < K && q >= K) v.add(limbs(eps(q) - eps(p)), d.t1[p * K + (q - K)]);
+    d.h[x] = limbs(shift_fix(v.value(), 4));
+  }
+  __syncthreads();
+  for (int x = tid; x < NF; x += NT) {  // normal order
+    const int p = x / NO, q = x % NO;
+    long long v = unlimb(d.h[x]);
+    for (int k = 0; k < K; ++k)
+      v += 2 * unlimb(d.g[((p * NO + q) * NO + k) * NO + k]) - unlimb(d.g[((p * NO + k) * NO + k) * NO + q]);
+    d.f[x] = limbs(v);
+  }
+  __syncthreads();
+  lin_fixed(sm, S + st + 4, st, S, 1, e0);
+  // W limbs relative to the largest element that is not (pp|rr)
+  const double unit = pow2(S - kFix);
+  long long big = 0;
+  for (int x = tid; x < C::NW; x += NT) {
+    const int pq = x / NF, rs = x % NF, p = pq / NO, q = pq % NO, r = rs / NO, t = rs % NO;
+    const long long v = d.W[x];
+    if (p == q && r == t) sm.J[p * NO + r] = (double)v * unit;
+    else big |= v < 0 ? ~v : v;
+    if (p == t && q == r) sm.X[p * NO + q] = (double)v * unit;
+  }
+  for (int x = tid; x < NF; x += NT) {
+    sm.F[x] = (double)d.F[x] * unit;
+    if (x / NO != x % NO) big |= d.F[x] < 0 ? ~d.F[x] : d.F[x];
+  }
+  const int lead = (int)block_max(sm, (unsigned)(64 - __clzll(big)), 0);  // |v| < 2^lead
+  const int up = lead > 0 ? kFix - lead : 0;                             // left shift to 54 bits
+  sx = S - up;
+  for (int x = tid; x < C::NW; x += NT) {
+    const int pq = x / NF, rs = x % NF;
+    const bool dd = (pq % (NO + 1)) == 0 && (rs % (NO + 1)) == 0;
+    const long long v = d.W[x];
+    sm.W[x] = dd ? make_int2(0, 0) : limbs(up >= 0 ? v << up : shift_fix(v, -up));
+  }
+  return true;
+}
+
+template <int K, bool DUCC>
 __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
   using C = FD<K>;
   constexpr int NS = C::NS, NORB = C::NORB, NF = C::NF, NT = C::NT, PER = C::PER;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  FSmem<K>& sm = *reinterpret_cast<FSmem<K>*>(smem_raw);
+  FSmem<K, DUCC>& sm = *reinterpret_cast<FSmem<K, DUCC>*>(smem_raw);
   const FTab<K>& tab = ftab<K>();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned n1 = (unsigned)a.n, n2 = n1 * n1, n3 = n2 * n1;
@@ -586,59 +1071,16 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
       const unsigned p = (unsigned)sm.orb[x / NORB], q = (unsigned)sm.orb[x % NORB];
       sm.off2[0][x] = p * n3 + q * n2;
       sm.off2[1][x] = p * n1 + q;
-      sm.F[x] = a.F[p * n1 + q];
     }
     __syncthreads();
-    double w[C::NG];
-    unsigned mx = 0;
-    bool fin = true;
-#pragma unroll
-    for (int i = 0; i < C::NG; ++i) {
-      const int x = tid + i * NT;
-      w[i] = 0.0;
-      if (x < C::NW) w[i] = a.W[sm.off2[0][x / NF] + sm.off2[1][x % NF]];
-    }
-#pragma unroll
-    for (int i = 0; i < C::NG; ++i) {
-      const int x = tid + i * NT;
-      if (x < C::NW) {
-        const int pq = x / NF, rs = x % NF;
-        const int p = pq / NORB, q = pq % NORB, r = rs / NORB, t = rs % NORB;
-        const unsigned hi = (unsigned)__double2hiint(w[i]) & 0x7fffffffu;
-        fin = fin && hi < 0x7ff00000u;
-        if (p == q && r == t) sm.J[p * NORB + r] = w[i];
-        else mx = max(mx, hi);
-        if (p == t && q == r) sm.X[p * NORB + q] = w[i];
-      }
-    }
-    for (int x = tid; x < NF; x += NT) {
-      const unsigned hi = (unsigned)__double2hiint(sm.F[x]) & 0x7fffffffu;
-      fin = fin && hi < 0x7ff00000u;
-      if (x / NORB != x % NORB) mx = max(mx, hi);
-    }
-    const double e0 = *a.e0;
-    fin = fin && isfinite(e0);
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    if (lane == 0) sm.imax[warp] = mx;
+    double e0 = *a.e0;
+    int sx = 0;
+    bool fin = isfinite(e0);
+    if constexpr (DUCC) fin = ducc_block(sm, a, e0, sx) && fin;
+    else fin = gather_block(sm, a, sx) && fin;
     if (!fin) sm.flag[1] = 1;
     __syncthreads();
-#pragma unroll
-    for (int v = 0; v < C::NWARP; ++v) mx = max(mx, sm.imax[v]);
-    // couplings are below 2^sx; a block without couplings (or only denormal ones) keeps sx = 0
-    const int ebits = (int)(mx >> 20);
-    const int sx = ebits > 0 ? ebits - 1022 : 0;
-    if (sx < -900 || sx > 900) fin = false;
-#pragma unroll
-    for (int i = 0; i < C::NG; ++i) {
-      const int x = tid + i * NT;
-      if (x < C::NW) {
-        const int pq = x / NF, rs = x % NF;
-        const bool dd = (pq % (NORB + 1)) == 0 && (rs % (NORB + 1)) == 0;
-        sm.W[x] = dd ? make_int2(0, 0) : limbs(to_fix(w[i], sx, kFix));
-      }
-    }
-    __syncthreads();
-    if (sm.flag[1] || !fin) {  // uniform: flag[1] is shared, sx is the same in every thread
+    if (sm.flag[1]) {
       if (tid == 0) a.status[oidx] = kSpaceDefer;
       __syncthreads();
       continue;
@@ -756,8 +1198,8 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
             double xv = 0.0, sv = 0.0;
             if (pin[r])
               for (int j = 0; j < C::KM; ++j) {
-                xv = fma(sm.y[j], sm.V[j][d], xv);
-                sv = fma(sm.y[j], sm.S[j][d], sv);
+                xv = fma(sm.y[j], sm.v.V[j][d], xv);
+                sv = fma(sm.y[j], sm.v.S[j][d], sv);
               }
             const double wt = pia[r] == pib[r] ? 1.0 : 2.0;
             xs[r] = xv;
@@ -765,14 +1207,14 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
             part2[0] = fma(wt * xv, xv, part2[0]);
             part2[1] = fma(wt * xv, sv, part2[1]);
           }
-          const double* o = sum_many<K, 8>(sm, part2, 2, buf);
+          const double* o = sum_many(sm, part2, 2, buf);
           const double inv = rsqrt_nr(o[0]);
           const double g00 = o[1] / o[0];
 #pragma unroll
           for (int r = 0; r < PER; ++r)
             if (pin[r]) {
-              sm.V[0][tid + r * NT] = xs[r] * inv;
-              sm.S[0][tid + r * NT] = ss[r] * inv;
+              sm.v.V[0][tid + r * NT] = xs[r] * inv;
+              sm.v.S[0][tid + r * NT] = ss[r] * inv;
             }
           __syncthreads();
           if (tid == 0) {
@@ -793,8 +1235,8 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
           double xv = 0.0, sv = 0.0;
           if (pin[r])
             for (int j = 0; j < k; ++j) {
-              xv = fma(sm.y[j], sm.V[j][d], xv);
-              sv = fma(sm.y[j], sm.S[j][d], sv);
+              xv = fma(sm.y[j], sm.v.V[j][d], xv);
+              sv = fma(sm.y[j], sm.v.S[j][d], sv);
             }
           const double res = fma(-th, xv, sv);
           const double wt = pia[r] == pib[r] ? 1.0 : 2.0;
@@ -804,7 +1246,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
           vk[r] = pin[r] ? res * recip(den) : 0.0;
           p1[1] = fma(wt * vk[r], vk[r], p1[1]);
         }
-        const double* o = sum_many<K, 8>(sm, p1, 2, buf);
+        const double* o = sum_many(sm, p1, 2, buf);
         const double rn2 = o[0], tt = o[1];
         if (!isfinite(rn2) || !isfinite(th)) {
           defer = true;
@@ -827,9 +1269,9 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
             if (pin[r])
 #pragma unroll
               for (int j = 0; j < C::KM - 1; ++j)
-                if (j < k) p2[j] = fma(sm.V[j][tid + r * NT], tw, p2[j]);
+                if (j < k) p2[j] = fma(sm.v.V[j][tid + r * NT], tw, p2[j]);
           }
-          const double* q = sum_many<K, 8>(sm, p2, k, buf);
+          const double* q = sum_many(sm, p2, k, buf);
           double p3[8];
 #pragma unroll
           for (int j = 0; j < 8; ++j) p3[j] = 0.0;
@@ -837,12 +1279,12 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
           for (int r = 0; r < PER; ++r) {
             double v = vk[r];
             if (pin[r])
-              for (int j = 0; j < k; ++j) v = fma(-q[j], sm.V[j][tid + r * NT], v);
+              for (int j = 0; j < k; ++j) v = fma(-q[j], sm.v.V[j][tid + r * NT], v);
             vk[r] = v;
             p3[0] = fma(pia[r] == pib[r] ? v : 2.0 * v, v, p3[0]);
           }
           const double prev = vn2;
-          vn2 = sum_many<K, 8>(sm, p3, 1, buf)[0];
+          vn2 = sum_many(sm, p3, 1, buf)[0];
           if (vn2 > 0.01 * prev) break;
         }
         if (!(vn2 > 1e-26)) {  // subspace cannot grow (complete or stagnated)
@@ -858,13 +1300,13 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
 #pragma unroll
       for (int r = 0; r < PER; ++r)
         if (pin[r]) {
-          sm.V[k][tid + r * NT] = vk[r];
+          sm.v.V[k][tid + r * NT] = vk[r];
           const int2 c = limbs(to_fix(vk[r], 0, kFix));
           sm.Cv[pia[r] * NS + pib[r]] = c;
           sm.Cv[pib[r] * NS + pia[r]] = c;
         }
       __syncthreads();
-      sigma_fixed<K>(sm, rep, row, part, mrow);
+      sigma_fixed(sm, rep, row, part, mrow);
       double p4[16];
 #pragma unroll
       for (int j = 0; j < 16; ++j) p4[j] = 0.0;
@@ -874,19 +1316,19 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
           const int d = tid + r * NT, ij = pia[r] * NS + pib[r], ji = pib[r] * NS + pia[r];
           const long long t = sm.B[ij] + sm.A[ij] + sm.A[ji];
           const double sk = fma(scale, (double)t, diag[r] * vk[r]);
-          sm.S[k][d] = sk;
+          sm.v.S[k][d] = sk;
           const double wt = pia[r] == pib[r] ? 1.0 : 2.0;
           const double ws = wt * sk, wv = wt * vk[r];
 #pragma unroll
           for (int j = 0; j < C::KM; ++j) {
             if (j < k) {
-              p4[j] = fma(sm.V[j][d], ws, p4[j]);            // G[j][k]
-              p4[8 + j] = fma(sm.S[j][d], wv, p4[8 + j]);    // G[k][j]
+              p4[j] = fma(sm.v.V[j][d], ws, p4[j]);            // G[j][k]
+              p4[8 + j] = fma(sm.v.S[j][d], wv, p4[8 + j]);    // G[k][j]
             }
             if (j == k) p4[j] = fma(vk[r], ws, p4[j]);
           }
         }
-      const double* o = sum_many<K, 16>(sm, p4, 16, buf);
+      const double* o = sum_many(sm, p4, 16, buf);
       if (warp == 0) {
         if (lane <= k) sm.G[lane * C::KM + k] = o[lane];
         if (lane < k) sm.G[k * C::KM + lane] = o[8 + lane];
@@ -898,7 +1340,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
           }
         } else {
           double thn = th;
-          const bool ok = newton_root(sm.G, C::KM, k + 1, th, sm.y, &thn);
+          const bool ok = newton_root<DUCC>(sm.G, C::KM, k + 1, th, sm.y, &thn, &sm.v.V[0][0], C::NP);
           if (lane == 0) {
             sm.theta = thn;
             if (!ok) sm.flag[1] = 1;
@@ -929,12 +1371,12 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
     for (int r = 0; r < PER; ++r)
       if (pin[r]) {
         double xv = 0.0;
-        for (int j = 0; j < k; ++j) xv = fma(sm.y[j], sm.V[j][tid + r * NT], xv);
+        for (int j = 0; j < k; ++j) xv = fma(sm.y[j], sm.v.V[j][tid + r * NT], xv);
         xf[pia[r] * NS + pib[r]] = xv;
         xf[pib[r] * NS + pia[r]] = xv;
         p5[0] = fma(pia[r] == pib[r] ? xv : 2.0 * xv, xv, p5[0]);
       }
-    const double xn2 = sum_many<K, 8>(sm, p5, 1, buf)[0];  // its barrier orders xf
+    const double xn2 = sum_many(sm, p5, 1, buf)[0];  // its barrier orders xf
     const double c0 = xf[0];
     if (st == kSpaceOk && !(c0 * c0 >= 1e-6 * xn2)) st = kSpaceRoot;
     if (!isfinite(c0) || !isfinite(th)) st = kSpaceNonFinite;
@@ -958,7 +1400,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
         for (int x = tid; x < K * K; x += NT) {
           const int i = x / K, aa = x % K;
           const size_t g = (size_t)sm.orb[i] * a.nvir + (sm.orb[K + aa] - a.nocc);
-          if (a.owner1[g] == sidx) a.t1_new[g] = a.t1_old[g] + x1(i, aa);
+          if (a.owner1[g] == sidx) a.t1_new[g] = (DUCC ? 0.0 : a.t1_old[g]) + x1(i, aa);  // DUCC: replaced
         }
       if (a.owner2)
         for (int x = tid; x < K * K * K * K; x += NT) {
@@ -968,7 +1410,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
           if (a.owner2[g] == sidx) {
             int sa, sb;
             const int ja = single(i, aa, &sa), jb = single(j, b, &sb);
-            a.t2_new[g] = a.t2_old[g] + ((double)(sa * sb) * xf[ja * NS + jb] * inv0 - x1(i, aa) * x1(j, b));
+            a.t2_new[g] = (DUCC ? 0.0 : a.t2_old[g]) + ((double)(sa * sb) * xf[ja * NS + jb] * inv0 - x1(i, aa) * x1(j, b));
           }
         }
     }
@@ -981,31 +1423,33 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
   }
 }
 
-template <int K>
+template <int K, bool DUCC>
 cudaError_t launch_fixed_k(const SolveArgs& a, cudaStream_t st) {
   if (a.nspaces <= 0) return cudaSuccess;
-  const size_t smem = sizeof(FSmem<K>);
-  cudaError_t e = cudaFuncSetAttribute(solve_fixed_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const size_t smem = sizeof(FSmem<K, DUCC>);
+  cudaError_t e =
+      cudaFuncSetAttribute(solve_fixed_kernel<K, DUCC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solve_fixed_kernel<K>, FD<K>::NT, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solve_fixed_kernel<K, DUCC>, FD<K>::NT, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) per_sm = 1;
   int64_t grid = (int64_t)sms * per_sm;
   if (grid > a.nspaces) grid = a.nspaces;
-  solve_fixed_kernel<K><<<(unsigned)grid, FD<K>::NT, smem, st>>>(a);
+  solve_fixed_kernel<K, DUCC><<<(unsigned)grid, FD<K>::NT, smem, st>>>(a);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_solve_fixed(int k, const SolveArgs& a, cudaStream_t st) {
+  const bool ducc = a.ducc_eri != nullptr && a.ducc_F0 != nullptr;
   switch (k) {
-    case 1: return launch_fixed_k<1>(a, st);
-    case 2: return launch_fixed_k<2>(a, st);
-    case 3: return launch_fixed_k<3>(a, st);
+    case 1: return ducc ? launch_fixed_k<1, true>(a, st) : launch_fixed_k<1, false>(a, st);
+    case 2: return ducc ? launch_fixed_k<2, true>(a, st) : launch_fixed_k<2, false>(a, st);
+    case 3: return ducc ? launch_fixed_k<3, true>(a, st) : launch_fixed_k<3, false>(a, st);
     default: return cudaErrorInvalidValue;
   }
 }
