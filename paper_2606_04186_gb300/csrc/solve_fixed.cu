@@ -69,7 +69,6 @@ struct FD {
   static constexpr int RPW = NS / NWARP;               // strings per warp
   static constexpr int NRS = NORB * (NORB - 1);        // (r, s), r != s
   static constexpr int NB = choose_c(NORB - 2, K - 1);  // strings each E_rs reaches
-  static constexpr int RA = (K == 3) ? 2 : 1, RB = (K == 3) ? 4 : (K == 2) ? 2 : 1;  // same-spin tile
   static constexpr int NG = (NW + NT - 1) / NT;        // gathered elements per thread
 };
 
@@ -85,6 +84,7 @@ struct FTab {
   int jb[C::NRS][C::NB] = {};
   int sg[C::NRS][C::NB] = {};
   unsigned rep[C::NS][C::NU] = {};    // per string: pq | J << 8 | (sign < 0) << 16
+  unsigned ex[C::NS] = {};            // <i| a+_r a_s |string 0>: rs | (sign < 0) << 16 | 1 << 17, else 0
   unsigned hs[C::NDET] = {};          // same-spin element kinds, see make_ftab
 };
 
@@ -128,6 +128,7 @@ constexpr FTab<K> make_ftab() {
         const int m1 = mi & ~(1 << p), mj = m1 | (1 << q);  // <i| a+_p a_q |j>
         const int neg = parity_below(mj, q) ^ parity_below(m1, p);
         t.rep[i][u++] = (unsigned)(p * C::NORB + q) | ((unsigned)t.idx[mj] << 8) | ((unsigned)neg << 16);
+        if (t.idx[mj] == 0) t.ex[i] = (unsigned)(p * C::NORB + q) | ((unsigned)neg << 16) | (1u << 17);
       }
   }
   // same-spin couplings <i|.|j>, i != j (Slater-Condon): bits 0-1 replacements (0: no coupling),
@@ -175,17 +176,27 @@ __device__ __forceinline__ const FTab<K>& ftab() {
 
 constexpr int kFix = 54;  // a number is t 2^-54 of its scale
 
-// 1 / x to about 2^-46: FP32 reciprocal and one Newton step (|x| within the FP32 range)
+// binary64 <-> binary32 by field arithmetic (a conversion holds the FP64 pipe, 64 cycles a warp): the
+// float is cut off after its 23 bits; for |x| in the normal FP32 range
+__device__ __forceinline__ float cut_float(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  return __uint_as_float((hi & 0x80000000u) | (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29));
+}
+__device__ __forceinline__ double wide(float x) {
+  const unsigned u = __float_as_uint(x);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+// 1 / x to about 2^-44: FP32 reciprocal and one Newton step (|x| well inside the FP32 range)
 __device__ __forceinline__ double recip(double x) {
-  const double y = (double)__frcp_rn((float)x);
+  const double y = wide(__frcp_rn(cut_float(x)));
   return fma(fma(-x, y, 1.0), y, y);
 }
-// 1 / sqrt(x) to FP64 rounding: FP32 estimate and two Newton steps (x within the FP32 range)
+// 1 / sqrt(x) to FP64 rounding: FP32 estimate y and one third-order step, with e = 1 - x y^2
+// y (1 + e / 2 + 3 e^2 / 8) (x within the FP32 range)
 __device__ __forceinline__ double rsqrt_nr(double x) {
-  double y = (double)rsqrtf((float)x);
-  const double h = 0.5 * x;
-  y = fma(y, fma(-h * y, y, 0.5), y);
-  return fma(y, fma(-h * y, y, 0.5), y);
+  const double y = wide(rsqrtf(cut_float(x)));
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // DUCC form: integrals and amplitudes of the space while its internal part is formed.
@@ -202,7 +213,7 @@ struct DuccFix {
 };
 template <int K>
 struct DavVectors {
-  double V[FD<K>::KM][FD<K>::NP];   // subspace basis (orthonormal), pair values
+  double V[FD<K>::KM][FD<K>::NP];   // subspace basis (orthonormal): pair values, times sqrt 2 for I < J
   double S[FD<K>::KM][FD<K>::NP];   // H applied to it
 };
 struct NoScratch {};
@@ -215,12 +226,12 @@ struct FSmem {
     std::conditional_t<DUCC, DuccFix<K>, NoScratch> d;  // only before the first vector
   };
   int2 W[C::NW];            // couplings W[pq][rs] in limbs, (pp|rr) zero
-  int2 Hs[C::NDET];         // same-spin couplings, diagonal zero
+  int2 Hs[C::NDET];         // same-spin couplings <I|.|L> at [L][I], diagonal zero
   int2 Cv[C::NDET];         // the vector sigma is applied to
-  long long A[C::NDET];     // parts of sigma that enter with their transpose
-  long long B[C::NDET];     // the other part
+  long long T[C::NDET];     // sigma's sums before they are made symmetric
   long long hfix[C::NF];    // folded one-body couplings
   double F[C::NF], J[C::NF], X[C::NF];  // F block, (pp|rr), (pr|rp)
+  double hd[C::NORB];       // folded one-body diagonal
   double hsd[C::NS];        // same-spin diagonal
   double JR[C::NS * C::NORB];  // sum of J over a string's orbitals
   double G[C::KM * C::KM];
@@ -276,132 +287,102 @@ __device__ __forceinline__ const double* sum_many(FSmem<K, DUCC>& sm, double (&v
 
 // ---- sigma ----------------------------------------------------------------------------------------
 
-template <int K, int RS, int M>
+// One replacement (r, s): the strings it reaches, as three runs of independent sums (the two cross
+// products of a string apart from each other, since they add to the same sum).
+template <int K, int RS, int M, int PART>
 __device__ __forceinline__ void rep_term(long long (&hh)[FD<K>::NS], long long (&xx)[FD<K>::NS], int2 w, int2 nw,
                                          const int (&ch)[FD<K>::NS], const int (&cl)[FD<K>::NS]) {
   constexpr int ib = FHold<K>::value.ib[RS][M], jb = FHold<K>::value.jb[RS][M];
-  if constexpr (FHold<K>::value.sg[RS][M] > 0) {
-    madw(hh[ib], w.x, ch[jb]);
-    madw(xx[ib], w.x, cl[jb]);
-    madw(xx[ib], w.y, ch[jb]);
-  } else {
-    madw(hh[ib], nw.x, ch[jb]);
-    madw(xx[ib], nw.x, cl[jb]);
-    madw(xx[ib], nw.y, ch[jb]);
-  }
+  constexpr bool plus = FHold<K>::value.sg[RS][M] > 0;
+  const int2 x = plus ? w : nw;
+  if constexpr (PART == 0) madw(hh[ib], x.x, ch[jb]);
+  else if constexpr (PART == 1) madw(xx[ib], x.x, cl[jb]);
+  else madw(xx[ib], x.y, ch[jb]);
 }
-template <int K, bool JROW, int RS, int... M>
-__device__ __forceinline__ void rep_rs(long long (&hh)[FD<K>::NS], long long (&xx)[FD<K>::NS],
-                                       const int2* (&row)[K], const int (&ch)[FD<K>::NS],
-                                       const int (&cl)[FD<K>::NS], std::integer_sequence<int, M...>) {
-  constexpr int rs = FHold<K>::value.rs[RS];
-  int2 w = row[0][rs];
-  if constexpr (JROW) {
-#pragma unroll
-    for (int i = 1; i < K; ++i) {
-      const int2 x = row[i][rs];
-      w.x += x.x;
-      w.y += x.y;
-    }
-  }
+template <int K, int RS, int... M>
+__device__ __forceinline__ void rep_rs(long long (&hh)[FD<K>::NS], long long (&xx)[FD<K>::NS], int2 w,
+                                       const int (&ch)[FD<K>::NS], const int (&cl)[FD<K>::NS],
+                                       std::integer_sequence<int, M...>) {
   const int2 nw = make_int2(-w.x, -w.y);
-  (rep_term<K, RS, M>(hh, xx, w, nw, ch, cl), ...);
+  (rep_term<K, RS, M, 0>(hh, xx, w, nw, ch, cl), ...);
+  (rep_term<K, RS, M, 1>(hh, xx, w, nw, ch, cl), ...);
+  (rep_term<K, RS, M, 2>(hh, xx, w, nw, ch, cl), ...);
 }
-template <int K, bool JROW, int... RS>
-__device__ __forceinline__ void rep_all(long long (&hh)[FD<K>::NS], long long (&xx)[FD<K>::NS],
-                                        const int2* (&row)[K], const int (&ch)[FD<K>::NS],
-                                        const int (&cl)[FD<K>::NS], std::integer_sequence<int, RS...>) {
-  (rep_rs<K, JROW, RS>(hh, xx, row, ch, cl, std::make_integer_sequence<int, FD<K>::NB>{}), ...);
-}
-// hh, xx [ib] += sum over beta replacements (r, s, jb) of w[rs] C[row][jb]; w = one row of W, or the
-// sum of the rows (pp|..) of a string's orbitals (JROW); sgn = 0 or -1 (the alpha sign)
-template <int K, bool JROW>
-__device__ __forceinline__ void apply_row(long long (&hh)[FD<K>::NS], long long (&xx)[FD<K>::NS],
-                                          const int2* (&row)[K], const int2* c, int sgn) {
-  int ch[FD<K>::NS], cl[FD<K>::NS];
-#pragma unroll
-  for (int j = 0; j < FD<K>::NS; ++j) {
-    const int2 x = c[j];
-    ch[j] = (x.x ^ sgn) - sgn;
-    cl[j] = (x.y ^ sgn) - sgn;
+template <int K, int RS>
+using RsOf = std::integral_constant<int, FHold<K>::value.rs[RS]>;
+// NORB - 1 replacements at a time, the next ones' couplings loaded ahead
+template <int K, int R, int... S>
+__device__ __forceinline__ void rep_group(long long (&hh)[FD<K>::NS], long long (&xx)[FD<K>::NS],
+                                          int2 (&w)[FD<K>::NORB - 1], const int2* row, const int (&ch)[FD<K>::NS],
+                                          const int (&cl)[FD<K>::NS], std::integer_sequence<int, S...>) {
+  constexpr int G = FD<K>::NORB - 1;
+  int2 next[G];
+  if constexpr (R + 1 < FD<K>::NORB) {
+    ((next[S] = row[RsOf<K, (R + 1 < FD<K>::NORB ? R + 1 : R) * G + S>::value]), ...);
   }
-  rep_all<K, JROW>(hh, xx, row, ch, cl, std::make_integer_sequence<int, FD<K>::NRS>{});
+  (rep_rs<K, R * G + S>(hh, xx, w[S], ch, cl, std::make_integer_sequence<int, FD<K>::NB>{}), ...);
+  if constexpr (R + 1 < FD<K>::NORB) {
+    ((w[S] = next[S]), ...);
+  }
+}
+template <int K, int... R, int... S>
+__device__ __forceinline__ void rep_all(long long (&hh)[FD<K>::NS], long long (&xx)[FD<K>::NS], const int2* row,
+                                        const int (&ch)[FD<K>::NS], const int (&cl)[FD<K>::NS],
+                                        std::integer_sequence<int, R...>, std::integer_sequence<int, S...> g) {
+  int2 w[FD<K>::NORB - 1];
+  ((w[S] = row[RsOf<K, S>::value]), ...);
+  (rep_group<K, R>(hh, xx, w, row, ch, cl, g), ...);
 }
 
-// Off-diagonal part of H C in fixed point: B[I][J] + A[I][J] + A[J][I].
+// Off-diagonal part of H C in fixed point, T with (T[I][J] + T[J][I]) / 2 = sigma[I][J].  A thread sums
+// for its alpha string I (row): its replacements I -> J with every beta replacement (symmetric in
+// itself), and, doubled since their transposes are not formed, the couplings of one of I's orbitals
+// with every beta replacement (W[pp][rs]) and its share of the same-spin part sum_L Hs[J][L] C[I][L].
 template <int K, bool DUCC>
-__device__ __noinline__ void sigma_fixed(FSmem<K, DUCC>& sm, const unsigned (&rep)[FD<K>::UPT], int row, int part, int mrow) {
+__device__ __forceinline__ void sigma_fixed(FSmem<K, DUCC>& sm, const unsigned (&rep)[FD<K>::UPT], unsigned own, int row,
+                                            int part) {
   using C = FD<K>;
   constexpr int NS = C::NS;
-  {
-    long long hh[NS], xx[NS];
+  long long hh[NS], xx[NS];
 #pragma unroll
-    for (int j = 0; j < NS; ++j) hh[j] = xx[j] = 0;
+  for (int j = 0; j < NS; ++j) hh[j] = xx[j] = 0;
 #pragma unroll 1
-    for (int u = 0; u < C::UPT; ++u) {
-      const unsigned e = u == 0 ? rep[0] : u == 1 ? rep[C::UPT > 1 ? 1 : 0] : rep[C::UPT - 1];
-      const int2* rows[K];
-#pragma unroll
-      for (int i = 0; i < K; ++i) rows[i] = sm.W + (e & 63u) * C::NF;
-      apply_row<K, false>(hh, xx, rows, sm.Cv + ((e >> 8) & 31u) * NS, -(int)((e >> 16) & 1u));
-    }
+  for (int u = 0; u <= C::UPT; ++u) {
+    const unsigned e = u == C::UPT ? own : u == 0 ? rep[0] : u == 1 ? rep[C::UPT > 1 ? 1 : 0] : rep[C::UPT - 1];
+    const int sgn = -(int)((e >> 16) & 1u), mul = (int)(e >> 17);  // 1; 2 for the string's own orbital, 0: none left
+    const int2* c = sm.Cv + ((e >> 8) & 31u) * NS;
+    int ch[NS], cl[NS];
 #pragma unroll
     for (int j = 0; j < NS; ++j) {
-      long long t = join(hh[j], xx[j]);
-      long long s = t;
+      const int2 x = c[j];
+      ch[j] = ((x.x ^ sgn) - sgn) * mul;
+      cl[j] = ((x.y ^ sgn) - sgn) * mul;
+    }
+    rep_all<K>(hh, xx, sm.W + (e & 63u) * C::NF, ch, cl, std::make_integer_sequence<int, C::NORB>{},
+               std::make_integer_sequence<int, C::NORB - 1>{});
+  }
+  if (part < C::TPR) {
+#pragma unroll 1
+    for (int l = part; l < NS; l += C::TPR) {
+      const int2 c = sm.Cv[row * NS + l];
+      const int c2 = 2 * c.x, d2 = 2 * c.y;
+      const int2* h = sm.Hs + l * NS;  // the transpose: Hs[J][l] over J
 #pragma unroll
-      for (int d = 1; d < C::TPR; ++d) s += __shfl_down_sync(0xffffffffu, t, d);
-      if (part == 0) sm.B[row * NS + j] = s;
+      for (int j = 0; j < NS; ++j) madw(hh[j], h[j].x, c2);
+#pragma unroll
+      for (int j = 0; j < NS; ++j) madw(xx[j], h[j].x, d2);
+#pragma unroll
+      for (int j = 0; j < NS; ++j) madw(xx[j], h[j].y, c2);
     }
   }
-  if (part == 0) {  // alpha occupations with beta replacements
-    long long hh[NS], xx[NS];
 #pragma unroll
-    for (int j = 0; j < NS; ++j) hh[j] = xx[j] = 0;
-    const int2* rows[K];
-    int m = mrow;
+  for (int j = 0; j < NS; ++j) {
+    const long long t = join(hh[j], xx[j]);
+    long long s = t;
 #pragma unroll
-    for (int i = 0; i < K; ++i) {
-      const int p = __ffs(m) - 1;
-      m &= m - 1;
-      rows[i] = sm.W + (p * C::NORB + p) * C::NF;
-    }
-    apply_row<K, true>(hh, xx, rows, sm.Cv + row * NS, 0);
-#pragma unroll
-    for (int j = 0; j < NS; ++j) sm.A[row * NS + j] = join(hh[j], xx[j]);
+    for (int d = 1; d < C::TPR; ++d) s += __shfl_down_sync(0xffffffffu, t, d);
+    if (part == 0) sm.T[row * NS + j] = s;
   }
-  __syncthreads();
-  // same-spin part: A[I][J] += sum_L Hs[J][L] C[I][L], an RA x RB tile per thread
-  constexpr int TB = NS / C::RB, TILES = (NS / C::RA) * TB;
-  if ((int)threadIdx.x < TILES) {
-    const int i0 = ((int)threadIdx.x / TB) * C::RA, j0 = ((int)threadIdx.x % TB) * C::RB;
-    long long hh[C::RA][C::RB], xx[C::RA][C::RB];
-#pragma unroll
-    for (int i = 0; i < C::RA; ++i)
-#pragma unroll
-      for (int j = 0; j < C::RB; ++j) hh[i][j] = xx[i][j] = 0;
-#pragma unroll 4
-    for (int l = 0; l < NS; ++l) {
-      int2 c[C::RA], h[C::RB];
-#pragma unroll
-      for (int i = 0; i < C::RA; ++i) c[i] = sm.Cv[(i0 + i) * NS + l];
-#pragma unroll
-      for (int j = 0; j < C::RB; ++j) h[j] = sm.Hs[(j0 + j) * NS + l];
-#pragma unroll
-      for (int i = 0; i < C::RA; ++i)
-#pragma unroll
-        for (int j = 0; j < C::RB; ++j) {
-          madw(hh[i][j], h[j].x, c[i].x);
-          madw(xx[i][j], h[j].x, c[i].y);
-          madw(xx[i][j], h[j].y, c[i].x);
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < C::RA; ++i)
-#pragma unroll
-      for (int j = 0; j < C::RB; ++j) sm.A[(i0 + i) * NS + j0 + j] += join(hh[i][j], xx[i][j]);
-  }
-  __syncthreads();
 }
 
 // ---- projected problem ------------------------------------------------------------------------------
@@ -409,133 +390,118 @@ __device__ __noinline__ void sigma_fixed(FSmem<K, DUCC>& sm, const unsigned (&re
 // Eigenpair (theta, y) of the kk x kk matrix G that continues the previous one (y_prev with kk - 1
 // coefficients, theta0), one warp, lane r < 8 owning row r.  Newton's method on
 //   f_r(w) = sum_c G_rc w_c - theta w_r,  theta = sum_c G_0c w_c,  w_0 = 1,
-// with the FP32 inverse of (G22 - theta0) corrected to first order in theta - theta0; f and w in
-// FP64.  solve.cu takes the eigenvalue nearest to theta0 - 1e-2: returns false (then that solver
+// with an FP32 inverse of (G22 - theta) as preconditioner: FP32 steps to single precision, then FP64
+// residuals (two or three steps).  solve.cu takes the eigenvalue nearest to theta0 - 1e-2: returns false (then that solver
 // decides) unless the rest of the spectrum is clearly farther from it than the found root, the root
 // is dominated by its first coefficient and the iteration settled.  SYM (DUCC form): of the
 // symmetrised matrix, the eigenvector with the largest Phi weight, which a vector with more than
 // half of the weight is (v0: the basis vectors' Phi coefficients, ld0 apart).
+// Lane l holds columns 2 (l / 8) and 2 (l / 8) + 1 of row l % 8; a vector's element r is in the four
+// lanes of row r.
 template <bool SYM>
 __device__ __forceinline__ bool newton_root(const double* G, int ld, int kk, double theta0, double* y, double* theta,
                                             const double* v0, int ld0) {
   const unsigned full = 0xffffffffu;
-  const int r = threadIdx.x & 31, rr = r & 7;
-  const bool in = rr < kk;
-  double g[8];
-  float gf[8], a[8], g0[8];
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    g[c] = (in && c < kk) ? (SYM ? 0.5 * (G[rr * ld + c] + G[c * ld + rr]) : G[rr * ld + c]) : 0.0;
-    g0[c] = (c < kk) ? (SYM ? (float)(0.5 * (G[c] + G[c * ld])) : (float)G[c]) : 0.f;
-    gf[c] = (float)g[c];
-    a[c] = (in && c < kk) ? gf[c] : 0.f;
-    if (c == rr) a[c] = in ? (float)(g[c] - theta0) : 1.f;
+  const int lane = threadIdx.x & 31, r = lane & 7, c0 = (lane >> 3) * 2, c1 = c0 + 1;
+  const bool in = r < kk, low = in && r >= 1;
+  auto elem = [&](int i, int j) -> double {
+    if (!(i < kk && j < kk)) return 0.0;
+    return SYM ? 0.5 * (G[i * ld + j] + G[j * ld + i]) : G[i * ld + j];
+  };
+  const double ga = elem(r, c0), gb = elem(r, c1);
+  const float fa = (float)ga, fb = (float)gb;
+  float top;  // G_0r
+  {
+    const float u = __shfl_sync(full, fa, (r >> 1) * 8), v = __shfl_sync(full, fb, (r >> 1) * 8);
+    top = r & 1 ? v : u;
   }
   bool ok = true;
-  // in-place inverse of the block 1..kk-1, last index first (no pivoting: its diagonal dominates
-  // wherever this path is taken; checked through the result)
-#pragma unroll
-  for (int p = 7; p >= 1; --p) {
-    if (p >= kk) continue;
-    const float piv = __shfl_sync(full, a[p], p);
-    if (!(fabsf(piv) > 1e-6f)) ok = false;
-    const float inv = 1.f / piv;
-    const float f = a[p] * inv;
-#pragma unroll
-    for (int c = 1; c < 8; ++c) {
-      if (c == p) continue;
-      const float rp = __shfl_sync(full, a[c], p);
-      a[c] = (rr == p) ? rp * inv : fmaf(-f, rp, a[c]);
+  float ma = 0.f, mb = 0.f;
+  // (ma, mb) = the inverse of the block 1..kk-1 of G - t, in place, last index first (no pivoting: its
+  // diagonal dominates wherever this path is taken; checked through the result), zero elsewhere
+  auto invert = [&](float t) {
+    ma = fa - (r == c0 ? t : 0.f);
+    mb = fb - (r == c1 ? t : 0.f);
+#pragma unroll 1
+    for (int p = kk - 1; p >= 1; --p) {
+      const int col = (p >> 1) * 8;
+      const float src = p & 1 ? mb : ma;
+      const float piv = __shfl_sync(full, src, col + p), mine = __shfl_sync(full, src, col + r);
+      const float ra = __shfl_sync(full, ma, (lane & 24) + p), rb = __shfl_sync(full, mb, (lane & 24) + p);
+      if (!(fabsf(piv) > 1e-6f)) ok = false;
+      const float inv = __frcp_rn(piv), f = mine * inv;
+      ma = c0 == p ? (r == p ? inv : -f) : r == p ? ra * inv : fmaf(-f, ra, ma);
+      mb = c1 == p ? (r == p ? inv : -f) : r == p ? rb * inv : fmaf(-f, rb, mb);
     }
-    a[p] = (rr == p) ? inv : -f;
-  }
-  float nrm = 0.f;
-#pragma unroll
-  for (int c = 1; c < 8; ++c)
-    if (c < kk) nrm += fabsf(a[c]);
-  if (rr == 0 || !in) nrm = 0.f;
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) nrm = fmaxf(nrm, __shfl_xor_sync(full, nrm, o));
-  // z = M v over rows 1..kk-1; row 0 receives g_0 . v of the returned z through dot0
-  auto mul = [&](float v) {
-    float z = 0.f;
-#pragma unroll
-    for (int c = 1; c < 8; ++c) {
-      const float vc = __shfl_sync(full, v, c);
-      if (c < kk) z = fmaf(a[c], vc, z);
-    }
-    return (rr >= 1 && in) ? z : 0.f;
+    if (!low || c0 < 1 || c0 >= kk) ma = 0.f;
+    if (!low || c1 >= kk) mb = 0.f;
   };
-  auto dot0 = [&](float v) {
-    float z = 0.f;
+  auto across = [&](float z) {  // sum over the columns' lanes
+    z += __shfl_xor_sync(full, z, 8);
+    return z + __shfl_xor_sync(full, z, 16);
+  };
+  auto mul = [&](float a, float b, float v) {
+    const float va = __shfl_sync(full, v, c0), vb = __shfl_sync(full, v, c1);
+    return across(fmaf(a, va, b * vb));
+  };
+  auto sum8 = [&](float z) {
 #pragma unroll
-    for (int c = 1; c < 8; ++c) {
-      const float vc = __shfl_sync(full, v, c);
-      if (c < kk) z = fmaf(g0[c], vc, z);
-    }
+    for (int o = 4; o > 0; o >>= 1) z += __shfl_xor_sync(full, z, o);
     return z;
   };
   const double y0 = y[0];
-  double w = (rr == 0) ? 1.0 : (rr < kk - 1 ? y[rr] * recip(y0) : 0.0);
-  double th = theta0;
-  // FP32 steps to single precision, then FP64 residuals
-  {
-    float wf = (float)w;
-    const float t0 = (float)theta0;
-    for (int it = 0; it < 4; ++it) {
-      float row = 0.f;
+  float wf = r == 0 ? 1.f : (r < kk - 1 ? (float)y[r] * __frcp_rn((float)y0) : 0.f);
+  float tf = (float)theta0, nrm = 0.f, b = 0.f, den = 1.f;
+  // FP32: three steps with the inverse at theta0, then two with the inverse at the value they reach
+#pragma unroll 1
+  for (int it = 0; it < 5; ++it) {
+    if (it == 0 || it == 3) {
+      invert(tf);
+      b = mul(ma, mb, wf);  // M w, for the change of theta within a step
+      den = __frcp_rn(1.f - sum8(top * b));
+      if (it == 0) {
+        nrm = across(fabsf(ma) + fabsf(mb));
 #pragma unroll
-      for (int c = 0; c < 8; ++c) row = fmaf(gf[c], __shfl_sync(full, wf, c), row);
-      const float tf = __shfl_sync(full, row, 0);
-      const float res = (rr >= 1 && in) ? row - tf * wf : 0.f;
-      const float dt = tf - t0;
-      const float x1 = mul(-res), x2 = mul(x1), xa = fmaf(dt, x2, x1);
-      const float b1 = mul(rr >= 1 ? wf : 0.f), b2 = mul(b1), xb = fmaf(dt, b2, b1);
-      const float s = dot0(xa) / (1.f - dot0(xb));
-      if (rr >= 1 && in) wf += fmaf(xb, s, xa);
+        for (int o = 4; o > 0; o >>= 1) nrm = fmaxf(nrm, __shfl_xor_sync(full, nrm, o));
+      }
     }
-    w = (rr == 0) ? 1.0 : (double)wf;
+    const float row = mul(fa, fb, wf);
+    tf = __shfl_sync(full, row, 0);
+    const float res = low ? fmaf(tf, wf, -row) : 0.f;
+    const float x = mul(ma, mb, res);
+    const float s = sum8(top * x) * den;
+    wf += fmaf(b, s, x);  // rows without an unknown have x = b = 0
   }
-  const float wf = (float)w;
-  const float bq1 = mul(rr >= 1 ? wf : 0.f), bq2 = mul(bq1);
+  // FP64 residuals and iterate
+  double w = (double)wf, th = theta0;
   bool settled = false;
-  for (int it = 0; it < 8; ++it) {
-    double row = 0.0;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const double wc = __shfl_sync(full, w, c);
-      if (c < kk) row = fma(g[c], wc, row);
-    }
+#pragma unroll 1
+  for (int it = 0; it < 10 && !settled; ++it) {
+    const double wa = __shfl_sync(full, w, c0), wb = __shfl_sync(full, w, c1);
+    double row = fma(ga, wa, gb * wb);
+    row += __shfl_xor_sync(full, row, 8);
+    row += __shfl_xor_sync(full, row, 16);
     th = __shfl_sync(full, row, 0);
-    const float dt = (float)(th - theta0);
-    const float res = (rr >= 1 && in) ? (float)fma(-th, w, row) : 0.f;
-    const float x1 = mul(-res), x2 = mul(x1), xa = fmaf(dt, x2, x1);
-    const float xb = fmaf(dt, bq2, bq1);
-    const float s = dot0(xa) / (1.f - dot0(xb));
-    float d = (rr >= 1 && in) ? fmaf(xb, s, xa) : 0.f;
+    const float res = low ? (float)fma(th, w, -row) : 0.f;
+    const float x = mul(ma, mb, res);
+    const float s = sum8(top * x) * den;
+    float d = fmaf(b, s, x);
     w += (double)d;
+    th += (double)sum8(top * d);
     d = fabsf(d);
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) d = fmaxf(d, __shfl_xor_sync(full, d, o));
-    // the next correction is smaller by the error of the preconditioner
-    const float q = nrm * fabsf(dt), rho = fmaxf(q * q, 1e-6f);
-    settled = d * rho < 1e-16f;
-    if (settled || !(d < 1e30f)) break;
+    // the step's own error is 1e-5 of it at most (FP32 inverse at the FP32 root)
+    settled = d < 1e-11f;
+    if (!(d < 1e30f)) break;
   }
   double n2 = w * w;
 #pragma unroll
   for (int o = 4; o > 0; o >>= 1) n2 += __shfl_xor_sync(full, n2, o);
-  double row = 0.0;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const double wc = __shfl_sync(full, w, c);
-    if (c < kk) row = fma(g[c], wc, row);
-  }
-  th = __shfl_sync(full, row, 0);
   ok = ok && settled && n2 < 1.5 && y0 > 0.5;
   const double inv = rsqrt_nr(n2);
   if constexpr (SYM) {
-    const double v = in ? v0[rr * ld0] : 0.0;
+    const double v = in ? v0[r * ld0] : 0.0;
     double c = w * inv * v, q = v * v;
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) {
@@ -547,7 +513,7 @@ __device__ __forceinline__ bool newton_root(const double* G, int ld, int kk, dou
     ok = ok && nrm * fabsf((float)(th - theta0 + 1e-2)) < 0.35f;
   }
   ok = __all_sync(full, ok);
-  if (r < kk) y[r] = w * inv;
+  if (lane < kk) y[lane] = w * inv;
   *theta = th;
   return ok;
 }
@@ -573,49 +539,52 @@ __device__ __forceinline__ int scale_of(unsigned mx) {
 }
 constexpr unsigned kInfHi = 0x7ff00000u;
 
+__device__ __forceinline__ void copy8_async(double* dst, const double* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // SES-CC: W limbs (relative to the largest element that is not (pp|rr)), J, X and the F block.
-// False (in some thread): an element is not finite or the scale is out of range.
+// False (in some thread): an element is not finite or the scale is out of range.  The elements come
+// by asynchronous copies (all of them in flight) and are converted in rolled loops: the kernel's
+// code has to stay within the instruction cache.
 template <int K>
 __device__ __forceinline__ bool gather_block(FSmem<K, false>& sm, const SolveArgs& a, int& sx) {
   using C = FD<K>;
   constexpr int NF = C::NF, NORB = C::NORB, NT = C::NT;
   const int tid = threadIdx.x;
-  double w[C::NG];
+  double* raw = reinterpret_cast<double*>(&sm.v);
+  static_assert(sizeof(double) * C::NW <= sizeof(DavVectors<K>), "the raw block fits the vectors' place");
+#pragma unroll 3
+  for (int x = tid; x < C::NW; x += NT) copy8_async(raw + x, a.W + (sm.off2[0][x / NF] + sm.off2[1][x % NF]));
   unsigned mx = 0, all = 0;
-#pragma unroll
-  for (int i = 0; i < C::NG; ++i) {
-    const int x = tid + i * NT;
-    w[i] = 0.0;
-    if (x < C::NW) w[i] = a.W[sm.off2[0][x / NF] + sm.off2[1][x % NF]];
-  }
+#pragma unroll 1
   for (int x = tid; x < NF; x += NT) {
     const double f = a.F[(unsigned)sm.orb[x / NORB] * (unsigned)a.n + (unsigned)sm.orb[x % NORB]];
     sm.F[x] = f;
     all = max(all, mag_hi(f));
     if (x / NORB != x % NORB) mx = max(mx, mag_hi(f));
   }
-#pragma unroll
-  for (int i = 0; i < C::NG; ++i) {
-    const int x = tid + i * NT;
-    if (x < C::NW) {
-      const int pq = x / NF, rs = x % NF;
-      const int p = pq / NORB, q = pq % NORB, r = rs / NORB, t = rs % NORB;
-      const unsigned hi = mag_hi(w[i]);
-      all = max(all, hi);
-      if (p == q && r == t) sm.J[p * NORB + r] = w[i];
-      else mx = max(mx, hi);
-      if (p == t && q == r) sm.X[p * NORB + q] = w[i];
-    }
+  copies_done();
+  // a thread reads back its own copies
+#pragma unroll 1
+  for (int x = tid; x < C::NW; x += NT) {
+    const double w = raw[x];
+    const int pq = x / NF, rs = x % NF;
+    const int p = pq / NORB, q = pq % NORB, r = rs / NORB, t = rs % NORB;
+    const unsigned hi = mag_hi(w);
+    all = max(all, hi);
+    if (p == q && r == t) sm.J[p * NORB + r] = w;
+    else mx = max(mx, hi);
+    if (p == t && q == r) sm.X[p * NORB + q] = w;
   }
   sx = scale_of(block_max(sm, mx, 0));
-#pragma unroll
-  for (int i = 0; i < C::NG; ++i) {
-    const int x = tid + i * NT;
-    if (x < C::NW) {
-      const int pq = x / NF, rs = x % NF;
-      const bool dd = (pq % (NORB + 1)) == 0 && (rs % (NORB + 1)) == 0;
-      sm.W[x] = dd ? make_int2(0, 0) : limbs(to_fix(w[i], sx, kFix));
-    }
+#pragma unroll 1
+  for (int x = tid; x < C::NW; x += NT) {
+    const int pq = x / NF, rs = x % NF;
+    const bool dd = (pq % (NORB + 1)) == 0 && (rs % (NORB + 1)) == 0;
+    sm.W[x] = dd ? make_int2(0, 0) : limbs(to_fix(raw[x], sx, kFix));
   }
   return all < kInfHi && sx > -900 && sx < 900;
 }
@@ -793,6 +762,7 @@ __device__ __forceinline__ void lin_fixed(FSmem<K, true>& sm, int so, int st, in
   long long* Wx = reinterpret_cast<long long*>(sm.W);
   const int tid = threadIdx.x;
   // elements block by block (16 o / v blocks of K^4), so that a warp takes one branch of w2
+#pragma unroll 1
   for (int x = tid; x < C::NW; x += NT) {
     const int blk = x / K4, y = x % K4;
     const int p = y / (K * K * K) + (blk & 8 ? K : 0), q = (y / (K * K)) % K + (blk & 4 ? K : 0);
@@ -802,6 +772,7 @@ __device__ __forceinline__ void lin_fixed(FSmem<K, true>& sm, int so, int st, in
     L.w2(v, blk, p, q, r, s);
     Wx[((p * NO + q) * NO + r) * NO + s] = v.value();
   }
+#pragma unroll 1
   for (int x = tid; x < C::NF; x += NT) {
     const int p = x / NO, q = x % NO;
     Acc v, w;
@@ -818,10 +789,12 @@ __device__ __forceinline__ void lin_fixed(FSmem<K, true>& sm, int so, int st, in
     d.Fx[x] = v.value() + w.value();
   }
   Acc e;
+#pragma unroll 1
   for (int x = tid; x < K4; x += NT) {
     const int i = x / (K * K * K), j = (x / K) % K, aa = (x / (K * K)) % K, b = x % K;  // (i a j b)
     e.add(L.g(i, K + aa, j, K + b), L.u(i, j, aa, b));
   }
+#pragma unroll 1
   for (int x = tid; x < K * K; x += NT) {
     const int k = x / K, l = x % K;
     Acc y, z;
@@ -841,10 +814,12 @@ __device__ __forceinline__ void lin_fixed(FSmem<K, true>& sm, int so, int st, in
   for (int v = 0; v < C::NWARP; ++v) ex += d.part[v];
   e0 -= (half ? 1.0 : 2.0) * ((double)ex * pow2(so + st - kFix));
   const int sh = S - so - st + half;
+#pragma unroll 1
   for (int x = tid; x < C::NW; x += NT) {
     const int p = x / (NO * NO * NO), q = (x / (NO * NO)) % NO, r = (x / NO) % NO, s = x % NO;
     d.W[x] -= shift_fix(Wx[x] + Wx[((q * NO + p) * NO + s) * NO + r], sh);
   }
+#pragma unroll 1
   for (int x = tid; x < C::NF; x += NT) d.F[x] -= shift_fix(d.Fx[x] + d.Fx[(x % NO) * NO + x / NO], sh);
   __syncthreads();
 }
@@ -930,12 +905,14 @@ __device__ __noinline__ bool ducc_block(FSmem<K, true>& sm, const SolveArgs& a, 
   const int S = scale_of(mx), st = scale_of(mt);
   if (mx >= kInfHi || mt >= kInfHi || S < -400 || S > 400 || st > 0 || st < -400) return false;
   __syncthreads();
+#pragma unroll 1
   for (int x = tid; x < K4; x += NT) {
     const int i = x / (K * K2), j = (x / K2) % K, aa = (x / K) % K, b = x % K;
     const int2 p = d.t2[x], q = d.t2[((i * K + j) * K + b) * K + aa];
     d.u[x] = make_int2(2 * p.x - q.x, 2 * p.y - q.y);
   }
   // X_A: H_A in vacuum order on the space
+#pragma unroll 1
   for (int x = tid; x < NF; x += NT) {
     const int p = x / NO, q = x % NO;
     long long v = d.f0[x];
@@ -948,6 +925,7 @@ __device__ __noinline__ bool ducc_block(FSmem<K, true>& sm, const SolveArgs& a, 
   // Y_A: B_A = D.T_A + (D.T_A)^+, D from the Fock diagonal; in units of 2^(S + st + 4 - 54), which
   // leaves the four orbital energies of D their room
   auto eps = [&](int p) { return d.f0[p * NO + p]; };
+#pragma unroll 1
   for (int x = tid; x < C::NW; x += NT) {
     const int p = x / (NO * NO * NO), q = (x / (NO * NO)) % NO, r = (x / NO) % NO, s = x % NO;
     Acc v;
@@ -957,6 +935,7 @@ __device__ __noinline__ bool ducc_block(FSmem<K, true>& sm, const SolveArgs& a, 
       v.add(limbs(eps(q) + eps(s) - eps(p) - eps(r)), d.t2[((p * K + r) * K + (q - K)) * K + (s - K)]);
     d.g[x] = limbs(shift_fix(v.value(), 4));
   }
+#pragma unroll 1
   for (int x = tid; x < NF; x += NT) {
     const int p = x / NO, q = x % NO;
     Acc v;
@@ -965,6 +944,7 @@ __device__ __noinline__ bool ducc_block(FSmem<K, true>& sm, const SolveArgs& a, 
     d.h[x] = limbs(shift_fix(v.value(), 4));
   }
   __syncthreads();
+#pragma unroll 1
   for (int x = tid; x < NF; x += NT) {  // normal order
     const int p = x / NO, q = x % NO;
     long long v = unlimb(d.h[x]);
@@ -977,6 +957,7 @@ __device__ __noinline__ bool ducc_block(FSmem<K, true>& sm, const SolveArgs& a, 
   // W limbs relative to the largest element that is not (pp|rr)
   const double unit = pow2(S - kFix);
   long long big = 0;
+#pragma unroll 1
   for (int x = tid; x < C::NW; x += NT) {
     const int pq = x / NF, rs = x % NF, p = pq / NO, q = pq % NO, r = rs / NO, t = rs % NO;
     const long long v = d.W[x];
@@ -984,6 +965,7 @@ __device__ __noinline__ bool ducc_block(FSmem<K, true>& sm, const SolveArgs& a, 
     else big |= v < 0 ? ~v : v;
     if (p == t && q == r) sm.X[p * NO + q] = (double)v * unit;
   }
+#pragma unroll 1
   for (int x = tid; x < NF; x += NT) {
     sm.F[x] = (double)d.F[x] * unit;
     if (x / NO != x % NO) big |= d.F[x] < 0 ? ~d.F[x] : d.F[x];
@@ -991,6 +973,7 @@ __device__ __noinline__ bool ducc_block(FSmem<K, true>& sm, const SolveArgs& a, 
   const int lead = (int)block_max(sm, (unsigned)(64 - __clzll(big)), 0);  // |v| < 2^lead
   const int up = lead > 0 ? kFix - lead : 0;                             // left shift to 54 bits
   sx = S - up;
+#pragma unroll 1
   for (int x = tid; x < C::NW; x += NT) {
     const int pq = x / NF, rs = x % NF;
     const bool dd = (pq % (NO + 1)) == 0 && (rs % (NO + 1)) == 0;
@@ -1015,19 +998,28 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
   const int rl = lane / C::TPR;
   const bool rowok = rl < C::RPW;
   const int row = warp * C::RPW + (rowok ? rl : 0);
-  const int part = rowok ? lane % C::TPR : C::TPR;  // C::TPR: idle lane (repeats row 0's work, stores nothing)
-  const int mrow = tab.mask[row];
-  unsigned rep[C::UPT];
+  const int part = rowok ? lane % C::TPR : C::TPR;  // C::TPR: idle lane (stores nothing)
+  unsigned rep[C::UPT], own = 0;
 #pragma unroll
-  for (int u = 0; u < C::UPT; ++u) rep[u] = tab.rep[row][(rowok ? part : 0) * C::UPT + u];
-  int pia[PER], pib[PER];
-  bool pin[PER];
+  for (int u = 0; u < C::UPT; ++u) rep[u] = tab.rep[row][(rowok ? part : 0) * C::UPT + u] | (1u << 17);
+  {  // the part-th orbital p of the string: row (pp) of W on the string's own row of C, twice
+    int m = tab.mask[row];
+    for (int i = 0; i < part; ++i) m &= m - 1;
+    if (m && part < C::TPR) own = (unsigned)((__ffs(m) - 1) * (NORB + 1)) | ((unsigned)row << 8) | (2u << 17);
+    else own = (unsigned)row << 8;
+  }
+  // pairs I <= J: index and strings; a pair I < J stands for two determinants, so vectors hold its
+  // value times sqrt 2 and sums over pairs are sums over determinants
+  int pd[PER], pia[PER], pib[PER];
+  bool has[PER];
+  constexpr double kRoot2 = 1.4142135623730951, kHalfRoot2 = 0.70710678118654757;
 #pragma unroll
   for (int r = 0; r < PER; ++r) {
     int d = tid + r * NT;
-    pin[r] = d < C::NP;
+    has[r] = d < C::NP;
+    if (!has[r]) d = 0;
+    pd[r] = d;
     int i = 0, len = NS;
-    if (!pin[r]) d = 0;
     while (d >= len) {
       d -= len;
       --len;
@@ -1067,6 +1059,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
       __syncthreads();
       continue;
     }
+#pragma unroll 1
     for (int x = tid; x < NF; x += NT) {
       const unsigned p = (unsigned)sm.orb[x / NORB], q = (unsigned)sm.orb[x % NORB];
       sm.off2[0][x] = p * n3 + q * n2;
@@ -1086,6 +1079,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
       continue;
     }
     // pair symmetry within 2^-44 of the largest coupling; folded one-body couplings
+#pragma unroll 1
     for (int x = tid; x < C::NW; x += NT) {
       const int pq = x / NF, rs = x % NF;
       if (pq < rs) {
@@ -1093,6 +1087,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
         if (df > 1024 || df < -1024) sm.flag[1] = 1;
       }
     }
+#pragma unroll 1
     for (int x = tid; x < NF; x += NT) {
       const int p = x / NORB, q = x % NORB;
       if (p != q) {
@@ -1104,18 +1099,15 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
         sm.hfix[x] = v;
       }
     }
-    if (tid < NORB) {  // folded one-body diagonal (FP64), kept in the F block's place below
+    if (tid < NORB) {  // folded one-body diagonal (FP64)
       double v = sm.F[tid * (NORB + 1)];
 #pragma unroll
       for (int k = 0; k < K; ++k) v -= 2.0 * sm.J[tid * NORB + k] - sm.X[tid * NORB + k];
-      sm.hsd[tid] = v;  // h_pp; NS >= NORB entries
+      sm.hd[tid] = v;
     }
     __syncthreads();
-    double hpp[NORB];
-#pragma unroll
-    for (int p = 0; p < NORB; ++p) hpp[p] = sm.hsd[p];
-    __syncthreads();
     // same-spin couplings (Slater-Condon rules) and diagonal, Coulomb rows of the strings
+#pragma unroll 1
     for (int x = tid; x < C::NDET; x += NT) {
       const unsigned e = tab.hs[x];
       const int p = (e >> 3) & 7, q = (e >> 6) & 7, r = (e >> 9) & 7, t = (e >> 12) & 7;
@@ -1127,25 +1119,37 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
       } else if ((e & 3u) == 2u) {
         v = unlimb(sm.W[(p * NORB + q) * NF + r * NORB + t]) - unlimb(sm.W[(p * NORB + t) * NF + r * NORB + q]);
       }
-      sm.Hs[x] = limbs((e & 4u) ? -v : v);
-      sm.Cv[x] = make_int2(0, 0);
+      sm.Hs[(x % NS) * NS + x / NS] = limbs((e & 4u) ? -v : v);
     }
+#pragma unroll 1
     for (int i = tid; i < NS; i += NT) {
-      double v = 0.0;
       const int m = tab.mask[i];
-      for (int p = 0; p < NORB; ++p) {
-        if (!((m >> p) & 1)) continue;
-        v += hpp[p];
-        for (int q = p + 1; q < NORB; ++q)
-          if ((m >> q) & 1) v += 0.5 * ((sm.J[p * NORB + q] + sm.J[q * NORB + p]) - (sm.X[p * NORB + q] + sm.X[q * NORB + p]));
+      int o[K];
+      int left = m;
+#pragma unroll
+      for (int x = 0; x < K; ++x) {
+        o[x] = __ffs(left) - 1;
+        left &= left - 1;
       }
-      sm.hsd[i] = v;
+      double v = 0.0, c = 0.0;
+#pragma unroll
+      for (int x = 0; x < K; ++x) {
+        v += sm.hd[o[x]];
+#pragma unroll
+        for (int z = x + 1; z < K; ++z) c += sm.J[o[x] * NORB + o[z]] - sm.X[o[x] * NORB + o[z]];
+      }
+      sm.hsd[i] = v + c;
     }
+#pragma unroll 1
     for (int x = tid; x < NS * NORB; x += NT) {
-      const int m = tab.mask[x / NORB], r = x % NORB;
+      const int r = x % NORB;
+      int left = tab.mask[x / NORB];
       double v = 0.0;
-      for (int p = 0; p < NORB; ++p)
-        if ((m >> p) & 1) v += sm.J[p * NORB + r];
+#pragma unroll
+      for (int z = 0; z < K; ++z) {
+        v += sm.J[(__ffs(left) - 1) * NORB + r];
+        left &= left - 1;
+      }
       sm.JR[x] = v;
     }
     __syncthreads();
@@ -1155,202 +1159,233 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
       continue;
     }
     auto diag_of = [&](int ia, int ib) {
-      double v = sm.hsd[ia] + sm.hsd[ib];
-      const int m = tab.mask[ib];
+      double v = 0.0;
+      int left = tab.mask[ib];
 #pragma unroll
-      for (int p = 0; p < NORB; ++p)
-        if ((m >> p) & 1) v += sm.JR[ia * NORB + p];
-      return v;
+      for (int z = 0; z < K; ++z) {
+        v += sm.JR[ia * NORB + __ffs(left) - 1];
+        left &= left - 1;
+      }
+      return (sm.hsd[ia] + sm.hsd[ib]) + v;
     };
     const double c00 = diag_of(0, 0);
     double eshift = 0.0;
     {
       double ec = e0;
 #pragma unroll
-      for (int k = 0; k < K; ++k) ec -= hpp[k] + sm.F[k * (NORB + 1)];
+      for (int k = 0; k < K; ++k) ec -= sm.hd[k] + sm.F[k * (NORB + 1)];
       eshift = ec + c00;
     }
+    // joined sums count 2^-54 of (2^sx)(1)
+    const double scale = pow2(sx - kFix);
     double diag[PER], vk[PER];
 #pragma unroll
     for (int r = 0; r < PER; ++r) {
-      diag[r] = pin[r] ? diag_of(pia[r], pib[r]) - c00 : 0.0;
-      vk[r] = (pin[r] && tid + r * NT == 0) ? 1.0 : 0.0;
+      diag[r] = diag_of(pia[r], pib[r]) - c00;
+      // first vector Phi; its sigma is Phi's column of the operator
+      const unsigned ea = tab.ex[pia[r]], eb = tab.ex[pib[r]];
+      long long t = 0;
+      if (pia[r] == 0) {
+        t = unlimb(sm.Hs[pib[r]]);
+        if (eb) {
+          long long c = 0;
+#pragma unroll
+          for (int p = 0; p < K; ++p) c += unlimb(sm.W[p * (NORB + 1) * NF + (eb & 63u)]);
+          t += (eb >> 16) & 1u ? -c : c;
+        }
+      } else if (ea && eb) {
+        t = unlimb(sm.W[(ea & 63u) * NF + (eb & 63u)]);
+        if (((ea ^ eb) >> 16) & 1u) t = -t;
+      }
+      if (has[r]) {
+        sm.v.V[0][pd[r]] = pd[r] == 0 ? 1.0 : 0.0;
+        sm.v.S[0][pd[r]] = (pia[r] == pib[r] ? scale : scale * kRoot2) * (double)t;
+      }
     }
-    // hh + cross sums count 2^-54 of (2^sx)(1): sigma's scale
-    const double scale = pow2(sx - kFix);
-    int k = 0;             // vectors in the subspace
+    if (tid == 0) {
+      sm.G[0] = 0.0;
+      sm.y[0] = 1.0;
+    }
+    int k = 1;             // vectors in the subspace
     double th = 0.0;
     int st = kSpaceNoConv, itn = 0;
     bool defer = false;
+    __syncthreads();
 
     // ---- Davidson -----------------------------------------------------------------------------
-    // `add`: vk (a unit vector) becomes V[k]; S[k] = H V[k]; new row and column of G
-    for (int it = -1; it < a.max_iter; ++it) {
-      if (it >= 0) {
-        if (k == C::KM) {  // restart on the current Ritz vector
-          double part2[8];
+    for (int it = 0; it < a.max_iter; ++it) {
+      if (k == C::KM) {  // restart on the current Ritz vector
+        double part2[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) part2[j] = 0.0;
-          double xs[PER], ss[PER];
-#pragma unroll
-          for (int r = 0; r < PER; ++r) {
-            const int d = tid + r * NT;
-            double xv = 0.0, sv = 0.0;
-            if (pin[r])
-              for (int j = 0; j < C::KM; ++j) {
-                xv = fma(sm.y[j], sm.v.V[j][d], xv);
-                sv = fma(sm.y[j], sm.v.S[j][d], sv);
-              }
-            const double wt = pia[r] == pib[r] ? 1.0 : 2.0;
-            xs[r] = xv;
-            ss[r] = sv;
-            part2[0] = fma(wt * xv, xv, part2[0]);
-            part2[1] = fma(wt * xv, sv, part2[1]);
-          }
-          const double* o = sum_many(sm, part2, 2, buf);
-          const double inv = rsqrt_nr(o[0]);
-          const double g00 = o[1] / o[0];
-#pragma unroll
-          for (int r = 0; r < PER; ++r)
-            if (pin[r]) {
-              sm.v.V[0][tid + r * NT] = xs[r] * inv;
-              sm.v.S[0][tid + r * NT] = ss[r] * inv;
-            }
-          __syncthreads();
-          if (tid == 0) {
-            sm.G[0] = g00;
-            sm.y[0] = 1.0;
-          }
-          th = g00;
-          k = 1;
-          __syncthreads();
-        }
-        // residual r = S y - theta V y; correction t = r / (theta - D)
-        double p1[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) p1[j] = 0.0;
+        for (int j = 0; j < 8; ++j) part2[j] = 0.0;
+        double xs[PER], ss[PER];
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
-          const int d = tid + r * NT;
           double xv = 0.0, sv = 0.0;
-          if (pin[r])
-            for (int j = 0; j < k; ++j) {
-              xv = fma(sm.y[j], sm.v.V[j][d], xv);
-              sv = fma(sm.y[j], sm.v.S[j][d], sv);
-            }
-          const double res = fma(-th, xv, sv);
-          const double wt = pia[r] == pib[r] ? 1.0 : 2.0;
-          p1[0] = fma(wt * res, res, p1[0]);
-          double den = th - diag[r];
-          if (fabs(den) < 1e-4) den = den < 0.0 ? -1e-4 : 1e-4;
-          vk[r] = pin[r] ? res * recip(den) : 0.0;
-          p1[1] = fma(wt * vk[r], vk[r], p1[1]);
-        }
-        const double* o = sum_many(sm, p1, 2, buf);
-        const double rn2 = o[0], tt = o[1];
-        if (!isfinite(rn2) || !isfinite(th)) {
-          defer = true;
-          break;
-        }
-        if (rn2 < tol2) {
-          st = kSpaceOk;
-          itn = it;
-          break;
-        }
-        // classical Gram-Schmidt; again where the first pass took most of the vector away
-        double vn2 = tt;
-        for (int pass = 0; pass < 2; ++pass) {
-          double p2[8];
-#pragma unroll
-          for (int j = 0; j < 8; ++j) p2[j] = 0.0;
-#pragma unroll
-          for (int r = 0; r < PER; ++r) {
-            const double tw = pia[r] == pib[r] ? vk[r] : 2.0 * vk[r];
-            if (pin[r])
-#pragma unroll
-              for (int j = 0; j < C::KM - 1; ++j)
-                if (j < k) p2[j] = fma(sm.v.V[j][tid + r * NT], tw, p2[j]);
+#pragma unroll 1
+          for (int j = 0; j < C::KM; ++j) {
+            xv = fma(sm.y[j], sm.v.V[j][pd[r]], xv);
+            sv = fma(sm.y[j], sm.v.S[j][pd[r]], sv);
           }
-          const double* q = sum_many(sm, p2, k, buf);
-          double p3[8];
+          xs[r] = xv;
+          ss[r] = sv;
+          if (!has[r]) xv = 0.0;
+          part2[0] = fma(xv, xv, part2[0]);
+          part2[1] = fma(xv, sv, part2[1]);
+        }
+        const double* o = sum_many(sm, part2, 2, buf);
+        const double inv = rsqrt_nr(o[0]);
+        const double g00 = o[1] / o[0];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) p3[j] = 0.0;
-#pragma unroll
-          for (int r = 0; r < PER; ++r) {
-            double v = vk[r];
-            if (pin[r])
-              for (int j = 0; j < k; ++j) v = fma(-q[j], sm.v.V[j][tid + r * NT], v);
-            vk[r] = v;
-            p3[0] = fma(pia[r] == pib[r] ? v : 2.0 * v, v, p3[0]);
+        for (int r = 0; r < PER; ++r)
+          if (has[r]) {
+            sm.v.V[0][pd[r]] = xs[r] * inv;
+            sm.v.S[0][pd[r]] = ss[r] * inv;
           }
-          const double prev = vn2;
-          vn2 = sum_many(sm, p3, 1, buf)[0];
-          if (vn2 > 0.01 * prev) break;
+        __syncthreads();
+        if (tid == 0) {
+          sm.G[0] = g00;
+          sm.y[0] = 1.0;
         }
-        if (!(vn2 > 1e-26)) {  // subspace cannot grow (complete or stagnated)
-          st = rn2 < 1e4 * tol2 ? kSpaceOk : kSpaceNoConv;
-          itn = it;
-          break;
-        }
-        const double inv = rsqrt_nr(vn2);
-#pragma unroll
-        for (int r = 0; r < PER; ++r) vk[r] *= inv;
+        th = g00;
+        k = 1;
+        __syncthreads();
       }
-      // V[k] = vk, S[k] = H vk
+      // residual r = S y - theta V y, correction t = r / (theta - D), and t's products with the basis
+      double xv[PER], sv[PER], p1[16];
 #pragma unroll
-      for (int r = 0; r < PER; ++r)
-        if (pin[r]) {
-          sm.v.V[k][tid + r * NT] = vk[r];
-          const int2 c = limbs(to_fix(vk[r], 0, kFix));
+      for (int r = 0; r < PER; ++r) xv[r] = sv[r] = 0.0;
+#pragma unroll 1
+      for (int j = 0; j < k; ++j) {
+        const double yj = sm.y[j];
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+          xv[r] = fma(yj, sm.v.V[j][pd[r]], xv[r]);
+          sv[r] = fma(yj, sm.v.S[j][pd[r]], sv[r]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 16; ++j) p1[j] = 0.0;
+#pragma unroll
+      for (int r = 0; r < PER; ++r) {
+        double res = fma(-th, xv[r], sv[r]);
+        if (!has[r]) res = 0.0;
+        double den = th - diag[r];
+        if (mag_hi(den) < 0x3f1a36e2u) den = den < 0.0 ? -1e-4 : 1e-4;  // |den| < 1e-4
+        vk[r] = res * recip(den);
+        p1[0] = fma(res, res, p1[0]);
+        p1[1] = fma(vk[r], vk[r], p1[1]);
+      }
+#pragma unroll
+      for (int j = 0; j < C::KM - 1; ++j)
+        if (j < k) {
+#pragma unroll
+          for (int r = 0; r < PER; ++r) p1[2 + j] = fma(sm.v.V[j][pd[r]], vk[r], p1[2 + j]);
+        }
+      const double* o = k + 2 <= 8 ? sum_many(sm, reinterpret_cast<double(&)[8]>(p1), k + 2, buf) : sum_many(sm, p1, k + 2, buf);
+      const double rn2 = o[0], tt = o[1];
+      if (!isfinite(rn2) || !isfinite(th)) {
+        defer = true;
+        break;
+      }
+      if (rn2 < tol2) {
+        st = kSpaceOk;
+        itn = it;
+        break;
+      }
+      // classical Gram-Schmidt; the norm of what is left from Pythagoras, or, where little is left, by a
+      // second pass and a sum of its own
+      double vn2 = tt;
+#pragma unroll 1
+      for (int j = 0; j < k; ++j) {
+        const double q = o[2 + j];
+        vn2 = fma(-q, q, vn2);
+#pragma unroll
+        for (int r = 0; r < PER; ++r) vk[r] = fma(-q, sm.v.V[j][pd[r]], vk[r]);
+      }
+      if (!(vn2 > 0.01 * tt)) {
+        double p2[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) p2[j] = 0.0;
+#pragma unroll
+        for (int j = 0; j < C::KM - 1; ++j)
+          if (j < k) {
+#pragma unroll
+            for (int r = 0; r < PER; ++r) p2[j] = fma(sm.v.V[j][pd[r]], vk[r], p2[j]);
+          }
+        const double* q = sum_many(sm, p2, k, buf);
+        double p3[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) p3[j] = 0.0;
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+#pragma unroll 1
+          for (int j = 0; j < k; ++j) vk[r] = fma(-q[j], sm.v.V[j][pd[r]], vk[r]);
+          if (!has[r]) vk[r] = 0.0;
+          p3[0] = fma(vk[r], vk[r], p3[0]);
+        }
+        vn2 = sum_many(sm, p3, 1, buf)[0];
+      }
+      if (!(vn2 > 1e-26)) {  // subspace cannot grow (complete or stagnated)
+        st = rn2 < 1e4 * tol2 ? kSpaceOk : kSpaceNoConv;
+        itn = it;
+        break;
+      }
+      // V[k] = vk (unit), S[k] = H vk
+      const double inv = rsqrt_nr(vn2);
+#pragma unroll
+      for (int r = 0; r < PER; ++r) {
+        vk[r] = has[r] ? vk[r] * inv : 0.0;
+        if (has[r]) {
+          sm.v.V[k][pd[r]] = vk[r];
+          const int2 c = limbs(to_fix(pia[r] == pib[r] ? vk[r] : vk[r] * kHalfRoot2, 0, kFix));
           sm.Cv[pia[r] * NS + pib[r]] = c;
           sm.Cv[pib[r] * NS + pia[r]] = c;
         }
+      }
       __syncthreads();
-      sigma_fixed(sm, rep, row, part, mrow);
-      double p4[16];
+      sigma_fixed(sm, rep, own, row, part);
+      __syncthreads();
+      // new row and column of the projected matrix: G[j][k] and G[k][j], j < k, then G[k][k]
+      double p4[16], sk[PER];
 #pragma unroll
       for (int j = 0; j < 16; ++j) p4[j] = 0.0;
 #pragma unroll
-      for (int r = 0; r < PER; ++r)
-        if (pin[r]) {
-          const int d = tid + r * NT, ij = pia[r] * NS + pib[r], ji = pib[r] * NS + pia[r];
-          const long long t = sm.B[ij] + sm.A[ij] + sm.A[ji];
-          const double sk = fma(scale, (double)t, diag[r] * vk[r]);
-          sm.v.S[k][d] = sk;
-          const double wt = pia[r] == pib[r] ? 1.0 : 2.0;
-          const double ws = wt * sk, wv = wt * vk[r];
+      for (int r = 0; r < PER; ++r) {
+        const long long t = sm.T[pia[r] * NS + pib[r]] + sm.T[pib[r] * NS + pia[r]];
+        sk[r] = fma(pia[r] == pib[r] ? 0.5 * scale : kHalfRoot2 * scale, (double)t, diag[r] * vk[r]);
+        if (has[r]) sm.v.S[k][pd[r]] = sk[r];
+        p4[0] = fma(vk[r], sk[r], p4[0]);  // vk is zero where there is no pair
+      }
 #pragma unroll
-          for (int j = 0; j < C::KM; ++j) {
-            if (j < k) {
-              p4[j] = fma(sm.v.V[j][d], ws, p4[j]);            // G[j][k]
-              p4[8 + j] = fma(sm.v.S[j][d], wv, p4[8 + j]);    // G[k][j]
-            }
-            if (j == k) p4[j] = fma(vk[r], ws, p4[j]);
+      for (int j = 0; j < C::KM - 1; ++j) {
+        if (j < k) {
+#pragma unroll
+          for (int r = 0; r < PER; ++r) {
+            p4[1 + 2 * j] = fma(sm.v.V[j][pd[r]], has[r] ? sk[r] : 0.0, p4[1 + 2 * j]);
+            p4[2 + 2 * j] = fma(sm.v.S[j][pd[r]], vk[r], p4[2 + 2 * j]);
           }
         }
-      const double* o = sum_many(sm, p4, 16, buf);
+      }
+      const double* g = 2 * k + 1 <= 8 ? sum_many(sm, reinterpret_cast<double(&)[8]>(p4), 2 * k + 1, buf) : sum_many(sm, p4, 2 * k + 1, buf);
       if (warp == 0) {
-        if (lane <= k) sm.G[lane * C::KM + k] = o[lane];
-        if (lane < k) sm.G[k * C::KM + lane] = o[8 + lane];
+        if (lane < k) {
+          sm.G[lane * C::KM + k] = g[1 + 2 * lane];
+          sm.G[k * C::KM + lane] = g[2 + 2 * lane];
+        }
+        if (lane == k) sm.G[k * C::KM + k] = g[0];
         __syncwarp();
-        if (k == 0) {
-          if (lane == 0) {
-            sm.y[0] = 1.0;
-            sm.theta = sm.G[0];
-          }
-        } else {
-          double thn = th;
-          const bool ok = newton_root<DUCC>(sm.G, C::KM, k + 1, th, sm.y, &thn, &sm.v.V[0][0], C::NP);
-          if (lane == 0) {
-            sm.theta = thn;
-            if (!ok) sm.flag[1] = 1;
-          }
+        double thn = th;
+        const bool ok = newton_root<DUCC>(sm.G, C::KM, k + 1, th, sm.y, &thn, &sm.v.V[0][0], C::NP);
+        if (lane == 0) {
+          sm.theta = thn;
+          if (!ok) sm.flag[1] = 1;
         }
       }
       __syncthreads();
       th = sm.theta;
       ++k;
-      if (it >= 0) itn = it + 1;
+      itn = it + 1;
       if (sm.flag[1]) {
         defer = true;
         break;
@@ -1363,19 +1398,22 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
     }
 
     // ---- root, increment, merge -----------------------------------------------------------------
-    double* xf = reinterpret_cast<double*>(sm.A);  // Ritz vector, [I][J]
+    double* xf = reinterpret_cast<double*>(sm.T);  // Ritz vector, [I][J]
     double p5[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) p5[j] = 0.0;
 #pragma unroll
-    for (int r = 0; r < PER; ++r)
-      if (pin[r]) {
-        double xv = 0.0;
-        for (int j = 0; j < k; ++j) xv = fma(sm.y[j], sm.v.V[j][tid + r * NT], xv);
-        xf[pia[r] * NS + pib[r]] = xv;
-        xf[pib[r] * NS + pia[r]] = xv;
-        p5[0] = fma(pia[r] == pib[r] ? xv : 2.0 * xv, xv, p5[0]);
+    for (int r = 0; r < PER; ++r) {
+      double xv = 0.0;
+#pragma unroll 1
+      for (int j = 0; j < k; ++j) xv = fma(sm.y[j], sm.v.V[j][pd[r]], xv);
+      if (has[r]) {
+        const double x = pia[r] == pib[r] ? xv : xv * kHalfRoot2;
+        xf[pia[r] * NS + pib[r]] = x;
+        xf[pib[r] * NS + pia[r]] = x;
+        p5[0] = fma(xv, xv, p5[0]);
       }
+    }
     const double xn2 = sum_many(sm, p5, 1, buf)[0];  // its barrier orders xf
     const double c0 = xf[0];
     if (st == kSpaceOk && !(c0 * c0 >= 1e-6 * xn2)) st = kSpaceRoot;
@@ -1397,12 +1435,14 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
         return sg * xf[j] * inv0;
       };
       if (a.owner1)
+#pragma unroll 1
         for (int x = tid; x < K * K; x += NT) {
           const int i = x / K, aa = x % K;
           const size_t g = (size_t)sm.orb[i] * a.nvir + (sm.orb[K + aa] - a.nocc);
           if (a.owner1[g] == sidx) a.t1_new[g] = (DUCC ? 0.0 : a.t1_old[g]) + x1(i, aa);  // DUCC: replaced
         }
       if (a.owner2)
+#pragma unroll 1
         for (int x = tid; x < K * K * K * K; x += NT) {
           const int i = x / (K * K * K), j = (x / (K * K)) % K, aa = (x / K) % K, b = x % K;
           const size_t g = (((size_t)sm.orb[i] * a.nocc + sm.orb[j]) * a.nvir + (sm.orb[K + aa] - a.nocc)) * a.nvir +
