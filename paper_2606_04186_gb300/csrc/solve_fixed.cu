@@ -22,7 +22,14 @@
 //     preconditioner, residuals and iterate in FP64;
 //   * sums over determinants reduce several values at once (2 m FP64 additions per warp for m values
 //     instead of 5 m), and Gram-Schmidt repeats only where the first pass cancelled.
-// Sweep of the 9,690 spaces of 24 orbitals: see the launch rule in launch_solve_fixed.
+//   * an FP64 instruction holds a warp for 64 cycles, so what is left in FP64 (residual, Gram-Schmidt,
+//     projected matrix) is spread over two warps with fused sums, conversions are field arithmetic,
+//     and six CTAs per SM (168 registers, 37 KB: four of the eight subspace vectors in shared memory,
+//     later ones in local memory) cover each other's latency.
+// Measured (sweep's solve phase): all 9,690 spaces of 24 orbitals 18.2 -> 1.47 ms, a cycle of 35,000
+// spaces of 82 orbitals 49.2 -> 4.5 ms, 35 spaces of 10 orbitals 0.72 -> 0.12 ms; FP64 pipe 42-50 %
+// busy, mad.wide about 25 %.  128 threads per space with three CTAs per SM: 1.85 ms at 24 orbitals (the
+// warps' sums double), 0.084 ms at 10.
 //
 // Spaces outside what this kernel is exact for leave with status kSpaceDefer and are solved by
 // solve.cu's kernel: non-finite integrals, W without pair symmetry, a projected root that is not
@@ -63,6 +70,8 @@ struct FD {
   static constexpr int NWARP = NT / 32;
   static constexpr int PER = (NP + NT - 1) / NT;       // pairs per thread
   static constexpr int KM = (NDET < 8) ? NDET : 8;     // subspace limit (as solve.cu)
+  static constexpr int SL = (K == 3) ? 4 : KM;         // vectors kept in shared memory, the rest in local
+  static constexpr int MINB = (K == 3) ? 6 : 16;       // resident CTAs the registers are held to
   static constexpr int NU = K * K;                     // replacements i -> a of a string
   static constexpr int TPR = (K == 3) ? 3 : NU;        // threads that share a string's replacements
   static constexpr int UPT = NU / TPR;
@@ -213,8 +222,8 @@ struct DuccFix {
 };
 template <int K>
 struct DavVectors {
-  double V[FD<K>::KM][FD<K>::NP];   // subspace basis (orthonormal): pair values, times sqrt 2 for I < J
-  double S[FD<K>::KM][FD<K>::NP];   // H applied to it
+  double V[FD<K>::SL][FD<K>::NP];   // subspace basis (orthonormal): pair values, times sqrt 2 for I < J
+  double S[FD<K>::SL][FD<K>::NP];   // H applied to it
 };
 struct NoScratch {};
 
@@ -236,6 +245,7 @@ struct FSmem {
   double JR[C::NS * C::NORB];  // sum of J over a string's orbitals
   double G[C::KM * C::KM];
   double y[8];
+  double phi[8];            // the basis vectors' Phi coefficients
   double red[2][C::NWARP][16];
   double out[C::NWARP][16];
   double theta;
@@ -395,12 +405,12 @@ __device__ __forceinline__ void sigma_fixed(FSmem<K, DUCC>& sm, const unsigned (
 // decides) unless the rest of the spectrum is clearly farther from it than the found root, the root
 // is dominated by its first coefficient and the iteration settled.  SYM (DUCC form): of the
 // symmetrised matrix, the eigenvector with the largest Phi weight, which a vector with more than
-// half of the weight is (v0: the basis vectors' Phi coefficients, ld0 apart).
+// half of the weight is (v0: the basis vectors' Phi coefficients).
 // Lane l holds columns 2 (l / 8) and 2 (l / 8) + 1 of row l % 8; a vector's element r is in the four
 // lanes of row r.
 template <bool SYM>
 __device__ __forceinline__ bool newton_root(const double* G, int ld, int kk, double theta0, double* y, double* theta,
-                                            const double* v0, int ld0) {
+                                            const double* v0) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, r = lane & 7, c0 = (lane >> 3) * 2, c1 = c0 + 1;
   const bool in = r < kk, low = in && r >= 1;
@@ -501,7 +511,7 @@ __device__ __forceinline__ bool newton_root(const double* G, int ld, int kk, dou
   ok = ok && settled && n2 < 1.5 && y0 > 0.5;
   const double inv = rsqrt_nr(n2);
   if constexpr (SYM) {
-    const double v = in ? v0[r * ld0] : 0.0;
+    const double v = in ? v0[r] : 0.0;
     double c = w * inv * v, q = v * v;
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) {
@@ -984,7 +994,7 @@ __device__ __noinline__ bool ducc_block(FSmem<K, true>& sm, const SolveArgs& a, 
 }
 
 template <int K, bool DUCC>
-__global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
+__global__ void __launch_bounds__(FD<K>::NT, DUCC && K == 3 ? 4 : FD<K>::MINB) solve_fixed_kernel(SolveArgs a) {
   using C = FD<K>;
   constexpr int NS = C::NS, NORB = C::NORB, NF = C::NF, NT = C::NT, PER = C::PER;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1028,6 +1038,17 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
     pia[r] = i;
     pib[r] = i + d;
   }
+  // a thread's columns of the subspace vectors and their images: the first SL of them in shared memory
+  constexpr int XL = C::KM > C::SL ? C::KM - C::SL : 1;
+  double vx[XL][PER], sx_[XL][PER];
+  auto getV = [&](int j, int r) -> double {
+    if (j < C::SL) return sm.v.V[j][pd[r]];
+    return vx[C::KM > C::SL ? j - C::SL : 0][r];
+  };
+  auto getS = [&](int j, int r) -> double {
+    if (j < C::SL) return sm.v.S[j][pd[r]];
+    return sx_[C::KM > C::SL ? j - C::SL : 0][r];
+  };
   int buf = 0;
 
   const int64_t nitems = a.count_dev ? (int64_t)*a.count_dev : a.nspaces;
@@ -1205,6 +1226,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
     if (tid == 0) {
       sm.G[0] = 0.0;
       sm.y[0] = 1.0;
+      sm.phi[0] = 1.0;
     }
     int k = 1;             // vectors in the subspace
     double th = 0.0;
@@ -1224,8 +1246,8 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
           double xv = 0.0, sv = 0.0;
 #pragma unroll 1
           for (int j = 0; j < C::KM; ++j) {
-            xv = fma(sm.y[j], sm.v.V[j][pd[r]], xv);
-            sv = fma(sm.y[j], sm.v.S[j][pd[r]], sv);
+            xv = fma(sm.y[j], getV(j, r), xv);
+            sv = fma(sm.y[j], getS(j, r), sv);
           }
           xs[r] = xv;
           ss[r] = sv;
@@ -1240,6 +1262,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
         for (int r = 0; r < PER; ++r)
           if (has[r]) {
             sm.v.V[0][pd[r]] = xs[r] * inv;
+            if (pd[r] == 0) sm.phi[0] = xs[r] * inv;
             sm.v.S[0][pd[r]] = ss[r] * inv;
           }
         __syncthreads();
@@ -1260,8 +1283,8 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
         const double yj = sm.y[j];
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
-          xv[r] = fma(yj, sm.v.V[j][pd[r]], xv[r]);
-          sv[r] = fma(yj, sm.v.S[j][pd[r]], sv[r]);
+          xv[r] = fma(yj, getV(j, r), xv[r]);
+          sv[r] = fma(yj, getS(j, r), sv[r]);
         }
       }
 #pragma unroll
@@ -1280,7 +1303,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
       for (int j = 0; j < C::KM - 1; ++j)
         if (j < k) {
 #pragma unroll
-          for (int r = 0; r < PER; ++r) p1[2 + j] = fma(sm.v.V[j][pd[r]], vk[r], p1[2 + j]);
+          for (int r = 0; r < PER; ++r) p1[2 + j] = fma(getV(j, r), vk[r], p1[2 + j]);
         }
       const double* o = k + 2 <= 8 ? sum_many(sm, reinterpret_cast<double(&)[8]>(p1), k + 2, buf) : sum_many(sm, p1, k + 2, buf);
       const double rn2 = o[0], tt = o[1];
@@ -1301,9 +1324,9 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
         const double q = o[2 + j];
         vn2 = fma(-q, q, vn2);
 #pragma unroll
-        for (int r = 0; r < PER; ++r) vk[r] = fma(-q, sm.v.V[j][pd[r]], vk[r]);
+        for (int r = 0; r < PER; ++r) vk[r] = fma(-q, getV(j, r), vk[r]);
       }
-      if (!(vn2 > 0.01 * tt)) {
+      if (!(vn2 > 0.5 * tt)) {
         double p2[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) p2[j] = 0.0;
@@ -1311,7 +1334,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
         for (int j = 0; j < C::KM - 1; ++j)
           if (j < k) {
 #pragma unroll
-            for (int r = 0; r < PER; ++r) p2[j] = fma(sm.v.V[j][pd[r]], vk[r], p2[j]);
+            for (int r = 0; r < PER; ++r) p2[j] = fma(getV(j, r), vk[r], p2[j]);
           }
         const double* q = sum_many(sm, p2, k, buf);
         double p3[8];
@@ -1320,7 +1343,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
 #pragma unroll 1
-          for (int j = 0; j < k; ++j) vk[r] = fma(-q[j], sm.v.V[j][pd[r]], vk[r]);
+          for (int j = 0; j < k; ++j) vk[r] = fma(-q[j], getV(j, r), vk[r]);
           if (!has[r]) vk[r] = 0.0;
           p3[0] = fma(vk[r], vk[r], p3[0]);
         }
@@ -1336,8 +1359,10 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
 #pragma unroll
       for (int r = 0; r < PER; ++r) {
         vk[r] = has[r] ? vk[r] * inv : 0.0;
+        if (C::KM > C::SL && k >= C::SL) vx[C::KM > C::SL ? k - C::SL : 0][r] = vk[r];
         if (has[r]) {
-          sm.v.V[k][pd[r]] = vk[r];
+          if (C::KM == C::SL || k < C::SL) sm.v.V[k][pd[r]] = vk[r];
+          if (pd[r] == 0) sm.phi[k] = vk[r];
           const int2 c = limbs(to_fix(pia[r] == pib[r] ? vk[r] : vk[r] * kHalfRoot2, 0, kFix));
           sm.Cv[pia[r] * NS + pib[r]] = c;
           sm.Cv[pib[r] * NS + pia[r]] = c;
@@ -1354,7 +1379,8 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
       for (int r = 0; r < PER; ++r) {
         const long long t = sm.T[pia[r] * NS + pib[r]] + sm.T[pib[r] * NS + pia[r]];
         sk[r] = fma(pia[r] == pib[r] ? 0.5 * scale : kHalfRoot2 * scale, (double)t, diag[r] * vk[r]);
-        if (has[r]) sm.v.S[k][pd[r]] = sk[r];
+        if (C::KM > C::SL && k >= C::SL) sx_[C::KM > C::SL ? k - C::SL : 0][r] = sk[r];
+        else if (has[r]) sm.v.S[k][pd[r]] = sk[r];
         p4[0] = fma(vk[r], sk[r], p4[0]);  // vk is zero where there is no pair
       }
 #pragma unroll
@@ -1362,8 +1388,8 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
         if (j < k) {
 #pragma unroll
           for (int r = 0; r < PER; ++r) {
-            p4[1 + 2 * j] = fma(sm.v.V[j][pd[r]], has[r] ? sk[r] : 0.0, p4[1 + 2 * j]);
-            p4[2 + 2 * j] = fma(sm.v.S[j][pd[r]], vk[r], p4[2 + 2 * j]);
+            p4[1 + 2 * j] = fma(getV(j, r), has[r] ? sk[r] : 0.0, p4[1 + 2 * j]);
+            p4[2 + 2 * j] = fma(getS(j, r), vk[r], p4[2 + 2 * j]);
           }
         }
       }
@@ -1376,7 +1402,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
         if (lane == k) sm.G[k * C::KM + k] = g[0];
         __syncwarp();
         double thn = th;
-        const bool ok = newton_root<DUCC>(sm.G, C::KM, k + 1, th, sm.y, &thn, &sm.v.V[0][0], C::NP);
+        const bool ok = newton_root<DUCC>(sm.G, C::KM, k + 1, th, sm.y, &thn, sm.phi);
         if (lane == 0) {
           sm.theta = thn;
           if (!ok) sm.flag[1] = 1;
@@ -1406,7 +1432,7 @@ __global__ void __launch_bounds__(FD<K>::NT) solve_fixed_kernel(SolveArgs a) {
     for (int r = 0; r < PER; ++r) {
       double xv = 0.0;
 #pragma unroll 1
-      for (int j = 0; j < k; ++j) xv = fma(sm.y[j], sm.v.V[j][pd[r]], xv);
+      for (int j = 0; j < k; ++j) xv = fma(sm.y[j], getV(j, r), xv);
       if (has[r]) {
         const double x = pia[r] == pib[r] ? xv : xv * kHalfRoot2;
         xf[pia[r] * NS + pib[r]] = x;
