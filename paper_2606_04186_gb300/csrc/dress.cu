@@ -158,7 +158,7 @@ __device__ __forceinline__ size_t t1_index(const Dims& d, int p, size_t rest) {
 }
 
 template <typename A, int POS>
-__global__ void __launch_bounds__(TPB, sizeof(A) == 4 ? kT1Blocks + 1 : 1) k_t1_creator_fast(double* __restrict__ W, const double* __restrict__ t1, Dims d) {
+__global__ void __launch_bounds__(TPB, kT1Blocks + 1) k_t1_creator_fast(double* __restrict__ W, const double* __restrict__ t1, Dims d) {
   extern __shared__ __align__(16) double t1raw[];  // [v][kT1Omax], in the accumulation type
   A* t1s = reinterpret_cast<A*>(t1raw);
   load_t1_t<A>(t1, t1s, d);
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(TPB, sizeof(A) == 4 ? kT1Blocks + 1 : 1) k_t1_
 // of W (occupied rows unchanged, virtual rows corrected), so no separate copy pass reads and
 // writes W first.  Same arithmetic as k_t1_creator_fast at POS 0.
 template <typename A>
-__global__ void __launch_bounds__(TPB, sizeof(A) == 4 ? kT1Blocks : 1) k_t1_creator_copy(const double* __restrict__ src, double* __restrict__ W, const double* __restrict__ t1,
+__global__ void __launch_bounds__(TPB, kT1Blocks) k_t1_creator_copy(const double* __restrict__ src, double* __restrict__ W, const double* __restrict__ t1,
                                   Dims d) {
   extern __shared__ __align__(16) double t1raw[];  // [v][kT1Omax], in the accumulation type
   A* t1s = reinterpret_cast<A*>(t1raw);
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(TPB, sizeof(A) == 4 ? kT1Blocks : 1) k_t1_crea
 }
 
 template <typename A, int POS>
-__global__ void __launch_bounds__(TPB, sizeof(A) == 4 ? kT1Blocks : 1) k_t1_annihilator_fast(double* __restrict__ W, const double* __restrict__ t1, Dims d) {
+__global__ void __launch_bounds__(TPB, kT1Blocks) k_t1_annihilator_fast(double* __restrict__ W, const double* __restrict__ t1, Dims d) {
   extern __shared__ __align__(16) double t1raw[];  // [v][kT1Omax], in the accumulation type
   A* t1s = reinterpret_cast<A*>(t1raw);
   load_t1_t<A>(t1, t1s, d);
@@ -238,17 +238,200 @@ __global__ void __launch_bounds__(TPB, sizeof(A) == 4 ? kT1Blocks : 1) k_t1_anni
   }
 }
 
+// FP64 passes on fixed-point products (fixed.cuh), o <= kT1Omax: the sums of a thread's triple share a
+// power-of-two scale taken from the values it reads, t1 one from its largest element, so a term is
+// exact to 2^-54 of the triple's largest element and the sums are exact.  The FP64 form of these
+// passes is bound by the FP64 pipe (0.4 G FMAs each at 82 orbitals: 1.15-1.2 ms against 0.11 ms of HBM
+// time); here a term is three mad.wide and an output element two FP64 operations.
+constexpr int kT1Bits = 54;
+
+// t1 in shared memory, transposed and padded with zeros: limbs t1s[a][0..16) in units of 2^(st - 54).
+// Returns false (every thread) when t1 has a non-finite element.
+__device__ __forceinline__ bool load_t1_fixed(const double* __restrict__ t1, int2* t1s, const Dims& d, int* st) {
+  __shared__ unsigned top;
+  if (threadIdx.x == 0) top = 0;
+  __syncthreads();
+  unsigned mx = 0;
+  for (int x = threadIdx.x; x < d.o * d.v; x += blockDim.x) mx = max(mx, (unsigned)__double2hiint(t1[x]) & 0x7fffffffu);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0) atomicMax(&top, mx);
+  __syncthreads();
+  mx = top;
+  const int e = (int)(mx >> 20);
+  *st = e > 0 ? e - 1022 : 0;
+  if (e == 0x7ff) return false;
+  for (int x = threadIdx.x; x < d.v * kT1Omax; x += blockDim.x) {
+    const int a = x / kT1Omax, i = x % kT1Omax;
+    t1s[x] = (i < d.o) ? limbs(to_fix(t1[i * d.v + a], *st, kT1Bits)) : make_int2(0, 0);
+  }
+  __syncthreads();
+  return true;
+}
+// 2^(sx + st - 54) within the double range (a scale below it belongs to sums below 1e-290)
+__device__ __forceinline__ double t1_unit(int sx, int st) {
+  const int e = sx + st - kT1Bits;
+  return pow2(e < -1021 ? -1021 : e > 1020 ? 1020 : e);
+}
+
+// Creator pass at POS: rows nocc + a get - sum_i t1[i][a] row_i; COPY: read from src, every row written.
+template <int POS, bool COPY>
+__global__ void __launch_bounds__(TPB, 2) k_t1_creator_fixed(const double* __restrict__ src, double* __restrict__ W,
+                                                              const double* __restrict__ t1, Dims d) {
+  extern __shared__ __align__(16) double t1raw[];
+  int2* t1s = reinterpret_cast<int2*>(t1raw);
+  int st;
+  const bool fine = load_t1_fixed(t1, t1s, d, &st);
+  const double* in = COPY ? src : W;
+  const size_t m = (size_t)d.n * d.n * d.n;
+  const size_t step = t1_index<double, POS>(d, 1, 0);  // distance of neighbouring rows
+  for (size_t rest = blockIdx.x * (size_t)blockDim.x + threadIdx.x; rest < m; rest += (size_t)gridDim.x * blockDim.x) {
+    const size_t base = t1_index<double, POS>(d, 0, rest);
+    int2 w[kT1Omax];
+    int sx;
+    bool ok = fine;
+    {
+      double x[kT1Omax];
+      unsigned mx = 0;
+#pragma unroll
+      for (int i = 0; i < kT1Omax; ++i) {
+        x[i] = 0.0;
+        if (i < d.o) {
+          x[i] = in[base + i * step];
+          if (COPY) W[base + i * step] = x[i];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kT1Omax; ++i) mx = max(mx, (unsigned)__double2hiint(x[i]) & 0x7fffffffu);
+      const int e = (int)(mx >> 20);
+      sx = e > 0 ? e - 1022 : 0;
+      ok = ok && e < 0x7ff;
+#pragma unroll
+      for (int i = 0; i < kT1Omax; ++i) w[i] = limbs(to_fix(x[i], sx, kT1Bits));
+    }
+    const size_t vb = base + d.o * step;
+    if (!ok) {  // NaN or infinity: plain sums
+      for (int a = 0; a < d.v; ++a) {
+        double acc = 0.0;
+        for (int i = 0; i < d.o; ++i) acc += t1[i * d.v + a] * in[base + i * step];
+        W[vb + a * step] = in[vb + a * step] - acc;
+      }
+      continue;
+    }
+    const double unit = t1_unit(sx, st);
+    constexpr int U = 8;  // rows whose loads are in flight
+    for (int a0 = 0; a0 < d.v; a0 += U) {
+      double x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) x[u] = a0 + u < d.v ? in[vb + (a0 + u) * step] : 0.0;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (a0 + u >= d.v) break;
+        const int4* c = reinterpret_cast<const int4*>(t1s + (a0 + u) * kT1Omax);
+        long long hh = 0, x0 = 0, x1 = 0;
+#pragma unroll
+        for (int i = 0; i < kT1Omax; i += 2) {
+          if (i < d.o) {
+            const int4 q = c[i / 2];
+            madw(hh, q.x, w[i].x);
+            madw(x0, q.x, w[i].y);
+            madw(x1, q.y, w[i].x);
+            madw(hh, q.z, w[i + 1].x);
+            madw(x0, q.z, w[i + 1].y);
+            madw(x1, q.w, w[i + 1].x);
+          }
+        }
+        W[vb + (a0 + u) * step] = fma(-unit, (double)join(hh, x0 + x1), x[u]);
+      }
+    }
+  }
+}
+
+// Annihilator pass at POS: rows q < nocc get + sum_a t1[q][a] row_(nocc + a).
+template <int POS>
+__global__ void __launch_bounds__(TPB, 2) k_t1_annihilator_fixed(double* __restrict__ W, const double* __restrict__ t1, Dims d) {
+  extern __shared__ __align__(16) double t1raw[];
+  int2* t1s = reinterpret_cast<int2*>(t1raw);
+  int st;
+  const bool fine = load_t1_fixed(t1, t1s, d, &st);
+  const size_t m = (size_t)d.n * d.n * d.n;
+  const size_t step = t1_index<double, POS>(d, 1, 0);
+  constexpr int U = 12;  // rows read at a time; they share a scale
+  for (size_t rest = blockIdx.x * (size_t)blockDim.x + threadIdx.x; rest < m; rest += (size_t)gridDim.x * blockDim.x) {
+    const size_t base = t1_index<double, POS>(d, 0, rest), vb = base + d.o * step;
+    double acc[kT1Omax];
+#pragma unroll
+    for (int q = 0; q < kT1Omax; ++q) acc[q] = 0.0;
+    for (int a0 = 0; a0 < d.v; a0 += U) {
+      int2 w[U];
+      int sx;
+      bool ok = fine;
+      {
+        double x[U];
+        unsigned mx = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) x[u] = a0 + u < d.v ? W[vb + (a0 + u) * step] : 0.0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) mx = max(mx, (unsigned)__double2hiint(x[u]) & 0x7fffffffu);
+        const int e = (int)(mx >> 20);
+        sx = e > 0 ? e - 1022 : 0;
+        ok = ok && e < 0x7ff;
+#pragma unroll
+        for (int u = 0; u < U; ++u) w[u] = limbs(to_fix(x[u], sx, kT1Bits));
+      }
+      const double unit = t1_unit(sx, st);
+#pragma unroll
+      for (int q = 0; q < kT1Omax; q += 2) {
+        if (q < d.o) {
+          if (ok) {
+            long long h0 = 0, h1 = 0, x0 = 0, x1 = 0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              if (a0 + u < d.v) {
+                const int4 c = reinterpret_cast<const int4*>(t1s + (a0 + u) * kT1Omax)[q / 2];
+                madw(h0, c.x, w[u].x);
+                madw(x0, c.x, w[u].y);
+                madw(x0, c.y, w[u].x);
+                madw(h1, c.z, w[u].x);
+                madw(x1, c.z, w[u].y);
+                madw(x1, c.w, w[u].x);
+              }
+            }
+            acc[q] = fma(unit, (double)join(h0, x0), acc[q]);
+            acc[q + 1] = fma(unit, (double)join(h1, x1), acc[q + 1]);
+          } else {
+            for (int u = 0; u < U && a0 + u < d.v; ++u) {
+              acc[q] += t1[q * d.v + a0 + u] * W[vb + (a0 + u) * step];
+              if (q + 1 < d.o) acc[q + 1] += t1[(q + 1) * d.v + a0 + u] * W[vb + (a0 + u) * step];
+            }
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kT1Omax; ++q)
+      if (q < d.o) W[base + q * step] += acc[q];
+  }
+}
+
 template <typename A>
 void t1_passes(const double* eri, double* W, const double* t1, const Dims& d, cudaStream_t st) {
   const size_t mc = (size_t)d.v * d.n * d.n * d.n, ma = (size_t)d.o * d.n * d.n * d.n;
   const size_t n3 = (size_t)d.n * d.n * d.n;
   if (d.o <= kT1Omax) {
-    const size_t sm = sizeof(A) * kT1Omax * d.v;
     const unsigned g = blocks_for(n3) > 152u * 16u ? 152u * 16u : blocks_for(n3);
-    k_t1_creator_copy<A><<<g, TPB, sm, st>>>(eri, W, t1, d);
-    k_t1_creator_fast<A, 2><<<g, TPB, sm, st>>>(W, t1, d);
-    k_t1_annihilator_fast<A, 1><<<g, TPB, sm, st>>>(W, t1, d);
-    k_t1_annihilator_fast<A, 3><<<g, TPB, sm, st>>>(W, t1, d);
+    if constexpr (sizeof(A) == 8) {
+      const size_t fm = sizeof(int2) * kT1Omax * d.v;
+      k_t1_creator_fixed<0, true><<<g, TPB, fm, st>>>(eri, W, t1, d);
+      k_t1_creator_fixed<2, false><<<g, TPB, fm, st>>>(nullptr, W, t1, d);
+      k_t1_annihilator_fixed<1><<<g, TPB, fm, st>>>(W, t1, d);
+      k_t1_annihilator_fixed<3><<<g, TPB, fm, st>>>(W, t1, d);
+    } else {
+      const size_t sm = sizeof(A) * kT1Omax * d.v;
+      k_t1_creator_copy<A><<<g, TPB, sm, st>>>(eri, W, t1, d);
+      k_t1_creator_fast<A, 2><<<g, TPB, sm, st>>>(W, t1, d);
+      k_t1_annihilator_fast<A, 1><<<g, TPB, sm, st>>>(W, t1, d);
+      k_t1_annihilator_fast<A, 3><<<g, TPB, sm, st>>>(W, t1, d);
+    }
   } else {
     const size_t n4 = n3 * d.n;
     k_copy<<<blocks_for(n4) > 152u * 64u ? 152u * 64u : blocks_for(n4), TPB, 0, st>>>(eri, W, n4);

@@ -29,7 +29,7 @@ def _dress(qf, h, g, t1, t2, no):
     return e0.item(), F.cpu().numpy(), W.cpu().numpy()
 
 
-@pytest.mark.parametrize("n,no", [(2, 1), (5, 1), (5, 4), (9, 8), (11, 3), (13, 6), (17, 2), (20, 9), (29, 5), (33, 8)])
+@pytest.mark.parametrize("n,no", [(2, 1), (5, 1), (5, 4), (9, 8), (11, 3), (13, 6), (17, 2), (20, 9), (20, 16), (22, 17), (29, 5), (33, 8)])
 def test_dressing_at_tile_edges(n, no):
     qf = library()
     _, h, g = synth.make_system(n, no, 4.0, 100 + n)
