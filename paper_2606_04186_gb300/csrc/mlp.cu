@@ -20,10 +20,16 @@
 #include <stdint.h>
 
 #include "qflow_internal.h"
+#include "rows_gemm.cuh"
 #include "tc_gemm.cuh"
 
 namespace qf {
 namespace {
+
+unsigned grid1(int64_t n, int threads) {
+  const int64_t g = (n + threads - 1) / threads;
+  return (unsigned)(g < 1 ? 1 : (g > 65536 ? 65536 : g));
+}
 
 // ---- matrix products on the tensor cores, with fused epilogues --------------------------------
 // C[M][N] = op(A) op(B) through the repo's tcgen05 engine (three-term TF32 products, FP32
@@ -53,35 +59,186 @@ struct StoreEpi {
     else if (EPI == kTanhGrad) v = v * (1.f - aux[x] * aux[x]);
     C[x] = v;
   }
+  // 32 consecutive columns of a row (cnt of them in range), in 16-byte stores where they are aligned
+  __device__ void run(int m, int n, const float (&v)[32], int cnt) const {
+    const size_t x = (size_t)m * ldc + n;
+    const bool wide = cnt == 32 && ((reinterpret_cast<uintptr_t>(C + x) | (EPI == kTanhGrad ? reinterpret_cast<uintptr_t>(aux + x) : 0)) & 15u) == 0;
+    if (wide) {
+#pragma unroll
+      for (int j = 0; j < 32; j += 4) {
+        float r[4];
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (EPI == kTanhGrad) a = *reinterpret_cast<const float4*>(aux + x + j);
+        const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          r[i] = v[j + i];
+          if (EPI == kBiasTanh) r[i] = tanhf(r[i] + bias[n + j + i]);
+          else if (EPI == kBias) r[i] = r[i] + bias[n + j + i];
+          else if (EPI == kTanhGrad) r[i] = r[i] * (1.f - av[i] * av[i]);
+        }
+        *reinterpret_cast<float4*>(C + x + j) = make_float4(r[0], r[1], r[2], r[3]);
+      }
+      return;
+    }
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (j < cnt) (*this)(m, n + j, v[j]);
+  }
 };
 
 __global__ void k_mlp_check(const int* __restrict__ err, float* __restrict__ y) {
   if (threadIdx.x == 0 && *err) y[0] = __int_as_float(0x7fc00000);
 }
 
+// out[c] = sum over rows r (ascending) of X[r][c]
+__global__ void k_colsum(const float* __restrict__ X, int rows, int cols, int ld, float* __restrict__ out) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= cols) return;
+  float s = 0.f;
+  for (int r = 0; r < rows; ++r) s += X[(size_t)r * ld + c];
+  out[c] = s;
+}
+
+// ---- small products: FP32 FMA tiles -------------------------------------------------------------
+// A training step multiplies 128-row batches: at most 4 x 4 tensor-core tiles with K up to 708, so the
+// tensor-core engines leave most SMs idle and run K serially (30-90 us a product).  Here a CTA owns a
+// 32 x 32 tile and its eight warps share every 64-k slab (eight k each, 4 x 8 outputs per lane, the
+// partial tiles summed in warp order at the end): 32 to 184 CTAs per product.  The next slab is in
+// registers while this one is multiplied.  With `colsum` (B's column sums, the bias gradient) the CTAs of
+// the first row tile also add up B.
+constexpr int ST = 32, SK = 64, STP = ST + 4;
+
+template <bool TA, bool TB, int EPI>
+__global__ void __launch_bounds__(256) k_gemm_small(int M, int N, int K, const float* __restrict__ A, int lda,
+                                                    const float* __restrict__ B, int ldb, StoreEpi<EPI> st,
+                                                    float* __restrict__ colsum) {
+  // the slabs, then (after the last one) the warps' partial tiles in the same place
+  __shared__ __align__(16) float raw[8 * ST * (ST + 1)];
+  static_assert(2 * SK * STP <= 8 * ST * (ST + 1), "slabs fit the partial tiles' place");
+  float(*as)[STP] = reinterpret_cast<float(*)[STP]>(raw);
+  float(*bs)[STP] = reinterpret_cast<float(*)[STP]>(raw + SK * STP);
+  float(*part)[ST][ST + 1] = reinterpret_cast<float(*)[ST][ST + 1]>(raw);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m0 = blockIdx.y * ST, n0 = blockIdx.x * ST;
+  const int lm = (lane >> 2) * 4, ln = (lane & 3) * 8;
+  const bool sums = colsum != nullptr && blockIdx.y == 0;
+  float acc[4][8], cs[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    cs[j] = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i][j] = 0.f;
+  }
+  // element (row, k) of an operand slab for this thread's x-th load: along k where k is contiguous
+  float ra[8], rb[8];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+      const int t = tid + x * 256;
+      {
+        const int r = TA ? t % ST : t / SK, k = TA ? t / ST : t % SK;
+        const bool in = m0 + r < M && k0 + k < K;
+        ra[x] = in ? (TA ? A[(size_t)(k0 + k) * lda + m0 + r] : A[(size_t)(m0 + r) * lda + k0 + k]) : 0.f;
+      }
+      {
+        const int r = TB ? t / SK : t % ST, k = TB ? t % SK : t / ST;
+        const bool in = n0 + r < N && k0 + k < K;
+        rb[x] = in ? (TB ? B[(size_t)(n0 + r) * ldb + k0 + k] : B[(size_t)(k0 + k) * ldb + n0 + r]) : 0.f;
+      }
+    }
+  };
+  load(0);
+  for (int k0 = 0; k0 < K; k0 += SK) {
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+      const int t = tid + x * 256;
+      as[TA ? t / ST : t % SK][TA ? t % ST : t / SK] = ra[x];
+      bs[TB ? t % SK : t / ST][TB ? t / SK : t % ST] = rb[x];
+    }
+    __syncthreads();
+    if (k0 + SK < K) load(k0 + SK);
+#pragma unroll
+    for (int q = 0; q < SK / 8; ++q) {
+      const int k = warp * (SK / 8) + q;
+      const float4 a4 = *reinterpret_cast<const float4*>(&as[k][lm]);
+      const float4 b0 = *reinterpret_cast<const float4*>(&bs[k][ln]), b1 = *reinterpret_cast<const float4*>(&bs[k][ln + 4]);
+      const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+      if (sums) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) cs[j] += bv[j];
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) part[warp][lm + i][ln + j] = acc[i][j];
+  __syncthreads();
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    const int t = tid + x * 256, r = t / ST, c = t % ST;
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) v += part[w][r][c];
+    if (m0 + r < M && n0 + c < N) st(m0 + r, n0 + c, v);
+  }
+  if (sums) {
+    __syncthreads();
+    if (lm == 0) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) part[0][warp][ln + j] = cs[j];
+    }
+    __syncthreads();
+    if (tid < ST && n0 + tid < N) {
+      float v = 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) v += part[0][w][tid];
+      colsum[n0 + tid] = v;
+    }
+  }
+}
+
+// Rows (of a batch) up to which the FMA tiles are the faster form: forward products of 708 x 256 at
+// 1,024 rows 20 us, on the tensor cores 23 us; the weight gradients' sums (K = rows) up to 8,192.
+constexpr int kSmallRows = 1024, kSmallSum = 8192;
+
+// C = op(A) op(B) with the epilogue; colsum (nullable): B's column sums.  `pack`: scratch for the split
+// weights of the row-streaming engine (op(B) is a weight matrix there), nullable where the call never
+// takes it (op(A) transposed).
 template <bool TA, bool TB, int EPI>
 cudaError_t gemm(int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C, int ldc,
-                 const float* bias, const float* aux, int* err, cudaStream_t st) {
+                 const float* bias, const float* aux, float* colsum, float* pack, int* err, cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
+  const StoreEpi<EPI> sv{C, ldc, bias, aux};
+  if (TA ? K <= kSmallSum : M <= kSmallRows) {
+    const dim3 g((unsigned)((N + ST - 1) / ST), (unsigned)((M + ST - 1) / ST));
+    k_gemm_small<TA, TB, EPI><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, sv, colsum);
+    return cudaGetLastError();
+  }
+  if (colsum) {
+    k_colsum<<<grid1(N, 128), 128, 0, st>>>(B, K, N, ldb, colsum);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  const LoadOp<!TB> lb{B, ldb};
+  if constexpr (!TA) {
+    if (tc::rows_streamable(A, lda)) return tc::gemm_rows(M, N, K, A, lda, lb, sv, pack, err, st);
+  }
   // the engine forms sum_k a(m, k) b(n, k): op(B)^T element (n, k) is B[k][n], or B[n][k] when TB.
   // Tile width: the widest that N fills while the tiles still cover every SM (op(A) streamed
   // fewer times); products with few 128-row tiles (the weight gradients, K = rows) take 64.
   const LoadOp<TA> la{A, lda};
-  const LoadOp<!TB> lb{B, ldb};
-  const StoreEpi<EPI> sv{C, ldc, bias, aux};
   const int mt = (M + 127) / 128;
   if (N > 128 && mt * ((N + 255) / 256) >= 152) return tc::gemm_tf32x3<256>(M, N, K, la, lb, sv, err, st);
   if (N > 64 && mt * ((N + 127) / 128) >= 152) return tc::gemm_tf32x3<128>(M, N, K, la, lb, sv, err, st);
   return tc::gemm_tf32x3<64>(M, N, K, la, lb, sv, err, st);
-}
-
-// out[c] = sum over rows r (ascending) of X[r][c]
-__global__ void k_colsum(const float* __restrict__ X, int rows, int cols, float* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  float s = 0.f;
-  for (int r = 0; r < rows; ++r) s += X[(size_t)r * cols + c];
-  out[c] = s;
 }
 
 constexpr int LB = 256;    // threads of the loss kernel
@@ -394,11 +551,6 @@ __global__ void k_rows(const float* __restrict__ X, int64_t rows, int cols, cons
   }
 }
 
-unsigned grid1(int64_t n, int threads) {
-  const int64_t g = (n + threads - 1) / threads;
-  return (unsigned)(g < 1 ? 1 : (g > 65536 ? 65536 : g));
-}
-
 struct Net {
   int I, H, O;
   const float *W1, *b1, *W2, *b2, *W3, *b3;
@@ -416,29 +568,58 @@ struct Net {
 
 int64_t mlp_param_count(int I, int H, int O) { return (int64_t)I * H + H + (int64_t)H * H + H + (int64_t)H * O + O; }
 
-size_t mlp_workspace_bytes(int I, int H, int O, int64_t rows) {
-  (void)I;
-  // H1, H2, dZ (rows x H each), Y, dY (rows x O each), loss partials + loss
-  return sizeof(float) * ((size_t)rows * (3 * (size_t)H + 2 * (size_t)O) + LGRID + 4) + 512;
-}
-// the products' timeout flag: the workspace's last 256 bytes
-int* mlp_err(void* work, int I, int H, int O, int64_t rows) {
-  return reinterpret_cast<int*>(static_cast<char*>(work) + mlp_workspace_bytes(I, H, O, rows) - 256);
-}
+namespace {
+
+// Row pitch of the hidden activations: rows start on 16 bytes, so TMA can read them.
+int hidden_pitch(int H) { return (H + 3) / 4 * 4; }
+
+// Workspace: H1, H2, dZ (rows x pitch each), Y, dY (rows x O each), loss partials, the split weights of
+// the row-streaming products, the products' timeout flag (the last 256 bytes).
+struct MlpWork {
+  float *H1, *H2, *dZ, *Y, *dY, *part, *pack;
+  int* err;
+  size_t bytes;
+  MlpWork(void* work, int I, int H, int O, int64_t rows) {
+    const size_t h = (size_t)rows * hidden_pitch(H), y = (size_t)rows * O;
+    const int wide = H > O ? H : O;
+    const size_t pk = rows > kSmallRows ? tc::rows_pack_floats(wide, I > wide ? I : wide) : 0;
+    size_t off = 0;
+    auto take = [&](size_t floats) {
+      float* p = work ? reinterpret_cast<float*>(static_cast<char*>(work) + off) : nullptr;
+      off += (floats * sizeof(float) + 255) / 256 * 256;
+      return p;
+    };
+    H1 = take(h);
+    H2 = take(h);
+    dZ = take(h);
+    Y = take(y);
+    dY = take(y);
+    part = take(LGRID + 4);
+    pack = take(pk);
+    err = reinterpret_cast<int*>(take(64));
+    bytes = off;
+  }
+};
+
+}  // namespace
+
+size_t mlp_workspace_bytes(int I, int H, int O, int64_t rows) { return MlpWork(nullptr, I, H, O, rows).bytes; }
 
 cudaError_t mlp_forward(int I, int H, int O, const float* params, const float* x, int64_t rows, float* y, void* work,
                         cudaStream_t st) {
   const Net net(I, H, O, params);
-  float* H1 = static_cast<float*>(work);
-  float* H2 = H1 + (size_t)rows * H;
-  const int R = (int)rows;
-  int* err = mlp_err(work, I, H, O, rows);
-  cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), st);
-  if (e == cudaSuccess) e = gemm<false, false, kBiasTanh>(R, H, I, x, I, net.W1, H, H1, H, net.b1, nullptr, err, st);
-  if (e == cudaSuccess) e = gemm<false, false, kBiasTanh>(R, H, H, H1, H, net.W2, H, H2, H, net.b2, nullptr, err, st);
-  if (e == cudaSuccess) e = gemm<false, false, kBias>(R, O, H, H2, H, net.W3, O, y, O, net.b3, nullptr, err, st);
-  if (e == cudaSuccess && R > 0) {
-    k_mlp_check<<<1, 32, 0, st>>>(err, y);
+  const MlpWork w(work, I, H, O, rows);
+  const int R = (int)rows, P = hidden_pitch(H);
+  const bool flag = R > kSmallRows;  // the FMA tiles wait on nothing
+  cudaError_t e = flag ? cudaMemsetAsync(w.err, 0, sizeof(int), st) : cudaSuccess;
+  if (e == cudaSuccess)
+    e = gemm<false, false, kBiasTanh>(R, H, I, x, I, net.W1, H, w.H1, P, net.b1, nullptr, nullptr, w.pack, w.err, st);
+  if (e == cudaSuccess)
+    e = gemm<false, false, kBiasTanh>(R, H, H, w.H1, P, net.W2, H, w.H2, P, net.b2, nullptr, nullptr, w.pack, w.err, st);
+  if (e == cudaSuccess)
+    e = gemm<false, false, kBias>(R, O, H, w.H2, P, net.W3, O, y, O, net.b3, nullptr, nullptr, w.pack, w.err, st);
+  if (e == cudaSuccess && R > 0 && flag) {
+    k_mlp_check<<<1, 32, 0, st>>>(w.err, y);
     e = cudaGetLastError();
   }
   return e;
@@ -447,43 +628,42 @@ cudaError_t mlp_forward(int I, int H, int O, const float* params, const float* x
 cudaError_t mlp_loss_grad(int I, int H, int O, const float* params, const float* x, const float* t,
                           const uint8_t* mask, int64_t rows, float* grad, float* loss, void* work, cudaStream_t st) {
   const Net net(I, H, O, params);
-  const int R = (int)rows;
-  float* H1 = static_cast<float*>(work);
-  float* H2 = H1 + (size_t)rows * H;
-  float* dZ = H2 + (size_t)rows * H;
-  float* Y = dZ + (size_t)rows * H;
-  float* dY = Y + (size_t)rows * O;
-  float* part = dY + (size_t)rows * O;
+  const MlpWork w(work, I, H, O, rows);
+  const int R = (int)rows, P = hidden_pitch(H);
   float* gW1 = grad;
   float* gb1 = gW1 + (size_t)I * H;
   float* gW2 = gb1 + H;
   float* gb2 = gW2 + (size_t)H * H;
   float* gW3 = gb2 + H;
   float* gb3 = gW3 + (size_t)H * O;
-  int* err = mlp_err(work, I, H, O, rows);
-  cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), st);
-  if (e == cudaSuccess) e = gemm<false, false, kBiasTanh>(R, H, I, x, I, net.W1, H, H1, H, net.b1, nullptr, err, st);
-  if (e == cudaSuccess) e = gemm<false, false, kBiasTanh>(R, H, H, H1, H, net.W2, H, H2, H, net.b2, nullptr, err, st);
-  if (e == cudaSuccess) e = gemm<false, false, kBias>(R, O, H, H2, H, net.W3, O, Y, O, net.b3, nullptr, err, st);
+  const bool flag = R > kSmallRows;
+  cudaError_t e = flag ? cudaMemsetAsync(w.err, 0, sizeof(int), st) : cudaSuccess;
+  if (e == cudaSuccess)
+    e = gemm<false, false, kBiasTanh>(R, H, I, x, I, net.W1, H, w.H1, P, net.b1, nullptr, nullptr, w.pack, w.err, st);
+  if (e == cudaSuccess)
+    e = gemm<false, false, kBiasTanh>(R, H, H, w.H1, P, net.W2, H, w.H2, P, net.b2, nullptr, nullptr, w.pack, w.err, st);
+  if (e == cudaSuccess)
+    e = gemm<false, false, kBias>(R, O, H, w.H2, P, net.W3, O, w.Y, O, net.b3, nullptr, nullptr, w.pack, w.err, st);
   if (e != cudaSuccess) return e;
-  k_loss_grad<<<LGRID, LB, 0, st>>>(Y, t, mask, R, O, dY, part);
-  k_loss_final<<<1, 32, 0, st>>>(part, R, loss);
+  k_loss_grad<<<LGRID, LB, 0, st>>>(w.Y, t, mask, R, O, w.dY, w.part);
+  k_loss_final<<<1, 32, 0, st>>>(w.part, R, loss);
   // layer 3: gW3 = H2^T dY, gb3 = colsum dY, dZ2 = (dY W3^T) (1 - H2^2)
-  e = gemm<true, false, kStore>(H, O, R, H2, H, dY, O, gW3, O, nullptr, nullptr, err, st);
-  if (e != cudaSuccess) return e;
-  k_colsum<<<grid1(O, 128), 128, 0, st>>>(dY, R, O, gb3);
-  e = gemm<false, true, kTanhGrad>(R, H, O, dY, O, net.W3, O, dZ, H, nullptr, H2, err, st);
+  e = gemm<true, false, kStore>(H, O, R, w.H2, P, w.dY, O, gW3, O, nullptr, nullptr, gb3, nullptr, w.err, st);
+  if (e == cudaSuccess)
+    e = gemm<false, true, kTanhGrad>(R, H, O, w.dY, O, net.W3, O, w.dZ, P, nullptr, w.H2, nullptr, w.pack, w.err, st);
   // layer 2: gW2 = H1^T dZ2, gb2 = colsum dZ2, dZ1 = (dZ2 W2^T) (1 - H1^2) (into H2's buffer)
-  if (e == cudaSuccess) e = gemm<true, false, kStore>(H, H, R, H1, H, dZ, H, gW2, H, nullptr, nullptr, err, st);
-  if (e != cudaSuccess) return e;
-  k_colsum<<<grid1(H, 128), 128, 0, st>>>(dZ, R, H, gb2);
-  e = gemm<false, true, kTanhGrad>(R, H, H, dZ, H, net.W2, H, H2, H, nullptr, H1, err, st);
+  if (e == cudaSuccess)
+    e = gemm<true, false, kStore>(H, H, R, w.H1, P, w.dZ, P, gW2, H, nullptr, nullptr, gb2, nullptr, w.err, st);
+  if (e == cudaSuccess)
+    e = gemm<false, true, kTanhGrad>(R, H, H, w.dZ, P, net.W2, H, w.H2, P, nullptr, w.H1, nullptr, w.pack, w.err, st);
   // layer 1: gW1 = X^T dZ1, gb1 = colsum dZ1
-  if (e == cudaSuccess) e = gemm<true, false, kStore>(I, H, R, x, I, H2, H, gW1, H, nullptr, nullptr, err, st);
-  if (e != cudaSuccess) return e;
-  k_colsum<<<grid1(H, 128), 128, 0, st>>>(H2, R, H, gb1);
-  k_mlp_check<<<1, 32, 0, st>>>(err, loss);  // a failed product shows as a NaN loss
-  return cudaGetLastError();
+  if (e == cudaSuccess)
+    e = gemm<true, false, kStore>(I, H, R, x, I, w.H2, P, gW1, H, nullptr, nullptr, gb1, nullptr, w.err, st);
+  if (e == cudaSuccess && flag) {
+    k_mlp_check<<<1, 32, 0, st>>>(w.err, loss);  // a failed product shows as a NaN loss
+    e = cudaGetLastError();
+  }
+  return e;
 }
 
 cudaError_t mlp_adam(int64_t n, float* p, const float* g, float* m, float* v, int step, float lr, float b1, float b2,
