@@ -360,11 +360,13 @@ int qflow_fma_peak(int32_t precision, double* tflops, void* stream);
  *
  * qflow_dress_device_static computes exactly what qflow_dress_device computes (same kernels,
  * same arguments except the workspace) but takes its scratch from a static device array of
- * QFLOW_STATIC_SCRATCH_BYTES bytes inside the library, so the call allocates nothing (no
+ * qflow_static_scratch_bytes() bytes inside the library, so the call allocates nothing (no
  * cudaMalloc, no cudaFree, no allocating library routine).  The array is held by every GPU
  * that loads the library until the process exits.
- *   - Limit: the call returns QFLOW_ERR_TOO_LARGE when qflow_dress_workspace(n, nocc) exceeds
- *     QFLOW_STATIC_SCRATCH_BYTES (4 MiB, e.g. 40 orbitals with 6 occupied fit, 82 do not).
+ *   - Limit: the call returns QFLOW_ERR_TOO_LARGE when its arrays (about 48 nocc^2 nvir^2 bytes)
+ *     exceed QFLOW_STATIC_SCRATCH_BYTES (4 MiB, e.g. 40 orbitals with 6 occupied fit, 82 do not).
+ *     qflow_dress_workspace(n, nocc) can be larger: with it the larger problems' products run on
+ *     operands packed for the tensor cores, here always without (equal up to FP64 rounding).
  *   - Set-up: the first call on a device looks up the device address of the array on that
  *     device (with it current) and keeps it for that device's current context; make that first
  *     call before any stream capture.  A call that would do the look-up while `stream` is
@@ -379,7 +381,7 @@ int qflow_fma_peak(int32_t precision, double* tflops, void* stream);
 #define QFLOW_STATIC_SCRATCH_BYTES (4u * 1024u * 1024u)
 int qflow_dress_device_static(const double* h, const double* eri, const double* t1, const double* t2, int32_t n,
                               int32_t nocc, double* e0, double* F, double* W, void* stream);
-/* Size of that static scratch array in bytes. */
+/* Size of that static scratch array in bytes (the limit, and room for scale factors). */
 size_t qflow_static_scratch_bytes(void);
 
 /* ---- warm-start network (not in the paper) -----------------------------------------------

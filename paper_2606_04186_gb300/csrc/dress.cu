@@ -21,6 +21,7 @@
 #include <stdint.h>
 
 #include "fix_gemm.cuh"
+#include "oz_gemm.cuh"
 #include "qflow_internal.h"
 #include "tc_gemm.cuh"
 
@@ -645,11 +646,14 @@ __global__ void k_finalize(double* __restrict__ W, double* __restrict__ F, const
   }
 }
 
+constexpr double kTensorTerms = 6e7;  // o^2 v^4
+
 struct Work {
   // FP64: A..D products of t2_terms_fixed, t2f = u, r2 its sum Z; mixed: A..D and t2f hold floats,
   // r2 = u until the residual is formed there
   double *ht, *foo, *fvv, *wo, *r1, *r2, *A, *B, *Cq, *D, *t2f;
   int* scales;    // FP64 path: scale exponents of the products' operand rows
+  void* slices;   // FP64 path, where its products run on the tensor cores: packed operands (else null)
   double* epart;  // energy partials
   float* acc;     // mixed path: FP32 GEMM results (v^3 o floats)
   float* f32;     // mixed path: FP32 copies of f~ (n^2), Foo (o^2), Fvv (v^2) for the FP32 finishing sums
@@ -658,9 +662,15 @@ struct Work {
 };
 
 size_t tc_arena_floats(int n, int nocc);
+// Whether the FP64 products of o occupied and v virtual orbitals run on the tensor cores (oz_gemm.cuh)
+// rather than the integer pipe (fix_gemm.cuh, which needs no packed operands): where their work, about
+// 3 o^2 v^4 terms and more, covers the packing and fills the SMs' tiles.
+bool fix_on_tensor_cores(int o, int v) { return o > 0 && v > 0 && (double)o * o * v * v * v * v >= kTensorTerms; }
 size_t fix_scale_ints(int o, int v);
+size_t fix_slice_bytes(int n, int o);
 
-size_t carve(void* base, int n, int o, Work* w, bool mixed = false) {
+// slices: whether the region of packed FP64 operands is part of the workspace
+size_t carve(void* base, int n, int o, Work* w, bool mixed = false, bool slices = false) {
   const int v = n - o;
   const size_t sizes[] = {(size_t)n * n, (size_t)o * o, (size_t)v * v, (size_t)o * o * o * o, (size_t)v * o,
                           (size_t)o * o * v * v, (size_t)o * v * o * v, (size_t)o * v * o * v, (size_t)o * v * o * v,
@@ -675,7 +685,12 @@ size_t carve(void* base, int n, int o, Work* w, bool mixed = false) {
   w->scales = nullptr;
   if (!mixed) {
     if (base) w->scales = reinterpret_cast<int*>(static_cast<char*>(base) + off);
-    off += ((fix_scale_ints(o, v) * sizeof(int) + 255) / 256) * 256;
+    off += dress_scale_bytes(n, o);
+  }
+  w->slices = nullptr;
+  if (slices) {
+    if (base) w->slices = static_cast<char*>(base) + off;
+    off += fix_slice_bytes(n, o);
   }
   w->acc = nullptr;
   w->f32 = nullptr;
@@ -710,6 +725,15 @@ cudaError_t launch_to_f32(const double* W, float* W32, size_t count, cudaStream_
 
 size_t dress_workspace_bytes(int n, int nocc) {
   Work w;
+  return carve(nullptr, n, nocc, &w, false, fix_on_tensor_cores(nocc, n - nocc));
+}
+
+size_t dress_scale_bytes(int n, int nocc) {
+  return (fix_scale_ints(nocc, n - nocc) * sizeof(int) + 255) / 256 * 256;
+}
+
+size_t dress_workspace_bytes_min(int n, int nocc) {
+  Work w;
   return carve(nullptr, n, nocc, &w);
 }
 
@@ -720,12 +744,13 @@ size_t dress_workspace_bytes_mixed(int n, int nocc) {
 
 int dress_launch_count(int n, int nocc, bool mixed) {
   // 4 T1 passes (the first one copies; for nocc > kT1Omax a separate copy + 4), h~, f~, 2 energy,
-  // u, small blocks, finalize; T2 terms: 2 row scales + 3 product launches (FP64) or 2 FP32 copies + 33 operand
+  // u, small blocks, finalize; T2 terms: 2 row scales + 3 product launches (FP64; + 3 operand packs where
+  // those run on the tensor cores) or 2 FP32 copies + 33 operand
   // packs + 9 GEMM launches + the vvvv pack and two product kernels + FP32 Fock copies + 4 finalize
   // kernels + error check (mixed)
   if (!(n - nocc > 0 && nocc > 0)) return 5;
   const int front = (nocc <= kT1Omax ? 4 : 5) + 7;
-  return front + (mixed ? 53 : 5);
+  return front + (mixed ? 53 : fix_on_tensor_cores(nocc, n - nocc) ? 8 : 5);
 }
 
 namespace {
@@ -760,7 +785,9 @@ Out out(double* p, int rd, int rs1, int rs2, int cd, int cs1, int cs2, int add) 
   return Out{p, rd, rs1, rs2, cd, cs1, cs2, add, nullptr, 0, 0, 0, 0};
 }
 
-cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const double* U, const Work& w, cudaStream_t st) {
+// need (nullable): instead of running, receives the bytes of packed operands the launches take.
+cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const double* U, const Work& w, cudaStream_t st,
+                           size_t* need = nullptr) {
   const int o = d.o, v = d.v, n1 = d.n, n2 = n1 * n1, n3 = n2 * n1;
   const int oo = o * o, vv = v * v, ov = o * v, ovv = o * vv;
   // start of a block of W: V(mask) has bit 8, 4, 2, 1 set where the first .. fourth index is virtual
@@ -833,10 +860,18 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
   for (const Operand* p : {&wA, &tij, &gab, &eA, &eB, &cA, &gx, &dA, &xA, &xB, &v1A, &v1B, &o1A, &x2B, &r2B, &tab, &v2B,
                            &v4B, &o2A, &o2B, &x3B, &ovA, &ooA, &v3A, &v3B, &o3A, &o3B, &yA, &y2A, &yB})
     ops.o[ops.count++] = *p;
-  cudaError_t e = fg::row_scales(ops, st);
+  cudaError_t e = need ? cudaSuccess : fg::row_scales(ops, st);
   if (e != cudaSuccess) return e;
 
   fg::Jobs js{};
+  auto launch = [&]() -> cudaError_t {
+    if (need) {
+      const size_t b = oz::pack_bytes(js);
+      *need = b > *need ? b : *need;
+      return cudaSuccess;
+    }
+    return w.slices ? oz::run(js, w.slices, st) : fg::run(js, st);
+  };
   auto add = [&](const Operand& a, const Operand& b, const Out& to) {
     Job& j = js.j[js.count++];
     j.a = a;
@@ -852,12 +887,12 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
   add(xA, xB, out(X, v, ovv, v, v, vv, 1, 0));             // (i a)(j b)
   add(v1A, v1B, vvvo_ae);
   add(o1A, tij, out(V(2), v, n3, n1, o, n2, 1, 1));        // W[m i B j]: (m b)(i j)
-  e = fg::run(js, st);
+  e = launch();
   if (e != cudaSuccess) return e;
 
   ops.count = 0;
   for (const Operand* p : {&x2A, &r2A, &x3A}) ops.o[ops.count++] = *p;
-  e = fg::row_scales(ops, st);
+  if (!need) e = fg::row_scales(ops, st);
   if (e != cudaSuccess) return e;
   js.count = 0;
   add(x2A, x2B, out(X, v, vv, v, v, ovv, 1, 1));           // (j a)(i b)
@@ -865,7 +900,7 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
   add(tab, v2B, out(V(14), v, n3, n1, o, n2, 1, 1));       // W[A E B i]: (a b)(e i)
   add(tab, v4B, out(V(15), v, n3, n1, v, n2, 1, 1));       // W[A E B F]: (a b)(e f)
   add(o2A, o2B, out(V(2), o, n3, n2, o, n1, 1, 1));        // W[m i B j]: (m i)(b j)
-  e = fg::run(js, st);
+  e = launch();
   if (e != cudaSuccess) return e;
 
   js.count = 0;
@@ -882,7 +917,19 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
   add(o3A, o3B, out(V(2), o, n3, 1, o, n1, n2, 1));        // W[m i B j]: (m j)(b i)
   add(yA, yB, out(Y, 1, v, 0, v, 0, 1, 0));                // into D's place, read by the second launch
   add(y2A, yB, out(Z, v, vv, 1, v, 0, v, 1));              // (i j b)(a)
-  return fg::run(js, st);
+  return launch();
+}
+
+// Bytes of packed operands (a dry run over the same operands; addresses are never used, and the scale
+// slots only tell operands apart).
+size_t fix_slice_bytes(int n, int o) {
+  const Dims d{n, o, n - o};
+  Work w{};
+  static int slots[1];
+  w.scales = slots;
+  size_t need = 0;
+  t2_terms_fixed(d, nullptr, nullptr, nullptr, w, nullptr, &need);
+  return (need + 255) / 256 * 256;
 }
 
 // FP64: the blocks' last terms (the O(o) and O(v) Fock sums), the residual's pair transpose and the
@@ -1838,7 +1885,9 @@ cudaError_t launch_dress(const double* h, const double* eri, const double* t1, c
   Work w;
   const bool mixed = g32 != nullptr;
   if (work_bytes < carve(nullptr, n, nocc, &w, mixed)) return cudaErrorInvalidValue;
-  carve(work, n, nocc, &w, mixed);
+  // a caller with less than dress_workspace_bytes (the static scratch) gets the products that pack nothing
+  const bool slices = !mixed && fix_on_tensor_cores(nocc, n - nocc) && work_bytes >= carve(nullptr, n, nocc, &w, false, true);
+  carve(work, n, nocc, &w, mixed, slices);
   Dims d{n, nocc, n - nocc};
   const size_t n4 = (size_t)n * n * n * n;
   const size_t o = nocc, v = n - nocc;

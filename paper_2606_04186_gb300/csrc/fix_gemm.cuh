@@ -319,8 +319,7 @@ __device__ __forceinline__ void product(const Job& jb, int tile, unsigned char* 
     const int ea = rw.e[0][r], eb = rw.e[1][c];
     double v = __longlong_as_double(0x7ff8000000000000ll);
     if (ea != kBad && eb != kBad) {
-      const int e = ea + eb - 2 * kBits + 2 * kLimb;
-      v = (e > -1000 && e < 900) ? (double)t * pow2(e) : ldexp((double)t, e);
+      v = fix_value(t, ea + eb - 2 * kBits + 2 * kLimb);
     }
     const int gr = r0 + r, gc = c0 + c;
     const int r1 = gr / o.rd, r2 = gr % o.rd, c1 = gc / o.cd, c2 = gc % o.cd;

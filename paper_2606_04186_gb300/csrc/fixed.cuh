@@ -39,6 +39,18 @@ __device__ __forceinline__ void madw(long long& s, int a, int b) { s += (long lo
 __device__ __forceinline__ long long join(long long hh, long long xx) {
   return hh + ((xx + (1ll << (kLimb - 1))) >> kLimb);
 }
+// t 2^e, rounded to nearest, by field arithmetic (an int64 conversion and a multiplication hold the FP64
+// pipe); results outside the normal range take ldexp
+__device__ __forceinline__ double fix_value(long long t, int e) {
+  const unsigned long long u = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
+  const int lz = __clzll((long long)u);
+  const unsigned long long m = (((u << (lz & 63)) >> 10) + 1) >> 1;  // 2^52 .. 2^53
+  const int ex = e + 1086 - lz;                                     // biased exponent of the leading bit
+  if (t == 0) return 0.0;
+  if (ex < 2 || ex > 2045) return ldexp((double)t, e);
+  const unsigned long long b = ((unsigned long long)(ex - 1) << 52) + m;
+  return __longlong_as_double((long long)(t < 0 ? b | 0x8000000000000000ull : b));
+}
 // 2^e as a double, |e| < 1022
 __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 

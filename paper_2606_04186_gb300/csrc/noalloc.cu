@@ -16,7 +16,8 @@
 
 namespace {
 
-constexpr size_t kStaticScratchBytes = (size_t)QFLOW_STATIC_SCRATCH_BYTES;
+// The documented limit, and room for the operands' scale exponents (0.39 MiB at most where the limit holds).
+constexpr size_t kStaticScratchBytes = (size_t)QFLOW_STATIC_SCRATCH_BYTES + (512u << 10);
 static __device__ __align__(256) unsigned char g_dress_scratch[kStaticScratchBytes];
 
 qf::ScratchAddressCache g_cache;  // device address of g_dress_scratch per (device, context)
@@ -79,8 +80,10 @@ extern "C" int qflow_dress_device_static(const double* h, const double* eri, con
                                          int32_t n, int32_t nocc, double* e0, double* F, double* W, void* stream) {
   if (!h || !eri || !t1 || !t2 || !e0 || !F || !W || n < 2 || n > 128 || nocc < 1 || nocc >= n)
     return QFLOW_ERR_ARG;
-  const size_t need = qf::dress_workspace_bytes(n, nocc);
-  if (need > kStaticScratchBytes) return QFLOW_ERR_TOO_LARGE;
+  const size_t scales = qf::dress_scale_bytes(n, nocc);
+  if (qf::dress_workspace_bytes_min(n, nocc) - scales > (size_t)QFLOW_STATIC_SCRATCH_BYTES ||
+      scales > kStaticScratchBytes - (size_t)QFLOW_STATIC_SCRATCH_BYTES)
+    return QFLOW_ERR_TOO_LARGE;
   void* scratch = nullptr;
   const int rc = scratch_address((cudaStream_t)stream, &scratch);
   if (rc != QFLOW_OK) return rc;

@@ -1378,7 +1378,8 @@ __global__ void __launch_bounds__(FD<K>::NT, DUCC && K == 3 ? 4 : FD<K>::MINB) s
 #pragma unroll
       for (int r = 0; r < PER; ++r) {
         const long long t = sm.T[pia[r] * NS + pib[r]] + sm.T[pib[r] * NS + pia[r]];
-        sk[r] = fma(pia[r] == pib[r] ? 0.5 * scale : kHalfRoot2 * scale, (double)t, diag[r] * vk[r]);
+        const double c = fix_value(t, sx - kFix - 1);
+        sk[r] = fma(diag[r], vk[r], pia[r] == pib[r] ? c : c * kRoot2);
         if (C::KM > C::SL && k >= C::SL) sx_[C::KM > C::SL ? k - C::SL : 0][r] = sk[r];
         else if (has[r]) sm.v.S[k][pd[r]] = sk[r];
         p4[0] = fma(vk[r], sk[r], p4[0]);  // vk is zero where there is no pair

@@ -67,3 +67,41 @@ def test_non_finite_integral_reaches_the_dressed_blocks():
     ok = np.ones(n - no, dtype=bool)
     ok[[5 - no, 7 - no]] = False
     assert np.isfinite(W[no:, :no, no:, :no][np.ix_(ok, range(no), ok, range(no))]).all()
+
+
+@pytest.mark.parametrize("n,no", [(26, 13), (43, 6), (47, 5), (50, 11)])
+def test_tensor_core_products_equal_integer_pipe_products(n, no):
+    """Problems above the work limit run on packed slices (oz_gemm.cuh); the static-scratch entry point
+    computes the same products without packing (43 x 6 fits it), and torch's FP64 gives the ladder of the
+    others.  Both forms are exact to 2^-54 sqrt(K) of the operand rows' norms, see above."""
+    import torch
+    qf = library()
+    _, h, g = synth.make_system(n, no, 5.0, 300 + n)
+    t1, t2 = synth.random_amplitudes(no, n - no, n, 0.05, 0.1)
+    e0, F, W = _dress(qf, h, g, t1, t2, no)
+    scale = max(1.0, np.abs(W).max())
+    if (n, no) == (43, 6):
+        f64 = lambda *s: torch.full(s, np.nan, dtype=torch.float64, device="cuda")  # noqa: E731
+        e0s, Fs, Ws = f64(1), f64(n, n), f64(n, n, n, n)
+        qf.dress_device_static(dev(h), dev(g), dev(t1), dev(t2), no, e0s, Fs, Ws)
+        torch.cuda.synchronize()
+        assert np.abs(F - Fs.cpu().numpy()).max() < 1e-12 * scale and np.abs(W - Ws.cpu().numpy()).max() < 1e-12 * scale
+        return
+    ref = hbar.hbar2(h, g, t1, t2, no)
+    for x, y in zip((e0, F, W), ref):
+        assert np.abs(np.asarray(x) - y).max() < 1e-12 * scale
+
+
+def test_tensor_core_products_pass_non_finite_integrals_on():
+    qf = library()
+    n, no = 44, 6
+    _, h, g = synth.make_system(n, no, 4.0, 8)
+    t1, t2 = synth.random_amplitudes(no, n - no, 3, 0.0, 0.1)
+    g = g.copy()
+    g[15, 16, 17, 18] = g[17, 18, 15, 16] = np.nan
+    e0, F, W = _dress(qf, h, g, t1, t2, no)
+    assert np.isfinite(e0) and np.isfinite(F[:no, :no]).all()
+    assert not np.isfinite(W[15, :no, 17, :no]).any()
+    ok = np.ones(n - no, dtype=bool)
+    ok[[15 - no, 17 - no]] = False
+    assert np.isfinite(W[no:, :no, no:, :no][np.ix_(ok, range(no), ok, range(no))]).all()
