@@ -30,8 +30,9 @@
 //     sweep.
 // Kernels: one per size class (grid-stride over that class), and a persistent kernel whose
 // warps take work items from one queue holding every class (largest spaces first).
-// Every loop is bounded; a warp never waits on another warp (the queue is a single atomic
-// counter).
+// Every loop is bounded; a warp waits for another one of its thread block at most for the few
+// accesses in which that one takes an item, and takes one from the global counter if it must wait
+// longer than a limit.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stddef.h>
@@ -44,9 +45,10 @@
 namespace qf {
 namespace {
 
-// Loop unrolling of the same-spin table loop (measured: 11 steps per iteration; 6, 22 and 66 were
-// not faster)
-constexpr int kHsUnroll = 11;
+// Loop unrolling of the same-spin table loop: the table's loads in flight.  The gathered blocks push
+// the table out of the L1 cache at large n, where more loads at once pay (82 orbitals, all spaces:
+// 68.8 / 68.2 / 67.7 ms with 11 / 22 / 33); at 24 and 40 orbitals 11 and 22 are equal, 33 is 1 % slower.
+constexpr int kHsUnroll = 22;
 constexpr int KM = 3;     // Davidson subspace limit (restart on the Ritz vector)
 // Spaces (warps) per CTA: a launch parameter up to kMaxWarps (the autotuner picks it); one CTA
 // fills the shared memory of an SM.  The register file is split over the SM's four
@@ -469,7 +471,7 @@ __device__ __forceinline__ void aa_first_terms(std::integer_sequence<int, I...>,
 // ---- shared memory -------------------------------------------------------------------------
 
 template <int K>
-struct Tabs {  // run-time string tables of one size class (bytes: they share the SM with warps)
+struct Tabs {  // string tables of one size class (bytes: they share the SM with warps)
   using D = Dim<K>;
   signed char J[D::NS * D::NSG];
   signed char pq[D::NS * D::NSG];
@@ -577,7 +579,7 @@ struct alignas(16) WarpState {  // 16-byte rows: the 6e6o sigma reads them as fl
   int ctrl[4];              // [0] subspace size, [1] valid, [2] status, [3] iterations
   // the small classes keep set-up data and gather offsets here (the 6e6o state keeps them in
   // the string operator's slot and the second S slot, which are free until they are filled)
-  alignas(16) unsigned char extra[K == 3 ? 16 : sizeof(SetupF32<K>) + 2 * D::NF * sizeof(long long)];
+  alignas(16) unsigned char extra[K == 3 ? 16 : sizeof(SetupF32<K>) + 2 * D::NF * sizeof(unsigned)];
   __device__ __forceinline__ float* hp() { return Wt + D::NW; }
   __device__ __forceinline__ const float* hp() const { return Wt + D::NW; }
 };
@@ -587,14 +589,14 @@ __device__ __forceinline__ SetupF32<K>& setup(WarpState<K>& ws) {
   if constexpr (K == 3) return *reinterpret_cast<SetupF32<K>*>(ws.Hs);
   else return *reinterpret_cast<SetupF32<K>*>(ws.extra);
 }
-// gather offsets: element (P, R) of the W block sits at off[P] + off[NF + R]
+// gather offsets: element (P, R) of the W block sits at off[P] + off[NF + R] (n <= 128: below 2^28)
 template <int K>
-__device__ __forceinline__ long long* gather_off(WarpState<K>& ws) {
-  if constexpr (K == 3) return reinterpret_cast<long long*>(ws.S + Dim<K>::NDET);
-  else return reinterpret_cast<long long*>(ws.extra + sizeof(SetupF32<K>));
+__device__ __forceinline__ unsigned* gather_off(WarpState<K>& ws) {
+  if constexpr (K == 3) return reinterpret_cast<unsigned*>(ws.S + Dim<K>::NDET);
+  else return reinterpret_cast<unsigned*>(ws.extra + sizeof(SetupF32<K>));
 }
 static_assert(KM == 3 && sizeof(SetupF32<3>) <= sizeof(WarpState<3>::Hs) &&
-                  2 * Dim<3>::NF * sizeof(long long) <= Dim<3>::NDET * sizeof(float),
+                  2 * Dim<3>::NF * sizeof(unsigned) <= Dim<3>::NDET * sizeof(float),
               "set-up data must fit the reused 6e6o slots");
 
 union alignas(16) AnyWarpState {
@@ -603,12 +605,22 @@ union alignas(16) AnyWarpState {
   WarpState<1> w1;
 };
 
+constexpr int kPairRounds = 11;  // 32 pairs a round
+
 // Shared memory of a CTA: the string tables, then one AnyWarpState per warp.
-struct alignas(16) CtaTabs {
+struct alignas(16) StringTabs {
   Tabs<3> t3;
   Tabs<2> t2;
   Tabs<1> t1;
-  unsigned short pair3[Dim<3>::NPAIR];  // (P, R) with P <= R, packed P | R << 8
+  // (P, R) with P <= R, packed P | R << 6 | (W_pprr ? 1 << 12 : 0): the 341 pairs with an index of
+  // the last orbital, then the 325 without; each part padded with its last pair to whole rounds of
+  // a warp
+  unsigned short pair3[2][kPairRounds * 32];
+};
+struct alignas(16) CtaTabs : StringTabs {
+  // items [q_next, q_end) of the work queue that the CTA's warps take one by one (take_item)
+  unsigned long long q_next, q_end;
+  int q_lock;
 };
 constexpr size_t kTabsBytes = (sizeof(CtaTabs) + 15) / 16 * 16;
 __host__ __device__ constexpr size_t cta_smem_bytes(int warps) { return kTabsBytes + (size_t)warps * sizeof(AnyWarpState); }
@@ -660,15 +672,17 @@ __device__ __forceinline__ float diag_at(const Tabs<K>& tb, const WarpState<K>& 
   return ws.dh[ia] + ws.dh[ib] + (jj - ws.j0);
 }
 
-// String tables of one class (single thread): strings by increasing bit mask (string 0 holds
-// the occupied orbitals), single replacements into each string, connections to the Phi string
-// and the single replacements i -> A of the Phi string.
+// String tables of one class, evaluated by the compiler: strings by increasing bit mask (string 0
+// holds the occupied orbitals), single replacements into each string, connections to the Phi string
+// and the single replacements i -> A of the Phi string.  Built on the device, one thread per class,
+// they cost every launch about 45 us before its first space.
 template <int K>
-__device__ void build_tabs(Tabs<K>& t) {
+__host__ __device__ constexpr Tabs<K> make_tabs() {
   using D = Dim<K>;
+  Tabs<K> t{};
   int c = 0;
   for (int m = 0; m < (1 << D::NORB); ++m)
-    if (__popc(m) == K) t.mask[c++] = m;
+    if (popc6(m) == K) t.mask[c++] = (signed char)m;
   for (int I = 0; I < D::NS; ++I) {
     int j = 0;
     for (int p = 0; p < D::NORB; ++p)
@@ -684,17 +698,17 @@ __device__ void build_tabs(Tabs<K>& t) {
         const int mj = (mi & ~(1 << p)) | (1 << q);
         int sgn = 1;
         if (p != q) {
-          int par = __popc(mj & ((1 << q) - 1)) & 1;
+          int par = popc6(mj & ((1 << q) - 1)) & 1;
           const int m1 = mj & ~(1 << q);
-          par ^= __popc(m1 & ((1 << p) - 1)) & 1;
+          par ^= popc6(m1 & ((1 << p) - 1)) & 1;
           sgn = par ? -1 : 1;
         }
         int J = 0;
         for (int x = 0; x < D::NS; ++x)
           if (t.mask[x] == mj) J = x;
-        t.J[I * D::NSG + u] = J;
-        t.pq[I * D::NSG + u] = p * D::NORB + q;
-        t.sg[I * D::NSG + u] = sgn;
+        t.J[I * D::NSG + u] = (signed char)J;
+        t.pq[I * D::NSG + u] = (signed char)(p * D::NORB + q);
+        t.sg[I * D::NSG + u] = (signed char)sgn;
         ++u;
       }
     }
@@ -707,29 +721,49 @@ __device__ void build_tabs(Tabs<K>& t) {
         t.c0sg[I][n0] = t.sg[I * D::NSG + u];
         ++n0;
       }
-    t.c0n[I] = n0;
+    t.c0n[I] = (signed char)n0;
   }
   for (int x = 0; x < K * K; ++x) {
     const int i = x / K, A = K + x % K, m0 = t.mask[0];
-    int par = __popc(m0 & ((1 << i) - 1)) & 1;
+    int par = popc6(m0 & ((1 << i) - 1)) & 1;
     const int m1 = m0 & ~(1 << i);
-    par ^= __popc(m1 & ((1 << A) - 1)) & 1;
+    par ^= popc6(m1 & ((1 << A) - 1)) & 1;
     int J = 0;
     for (int q = 0; q < D::NS; ++q)
       if (t.mask[q] == (m1 | (1 << A))) J = q;
-    t.xJ[x] = J;
-    t.xs[x] = par ? -1 : 1;
+    t.xJ[x] = (signed char)J;
+    t.xs[x] = (signed char)(par ? -1 : 1);
   }
+  return t;
 }
 
-__device__ void build_all_tabs(CtaTabs& cs) {
-  if (threadIdx.x == 0) build_tabs<3>(cs.t3);
-  if (threadIdx.x == 32) build_tabs<2>(cs.t2);
-  if (threadIdx.x == 64) build_tabs<1>(cs.t1);
-  if (threadIdx.x == 96) {
-    int t = 0;
-    for (int P = 0; P < Dim<3>::NF; ++P)
-      for (int R = P; R < Dim<3>::NF; ++R) cs.pair3[t++] = (unsigned short)(P | (R << 8));
+__host__ __device__ constexpr StringTabs make_string_tabs() {
+  StringTabs t{};
+  t.t3 = make_tabs<3>();
+  t.t2 = make_tabs<2>();
+  t.t1 = make_tabs<1>();
+  constexpr int NORB = Dim<3>::NORB, NF = Dim<3>::NF, L = NORB - 1;
+  int cnt[2] = {0, 0};
+  for (int P = 0; P < NF; ++P)
+    for (int R = P; R < NF; ++R) {
+      const int part = !(P % NORB == L || P / NORB == L || R % NORB == L || R / NORB == L);
+      const int jj = P % (NORB + 1) == 0 && R % (NORB + 1) == 0;  // W_pprr
+      t.pair3[part][cnt[part]++] = (unsigned short)(P | (R << 6) | (jj << 12));
+    }
+  for (int part = 0; part < 2; ++part)
+    for (int x = cnt[part]; x < kPairRounds * 32; ++x) t.pair3[part][x] = t.pair3[part][cnt[part] - 1];
+  return t;
+}
+__device__ const StringTabs g_string_tabs = make_string_tabs();
+
+__device__ void load_tabs(CtaTabs& cs) {
+  static_assert(sizeof(StringTabs) % 16 == 0, "copied in 16-byte words");
+  const uint4* src = reinterpret_cast<const uint4*>(&g_string_tabs);
+  uint4* dst = reinterpret_cast<uint4*>(static_cast<StringTabs*>(&cs));
+  for (int x = threadIdx.x; x < (int)(sizeof(StringTabs) / 16); x += blockDim.x) dst[x] = src[x];
+  if (threadIdx.x == 0) {
+    cs.q_next = cs.q_end = 0;
+    cs.q_lock = 0;
   }
   __syncthreads();
 }
@@ -1298,9 +1332,9 @@ __device__ void solve_one(const Tabs<K>& tb, const CtaTabs& cs, WarpState<K>& ws
                           float* __restrict__ guess_out, int64_t s, int lane) {
   using D = Dim<K>;
   constexpr int NS = D::NS, NSG = D::NSG, NDET = D::NDET, NORB = D::NORB, NF = D::NF;
-  const unsigned short* __restrict__ pair3 = cs.pair3;
+  const unsigned short(*__restrict__ pair3)[kPairRounds * 32] = cs.pair3;
   const int n = a.n;
-  const size_t n1 = (size_t)n, n2 = n1 * n1, n3 = n2 * n1;
+  const size_t n1 = (size_t)n, n2 = n1 * n1;
   const float tol = (float)a.tol;
   // ---- validate -------------------------------------------------------------------------
   // (the sorted index and the owner flag are loaded beside the record: neither waits on it)
@@ -1308,19 +1342,27 @@ __device__ void solve_one(const Tabs<K>& tb, const CtaTabs& cs, WarpState<K>& ws
   const int64_t oidx = a.sorted_index ? sidx : s;
   // only a space that owns an amplitude forms its increment (loaded here, used at the merge)
   const bool owner = !a.owns || a.owns[s] != 0;
-  if (lane == 0) {
-    const qflow_space& q = a.spaces[s];
-    int ok = (q.no == K && q.nv == K), same = (K == 3);
-    for (int t = 0; t < NORB; ++t) {
-      const int o = q.orb[t];
-      if (t < NORB - 1) same &= (o == ws.orb[t]);
-      ws.orb[t] = o;
-      if (t < K) ok &= (o >= 0 && o < a.nocc);
-      else ok &= (o >= a.nocc && o < a.n);
+  {  // lane t reads orbital t (the class lists hold one class, so lanes 6 and 7 take no and nv)
+    const qflow_space* q = a.spaces + s;
+    int ok = 1, same = 1;
+    if (lane < NORB) {
+      const int o = q->orb[lane];
+      ok = lane < K ? (o >= 0 && o < a.nocc) : (o >= a.nocc && o < a.n);
+      same = lane == NORB - 1 || o == ws.orb[lane];
+      ws.orb[lane] = o;
+    } else if (lane == NORB) {
+      ok = q->no == K;
+    } else if (lane == NORB + 1) {
+      ok = q->nv == K;
     }
-    if (!ok) ws.orb[0] = -1;  // the W block below is not this record's: nothing to reuse next
-    ws.ctrl[1] = ok;
-    ws.ctrl[0] = same && ok;
+    ok = __all_sync(0xffffffffu, ok);
+    same = __all_sync(0xffffffffu, same);
+    __syncwarp();
+    if (lane == 0) {
+      if (!ok) ws.orb[0] = -1;  // the W block below is not this record's: nothing to reuse next
+      ws.ctrl[1] = ok;
+      ws.ctrl[0] = K == 3 && same && ok;
+    }
   }
   __syncwarp();
   if (!ws.ctrl[1]) {
@@ -1337,11 +1379,11 @@ __device__ void solve_one(const Tabs<K>& tb, const CtaTabs& cs, WarpState<K>& ws
   // block.  Element (P, R) of the W block is at off[P] + off[NF + R] (pair offsets built first).
   SetupF32<K>& su = setup(ws);
   {
-    long long* off = gather_off(ws);
+    unsigned* off = gather_off(ws);
     for (int t = lane; t < 2 * NF; t += 32) {
       const int P = t % NF;
-      const long long o0 = ws.orb[P / NORB], o1 = ws.orb[P % NORB];
-      off[t] = (t < NF) ? o0 * (long long)n3 + o1 * (long long)n2 : o0 * (long long)n1 + o1;
+      const unsigned o0 = (unsigned)ws.orb[P / NORB], o1 = (unsigned)ws.orb[P % NORB];
+      off[t] = (o0 * (unsigned)n + o1) * (t < NF ? (unsigned)n2 : 1u);
     }
     __syncwarp();
     static_assert(NF <= 64, "two rounds of F");
@@ -1357,44 +1399,52 @@ __device__ void solve_one(const Tabs<K>& tb, const CtaTabs& cs, WarpState<K>& ws
     if constexpr (K == 3) {  // the 666 unique elements of the pair-symmetric block
       // A space whose first five orbitals are those of this warp's previous space (consecutive
       // spaces of the sorted list differ in the last virtual) keeps the 325 elements without
-      // orbital 5 from it: W_t and J_c still hold them.
+      // orbital 5 from it: W_t and J_c still hold them.  The pair list holds the others first, so
+      // such a space takes 11 rounds of 32 loads instead of 21 partly idle ones (40 orbitals, 60,000
+      // spaces: 0.73 -> 0.69 ms).
       const bool reuse = ws.ctrl[0] != 0;
-      constexpr int PER = (D::NPAIR + 31) / 32;
-      float wv[PER];
+      float wv[2][kPairRounds];
+      auto element = [&](int part, int k) {
+        const int pr = pair3[part][32 * k + lane];
+        return off[pr & 63] + off[NF + ((pr >> 6) & 63)];
+      };
+      auto put = [&](int part, int k) {
+        const int pr = pair3[part][32 * k + lane], P = pr & 63, R = (pr >> 6) & 63;
+        float wf = wv[part][k];
+        if (pr >> 12) {  // W_pprr: diagonal only
+          const int p = P / (NORB + 1), r = R / (NORB + 1);
+          ws.Jc[p * NORB + r] = wf;
+          ws.Jc[r * NORB + p] = wf;
+          wf = 0.f;
+        }
+        ws.Wt[P * NF + R] = wf;
+        ws.Wt[R * NF + P] = wf;
+      };
+      if (W32) {
 #pragma unroll
-      for (int k = 0; k < PER; ++k) {
-        const int t = lane + 32 * k;
-        wv[k] = 0.f;
-        if (t < D::NPAIR) {
-          const int pr = pair3[t], P = pr & 255, R = pr >> 8;
-          if (!reuse || P % NORB == NORB - 1 || P >= NF - NORB || R % NORB == NORB - 1 || R >= NF - NORB) {
-            const size_t g = (size_t)(off[P] + off[NF + R]);
-            wv[k] = W32 ? W32[g] : (float)a.W[g];
-          }
+        for (int k = 0; k < kPairRounds; ++k) wv[0][k] = W32[element(0, k)];
+        if (!reuse) {
+#pragma unroll
+          for (int k = 0; k < kPairRounds; ++k) wv[1][k] = W32[element(1, k)];
+#pragma unroll
+          for (int k = 0; k < kPairRounds; ++k) put(1, k);
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < kPairRounds; ++k) wv[0][k] = (float)a.W[element(0, k)];
+        if (!reuse) {
+#pragma unroll
+          for (int k = 0; k < kPairRounds; ++k) wv[1][k] = (float)a.W[element(1, k)];
+#pragma unroll
+          for (int k = 0; k < kPairRounds; ++k) put(1, k);
         }
       }
 #pragma unroll
-      for (int k = 0; k < PER; ++k) {
-        const int t = lane + 32 * k;
-        if (t < D::NPAIR) {
-          const int pr = pair3[t], P = pr & 255, R = pr >> 8;
-          if (!reuse || P % NORB == NORB - 1 || P >= NF - NORB || R % NORB == NORB - 1 || R >= NF - NORB) {
-            const int p = P / NORB, r = R / NORB;
-            const bool jj = (P == p * (NORB + 1)) && (R == r * (NORB + 1));  // W_pprr: diagonal only
-            if (jj) {
-              ws.Jc[p * NORB + r] = wv[k];
-              ws.Jc[r * NORB + p] = wv[k];
-            }
-            const float wf = jj ? 0.f : wv[k];
-            ws.Wt[P * NF + R] = wf;
-            ws.Wt[R * NF + P] = wf;
-          }
-        }
-      }
+      for (int k = 0; k < kPairRounds; ++k) put(0, k);
     } else {
       for (int t = lane; t < D::NW; t += 32) {
         const int P = t / NF, R = t % NF;
-        const size_t g = (size_t)(off[P] + off[NF + R]);
+        const unsigned g = off[P] + off[NF + R];
         const int p = P / NORB, r = R / NORB;
         const bool jj = (P == p * (NORB + 1)) && (R == r * (NORB + 1));
         const float w = W32 ? W32[g] : (float)a.W[g];
@@ -1975,7 +2025,7 @@ __global__ void __maxnreg__(kMaxRegs) solve_class_kernel(SolveArgs a, const floa
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CtaTabs& cs = *reinterpret_cast<CtaTabs*>(smem_raw);
   AnyWarpState* wst = reinterpret_cast<AnyWarpState*>(smem_raw + kTabsBytes);
-  build_all_tabs(cs);
+  load_tabs(cs);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   WarpState<K>& ws = state<K>(wst[warp]);
   if (lane == 0) ws.orb[0] = -1;  // no previous space: nothing to reuse
@@ -1988,38 +2038,90 @@ struct PersistentArgs {
   SolveArgs cls[4];           // [k] for k = 1..3 (cls[0] unused)
   const float* W32;
   unsigned long long* queue;  // work counter, zero at launch
-  int chunk;                  // work items taken per atomic
+  int chunk;                  // work items per warp that a CTA takes at once
 };
+
+// The next work item of a warp (every lane calls).  A CTA takes `block` consecutive items at a time
+// and its warps share them, so they work on spaces that differ in the last virtual or two: the
+// elements without it and the 32-byte sectors of those with it meet in the L1 cache (40 orbitals:
+// 0.69 -> 0.68 ms; 114 orbitals with 12 warps: 32.4 -> 31.4 ms; 4 items per warp and block no longer
+// cost a ragged end: 0.85 instead of 1.19 ms at 40 orbitals, and are the best choice at 82).  The
+// lock is held for a few shared-memory accesses, once per block for the global atomic; a warp that does
+// not get it within the limit takes an item of its own.
+constexpr int kTakeTries = 4096;
+__device__ __forceinline__ unsigned long long take_item(CtaTabs& cs, unsigned long long* queue, unsigned block,
+                                                        int lane) {
+  volatile unsigned long long* next = &cs.q_next;
+  volatile unsigned long long* end = &cs.q_end;
+  unsigned long long x = 0;
+  int held = 1;
+#pragma unroll 1
+  for (int t = 0; t < kTakeTries; ++t) {
+    if (lane == 0) held = atomicCAS_block(&cs.q_lock, 0, 1);
+    held = __shfl_sync(0xffffffffu, held, 0);
+    if (held == 0) break;
+    __nanosleep(32);
+  }
+  if (held == 0) {
+    __threadfence_block();
+    x = *next;
+    const bool more = x < *end;
+    __syncwarp();
+    if (!more) {
+      if (lane == 0) x = atomicAdd(queue, (unsigned long long)block);
+      x = __shfl_sync(0xffffffffu, x, 0);
+      if (lane == 0) *end = x + block;
+    }
+    if (lane == 0) {
+      *next = x + 1;
+      __threadfence_block();
+      atomicExch_block(&cs.q_lock, 0);
+    }
+  } else {
+    if (lane == 0) x = atomicAdd(queue, 1ull);
+    x = __shfl_sync(0xffffffffu, x, 0);
+  }
+  __syncwarp();
+  return x;
+}
+
+// The record a warp takes about one round of the grid later, its index and its owner flag, into the
+// L2 cache: the class list streams from HBM, a latency per space that nothing else covers (82
+// orbitals, all 7.2 M spaces: 71.5 -> 68.9 ms).
+__device__ __forceinline__ void prefetch_record(const SolveArgs& a, int64_t s, int64_t n, int lane) {
+  if (a.items || s >= n) return;
+  const void* p = nullptr;
+  if (lane == 0) p = a.spaces + s;
+  else if (lane == 1 && a.sorted_index) p = a.sorted_index + s;
+  else if (lane == 2 && a.owns) p = a.owns + s;
+  if (p) asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+  __syncwarp();
+}
 
 // One queue over every size class: items [0, n3) are 6e6o spaces, then 4e4o, then 2e2o.
 __global__ void __maxnreg__(kMaxRegs) solve_persistent_kernel(PersistentArgs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CtaTabs& cs = *reinterpret_cast<CtaTabs*>(smem_raw);
   AnyWarpState* wst = reinterpret_cast<AnyWarpState*>(smem_raw + kTabsBytes);
-  build_all_tabs(cs);
+  load_tabs(cs);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // no previous 6e6o space: nothing to reuse (a warp's items only increase, so after its first
-  // smaller space it never meets a 6e6o space again)
-  if (lane == 0) state<3>(wst[warp]).orb[0] = -1;
+  if (lane == 0) state<3>(wst[warp]).orb[0] = -1;  // no previous 6e6o space: nothing to reuse
   const int64_t n3 = p.cls[3].nspaces, n2 = p.cls[2].nspaces, n1 = p.cls[1].nspaces;
   const unsigned long long total = (unsigned long long)(n3 + n2 + n1);
-  // each pass takes `chunk` new items, so the loop ends after at most total / chunk + 1 passes
+  const unsigned block = (unsigned)p.chunk * (blockDim.x >> 5);
+  // each pass takes a new item, so the loop ends after at most total + 1 passes
 #pragma unroll 1
   for (unsigned long long pass = 0; pass <= total; ++pass) {
-    unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(p.queue, (unsigned long long)p.chunk);
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (base >= total) break;
-#pragma unroll 1
-    for (int c = 0; c < p.chunk; ++c) {
-      const unsigned long long item = base + (unsigned long long)c;
-      if (item >= total) break;
-      const int64_t it = (int64_t)item;
-      if (it < n3) {
-        const SolveArgs& a = p.cls[3];
-        solve_one<3>(cs.t3, cs, state<3>(wst[warp]), a, p.W32, static_cast<const float*>(a.guess),
-                     static_cast<float*>(a.root_out), a.items ? a.items[it] : it, lane);
-      } else if (it < n3 + n2) {
+    const unsigned long long item = take_item(cs, p.queue, block, lane);
+    if (item >= total) break;
+    const int64_t it = (int64_t)item;
+    if (it < n3) {
+      const SolveArgs& a = p.cls[3];
+      prefetch_record(a, it + (int64_t)gridDim.x * block, n3, lane);
+      solve_one<3>(cs.t3, cs, state<3>(wst[warp]), a, p.W32, static_cast<const float*>(a.guess),
+                   static_cast<float*>(a.root_out), a.items ? a.items[it] : it, lane);
+    } else {
+      if (it < n3 + n2) {
         const SolveArgs& a = p.cls[2];
         const int64_t l = it - n3;
         solve_one<2>(cs.t2, cs, state<2>(wst[warp]), a, p.W32, static_cast<const float*>(a.guess),
@@ -2030,6 +2132,8 @@ __global__ void __maxnreg__(kMaxRegs) solve_persistent_kernel(PersistentArgs p) 
         solve_one<1>(cs.t1, cs, state<1>(wst[warp]), a, p.W32, static_cast<const float*>(a.guess),
                      static_cast<float*>(a.root_out), a.items ? a.items[l] : l, lane);
       }
+      if (lane == 0) state<3>(wst[warp]).orb[0] = -1;  // the slot holds another class's state now
+      __syncwarp();
     }
   }
 }
