@@ -123,9 +123,12 @@ __global__ void k_t1_annihilator(double* __restrict__ W, const double* __restric
 // Shared t1 is stored transposed, t1s[a][i] with rows padded to kT1Omax (zeros), so the o
 // coefficients of one virtual index come in 16-byte loads that every lane shares.
 constexpr int kT1Omax = 16;
-// FP32 sums: resident CTAs per SM the register budget keeps (5 x 256 threads; the creator
-// pass, which holds no accumulators, 6)
-constexpr int kT1Blocks = 5;
+// FP32 sums: rows whose loads a thread has in flight, and the CTAs per SM that its registers leave
+// (annihilator passes, with o sums in registers, one less).  One
+// row at a time (5 and 6 CTAs), a store between each load and the next, these passes took 0.68-0.74 ms
+// each at 114 orbitals (HBM: 0.2-0.4) and 20-31 us at 40; now 0.48-0.61 ms and 18-23 us.
+constexpr int kT1Rows = 8;
+constexpr int kT1Blocks = 4;
 
 template <typename A>
 __device__ __forceinline__ void load_t1_t(const double* __restrict__ t1, A* t1s, const Dims& d) {
@@ -159,23 +162,32 @@ __device__ __forceinline__ size_t t1_index(const Dims& d, int p, size_t rest) {
 }
 
 template <typename A, int POS>
-__global__ void __launch_bounds__(TPB, kT1Blocks + 1) k_t1_creator_fast(double* __restrict__ W, const double* __restrict__ t1, Dims d) {
+__global__ void __launch_bounds__(TPB, kT1Blocks) k_t1_creator_fast(double* __restrict__ W, const double* __restrict__ t1, Dims d) {
   extern __shared__ __align__(16) double t1raw[];  // [v][kT1Omax], in the accumulation type
   A* t1s = reinterpret_cast<A*>(t1raw);
   load_t1_t<A>(t1, t1s, d);
   const size_t m = (size_t)d.n * d.n * d.n;
+  const size_t step = t1_index<A, POS>(d, 1, 0);  // distance of neighbouring rows
   for (size_t rest = blockIdx.x * (size_t)blockDim.x + threadIdx.x; rest < m; rest += (size_t)gridDim.x * blockDim.x) {
+    const size_t base = t1_index<A, POS>(d, 0, rest), vb = base + d.o * step;
     A wi[kT1Omax];
 #pragma unroll
-    for (int i = 0; i < kT1Omax; ++i) wi[i] = (i < d.o) ? to_acc<A>(W[t1_index<A, POS>(d, i, rest)]) : (A)0;
-    for (int a = 0; a < d.v; ++a) {
-      A c[kT1Omax];
-      t1_row<A>(t1s, a, c);
-      A acc = 0;
+    for (int i = 0; i < kT1Omax; ++i) wi[i] = (i < d.o) ? to_acc<A>(W[base + i * step]) : (A)0;
+    for (int a0 = 0; a0 < d.v; a0 += kT1Rows) {
+      double x[kT1Rows];
 #pragma unroll
-      for (int i = 0; i < kT1Omax; ++i)
-        if (i < d.o) acc += c[i] * wi[i];
-      W[t1_index<A, POS>(d, d.o + a, rest)] -= from_acc<A>(acc);
+      for (int u = 0; u < kT1Rows; ++u) x[u] = a0 + u < d.v ? W[vb + (a0 + u) * step] : 0.0;
+#pragma unroll
+      for (int u = 0; u < kT1Rows; ++u) {
+        if (a0 + u >= d.v) break;
+        A c[kT1Omax];
+        t1_row<A>(t1s, a0 + u, c);
+        A acc = 0;
+#pragma unroll
+        for (int i = 0; i < kT1Omax; ++i)
+          if (i < d.o) acc += c[i] * wi[i];
+        W[vb + (a0 + u) * step] = x[u] - from_acc<A>(acc);
+      }
     }
   }
 }
@@ -190,52 +202,69 @@ __global__ void __launch_bounds__(TPB, kT1Blocks) k_t1_creator_copy(const double
   A* t1s = reinterpret_cast<A*>(t1raw);
   load_t1_t<A>(t1, t1s, d);
   const size_t m = (size_t)d.n * d.n * d.n;
+  const size_t step = t1_index<A, 0>(d, 1, 0);  // distance of neighbouring rows
   for (size_t rest = blockIdx.x * (size_t)blockDim.x + threadIdx.x; rest < m; rest += (size_t)gridDim.x * blockDim.x) {
+    const size_t base = t1_index<A, 0>(d, 0, rest), vb = base + d.o * step;
     A wi[kT1Omax];
 #pragma unroll
     for (int i = 0; i < kT1Omax; ++i) {
       wi[i] = (A)0;
       if (i < d.o) {
-        const size_t g = t1_index<A, 0>(d, i, rest);
+        const size_t g = base + i * step;
         const double x = src[g];
         W[g] = x;
         wi[i] = to_acc<A>(x);
       }
     }
-    for (int a = 0; a < d.v; ++a) {
-      A c[kT1Omax];
-      t1_row<A>(t1s, a, c);
-      A acc = 0;
+    for (int a0 = 0; a0 < d.v; a0 += kT1Rows) {
+      double x[kT1Rows];
 #pragma unroll
-      for (int i = 0; i < kT1Omax; ++i)
-        if (i < d.o) acc += c[i] * wi[i];
-      const size_t g = t1_index<A, 0>(d, d.o + a, rest);
-      W[g] = src[g] - from_acc<A>(acc);
+      for (int u = 0; u < kT1Rows; ++u) x[u] = a0 + u < d.v ? src[vb + (a0 + u) * step] : 0.0;
+#pragma unroll
+      for (int u = 0; u < kT1Rows; ++u) {
+        if (a0 + u >= d.v) break;
+        A c[kT1Omax];
+        t1_row<A>(t1s, a0 + u, c);
+        A acc = 0;
+#pragma unroll
+        for (int i = 0; i < kT1Omax; ++i)
+          if (i < d.o) acc += c[i] * wi[i];
+        W[vb + (a0 + u) * step] = x[u] - from_acc<A>(acc);
+      }
     }
   }
 }
 
 template <typename A, int POS>
-__global__ void __launch_bounds__(TPB, kT1Blocks) k_t1_annihilator_fast(double* __restrict__ W, const double* __restrict__ t1, Dims d) {
+__global__ void __launch_bounds__(TPB, kT1Blocks - 1) k_t1_annihilator_fast(double* __restrict__ W, const double* __restrict__ t1, Dims d) {
   extern __shared__ __align__(16) double t1raw[];  // [v][kT1Omax], in the accumulation type
   A* t1s = reinterpret_cast<A*>(t1raw);
   load_t1_t<A>(t1, t1s, d);
   const size_t m = (size_t)d.n * d.n * d.n;
+  const size_t step = t1_index<A, POS>(d, 1, 0);  // distance of neighbouring rows
   for (size_t rest = blockIdx.x * (size_t)blockDim.x + threadIdx.x; rest < m; rest += (size_t)gridDim.x * blockDim.x) {
+    const size_t base = t1_index<A, POS>(d, 0, rest), vb = base + d.o * step;
     A acc[kT1Omax];
 #pragma unroll
     for (int q = 0; q < kT1Omax; ++q) acc[q] = 0;
-    for (int a = 0; a < d.v; ++a) {
-      const A wa = to_acc<A>(W[t1_index<A, POS>(d, d.o + a, rest)]);
-      A c[kT1Omax];
-      t1_row<A>(t1s, a, c);
+    for (int a0 = 0; a0 < d.v; a0 += kT1Rows) {
+      double x[kT1Rows];
 #pragma unroll
-      for (int q = 0; q < kT1Omax; ++q)
-        if (q < d.o) acc[q] += c[q] * wa;
+      for (int u = 0; u < kT1Rows; ++u) x[u] = a0 + u < d.v ? W[vb + (a0 + u) * step] : 0.0;
+#pragma unroll
+      for (int u = 0; u < kT1Rows; ++u) {
+        if (a0 + u >= d.v) break;
+        const A wa = to_acc<A>(x[u]);
+        A c[kT1Omax];
+        t1_row<A>(t1s, a0 + u, c);
+#pragma unroll
+        for (int q = 0; q < kT1Omax; ++q)
+          if (q < d.o) acc[q] += c[q] * wa;
+      }
     }
 #pragma unroll
     for (int q = 0; q < kT1Omax; ++q)
-      if (q < d.o) W[t1_index<A, POS>(d, q, rest)] += from_acc<A>(acc[q]);
+      if (q < d.o) W[base + q * step] += from_acc<A>(acc[q]);
   }
 }
 
@@ -428,10 +457,13 @@ void t1_passes(const double* eri, double* W, const double* t1, const Dims& d, cu
       k_t1_annihilator_fixed<3><<<g, TPB, fm, st>>>(W, t1, d);
     } else {
       const size_t sm = sizeof(A) * kT1Omax * d.v;
-      k_t1_creator_copy<A><<<g, TPB, sm, st>>>(eri, W, t1, d);
-      k_t1_creator_fast<A, 2><<<g, TPB, sm, st>>>(W, t1, d);
-      k_t1_annihilator_fast<A, 1><<<g, TPB, sm, st>>>(W, t1, d);
-      k_t1_annihilator_fast<A, 3><<<g, TPB, sm, st>>>(W, t1, d);
+      // up to 53 orbitals blocks of 64: every SM gets some of the n^3 threads
+      const unsigned tpb = n3 < 152u * 1024u ? 64u : (unsigned)TPB;
+      const unsigned gs = tpb == 64u ? (unsigned)((n3 + 63) / 64) : g;
+      k_t1_creator_copy<A><<<gs, tpb, sm, st>>>(eri, W, t1, d);
+      k_t1_creator_fast<A, 2><<<gs, tpb, sm, st>>>(W, t1, d);
+      k_t1_annihilator_fast<A, 1><<<gs, tpb, sm, st>>>(W, t1, d);
+      k_t1_annihilator_fast<A, 3><<<gs, tpb, sm, st>>>(W, t1, d);
     }
   } else {
     const size_t n4 = n3 * d.n;
@@ -443,22 +475,22 @@ void t1_passes(const double* eri, double* W, const double* t1, const Dims& d, cu
   }
 }
 
-// h~ = (1 - K) h (1 + K)
+// h~ = (1 - K) h (1 + K), a block per column s (n <= 128 threads): (h (1+K))_{p s} of every row p once,
+// in shared memory, then the occupied rows' part.  Bound by the latency of the FP64 sums (v terms,
+// then o); with a thread per element and o + 1 sums of v terms in each it took 69 us at 114 orbitals
+// and 11 us at 24; now 15 and 6.
 __global__ void k_h_tilde(const double* __restrict__ h, const double* __restrict__ t1, double* __restrict__ ht, Dims d) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= d.n * d.n) return;
-  const int r = x / d.n, s = x % d.n;
+  extern __shared__ __align__(16) double hks[];  // [n]
+  const int s = blockIdx.x, p = threadIdx.x;
   // (h (1+K))_{p s} = h_ps + [s occ] sum_a h_{p,nocc+a} t1[s][a]
-  auto hk = [&](int p) {
-    double v = h[p * d.n + s];
-    if (s < d.o)
-      for (int a = 0; a < d.v; ++a) v += h[p * d.n + d.o + a] * t1[s * d.v + a];
-    return v;
-  };
-  double v = hk(r);
-  if (r >= d.o)
-    for (int i = 0; i < d.o; ++i) v -= t1[i * d.v + (r - d.o)] * hk(i);
-  ht[x] = v;
+  double v = h[p * d.n + s];
+  if (s < d.o)
+    for (int a = 0; a < d.v; ++a) v += h[p * d.n + d.o + a] * t1[s * d.v + a];
+  hks[p] = v;
+  __syncthreads();
+  if (p >= d.o)
+    for (int i = 0; i < d.o; ++i) v -= t1[i * d.v + (p - d.o)] * hks[i];
+  ht[p * d.n + s] = v;
 }
 
 // f~ = h~ + sum_k [2 g~_pqkk - g~_pkkq]
@@ -662,6 +694,7 @@ struct Work {
 };
 
 size_t tc_arena_floats(int n, int nocc);
+bool vvvo_shares_launch(int o, int v);
 // Whether the FP64 products of o occupied and v virtual orbitals run on the tensor cores (oz_gemm.cuh)
 // rather than the integer pipe (fix_gemm.cuh, which needs no packed operands): where their work, about
 // 3 o^2 v^4 terms and more, covers the packing and fills the SMs' tiles.
@@ -745,12 +778,12 @@ size_t dress_workspace_bytes_mixed(int n, int nocc) {
 int dress_launch_count(int n, int nocc, bool mixed) {
   // 4 T1 passes (the first one copies; for nocc > kT1Omax a separate copy + 4), h~, f~, 2 energy,
   // u, small blocks, finalize; T2 terms: 2 row scales + 3 product launches (FP64; + 3 operand packs where
-  // those run on the tensor cores) or 2 FP32 copies + 33 operand
-  // packs + 9 GEMM launches + the vvvv pack and two product kernels + FP32 Fock copies + 4 finalize
-  // kernels + error check (mixed)
+  // those run on the tensor cores) or 2 FP32 copies + 3 operand
+  // packs + 3 GEMM launches (4 where vvvo has its own) + the vvvv pack and two product kernels + FP32
+  // Fock copies + 4 finalize kernels + error check (mixed)
   if (!(n - nocc > 0 && nocc > 0)) return 5;
   const int front = (nocc <= kT1Omax ? 4 : 5) + 7;
-  return front + (mixed ? 53 : fix_on_tensor_cores(nocc, n - nocc) ? 8 : 5);
+  return front + (mixed ? 17 + (vvvo_shares_launch(nocc, n - nocc) ? 0 : 1) : fix_on_tensor_cores(nocc, n - nocc) ? 8 : 5);
 }
 
 namespace {
@@ -1445,10 +1478,12 @@ __global__ void k_oovo_fin(double* __restrict__ W, const float* __restrict__ F, 
   const int b = (int)((x / d.o) % d.v), j = (int)(x % d.o);
   const int B_ = d.o + b;
   float v = 0.f;
+#pragma unroll 6
   for (int z = 0; z < nsplit; ++z) v += part[(size_t)z * m_all + x];  // split-K partials, in order
   // the O(o v) maps: [m i][b j] (same order as x) and [m j][b i]
   v += part[(size_t)nsplit * m_all + x];
   v += part[(size_t)(nsplit + 1) * m_all + (((size_t)m * d.o + j) * d.v + b) * d.o + i];
+#pragma unroll 8
   for (int e = 0; e < d.v; ++e) v += F[m * d.n + d.o + e] * t2[ti(d, i, j, e, b)];
   const double w = W[gi(d, m, i, B_, j)] + (double)v;
   W[gi(d, m, i, B_, j)] = w;
@@ -1503,14 +1538,22 @@ __global__ void k_pack_vvvv(const float* __restrict__ g, const float* __restrict
   }
 }
 
-constexpr int kV4Tile = 128;  // v <= 128: one CTA holds a family's whole v x v product
-constexpr int kV4K = 32;      // K chunk staged in shared memory
+constexpr int kV4K = 32;  // K chunk staged in shared memory
 
+// A block holds a T x T tile of one family's v x v product, T / 16 x T / 16 outputs per thread (rows
+// ty + 16 r, columns tx + 16 c).  A warp stages 32 consecutive k of one operand row at a time (whole
+// 128-byte lines), and rows of 36 floats let eight rows be read as float4 along k without bank
+// conflicts.  Bound by the latency of that staging and by the scattered read-modify-writes: 15 us at 40
+// orbitals, 190 us at 114 (a 128 x 128 tile per product whatever v is, lanes along the rows: 71 and
+// 247 us, and 55 at 24).  Tiles of 32 where one covers v, which leaves less of a tile unused; 64 else.
+template <int T>
 __global__ void __launch_bounds__(256) k_vvvv_restricted(double* __restrict__ W, const float* __restrict__ Gt,
                                                          const float* __restrict__ Tt, Dims d) {
-  __shared__ float ts[kV4K][kV4Tile + 4], gs[kV4K][kV4Tile + 4];  // [k][row]
+  constexpr int R = T / 16;
+  __shared__ __align__(16) float ts[T][kV4K + 4], gs[T][kV4K + 4];  // [row][k]
   const int o = d.o, v = d.v, oo = o * o;
   const int fam = 1 + blockIdx.x / v, x = blockIdx.x % v;  // families 1..5 (0: k_vvvv_diag)
+  const int tiles = (v + T - 1) / T, i0 = (int)(blockIdx.y / tiles) * T, j0 = (int)(blockIdx.y % tiles) * T;
   const size_t n1 = d.n, n2 = n1 * n1, n3 = n2 * n1;
   // row selectors of the batch: T row i, G row j
   auto trow = [&](int i) -> int { return (fam == 1 || fam == 3 || fam == 5) ? x * v + i : i * v + x; };
@@ -1521,45 +1564,56 @@ __global__ void __launch_bounds__(256) k_vvvv_restricted(double* __restrict__ W,
       default: return j * (v + 1);  // 5
     }
   };
-  const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;  // 16 x 16 threads, 8 x 8 outputs each
-  float acc[8][8];
+  const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16, lane = tid & 31;
+  float acc[R][R];
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
+  for (int r = 0; r < R; ++r)
 #pragma unroll
-    for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
+    for (int c = 0; c < R; ++c) acc[r][c] = 0.f;
   for (int k0 = 0; k0 < oo; k0 += kV4K) {
-    __syncthreads();
-    for (int t = tid; t < kV4K * kV4Tile; t += 256) {
-      const int kk = t / kV4Tile, r = t % kV4Tile, k = k0 + kk;
-      float tv = 0.f, gv = 0.f;
-      if (r < v && k < oo) {
-        tv = Tt[(size_t)trow(r) * oo + k];
-        gv = Gt[(size_t)grow(r) * oo + k];
-      }
-      ts[kk][r] = tv;
-      gs[kk][r] = gv;
+    const int k = k0 + lane;
+    float tv[T / 8], gv[T / 8];
+#pragma unroll
+    for (int q = 0; q < T / 8; ++q) {
+      const int r = (tid >> 5) + 8 * q;
+      tv[q] = (i0 + r < v && k < oo) ? Tt[(size_t)trow(i0 + r) * oo + k] : 0.f;
+      gv[q] = (j0 + r < v && k < oo) ? Gt[(size_t)grow(j0 + r) * oo + k] : 0.f;
     }
     __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < kV4K; ++kk) {
-      float a[8], b[8];
 #pragma unroll
-      for (int r = 0; r < 8; ++r) a[r] = ts[kk][ty * 8 + r];
+    for (int q = 0; q < T / 8; ++q) {
+      const int r = (tid >> 5) + 8 * q;
+      ts[r][lane] = tv[q];
+      gs[r][lane] = gv[q];
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int kk = 0; kk < kV4K; kk += 4) {
+      float4 a[R], b[R];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) b[c] = gs[kk][tx * 8 + c];
+      for (int r = 0; r < R; ++r) {
+        a[r] = *reinterpret_cast<const float4*>(&ts[ty + 16 * r][kk]);
+        b[r] = *reinterpret_cast<const float4*>(&gs[tx + 16 * r][kk]);
+      }
 #pragma unroll
-      for (int r = 0; r < 8; ++r)
+      for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int c = 0; c < 8; ++c) acc[r][c] = fmaf(a[r], b[c], acc[r][c]);
+        for (int c = 0; c < R; ++c) {
+          float s = acc[r][c];
+          s = fmaf(a[r].x, b[c].x, s);
+          s = fmaf(a[r].y, b[c].y, s);
+          s = fmaf(a[r].z, b[c].z, s);
+          acc[r][c] = fmaf(a[r].w, b[c].w, s);
+        }
     }
   }
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int i = ty * 8 + r;
+  for (int r = 0; r < R; ++r) {
+    const int i = i0 + ty + 16 * r;
     if (i >= v) continue;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int j = tx * 8 + c;
+    for (int c = 0; c < R; ++c) {
+      const int j = j0 + tx + 16 * c;
       if (j >= v) continue;
       int a, e, b, f;
       bool keep;
@@ -1578,30 +1632,90 @@ __global__ void __launch_bounds__(256) k_vvvv_restricted(double* __restrict__ W,
   }
 }
 
-// Family 0 (a = b, every (e, f)): C[e][f] = Tt(a,a).Gt(e v + f), a warp per output streaming
-// Gt's rows (contiguous) with Tt(a,a) in registers; kV4Diag blocks share one a.
-constexpr int kV4Diag = 8;
+// Family 0 (a = b, every (e, f)): C[e][f] = Tt(a,a).Gt(e v + f).  A warp takes two rows of Gt and kV4A
+// values of a at a time (6 loads for 8 outputs instead of 16) and reduces the eight sums together:
+// each step halves the values a lane holds, 9 shuffles instead of 40, with the same tree of
+// additions per output as a butterfly of its own (114 orbitals: 234 -> 69 us, 40: 21 -> 6.5).
+constexpr int kV4A = 4;
+inline int v4_parts(int v) {  // blocks per group of a: about four blocks per SM, at least a row pair per warp
+  const int groups = (v + kV4A - 1) / kV4A, want = (4 * 152 + groups - 1) / groups, most = (v * v + 15) / 16;
+  return want < most ? want : most;
+}
 __global__ void __launch_bounds__(256) k_vvvv_diag(double* __restrict__ W, const float* __restrict__ Gt,
-                                                   const float* __restrict__ Tt, Dims d) {
+                                                   const float* __restrict__ Tt, Dims d, int parts) {
   const int o = d.o, v = d.v, oo = o * o, lane = threadIdx.x & 31;
-  const int a = blockIdx.x / kV4Diag, part = blockIdx.x % kV4Diag;
+  const int a0 = (int)(blockIdx.x / parts) * kV4A, part = blockIdx.x % parts;
   const size_t n1 = d.n, n2 = n1 * n1, n3 = n2 * n1;
-  const float* trow = Tt + (size_t)(a * v + a) * oo;
-  const int rows = v * v, per = (rows + kV4Diag - 1) / kV4Diag;
-  const int r1 = (part + 1) * per < rows ? (part + 1) * per : rows;
-  for (int r = part * per + (int)(threadIdx.x >> 5); r < r1; r += (int)(blockDim.x >> 5)) {
-    const float* gr = Gt + (size_t)r * oo;
-    float acc = 0.f;
-    for (int k = lane; k < oo; k += 32) acc = fmaf(trow[k], gr[k], acc);
+  const float* trow[kV4A];
 #pragma unroll
-    for (int s2 = 16; s2 > 0; s2 >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s2);
-    if (lane == 0) {
-      const int e = r / v, f = r % v;
+  for (int q = 0; q < kV4A; ++q) {
+    const int a = a0 + q < v ? a0 + q : v - 1;
+    trow[q] = Tt + (size_t)(a * v + a) * oo;
+  }
+  const int rows = v * v;
+  for (int r = 2 * (part * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5)); r < rows;
+       r += 2 * parts * (int)(blockDim.x >> 5)) {
+    const float* g0 = Gt + (size_t)r * oo;
+    const float* g1 = r + 1 < rows ? g0 + oo : g0;
+    float s[2 * kV4A];
+#pragma unroll
+    for (int q = 0; q < 2 * kV4A; ++q) s[q] = 0.f;
+#pragma unroll 2
+    for (int k = lane; k < oo; k += 32) {
+      const float x0 = g0[k], x1 = g1[k];
+#pragma unroll
+      for (int q = 0; q < kV4A; ++q) {
+        const float t = trow[q][k];
+        s[q] = fmaf(t, x0, s[q]);
+        s[kV4A + q] = fmaf(t, x1, s[kV4A + q]);
+      }
+    }
+#pragma unroll
+    for (int h = 4; h >= 1; h >>= 1) {  // lanes with bit 4 h keep the upper half of the values
+      const bool up = lane & (4 * h);
+#pragma unroll
+      for (int q = 0; q < h; ++q) {
+        const float give = up ? s[q] : s[q + h], keep = up ? s[q + h] : s[q];
+        s[q] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * h);
+      }
+    }
+    s[0] += __shfl_xor_sync(0xffffffffu, s[0], 2);
+    s[0] += __shfl_xor_sync(0xffffffffu, s[0], 1);
+    const int a = a0 + ((lane >> 2) & 3), rr = r + (lane >> 4);
+    if ((lane & 3) == 0 && a < v && rr < rows) {
+      const int e = rr / v, f = rr % v;
       const size_t w = (size_t)(o + a) * n3 + (size_t)(o + e) * n2 + (size_t)(o + a) * n1 + (size_t)(o + f);
-      W[w] += (double)acc;
+      W[w] += (double)s[0];
     }
   }
 }
+
+// The stores of the block products that share a launch.
+struct StoreAny {
+  int kind;
+  union {
+    StoreOV ov;
+    StoreOO oo;
+    StoreOVO ovo;
+    StoreRows rows;
+    StoreVV vv;
+  };
+  StoreAny() = default;
+  StoreAny(StoreOV s) : kind(0), ov(s) {}
+  StoreAny(StoreOO s) : kind(1), oo(s) {}
+  StoreAny(StoreOVO s) : kind(2), ovo(s) {}
+  StoreAny(StoreRows s) : kind(3), rows(s) {}
+  StoreAny(StoreVV s) : kind(4), vv(s) {}
+  __device__ void run(int r, int col, const float (&v)[32], int cnt) const {
+    switch (kind) {
+      case 0: ov.run(r, col, v, cnt); break;
+      case 1: oo.run(r, col, v, cnt); break;
+      case 2: ovo.run(r, col, v, cnt); break;
+      case 3: rows.run(r, col, v, cnt); break;
+      default: vv.run(r, col, v, cnt); break;
+    }
+  }
+};
 
 struct Arena {
   float* base;
@@ -1620,8 +1734,9 @@ struct Op {  // a packed operand: hi / lo parts, rows padded to the tile (rows_p
   int rows, rows_p, K, ld;
 };
 
+// Carves one operand and describes its packing.
 template <class L>
-cudaError_t pack_op(L ld, int rows, int K, int tile, Arena& ar, Op* out, cudaStream_t st) {
+tc::PackJob<L> operand(L ld, int rows, int K, int tile, Arena& ar, Op* out) {
   const int rows_p = tc::pad_to(rows, tile), Kp = tc::pad_to(K, tc::BK);
   out->rows = rows;
   out->rows_p = rows_p;
@@ -1629,8 +1744,11 @@ cudaError_t pack_op(L ld, int rows, int K, int tile, Arena& ar, Op* out, cudaStr
   out->ld = Kp;
   out->hi = ar.take((size_t)rows_p * Kp);
   out->lo = ar.take((size_t)rows_p * Kp);
-  if (!ar.base) return cudaSuccess;
-  return tc::pack(ld, rows, K, rows_p, Kp, out->hi, out->lo, st);
+  return tc::PackJob<L>{ld, rows, K, rows_p, Kp, out->hi, out->lo, 0, 0};
+}
+template <class... L>
+cudaError_t pack_all(const Arena& ar, cudaStream_t st, const tc::PackJob<L>&... jobs) {
+  return ar.base ? tc::pack(st, jobs...) : cudaSuccess;
 }
 
 // operand tiles: A rows pad to 128; B rows pad to the launch's BN
@@ -1679,12 +1797,22 @@ cudaError_t run_ladder(tc::PackedJobs<StoreR2>& js, const Arena& ar, int* err, i
 // (m, n).
 cudaError_t pack_ladder(const TcCtx& c, int o, int v, Arena& ar, Op* a1, Op* b1, cudaStream_t st) {
   const int oo = o * o, vv = v * v;
-  cudaError_t e = pack_op(LR2G1A{c}, oo, vv + oo, kTileM, ar, a1, st);
-  if (e == cudaSuccess) e = pack_op(LR2G1B{c}, vv, vv + oo, kLadderPad, ar, b1, st);
-  return e;
+  const auto ja = operand(LR2G1A{c}, oo, vv + oo, kTileM, ar, a1);
+  const auto jb = operand(LR2G1B{c}, vv, vv + oo, kLadderPad, ar, b1);
+  return pack_all(ar, st, ja, jb);
 }
 
 constexpr int kOvoSplit = 6;  // split K of the oovo v^2 product (720 x 100 x v^2)
+
+// Whether the vvvo products take 32-column tiles in the launch of the other blocks (else 128-column
+// tiles in one of their own): where 32-column tiles of all of them are at most two per SM, so that the
+// launch is a chain of latencies rather than a stream of operands (40 orbitals: 35 us for all, 82 with
+// a launch per block and 22 of them for vvvo; at 114, 32-column tiles would re-read the v^2-row operand
+// four times as often: 0.55 ms with 128).
+bool vvvo_shares_launch(int o, int v) {
+  const long long m = (v * v + tc::BM - 1) / tc::BM, n = (o * v + 31) / 32;
+  return 3 * m * n <= 2 * 152;
+}
 
 // The T2 terms of the mixed path; with ar.base == nullptr only sizes the packed scratch.
 cudaError_t t2_terms_tc(const Dims& d, double* W, const float* G, const double* F, const float* t2, const Work& w,
@@ -1703,70 +1831,58 @@ cudaError_t t2_terms_tc(const Dims& d, double* W, const float* G, const double* 
   do {                                  \
     if (e == cudaSuccess) e = (x);      \
   } while (0)
-  // Woooo first: the ladder + oooo map reads it
+  // Woooo (the ladder + oooo map reads it) and the ring intermediates
   {
     ar.reset();
-    Op a, b;
-    QF_TRY(pack_op(LWOA{c}, oo, vv, kTileM, ar, &a, st));
-    QF_TRY(pack_op(LWOB{c}, oo, vv, 32, ar, &b, st));
+    Op a, b, au, at, atx, b0, b1;
+    const auto p0 = operand(LWOA{c}, oo, vv, kTileM, ar, &a);
+    const auto p1 = operand(LWOB{c}, oo, vv, 64, ar, &b);
+    const auto p2 = operand(LRingA{c, 0}, ov, ov, kTileM, ar, &au);
+    const auto p3 = operand(LRingA{c, 1}, ov, ov, kTileM, ar, &at);
+    const auto p4 = operand(LRingA{c, 2}, ov, ov, kTileM, ar, &atx);
+    const auto p5 = operand(LRingB{c, 0}, ov, ov, 64, ar, &b0);
+    const auto p6 = operand(LRingB{c, 1}, ov, ov, 64, ar, &b1);
+    QF_TRY(pack_all(ar, st, p0, p1, p2, p3, p4, p5, p6));
     float* wp = ar.take((size_t)oo * oo * kWoSplit);
-    tc::PackedJobs<StoreRows> js{};
-    for (int z = 0; z < kWoSplit; ++z) js.j[z] = job(a, b, StoreRows{wp + (run ? (size_t)oo * oo * z : 0), oo}, z, kWoSplit);
-    js.count = kWoSplit;
-    QF_TRY((run_jobs<32>(js, ar, err, st)));
-    if (run && e == cudaSuccess) {
-      k_wo_fin<<<blocks_for((size_t)oo * oo), TPB, 0, st>>>(W, wp, w.wo, d);
-      e = cudaGetLastError();
-    }
-  }
-  // ring intermediates: one launch of four jobs sharing packed operands
-  {
-    ar.reset();
-    Op au, at, atx, b0, b1;
-    QF_TRY(pack_op(LRingA{c, 0}, ov, ov, kTileM, ar, &au, st));
-    QF_TRY(pack_op(LRingA{c, 1}, ov, ov, kTileM, ar, &at, st));
-    QF_TRY(pack_op(LRingA{c, 2}, ov, ov, kTileM, ar, &atx, st));
-    QF_TRY(pack_op(LRingB{c, 0}, ov, ov, 64, ar, &b0, st));
-    QF_TRY(pack_op(LRingB{c, 1}, ov, ov, 64, ar, &b1, st));
     tc::PackedJobs<StoreRows> js{};
     js.j[0] = job(au, b0, StoreRows{A, ov});
     js.j[1] = job(au, b1, StoreRows{B, ov});
     js.j[2] = job(at, b1, StoreRows{Cq, ov});
     js.j[3] = job(atx, b1, StoreRows{D, ov});
-    js.count = 4;
+    for (int z = 0; z < kWoSplit; ++z)
+      js.j[4 + z] = job(a, b, StoreRows{wp + (run ? (size_t)oo * oo * z : 0), oo}, z, kWoSplit);
+    js.count = 4 + kWoSplit;
     QF_TRY((run_jobs<64>(js, ar, err, st)));
+    if (run && e == cudaSuccess) {
+      k_wo_fin<<<blocks_for((size_t)oo * oo), TPB, 0, st>>>(W, wp, w.wo, d);
+      e = cudaGetLastError();
+    }
   }
-  // r2: ladder + oooo term
+  // r2: ladder + oooo term, and the rings (four output maps)
   {
     ar.reset();
-    Op a1, b1;
-    QF_TRY(pack_ladder(c, o, v, ar, &a1, &b1, st));
-    tc::PackedJobs<StoreR2> js{};
-    js.j[0] = job(a1, b1, StoreR2{acc, o, v, 4});
-    js.count = 1;
-    QF_TRY(run_ladder(js, ar, err, ladder_bn, st));
-  }
-  // r2: rings (four output maps, one launch)
-  {
-    ar.reset();
-    Op a3, b3, a4, b4, a5, b5, a6, b6;
-    QF_TRY(pack_op(LR2G3A{c}, ov, 5 * ov, kTileM, ar, &a3, st));
-    QF_TRY(pack_op(LR2G3B{c}, ov, 5 * ov, 64, ar, &b3, st));
-    QF_TRY(pack_op(LR2G4A{c}, ov, 2 * ov, kTileM, ar, &a4, st));
-    QF_TRY(pack_op(LR2G4B{c}, ov, 2 * ov, 64, ar, &b4, st));
-    QF_TRY(pack_op(LR2G5A{c}, ov, ov, kTileM, ar, &a5, st));
-    QF_TRY(pack_op(LR2G5B{c}, ov, ov, 64, ar, &b5, st));
-    QF_TRY(pack_op(LR2G6A{c}, ov, 2 * ov, kTileM, ar, &a6, st));
-    QF_TRY(pack_op(LR2G6B{c}, ov, 2 * ov, 64, ar, &b6, st));
+    Op a1, b1, a3, b3, a4, b4, a5, b5, a6, b6;
+    const auto p0 = operand(LR2G1A{c}, oo, vv + oo, kTileM, ar, &a1);
+    const auto p1 = operand(LR2G1B{c}, vv, vv + oo, kLadderPad, ar, &b1);
+    const auto p2 = operand(LR2G3A{c}, ov, 5 * ov, kTileM, ar, &a3);
+    const auto p3 = operand(LR2G3B{c}, ov, 5 * ov, kLadderPad, ar, &b3);
+    const auto p4 = operand(LR2G4A{c}, ov, 2 * ov, kTileM, ar, &a4);
+    const auto p5 = operand(LR2G4B{c}, ov, 2 * ov, kLadderPad, ar, &b4);
+    const auto p6 = operand(LR2G5A{c}, ov, ov, kTileM, ar, &a5);
+    const auto p7 = operand(LR2G5B{c}, ov, ov, kLadderPad, ar, &b5);
+    const auto p8 = operand(LR2G6A{c}, ov, 2 * ov, kTileM, ar, &a6);
+    const auto p9 = operand(LR2G6B{c}, ov, 2 * ov, kLadderPad, ar, &b6);
+    QF_TRY(pack_all(ar, st, p0, p1, p2, p3, p4, p5, p6, p7, p8, p9));
     const size_t n_r2 = (size_t)oo * vv;
     float* part = ar.take(4 * n_r2);
     tc::PackedJobs<StoreR2> js{};
-    js.j[0] = job(a3, b3, StoreR2{part, o, v, 0});
-    js.j[1] = job(a4, b4, StoreR2{run ? part + n_r2 : nullptr, o, v, 1});
-    js.j[2] = job(a5, b5, StoreR2{run ? part + 2 * n_r2 : nullptr, o, v, 2});
-    js.j[3] = job(a6, b6, StoreR2{run ? part + 3 * n_r2 : nullptr, o, v, 3});
-    js.count = 4;
-    QF_TRY((run_jobs<64>(js, ar, err, st)));
+    js.j[0] = job(a1, b1, StoreR2{acc, o, v, 4});
+    js.j[1] = job(a3, b3, StoreR2{part, o, v, 0});
+    js.j[2] = job(a4, b4, StoreR2{run ? part + n_r2 : nullptr, o, v, 1});
+    js.j[3] = job(a5, b5, StoreR2{run ? part + 2 * n_r2 : nullptr, o, v, 2});
+    js.j[4] = job(a6, b6, StoreR2{run ? part + 3 * n_r2 : nullptr, o, v, 3});
+    js.count = 5;
+    QF_TRY(run_ladder(js, ar, err, ladder_bn, st));
     if (run && e == cudaSuccess) {
       const float* f32 = w.f32;
       k_fock_f32<<<blocks_for((size_t)d.n * d.n + oo + vv), TPB, 0, st>>>(F, w.foo, w.fvv, w.f32, d);
@@ -1776,89 +1892,75 @@ cudaError_t t2_terms_tc(const Dims& d, double* W, const float* G, const double* 
     }
   }
   // blocks written in place (their bases are read from W by the store of their single job)
-  {  // vvvv: only the elements (k, k) spaces read, six batched SIMT products (v <= 128)
-    static_assert(kV4Tile >= 128, "n <= 128 orbitals: v fits one tile");
+  {  // vvvv: only the elements (k, k) spaces read, six batched SIMT products
     ar.reset();
     float* Gt = ar.take((size_t)vv * oo);
     float* Tt = ar.take((size_t)vv * oo);
     if (run && e == cudaSuccess) {
       const size_t m_all = (size_t)vv * oo;
       k_pack_vvvv<<<blocks_for(m_all) > 152u * 32u ? 152u * 32u : blocks_for(m_all), TPB, 0, st>>>(G, t2, Gt, Tt, d);
-      k_vvvv_diag<<<kV4Diag * v, 256, 0, st>>>(W, Gt, Tt, d);
-      k_vvvv_restricted<<<5 * v, 256, 0, st>>>(W, Gt, Tt, d);
+      const int groups = (v + kV4A - 1) / kV4A, parts = v4_parts(v);
+      k_vvvv_diag<<<(unsigned)(groups * parts), 256, 0, st>>>(W, Gt, Tt, d, parts);
+      if (v <= 32) {
+        k_vvvv_restricted<32><<<5 * v, 256, 0, st>>>(W, Gt, Tt, d);
+      } else {
+        const unsigned t = (unsigned)(v + 63) / 64;
+        k_vvvv_restricted<64><<<dim3(5 * v, t * t), 256, 0, st>>>(W, Gt, Tt, d);
+      }
       e = cudaGetLastError();
     }
   }
+  // ovov, oovv (in place), oovo (the v^2 term split over K into partial outputs summed in order by
+  // k_oovo_fin, and its two O(o v) maps) and vvvo (three output maps, each its own buffer, summed by
+  // k_vvvo_fin)
   {
     ar.reset();
-    Op a, b;
-    QF_TRY(pack_op(LOVA{c}, ov, 2 * ov, kTileM, ar, &a, st));
-    QF_TRY(pack_op(LOVB{c}, ov, 2 * ov, 32, ar, &b, st));
-    tc::PackedJobs<StoreOV> js{};
-    js.j[0] = job(a, b, StoreOV{W, d.n, o, v});
-    js.count = 1;
-    QF_TRY((run_jobs<32>(js, ar, err, st)));
-  }
-  {
-    ar.reset();
-    Op a, b;
-    QF_TRY(pack_op(LOOA{c}, ov, ov, kTileM, ar, &a, st));
-    QF_TRY(pack_op(LOOB{c}, ov, ov, 32, ar, &b, st));
-    tc::PackedJobs<StoreOO> js{};
-    js.j[0] = job(a, b, StoreOO{W, d.n, o, v});
-    js.count = 1;
-    QF_TRY((run_jobs<32>(js, ar, err, st)));
-  }
-  // oovo v^2 term, split K into partial outputs summed in order by k_oovo_fin
-  float* part = nullptr;
-  {
-    ar.reset();
-    Op a, b;
-    QF_TRY(pack_op(LOVOA{c}, ov, vv, kTileM, ar, &a, st));
-    QF_TRY(pack_op(LOVOB{c}, oo, vv, 32, ar, &b, st));
-    const size_t n_ovo = (size_t)oo * v * o;
-    part = ar.take(n_ovo * (kOvoSplit + 2));  // + the two O(o v) maps
-    tc::PackedJobs<StoreOVO> js{};
-    for (int z = 0; z < kOvoSplit; ++z) js.j[z] = job(a, b, StoreOVO{part + (run ? n_ovo * z : 0), o, v}, z, kOvoSplit);
-    js.count = kOvoSplit;
-    QF_TRY((run_jobs<32>(js, ar, err, st)));
-    Op a2, b2, a3, b3;
-    QF_TRY(pack_op(LOV2A{c}, oo, 2 * ov, kTileM, ar, &a2, st));
-    QF_TRY(pack_op(LOV2B{c}, ov, 2 * ov, 32, ar, &b2, st));
-    QF_TRY(pack_op(LOV3A{c}, oo, ov, kTileM, ar, &a3, st));
-    QF_TRY(pack_op(LOV3B{c}, ov, ov, 32, ar, &b3, st));
-    tc::PackedJobs<StoreRows> jr{};
-    jr.j[0] = job(a2, b2, StoreRows{part + (run ? n_ovo * kOvoSplit : 0), ov});
-    jr.j[1] = job(a3, b3, StoreRows{part + (run ? n_ovo * (kOvoSplit + 1) : 0), ov});
-    jr.count = 2;
-    QF_TRY((run_jobs<32>(jr, ar, err, st)));
-  }
-  if (run && e == cudaSuccess) {
-    k_oovo_fin<<<blocks_for((size_t)oo * v * o), TPB, 0, st>>>(W, w.f32, t2, part, kOvoSplit, d);
-    e = cudaGetLastError();
-  }
-  // vvvo: three output maps, one launch; each job its own buffer, summed by k_vvvo_fin
-  {
-    ar.reset();
-    Op a1, b1, a2, b2, a3, b3;
-    QF_TRY(pack_op(LVV1A{c}, vv, 2 * ov, kTileM, ar, &a1, st));
-    QF_TRY(pack_op(LVV1B{c}, v * o, 2 * ov, 128, ar, &b1, st));
-    QF_TRY(pack_op(LVV2A{c}, vv, oo, kTileM, ar, &a2, st));
-    QF_TRY(pack_op(LVV2B{c}, v * o, oo, 128, ar, &b2, st));
-    QF_TRY(pack_op(LVV3A{c}, vv, ov, kTileM, ar, &a3, st));
-    QF_TRY(pack_op(LVV3B{c}, v * o, ov, 128, ar, &b3, st));
-    const size_t n_vvvo = (size_t)vv * v * o;
-    float* p1 = ar.take(n_vvvo);
-    float* p2 = ar.take(n_vvvo);
-    tc::PackedJobs<StoreVV> js{};
-    js.j[0] = job(a1, b1, StoreVV{acc, o, v, 0});
-    js.j[1] = job(a2, b2, StoreVV{p1, o, v, 1});
-    js.j[2] = job(a3, b3, StoreVV{p2, o, v, 2});
-    js.count = 3;
-    // 128-column tiles: half the re-reads of the v^2-row operand from L2
-    QF_TRY((run_jobs<128>(js, ar, err, st)));
+    Op a0, b0, a1, b1, a2, b2, a3, b3, a4, b4, a5, b5, a6, b6, a7, b7;
+    const auto p0 = operand(LOVA{c}, ov, 2 * ov, kTileM, ar, &a0);
+    const auto p1 = operand(LOVB{c}, ov, 2 * ov, 32, ar, &b0);
+    const auto p2 = operand(LOOA{c}, ov, ov, kTileM, ar, &a1);
+    const auto p3 = operand(LOOB{c}, ov, ov, 32, ar, &b1);
+    const auto p4 = operand(LOVOA{c}, ov, vv, kTileM, ar, &a2);
+    const auto p5 = operand(LOVOB{c}, oo, vv, 32, ar, &b2);
+    const auto p6 = operand(LOV2A{c}, oo, 2 * ov, kTileM, ar, &a3);
+    const auto p7 = operand(LOV2B{c}, ov, 2 * ov, 32, ar, &b3);
+    const auto p8 = operand(LOV3A{c}, oo, ov, kTileM, ar, &a4);
+    const auto p9 = operand(LOV3B{c}, ov, ov, 32, ar, &b4);
+    const auto q0 = operand(LVV1A{c}, vv, 2 * ov, kTileM, ar, &a5);
+    const auto q1 = operand(LVV1B{c}, ov, 2 * ov, 128, ar, &b5);
+    const auto q2 = operand(LVV2A{c}, vv, oo, kTileM, ar, &a6);
+    const auto q3 = operand(LVV2B{c}, ov, oo, 128, ar, &b6);
+    const auto q4 = operand(LVV3A{c}, vv, ov, kTileM, ar, &a7);
+    const auto q5 = operand(LVV3B{c}, ov, ov, 128, ar, &b7);
+    QF_TRY(pack_all(ar, st, p0, p1, p2, p3, p4, p5, p6, p7, p8, p9, q0, q1, q2, q3, q4, q5));
+    const size_t n_ovo = (size_t)oo * v * o, n_vvvo = (size_t)vv * v * o;
+    float* part = ar.take(n_ovo * (kOvoSplit + 2));
+    float* v1 = ar.take(n_vvvo);
+    float* v2 = ar.take(n_vvvo);
+    tc::PackedJobs<StoreAny> js{};
+    js.j[0] = job<StoreAny>(a0, b0, StoreOV{W, d.n, o, v});
+    js.j[1] = job<StoreAny>(a1, b1, StoreOO{W, d.n, o, v});
+    for (int z = 0; z < kOvoSplit; ++z)
+      js.j[2 + z] = job<StoreAny>(a2, b2, StoreOVO{part + (run ? n_ovo * z : 0), o, v}, z, kOvoSplit);
+    js.j[2 + kOvoSplit] = job<StoreAny>(a3, b3, StoreRows{part + (run ? n_ovo * kOvoSplit : 0), ov});
+    js.j[3 + kOvoSplit] = job<StoreAny>(a4, b4, StoreRows{part + (run ? n_ovo * (kOvoSplit + 1) : 0), ov});
+    js.count = 4 + kOvoSplit;
+    tc::PackedJobs<StoreAny> jv{};
+    jv.j[0] = job<StoreAny>(a5, b5, StoreVV{acc, o, v, 0});
+    jv.j[1] = job<StoreAny>(a6, b6, StoreVV{v1, o, v, 1});
+    jv.j[2] = job<StoreAny>(a7, b7, StoreVV{v2, o, v, 2});
+    jv.count = 3;
+    if (vvvo_shares_launch(o, v)) {
+      for (int z = 0; z < 3; ++z) js.j[js.count++] = jv.j[z];
+      QF_TRY((run_jobs<32>(js, ar, err, st)));
+    } else {
+      QF_TRY((run_jobs<32>(js, ar, err, st)));
+      // 128-column tiles: half the re-reads of the v^2-row operand from L2
+      QF_TRY((run_jobs<128>(jv, ar, err, st)));
+    }
     if (run && e == cudaSuccess) {
-      k_vvvo_fin<<<blocks_for(n_vvvo), TPB, 0, st>>>(W, w.f32, t2, acc, p1, p2, d);
+      k_oovo_fin<<<(unsigned)(((size_t)oo * v * o + 63) / 64), 64, 0, st>>>(W, w.f32, t2, part, kOvoSplit, d);
+      k_vvvo_fin<<<blocks_for(n_vvvo), TPB, 0, st>>>(W, w.f32, t2, acc, v1, v2, d);
       e = cudaGetLastError();
     }
   }
@@ -1897,8 +1999,8 @@ cudaError_t launch_dress(const double* h, const double* eri, const double* t1, c
   } else {
     k_copy<<<blocks_for(n4) > 152u * 64u ? 152u * 64u : blocks_for(n4), TPB, 0, st>>>(eri, W, n4);
   }
-  k_h_tilde<<<blocks_for((size_t)n * n), TPB, 0, st>>>(h, t1, w.ht, d);
-  k_fock<<<blocks_for((size_t)n * n), TPB, 0, st>>>(w.ht, W, F, d);
+  k_h_tilde<<<n, n, n * sizeof(double), st>>>(h, t1, w.ht, d);
+  k_fock<<<(n * n + 31) / 32, 32, 0, st>>>(w.ht, W, F, d);  // a warp per block: all SMs take part
   k_energy_part<<<EGRID, TPB, 0, st>>>(w.ht, W, t2, w.epart, d);
   k_energy_sum<<<1, EGRID, 0, st>>>(w.epart, e0);
   if (v > 0 && o > 0) {

@@ -224,7 +224,7 @@ cudaError_t gemm_rows(int M, int N, int K, const float* A, int lda, LoadB lb, St
   const int rows_p = pad_to(N, bn), ld = pad_to(K, BK);
   float* bh = pack_buf;
   float* bl = bh + (size_t)rows_p * ld;
-  cudaError_t e = pack(lb, N, K, rows_p, ld, bh, bl, stream);
+  cudaError_t e = pack(stream, PackJob<LoadB>{lb, N, K, rows_p, ld, bh, bl, 0, 0});
   if (e != cudaSuccess) return e;
   RowsArgs g{};
   g.M = M;

@@ -304,34 +304,55 @@ namespace tc {
 
 constexpr int PTHREADS = 256;  // threads of a packed-engine CTA
 
-// out_hi/out_lo[r][k] = split(L(r, k)) for r < rows, k < K; zero in the padding.
+// One operand to pack: hi/lo[r][k] = split(L(r, k)) for r < rows, k < K; zero in the padding.
+template <class L>
+struct PackJob {
+  L ld;
+  int rows, K, rows_p, Kp;
+  float *hi, *lo;
+  unsigned b0, nb;  // its blocks of the launch (set by pack)
+};
+
 // (r, k) of the grid-stride index x = r Kp + k advance by the stride's own digits with a carry,
 // so no 64-bit division runs per element.
 template <class L>
-__global__ void k_pack(L ld, int rows, int K, int rows_p, int Kp, float* __restrict__ hi, float* __restrict__ lo) {
-  const size_t total = (size_t)rows_p * Kp;
-  const size_t x0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
-  int r = (int)(x0 / Kp), k = (int)(x0 % Kp);
-  const int sr = (int)(step / Kp), sk = (int)(step % Kp);
+__device__ __forceinline__ void pack_body(const PackJob<L>& j) {
+  const size_t total = (size_t)j.rows_p * j.Kp;
+  const size_t x0 = (blockIdx.x - j.b0) * (size_t)blockDim.x + threadIdx.x, step = (size_t)j.nb * blockDim.x;
+  int r = (int)(x0 / j.Kp), k = (int)(x0 % j.Kp);
+  const int sr = (int)(step / j.Kp), sk = (int)(step % j.Kp);
   for (size_t x = x0; x < total; x += step) {
-    const float v = (r < rows && k < K) ? ld(r, k) : 0.f;
+    const float v = (r < j.rows && k < j.K) ? j.ld(r, k) : 0.f;
     const float h = tf32_round(v);
-    hi[x] = h;
-    lo[x] = tf32_round(v - h);
+    j.hi[x] = h;
+    j.lo[x] = tf32_round(v - h);
     k += sk;
-    const int c = k >= Kp;
-    k -= c ? Kp : 0;
+    const int c = k >= j.Kp;
+    k -= c ? j.Kp : 0;
     r += sr + c;
   }
 }
 
-template <class L>
-cudaError_t pack(L ld, int rows, int K, int rows_p, int Kp, float* hi, float* lo, cudaStream_t st) {
-  const size_t total = (size_t)rows_p * Kp;
-  size_t g = (total + 255) / 256;
-  if (g > 152 * 64) g = 152 * 64;
-  if (g < 1) g = 1;
-  k_pack<L><<<(unsigned)g, 256, 0, st>>>(ld, rows, K, rows_p, Kp, hi, lo);
+// Operands of one or more products in one launch, each with blocks of its own: below about 40 orbitals
+// an operand costs the 2 to 3 us of a launch, whatever its size (a common grid for all, indexed by
+// operand, spent longer on empty blocks: 53 instead of 17 us for the ten operands of the residual at
+// 40 orbitals).
+template <class... L>
+__global__ void k_pack(const PackJob<L>... jobs) {
+  ((blockIdx.x - jobs.b0 < jobs.nb ? pack_body(jobs) : void()), ...);
+}
+
+template <class... L>
+cudaError_t pack(cudaStream_t st, PackJob<L>... jobs) {
+  unsigned blocks = 0;
+  auto place = [&](auto& j) {
+    const size_t g = ((size_t)j.rows_p * j.Kp + 511) / 512;  // two elements per thread
+    j.b0 = blocks;
+    j.nb = (unsigned)(g > 152 * 64 ? 152 * 64 : g < 1 ? 1 : g);
+    blocks += j.nb;
+  };
+  (place(jobs), ...);
+  k_pack<L...><<<blocks, 256, 0, st>>>(jobs...);
   return cudaGetLastError();
 }
 
@@ -349,7 +370,7 @@ struct PackedJob {
   Store st;
 };
 
-constexpr int kMaxJobs = 8;
+constexpr int kMaxJobs = 13;
 template <class Store>
 struct PackedJobs {
   PackedJob<Store> j[kMaxJobs];
