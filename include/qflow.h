@@ -125,11 +125,12 @@ typedef struct {
   int32_t form;               /* qflow_form: the downfolding form (default QFLOW_FORM_SESCC)  */
   int32_t warps;              /* mixed precision: spaces (warps) per CTA of the solver, 1..15;
                                  0 = chosen by the autotuner (QFLOW_SCHED_AUTO) or 15        */
-  int32_t chunk;              /* mixed precision, persistent queue: consecutive spaces a warp
-                                 takes per fetch, 1..16; 0 = chosen by the autotuner
-                                 (QFLOW_SCHED_AUTO) or 1                                     */
+  int32_t chunk;              /* mixed precision, persistent queue: a CTA takes chunk x warps
+                                 consecutive spaces per fetch, its warps one after another,
+                                 1..16; 0 = chosen by the autotuner (QFLOW_SCHED_AUTO) or 1  */
   int32_t ladder_bn;          /* mixed precision, SES-CC form: tile width (columns) of the
-                                 dressing's ladder + oooo tensor-core product, 32, 64 or 128;
+                                 dressing's ladder + oooo tensor-core product (and of the
+                                 rings, which share its launch), 32, 64 or 128;
                                  0 = chosen by the autotuner (QFLOW_SCHED_AUTO) or 64.  Every
                                  width gives the same products bit for bit.                  */
   int32_t reserved[2];

@@ -697,7 +697,9 @@ size_t tc_arena_floats(int n, int nocc);
 bool vvvo_shares_launch(int o, int v);
 // Whether the FP64 products of o occupied and v virtual orbitals run on the tensor cores (oz_gemm.cuh)
 // rather than the integer pipe (fix_gemm.cuh, which needs no packed operands): where their work, about
-// 3 o^2 v^4 terms and more, covers the packing and fills the SMs' tiles.
+// 3 o^2 v^4 terms and more, covers the packing and fills the SMs' tiles.  Dressings on the tensor cores /
+// the integer pipe: o^2 v^4 = 4.8e7 (40 orbitals, 6 occupied) 0.729 / 0.714 ms, 7.5e7 (44, 6) 0.917 / 0.992,
+// 1.7e8 (50, 7) 1.22 / 1.66, 2.7e9 (82, 10) 6.6 / 13.7.
 bool fix_on_tensor_cores(int o, int v) { return o > 0 && v > 0 && (double)o * o * v * v * v * v >= kTensorTerms; }
 size_t fix_scale_ints(int o, int v);
 size_t fix_slice_bytes(int n, int o);

@@ -377,7 +377,9 @@ inline cudaError_t row_scales(Ops& ops, cudaStream_t st) {
 
 // Runs the jobs of one launch, longest sums first.  Tile size: a 64 x 64 tile takes time ~ K; a
 // product whose tile would take more than half of the launch's share of one of the 2 x 152 CTA
-// slots gets 32 x 32 tiles (a quarter of the time per tile, twice the conversions per term).
+// slots gets 32 x 32 tiles (a quarter of the time per tile, twice the conversions per term).  Dressings
+// with 64 x 64 tiles only / 32 x 32 only / this rule: 10 orbitals 0.201 / 0.146 / 0.146 ms, 24 orbitals 0.413 /
+// 0.270 / 0.272, 32 orbitals 0.682 / 0.430 / 0.429, 40 orbitals 1.008 / 0.732 / 0.707.
 inline cudaError_t run(Jobs& js, cudaStream_t st) {
   auto klen = [](const Job& j) {
     long k = 0;

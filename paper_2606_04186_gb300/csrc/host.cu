@@ -220,7 +220,7 @@ struct qflow_ctx {
   int64_t* rescue_items = nullptr;  // mixed path: positions of spaces the warp pass left unconverged
   unsigned long long* rescue_count = nullptr;  // and their count (device)
   // launch schedule of the mixed-precision solver: persistent queue or one launch per class
-  int sched_persistent = 1, sched_chunk = 1, sched_warps = 15;  // items per fetch, warps (spaces) per CTA
+  int sched_persistent = 1, sched_chunk = 1, sched_warps = 15;  // items per warp and fetch, warps (spaces) per CTA
   bool tuned = false;
   int64_t sweeps = 0;  // sweeps run so far
   float tune_ms[QFLOW_TUNE_MAX] = {0};
@@ -758,7 +758,7 @@ cudaError_t autotune(qflow_ctx* c) {
       return cudaSuccess;
     }
   }
-  // candidates: (persistent, items per fetch, warps per CTA).  Only the persistent queue: the
+  // candidates: (persistent, items per warp and fetch of a CTA, warps per CTA).  Only the persistent queue: the
   // per-class grid-stride launch, which can tie on a calibration prefix, loses its L2 locality
   // over a whole list (n82: 90 ms against 76 ms).  Fewer warps per CTA leave more of the SM's
   // 256 KB to the L1 cache (the coupling tables and the gathered blocks) at the cost of latency
