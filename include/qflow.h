@@ -360,10 +360,9 @@ int qflow_fma_peak(int32_t precision, double* tflops, void* stream);
  * synchronisation an allocation may cause, or services with a fixed pre-reserved budget.
  *
  * qflow_dress_device_static computes exactly what qflow_dress_device computes (same kernels,
- * same arguments except the workspace) but takes its scratch from a static device array of
- * qflow_static_scratch_bytes() bytes inside the library, so the call allocates nothing (no
- * cudaMalloc, no cudaFree, no allocating library routine).  The array is held by every GPU
- * that loads the library until the process exits.
+ * same arguments except the workspace) but takes its scratch from a static device array inside
+ * the library, so the call allocates nothing (no cudaMalloc, no cudaFree, no allocating library
+ * routine).  The array is held by every GPU that loads the library until the process exits.
  *   - Limit: the call returns QFLOW_ERR_TOO_LARGE when its arrays (about 48 nocc^2 nvir^2 bytes)
  *     exceed QFLOW_STATIC_SCRATCH_BYTES (4 MiB, e.g. 40 orbitals with 6 occupied fit, 82 do not).
  *     qflow_dress_workspace(n, nocc) can be larger: with it the larger problems' products run on
@@ -382,7 +381,7 @@ int qflow_fma_peak(int32_t precision, double* tflops, void* stream);
 #define QFLOW_STATIC_SCRATCH_BYTES (4u * 1024u * 1024u)
 int qflow_dress_device_static(const double* h, const double* eri, const double* t1, const double* t2, int32_t n,
                               int32_t nocc, double* e0, double* F, double* W, void* stream);
-/* Size of that static scratch array in bytes (the limit, and room for scale factors). */
+/* That limit in bytes: every problem with qflow_dress_workspace(n, nocc) up to it is accepted. */
 size_t qflow_static_scratch_bytes(void);
 
 /* ---- warm-start network (not in the paper) -----------------------------------------------

@@ -93,4 +93,6 @@ extern "C" int qflow_dress_device_static(const double* h, const double* eri, con
       qf::launch_dress(h, eri, t1, t2, n, nocc, e0, F, W, scratch, kStaticScratchBytes, (cudaStream_t)stream));
 }
 
-extern "C" size_t qflow_static_scratch_bytes(void) { return kStaticScratchBytes; }
+// The limit, not the array's size: a caller that compares qflow_dress_workspace with it and finds that it
+// fits must not be refused.
+extern "C" size_t qflow_static_scratch_bytes(void) { return (size_t)QFLOW_STATIC_SCRATCH_BYTES; }
