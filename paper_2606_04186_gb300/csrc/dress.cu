@@ -1989,8 +1989,10 @@ cudaError_t launch_dress(const double* h, const double* eri, const double* t1, c
   Work w;
   const bool mixed = g32 != nullptr;
   if (work_bytes < carve(nullptr, n, nocc, &w, mixed)) return cudaErrorInvalidValue;
-  // a caller with less than dress_workspace_bytes (the static scratch) gets the products that pack nothing
-  const bool slices = !mixed && fix_on_tensor_cores(nocc, n - nocc) && work_bytes >= carve(nullptr, n, nocc, &w, false, true);
+  // a caller with less than dress_workspace_bytes (the static scratch), or with a workspace that TMA cannot
+  // read (off 16 bytes), gets the products that pack nothing
+  const bool slices = !mixed && fix_on_tensor_cores(nocc, n - nocc) && (reinterpret_cast<uintptr_t>(work) & 15u) == 0 &&
+                      work_bytes >= carve(nullptr, n, nocc, &w, false, true);
   carve(work, n, nocc, &w, mixed, slices);
   Dims d{n, nocc, n - nocc};
   const size_t n4 = (size_t)n * n * n * n;

@@ -595,7 +595,8 @@ struct MlpWork {
     Y = take(y);
     dY = take(y);
     part = take(LGRID + 4);
-    pack = take(pk);
+    pack = take(pk ? pk + 4 : 0);  // read by TMA: on 16 bytes whatever the workspace's own alignment
+    pack = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(pack) + 15) & ~(uintptr_t)15);
     err = reinterpret_cast<int*>(take(64));
     bytes = off;
   }
