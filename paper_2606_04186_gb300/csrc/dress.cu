@@ -699,8 +699,10 @@ bool vvvo_shares_launch(int o, int v);
 // rather than the integer pipe (fix_gemm.cuh, which needs no packed operands): where their work, about
 // 3 o^2 v^4 terms and more, covers the packing and fills the SMs' tiles.  Dressings on the tensor cores /
 // the integer pipe: o^2 v^4 = 4.8e7 (40 orbitals, 6 occupied) 0.729 / 0.714 ms, 7.5e7 (44, 6) 0.917 / 0.992,
-// 1.7e8 (50, 7) 1.22 / 1.66, 2.7e9 (82, 10) 6.6 / 13.7.
-bool fix_on_tensor_cores(int o, int v) { return o > 0 && v > 0 && (double)o * o * v * v * v * v >= kTensorTerms; }
+// 1.7e8 (50, 7) 1.22 / 1.66, 2.7e9 (82, 10) 6.6 / 13.7.  One or two occupied orbitals fill at most 4 of a
+// tile's 128 rows, and the packed v^4 operand (4.4 GB at 128 orbitals) costs more than it saves: (128, 1)
+// 18.8 / 17.8, (96, 2) 6.48 / 6.27, against (96, 3) 7.08 / 7.42, (96, 6) 8.5 / 13.4.
+bool fix_on_tensor_cores(int o, int v) { return o >= 3 && v > 0 && (double)o * o * v * v * v * v >= kTensorTerms; }
 size_t fix_scale_ints(int o, int v);
 size_t fix_slice_bytes(int n, int o);
 
