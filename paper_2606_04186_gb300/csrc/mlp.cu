@@ -101,18 +101,17 @@ __global__ void k_colsum(const float* __restrict__ X, int rows, int cols, int ld
 }
 
 // ---- small products: FP32 FMA tiles -------------------------------------------------------------
-// A training step multiplies 128-row batches: at most 4 x 4 tensor-core tiles with K up to 708, so the
-// tensor-core engines leave most SMs idle and run K serially (30-90 us a product).  Here a CTA owns a
-// 32 x 32 tile and its eight warps share every 64-k slab (eight k each, 4 x 8 outputs per lane, the
-// partial tiles summed in warp order at the end): 32 to 184 CTAs per product.  The next slab is in
-// registers while this one is multiplied.  With `colsum` (B's column sums, the bias gradient) the CTAs of
-// the first row tile also add up B.
+// Inference of a small batch: 128 rows are one row tile of the tensor-core engines, which run K (up to 708)
+// serially on a few SMs (30-90 us a product).  Here a CTA owns a 32 x 32 tile and its eight warps share every
+// 64-k slab (eight k each, 4 x 8 outputs per lane, the partial tiles summed in warp order at the end).  The
+// next slab is in registers while this one is multiplied.  A training step keeps the tensor-core products
+// at every row count: Adam's first steps divide by |g|, which carries the rounding of gradients near its
+// epsilon into the weights.
 constexpr int ST = 32, SK = 64, STP = ST + 4;
 
-template <bool TA, bool TB, int EPI>
+template <bool TB, int EPI>
 __global__ void __launch_bounds__(256) k_gemm_small(int M, int N, int K, const float* __restrict__ A, int lda,
-                                                    const float* __restrict__ B, int ldb, StoreEpi<EPI> st,
-                                                    float* __restrict__ colsum) {
+                                                    const float* __restrict__ B, int ldb, StoreEpi<EPI> st) {
   // the slabs, then (after the last one) the warps' partial tiles in the same place
   __shared__ __align__(16) float raw[8 * ST * (ST + 1)];
   static_assert(2 * SK * STP <= 8 * ST * (ST + 1), "slabs fit the partial tiles' place");
@@ -122,14 +121,11 @@ __global__ void __launch_bounds__(256) k_gemm_small(int M, int N, int K, const f
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m0 = blockIdx.y * ST, n0 = blockIdx.x * ST;
   const int lm = (lane >> 2) * 4, ln = (lane & 3) * 8;
-  const bool sums = colsum != nullptr && blockIdx.y == 0;
-  float acc[4][8], cs[8];
+  float acc[4][8];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    cs[j] = 0.f;
+  for (int j = 0; j < 8; ++j)
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[i][j] = 0.f;
-  }
   // element (row, k) of an operand slab for this thread's x-th load: along k where k is contiguous
   float ra[8], rb[8];
   auto load = [&](int k0) {
@@ -137,9 +133,9 @@ __global__ void __launch_bounds__(256) k_gemm_small(int M, int N, int K, const f
     for (int x = 0; x < 8; ++x) {
       const int t = tid + x * 256;
       {
-        const int r = TA ? t % ST : t / SK, k = TA ? t / ST : t % SK;
+        const int r = t / SK, k = t % SK;
         const bool in = m0 + r < M && k0 + k < K;
-        ra[x] = in ? (TA ? A[(size_t)(k0 + k) * lda + m0 + r] : A[(size_t)(m0 + r) * lda + k0 + k]) : 0.f;
+        ra[x] = in ? A[(size_t)(m0 + r) * lda + k0 + k] : 0.f;
       }
       {
         const int r = TB ? t / SK : t % ST, k = TB ? t % SK : t / ST;
@@ -154,7 +150,7 @@ __global__ void __launch_bounds__(256) k_gemm_small(int M, int N, int K, const f
 #pragma unroll
     for (int x = 0; x < 8; ++x) {
       const int t = tid + x * 256;
-      as[TA ? t / ST : t % SK][TA ? t % ST : t / SK] = ra[x];
+      as[t % SK][t / SK] = ra[x];
       bs[TB ? t % SK : t / ST][TB ? t / SK : t % ST] = rb[x];
     }
     __syncthreads();
@@ -169,10 +165,6 @@ __global__ void __launch_bounds__(256) k_gemm_small(int M, int N, int K, const f
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-      if (sums) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) cs[j] += bv[j];
-      }
     }
   }
   __syncthreads();
@@ -189,38 +181,26 @@ __global__ void __launch_bounds__(256) k_gemm_small(int M, int N, int K, const f
     for (int w = 0; w < 8; ++w) v += part[w][r][c];
     if (m0 + r < M && n0 + c < N) st(m0 + r, n0 + c, v);
   }
-  if (sums) {
-    __syncthreads();
-    if (lm == 0) {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) part[0][warp][ln + j] = cs[j];
-    }
-    __syncthreads();
-    if (tid < ST && n0 + tid < N) {
-      float v = 0.f;
-#pragma unroll
-      for (int w = 0; w < 8; ++w) v += part[0][w][tid];
-      colsum[n0 + tid] = v;
-    }
-  }
 }
 
-// Rows (of a batch) up to which the FMA tiles are the faster form: forward products of 708 x 256 at
-// 1,024 rows 20 us, on the tensor cores 23 us; the weight gradients' sums (K = rows) up to 8,192.
-constexpr int kSmallRows = 1024, kSmallSum = 8192;
+// Rows (of a batch) up to which the FMA tiles are inference's faster form: forward products of 708 x 256 at
+// 1,024 rows 20 us, on the tensor cores 23 us.
+constexpr int kSmallRows = 1024;
 
-// C = op(A) op(B) with the epilogue; colsum (nullable): B's column sums.  `pack`: scratch for the split
-// weights of the row-streaming engine (op(B) is a weight matrix there), nullable where the call never
-// takes it (op(A) transposed).
+// C = op(A) op(B) with the epilogue; colsum (nullable): B's column sums.  `tiles`: small batches may take the
+// FMA tiles.  `pack`: scratch for the split weights of the row-streaming engine (op(B) is a weight matrix
+// there), null up to kSmallRows rows and where op(A) is transposed: those take the functor engine.
 template <bool TA, bool TB, int EPI>
 cudaError_t gemm(int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C, int ldc,
-                 const float* bias, const float* aux, float* colsum, float* pack, int* err, cudaStream_t st) {
+                 const float* bias, const float* aux, float* colsum, float* pack, int* err, cudaStream_t st, bool tiles = false) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   const StoreEpi<EPI> sv{C, ldc, bias, aux};
-  if (TA ? K <= kSmallSum : M <= kSmallRows) {
-    const dim3 g((unsigned)((N + ST - 1) / ST), (unsigned)((M + ST - 1) / ST));
-    k_gemm_small<TA, TB, EPI><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, sv, colsum);
-    return cudaGetLastError();
+  if constexpr (!TA) {
+    if (tiles && M <= kSmallRows) {
+      const dim3 g((unsigned)((N + ST - 1) / ST), (unsigned)((M + ST - 1) / ST));
+      k_gemm_small<TB, EPI><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, sv);
+      return cudaGetLastError();
+    }
   }
   if (colsum) {
     k_colsum<<<grid1(N, 128), 128, 0, st>>>(B, K, N, ldb, colsum);
@@ -229,7 +209,7 @@ cudaError_t gemm(int M, int N, int K, const float* A, int lda, const float* B, i
   }
   const LoadOp<!TB> lb{B, ldb};
   if constexpr (!TA) {
-    if (tc::rows_streamable(A, lda)) return tc::gemm_rows(M, N, K, A, lda, lb, sv, pack, err, st);
+    if (pack && tc::rows_streamable(A, lda)) return tc::gemm_rows(M, N, K, A, lda, lb, sv, pack, err, st);
   }
   // the engine forms sum_k a(m, k) b(n, k): op(B)^T element (n, k) is B[k][n], or B[n][k] when TB.
   // Tile width: the widest that N fills while the tiles still cover every SM (op(A) streamed
@@ -596,7 +576,7 @@ struct MlpWork {
     dY = take(y);
     part = take(LGRID + 4);
     pack = take(pk ? pk + 4 : 0);  // read by TMA: on 16 bytes whatever the workspace's own alignment
-    pack = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(pack) + 15) & ~(uintptr_t)15);
+    pack = pk ? reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(pack) + 15) & ~(uintptr_t)15) : nullptr;
     err = reinterpret_cast<int*>(take(64));
     bytes = off;
   }
@@ -614,11 +594,11 @@ cudaError_t mlp_forward(int I, int H, int O, const float* params, const float* x
   const bool flag = R > kSmallRows;  // the FMA tiles wait on nothing
   cudaError_t e = flag ? cudaMemsetAsync(w.err, 0, sizeof(int), st) : cudaSuccess;
   if (e == cudaSuccess)
-    e = gemm<false, false, kBiasTanh>(R, H, I, x, I, net.W1, H, w.H1, P, net.b1, nullptr, nullptr, w.pack, w.err, st);
+    e = gemm<false, false, kBiasTanh>(R, H, I, x, I, net.W1, H, w.H1, P, net.b1, nullptr, nullptr, w.pack, w.err, st, true);
   if (e == cudaSuccess)
-    e = gemm<false, false, kBiasTanh>(R, H, H, w.H1, P, net.W2, H, w.H2, P, net.b2, nullptr, nullptr, w.pack, w.err, st);
+    e = gemm<false, false, kBiasTanh>(R, H, H, w.H1, P, net.W2, H, w.H2, P, net.b2, nullptr, nullptr, w.pack, w.err, st, true);
   if (e == cudaSuccess)
-    e = gemm<false, false, kBias>(R, O, H, w.H2, P, net.W3, O, y, O, net.b3, nullptr, nullptr, w.pack, w.err, st);
+    e = gemm<false, false, kBias>(R, O, H, w.H2, P, net.W3, O, y, O, net.b3, nullptr, nullptr, w.pack, w.err, st, true);
   if (e == cudaSuccess && R > 0 && flag) {
     k_mlp_check<<<1, 32, 0, st>>>(w.err, y);
     e = cudaGetLastError();
@@ -637,8 +617,7 @@ cudaError_t mlp_loss_grad(int I, int H, int O, const float* params, const float*
   float* gb2 = gW2 + (size_t)H * H;
   float* gW3 = gb2 + H;
   float* gb3 = gW3 + (size_t)H * O;
-  const bool flag = R > kSmallRows;
-  cudaError_t e = flag ? cudaMemsetAsync(w.err, 0, sizeof(int), st) : cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(w.err, 0, sizeof(int), st);
   if (e == cudaSuccess)
     e = gemm<false, false, kBiasTanh>(R, H, I, x, I, net.W1, H, w.H1, P, net.b1, nullptr, nullptr, w.pack, w.err, st);
   if (e == cudaSuccess)
@@ -660,7 +639,7 @@ cudaError_t mlp_loss_grad(int I, int H, int O, const float* params, const float*
   // layer 1: gW1 = X^T dZ1, gb1 = colsum dZ1
   if (e == cudaSuccess)
     e = gemm<true, false, kStore>(I, H, R, x, I, w.H2, P, gW1, H, nullptr, nullptr, gb1, nullptr, w.err, st);
-  if (e == cudaSuccess && flag) {
+  if (e == cudaSuccess) {
     k_mlp_check<<<1, 32, 0, st>>>(w.err, loss);  // a failed product shows as a NaN loss
     e = cudaGetLastError();
   }
