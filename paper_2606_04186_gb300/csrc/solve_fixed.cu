@@ -1092,9 +1092,8 @@ __global__ void __launch_bounds__(FD<K>::NT, DUCC && K == 3 ? 4 : FD<K>::MINB) s
     bool fin = isfinite(e0);
     if constexpr (DUCC) fin = ducc_block(sm, a, e0, sx) && fin;
     else fin = gather_block(sm, a, sx) && fin;
-    if (!fin) sm.flag[1] = 1;
-    __syncthreads();
-    if (sm.flag[1]) {
+    // the barrier's own vote: the symmetry test below sets flag[1] while the other warp may still be here
+    if (__syncthreads_or(!fin)) {
       if (tid == 0) a.status[oidx] = kSpaceDefer;
       __syncthreads();
       continue;
