@@ -5,6 +5,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 namespace qf {
@@ -53,6 +54,32 @@ __device__ __forceinline__ double fix_value(long long t, int e) {
 }
 // 2^e as a double, |e| < 1022
 __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+
+// binary64 <-> binary32 by field arithmetic (a conversion holds the FP64 pipe, 64 cycles a warp): the
+// float is cut off after its 23 bits.  Only for |x| in the normal FP32 range (2^-126 .. 2^127): outside it the
+// exponent field wraps, so callers bound their arguments first.
+__device__ __forceinline__ float cut_float(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  return __uint_as_float((hi & 0x80000000u) | (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29));
+}
+__device__ __forceinline__ double wide(float x) {
+  const unsigned u = __float_as_uint(x);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+// 1 / x: FP32 reciprocal y of the cut x, off by d <= 2^-23 + 2^-24, and one Newton step (y += y (1 - x y)),
+// which leaves d^2 < 2^-44; 2^-125 <= |x| <= 2^125.
+__device__ __forceinline__ double recip(double x) {
+  const double y = wide(__frcp_rn(cut_float(x)));
+  return fma(fma(-x, y, 1.0), y, y);
+}
+// 1 / sqrt(x): FP32 estimate y (off by less than 2^-21) and the binomial series of (1 - e)^(-1/2), e = 1 - x y^2,
+// y (1 + e / 2 + 3 e^2 / 8), whose next term 5 e^3 / 16 is below 2^-61: rounding is what is left, below
+// 2^-52; 2^-125 <= x <= 2^125.
+__device__ __forceinline__ double rsqrt_nr(double x) {
+  const double y = wide(rsqrtf(cut_float(x)));
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
 
 }  // namespace
 }  // namespace qf

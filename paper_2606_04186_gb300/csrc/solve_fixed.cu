@@ -32,8 +32,8 @@
 // warps' sums double), 0.084 ms at 10.
 //
 // Spaces outside what this kernel is exact for leave with status kSpaceDefer and are solved by
-// solve.cu's kernel: non-finite integrals, W without pair symmetry, a projected root that is not
-// clearly the one solve.cu's shifted inverse iteration picks.
+// solve.cu's kernel: non-finite integrals or ones of 2^30 and more, W without pair symmetry, a projected
+// root that is not clearly the one solve.cu's shifted inverse iteration picks.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -184,29 +184,6 @@ __device__ __forceinline__ const FTab<K>& ftab() {
 }
 
 constexpr int kFix = 54;  // a number is t 2^-54 of its scale
-
-// binary64 <-> binary32 by field arithmetic (a conversion holds the FP64 pipe, 64 cycles a warp): the
-// float is cut off after its 23 bits; for |x| in the normal FP32 range
-__device__ __forceinline__ float cut_float(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  return __uint_as_float((hi & 0x80000000u) | (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29));
-}
-__device__ __forceinline__ double wide(float x) {
-  const unsigned u = __float_as_uint(x);
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
-}
-// 1 / x to about 2^-44: FP32 reciprocal and one Newton step (|x| well inside the FP32 range)
-__device__ __forceinline__ double recip(double x) {
-  const double y = wide(__frcp_rn(cut_float(x)));
-  return fma(fma(-x, y, 1.0), y, y);
-}
-// 1 / sqrt(x) to FP64 rounding: FP32 estimate y and one third-order step, with e = 1 - x y^2
-// y (1 + e / 2 + 3 e^2 / 8) (x within the FP32 range)
-__device__ __forceinline__ double rsqrt_nr(double x) {
-  const double y = wide(rsqrtf(cut_float(x)));
-  const double e = fma(-x * y, y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
 
 // DUCC form: integrals and amplitudes of the space while its internal part is formed.
 template <int K>
@@ -548,6 +525,11 @@ __device__ __forceinline__ int scale_of(unsigned mx) {
   return e > 0 ? e - 1022 : 0;
 }
 constexpr unsigned kInfHi = 0x7ff00000u;
+// Integrals of a space stay below 2^kMaxScale: its diagonal and sigma below 2^38, a correction (divided by
+// 1e-4 at least) below 2^52 and sums of its squares below 2^113, inside the FP32 range that cut_float and
+// wide work in.
+constexpr int kMaxScale = 30;
+constexpr unsigned kMaxHi = (unsigned)(1023 + kMaxScale) << 20;
 
 __device__ __forceinline__ void copy8_async(double* dst, const double* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -556,7 +538,7 @@ __device__ __forceinline__ void copy8_async(double* dst, const double* src) {
 __device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // SES-CC: W limbs (relative to the largest element that is not (pp|rr)), J, X and the F block.
-// False (in some thread): an element is not finite or the scale is out of range.  The elements come
+// False (in some thread): an element is not finite or out of range (kMaxScale).  The elements come
 // by asynchronous copies (all of them in flight) and are converted in rolled loops: the kernel's
 // code has to stay within the instruction cache.
 template <int K>
@@ -596,7 +578,7 @@ __device__ __forceinline__ bool gather_block(FSmem<K, false>& sm, const SolveArg
     const bool dd = (pq % (NORB + 1)) == 0 && (rs % (NORB + 1)) == 0;
     sm.W[x] = dd ? make_int2(0, 0) : limbs(to_fix(raw[x], sx, kFix));
   }
-  return all < kInfHi && sx > -900 && sx < 900;
+  return all < kMaxHi && sx > -900;
 }
 
 // Sum of products of limbs.
@@ -913,7 +895,7 @@ __device__ __noinline__ bool ducc_block(FSmem<K, true>& sm, const SolveArgs& a, 
   // uniform: both maxima are the block's.  An amplitude of 1 or more leaves the range in which the
   // sums below cannot overflow (up to 100 products of 2^54, with t below 1)
   const int S = scale_of(mx), st = scale_of(mt);
-  if (mx >= kInfHi || mt >= kInfHi || S < -400 || S > 400 || st > 0 || st < -400) return false;
+  if (mx >= kMaxHi || mt >= kInfHi || S < -400 || st > 0 || st < -400) return false;
   __syncthreads();
 #pragma unroll 1
   for (int x = tid; x < K4; x += NT) {

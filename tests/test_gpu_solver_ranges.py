@@ -1,0 +1,50 @@
+"""The FP64 solver's FP32-seeded helpers and what keeps their arguments in range: a space whose integrals are
+2^30 and more goes to the general kernel, so both forms of the call give the same bits there, and large scales
+below that limit agree to rounding.
+
+Tolerances: recip and rsqrt_nr as derived beside them in csrc/fixed.cuh (2^-44 and 2^-52; the references
+are themselves within 2^-52); scaled solves as in test_gpu_fixed_solver.py, times the scale.
+"""
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2606_04186_gb300 import build, synth
+
+from gpu_util import dev
+from test_gpu_fixed_solver import _solve, _system
+
+pytestmark = pytest.mark.gpu
+
+
+def test_seeded_reciprocal_and_root(tmp_path):
+    exe = str(tmp_path / "seed_check")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "native", "seed_check.cu")
+    subprocess.run([build.nvcc(), *build.ARCH, "-O2", "-std=c++17", "-I", build.CSRC, src, "-o", exe], check=True)
+    out = subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split()
+    assert float(out[0]) < 2.0 ** -44 + 2.0 ** -52 and float(out[1]) < 2.0 ** -52 + 2.0 ** -52
+
+
+@pytest.mark.parametrize("k", [1, 2, 3])
+@pytest.mark.parametrize("bits", [20, 36, 140, 700])
+def test_solver_at_large_scales(k, bits):
+    """Integrals times 2^bits with the tolerance scaled along."""
+    n, no = 13, 4
+    qf, h, g, t1, t2, e0, F, W = _system(n, no, 5.0, 5, 0.02)
+    sp = synth.sampled_spaces(n, no, 36, 4, no=k, nv=k)
+    perm, o1, o2, _ = qf.plan(h, g, no, sp)
+    sp, own = dev(sp[perm]), (dev(o1), dev(o2))
+    s = 2.0 ** bits
+    kw = {"tol": 1e-9 * s}
+    a = _solve(qf, n, no, e0 * s, F * s, W * s, k, sp, t1, t2, own, False, **kw)
+    b = _solve(qf, n, no, e0 * s, F * s, W * s, k, sp, t1, t2, own, True, **kw)
+    assert np.array_equal(a[1], b[1]) and np.array_equal(a[2], b[2])
+    if bits > 32:  # the largest integrals (about 0.2) are above 2^30: the general kernel both times
+        for x, y in zip((a[0], a[3], a[4]), (b[0], b[3], b[4])):
+            assert np.array_equal(x, y, equal_nan=True)
+    else:
+        assert (a[1] == 0).all()
+        for x, y, u in ((a[0], b[0], s), (a[3], b[3], 1.0), (a[4], b[4], 1.0)):
+            assert np.abs(x - y).max() < 1e-12 * u
