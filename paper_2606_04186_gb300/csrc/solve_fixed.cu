@@ -32,8 +32,9 @@
 // warps' sums double), 0.084 ms at 10.
 //
 // Spaces outside what this kernel is exact for leave with status kSpaceDefer and are solved by
-// solve.cu's kernel: non-finite integrals or ones of 2^30 and more, W without pair symmetry, a projected
-// root that is not clearly the one solve.cu's shifted inverse iteration picks.
+// solve.cu's kernel: non-finite integrals or ones of 2^30 and more, couplings so large that their rounding
+// here comes near the tolerance, W without pair symmetry to rounding, a projected root that is not
+// clearly the one solve.cu's shifted inverse iteration picks.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -1080,20 +1081,27 @@ __global__ void __launch_bounds__(FD<K>::NT, DUCC && K == 3 ? 4 : FD<K>::MINB) s
       __syncthreads();
       continue;
     }
-    // pair symmetry within 2^-44 of the largest coupling; folded one-body couplings
+    // sigma's rounding (at most a few hundred terms of 2^-55 of the largest coupling, below 2^(sx - 50) in the
+    // norms met) has to stay far below the residual asked for: where integrals of graded orbitals span so
+    // many decades that it does not, the general kernel's relative rounding decides
+    if (tid == 0 && pow2(sx - 46) > a.tol) sm.flag[1] = 1;
+    // pair symmetry to rounding: 64 units of 2^-54 of the largest coupling (dressed blocks: at most 2.5 at 24 to
+    // 82 orbitals, 9 with amplitudes of 0.2); folded one-body couplings
+    const double near = pow2(sx - 48);
 #pragma unroll 1
     for (int x = tid; x < C::NW; x += NT) {
       const int pq = x / NF, rs = x % NF;
       if (pq < rs) {
         const long long df = unlimb(sm.W[x]) - unlimb(sm.W[rs * NF + pq]);
-        if (df > 1024 || df < -1024) sm.flag[1] = 1;
+        if (df > 64 || df < -64) sm.flag[1] = 1;
       }
     }
 #pragma unroll 1
     for (int x = tid; x < NF; x += NT) {
       const int p = x / NORB, q = x % NORB;
       if (p != q) {
-        if (!(fabs(sm.J[x] - sm.J[q * NORB + p]) <= 1e-13 * (fabs(sm.J[x]) + fabs(sm.J[q * NORB + p])) + 1e-300)) sm.flag[1] = 1;
+        const double ja = sm.J[x], jb = sm.J[q * NORB + p];
+        if (!(fabs(ja - jb) <= fmax(near, 0x1p-48 * fabs(ja)))) sm.flag[1] = 1;
         long long v = to_fix(sm.F[x], sx, kFix);
 #pragma unroll
         for (int k = 0; k < K; ++k)

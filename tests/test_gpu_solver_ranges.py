@@ -1,6 +1,7 @@
 """The FP64 solver's FP32-seeded helpers and what keeps their arguments in range: a space whose integrals are
 2^30 and more goes to the general kernel, so both forms of the call give the same bits there, and large scales
-below that limit agree to rounding.
+below that limit agree to rounding.  So do spaces whose couplings' rounding comes near the tolerance and spaces with
+pair asymmetry above rounding (64 units of 2^-54 of the largest coupling).
 
 Tolerances: recip and rsqrt_nr as derived beside them in csrc/fixed.cuh (2^-44 and 2^-52; the references
 are themselves within 2^-52); scaled solves as in test_gpu_fixed_solver.py, times the scale.
@@ -48,3 +49,44 @@ def test_solver_at_large_scales(k, bits):
         assert (a[1] == 0).all()
         for x, y, u in ((a[0], b[0], s), (a[3], b[3], 1.0), (a[4], b[4], 1.0)):
             assert np.abs(x - y).max() < 1e-12 * u
+
+
+def _system13(seed, k):
+    n, no = 13, 4
+    qf, h, g, t1, t2, e0, F, W = _system(n, no, 5.0, seed, 0.02)
+    sp = synth.sampled_spaces(n, no, 36, 4, no=k, nv=k)
+    perm, o1, o2, _ = qf.plan(h, g, no, sp)
+    return qf, n, no, t1, t2, e0, F, W, sp[perm], (dev(o1), dev(o2))
+
+
+@pytest.mark.parametrize("k", [1, 2, 3])
+def test_pair_asymmetry_above_rounding(k):
+    """4e-15 on one element of each pair: 140 to 1,200 units of 2^-54 of couplings between 0.06 and 0.5."""
+    import torch
+    qf, n, no, t1, t2, e0, F, W, sp, own = _system13(5, k)
+    pq = torch.arange(n * n, device="cuda").reshape(n, n)
+    upper = pq[:, :, None, None] < pq[None, None, :, :]
+    w = W + 4e-15 * upper.to(torch.float64)
+    a = _solve(qf, n, no, e0, F, w, k, dev(sp), t1, t2, own, False)
+    b = _solve(qf, n, no, e0, F, w, k, dev(sp), t1, t2, own, True)
+    assert (a[1] == 0).all()
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("k", [2, 3])
+def test_couplings_that_span_many_decades(k):
+    """A diagonal similarity transform of the operator (creators times d, annihilators by 1 / d, d = 2^-20 on
+    two virtuals): couplings out of the scaled orbitals reach 2^40, those into them 2^-40."""
+    import torch
+    qf, n, no, t1, t2, e0, F, W, sp, own = _system13(6, k)
+    d = torch.ones(n, dtype=torch.float64, device="cuda")
+    d[no] = d[no + 3] = 2.0 ** -20
+    f = F * d[:, None] / d[None, :]
+    w = W * torch.einsum("p,q,r,s->pqrs", d, 1 / d, d, 1 / d)
+    a = _solve(qf, n, no, e0, f, w, k, dev(sp), t1, t2, own, False)
+    b = _solve(qf, n, no, e0, f, w, k, dev(sp), t1, t2, own, True)
+    for x, y in zip(a, b):
+        assert np.abs(x - y).max() < 1e-12
+    assert np.array_equal(a[1], b[1]) and np.array_equal(a[2], b[2])
+    assert (b[1] == 0).mean() > 0.3
