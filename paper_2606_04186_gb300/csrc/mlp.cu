@@ -19,6 +19,9 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <utility>
+
 #include "qflow_internal.h"
 #include "rows_gemm.cuh"
 #include "tc_gemm.cuh"
@@ -187,6 +190,12 @@ __global__ void __launch_bounds__(256) k_gemm_small(int M, int N, int K, const f
 // 1,024 rows 20 us, on the tensor cores 23 us.
 constexpr int kSmallRows = 1024;
 
+// Split weights are held in the workspace up to 128 MiB (4,096 x 4,096, the widest hidden layer); a larger
+// product stays on the functor engine, which needs no scratch and gives the same bits, so that the
+// workspace of a network with 65,536 inputs or outputs stays near its activations.
+constexpr size_t kPackFloats = (size_t)32 << 20;
+bool streams_weights(int N, int K) { return tc::rows_pack_floats(N, K) <= kPackFloats; }
+
 // C = op(A) op(B) with the epilogue; colsum (nullable): B's column sums.  `tiles`: small batches may take the
 // FMA tiles.  `pack`: scratch for the split weights of the row-streaming engine (op(B) is a weight matrix
 // there; a gradient of 128 rows 366 -> 215 us, 1,000 rows 713 -> 559 us, same bits), null where op(A) is transposed.
@@ -209,7 +218,7 @@ cudaError_t gemm(int M, int N, int K, const float* A, int lda, const float* B, i
   }
   const LoadOp<!TB> lb{B, ldb};
   if constexpr (!TA) {
-    if (pack && tc::rows_streamable(A, lda)) return tc::gemm_rows(M, N, K, A, lda, lb, sv, pack, err, st);
+    if (pack && streams_weights(N, K) && tc::rows_streamable(A, lda)) return tc::gemm_rows(M, N, K, A, lda, lb, sv, pack, err, st);
   }
   // the engine forms sum_k a(m, k) b(n, k): op(B)^T element (n, k) is B[k][n], or B[n][k] when TB.
   // Tile width: the widest that N fills while the tiles still cover every SM (op(A) streamed
@@ -561,8 +570,9 @@ struct MlpWork {
   size_t bytes;
   MlpWork(void* work, int I, int H, int O, int64_t rows) {
     const size_t h = (size_t)rows * hidden_pitch(H), y = (size_t)rows * O;
-    const int wide = H > O ? H : O;
-    const size_t pk = tc::rows_pack_floats(wide, I > wide ? I : wide);
+    size_t pk = 0;  // the largest of the products that stream rows: (columns, terms) of each layer
+    for (const auto& p : {std::pair<int, int>{H, I}, {H, H}, {O, H}, {H, O}})
+      if (streams_weights(p.first, p.second)) pk = std::max(pk, tc::rows_pack_floats(p.first, p.second));
     size_t off = 0;
     auto take = [&](size_t floats) {
       float* p = work ? reinterpret_cast<float*>(static_cast<char*>(work) + off) : nullptr;
