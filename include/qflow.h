@@ -298,11 +298,17 @@ const char* qflow_strerror(int code);
  * calls are asynchronous; errors of the launch are returned, errors of the kernels surface at
  * the next synchronisation.                                                                 */
 
-/* Scratch bytes qflow_dress_device needs for n orbitals. */
+/* Scratch bytes with which qflow_dress_device is fastest for n orbitals.  From nocc^2 nvir^4 = 6e7
+ * on (three occupied orbitals and more) most of them are operands packed for the tensor cores: 184 MiB
+ * at 57 orbitals, 750 MiB at 82, up to 4.2 GiB at 128. */
 size_t qflow_dress_workspace(int32_t n, int32_t nocc);
 
 /* Step (a): e0[1], F[n*n], W[n^4] of H-bar_<=2 for the pool (t1, t2); FP64.
- * work: qflow_dress_workspace(n, nocc) bytes of device scratch. */
+ * work: qflow_dress_workspace(n, nocc) bytes of device scratch.  Less is accepted down to the
+ * arrays alone, n^2 + nocc^2 + nvir^2 + nocc^4 + nocc nvir + 6 nocc^2 nvir^2 + 256 doubles with each of
+ * the twelve arrays rounded up to 256 bytes (24 MiB at 82 orbitals): the products then run without
+ * packed operands, and one after another where there is no room for their scale exponents (equal
+ * up to FP64 rounding, slower: twice as long at 82 orbitals). */
 int qflow_dress_device(const double* h, const double* eri, const double* t1, const double* t2, int32_t n,
                        int32_t nocc, double* e0, double* F, double* W, void* work, size_t work_bytes,
                        void* stream);

@@ -684,7 +684,7 @@ struct Work {
   // FP64: A..D products of t2_terms_fixed, t2f = u, r2 its sum Z; mixed: A..D and t2f hold floats,
   // r2 = u until the residual is formed there
   double *ht, *foo, *fvv, *wo, *r1, *r2, *A, *B, *Cq, *D, *t2f;
-  int* scales;    // FP64 path: scale exponents of the products' operand rows
+  int* scales;    // FP64 path: scale exponents of the products' operand rows (null: kArrays)
   void* slices;   // FP64 path, where its products run on the tensor cores: packed operands (else null)
   double* epart;  // energy partials
   float* acc;     // mixed path: FP32 GEMM results (v^3 o floats)
@@ -705,9 +705,14 @@ bool vvvo_shares_launch(int o, int v);
 bool fix_on_tensor_cores(int o, int v) { return o >= 3 && v > 0 && (double)o * o * v * v * v * v >= kTensorTerms; }
 size_t fix_scale_ints(int o, int v);
 size_t fix_slice_bytes(int n, int o);
+constexpr int kFixProducts = 20;  // products of t2_terms_fixed
 
-// slices: whether the region of packed FP64 operands is part of the workspace
-size_t carve(void* base, int n, int o, Work* w, bool mixed = false, bool slices = false) {
+// What of a workspace the FP64 form has: its arrays alone (products one at a time, their scale exponents in
+// an array that is free then), room for the scale exponents of a launch's products too, or also the packed
+// operands of the tensor-core products.
+enum Room { kArrays, kScales, kSlices };
+
+size_t carve(void* base, int n, int o, Work* w, bool mixed = false, Room room = kScales) {
   const int v = n - o;
   const size_t sizes[] = {(size_t)n * n, (size_t)o * o, (size_t)v * v, (size_t)o * o * o * o, (size_t)v * o,
                           (size_t)o * o * v * v, (size_t)o * v * o * v, (size_t)o * v * o * v, (size_t)o * v * o * v,
@@ -720,12 +725,12 @@ size_t carve(void* base, int n, int o, Work* w, bool mixed = false, bool slices 
     off += ((sizes[k] * sizeof(double) + 255) / 256) * 256;
   }
   w->scales = nullptr;
-  if (!mixed) {
+  if (!mixed && room >= kScales) {
     if (base) w->scales = reinterpret_cast<int*>(static_cast<char*>(base) + off);
     off += dress_scale_bytes(n, o);
   }
   w->slices = nullptr;
-  if (slices) {
+  if (!mixed && room == kSlices) {
     if (base) w->slices = static_cast<char*>(base) + off;
     off += fix_slice_bytes(n, o);
   }
@@ -762,7 +767,7 @@ cudaError_t launch_to_f32(const double* W, float* W32, size_t count, cudaStream_
 
 size_t dress_workspace_bytes(int n, int nocc) {
   Work w;
-  return carve(nullptr, n, nocc, &w, false, fix_on_tensor_cores(nocc, n - nocc));
+  return carve(nullptr, n, nocc, &w, false, fix_on_tensor_cores(nocc, n - nocc) ? kSlices : kScales);
 }
 
 size_t dress_scale_bytes(int n, int nocc) {
@@ -771,23 +776,41 @@ size_t dress_scale_bytes(int n, int nocc) {
 
 size_t dress_workspace_bytes_min(int n, int nocc) {
   Work w;
-  return carve(nullptr, n, nocc, &w);
+  return carve(nullptr, n, nocc, &w, false, kArrays);
 }
+
+namespace {
+// The most that a FP64 dressing can use of a workspace: the products that pack nothing also take one that TMA
+// cannot read (off 16 bytes).
+Room room_of(int n, int nocc, const void* work, size_t bytes) {
+  Work w;
+  if (fix_on_tensor_cores(nocc, n - nocc) && (reinterpret_cast<uintptr_t>(work) & 15u) == 0 &&
+      bytes >= carve(nullptr, n, nocc, &w, false, kSlices))
+    return kSlices;
+  return bytes >= carve(nullptr, n, nocc, &w, false, kScales) ? kScales : kArrays;
+}
+}  // namespace
 
 size_t dress_workspace_bytes_mixed(int n, int nocc) {
   Work w;
   return carve(nullptr, n, nocc, &w, true);
 }
 
-int dress_launch_count(int n, int nocc, bool mixed) {
+int dress_launch_count(int n, int nocc, bool mixed, size_t work_bytes) {
   // 4 T1 passes (the first one copies; for nocc > kT1Omax a separate copy + 4), h~, f~, 2 energy,
   // u, small blocks, finalize; T2 terms: 2 row scales + 3 product launches (FP64; + 3 operand packs where
-  // those run on the tensor cores) or 2 FP32 copies + 3 operand
+  // those run on the tensor cores; scales and launch per product where the workspace holds the arrays alone)
+  // or 2 FP32 copies + 3 operand
   // packs + 3 GEMM launches (4 where vvvo has its own) + the vvvv pack and two product kernels + FP32
   // Fock copies + 4 finalize kernels + error check (mixed)
   if (!(n - nocc > 0 && nocc > 0)) return 5;
   const int front = (nocc <= kT1Omax ? 4 : 5) + 7;
-  return front + (mixed ? 17 + (vvvo_shares_launch(nocc, n - nocc) ? 0 : 1) : fix_on_tensor_cores(nocc, n - nocc) ? 8 : 5);
+  if (mixed) return front + 17 + (vvvo_shares_launch(nocc, n - nocc) ? 0 : 1);
+  switch (room_of(n, nocc, nullptr, work_bytes)) {
+    case kSlices: return front + 8;
+    case kScales: return front + 5;
+    default: return front + 2 * kFixProducts;
+  }
 }
 
 namespace {
@@ -832,6 +855,7 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
     return W + (size_t)o * ((mask & 8 ? n3 : 0) + (mask & 4 ? n2 : 0) + (mask & 2 ? n1 : 0) + (mask & 1));
   };
   double *E = w.A, *C = w.B, *D = w.Cq, *X = w.D, *Y = w.Cq, *Z = w.r2;
+  const bool alone = !need && !w.scales;  // one product at a time
   int* next = w.scales;
   auto operand = [&](int rows, Seg a) {
     Operand x{};
@@ -839,7 +863,7 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
     x.nseg = 1;
     x.rows = rows;
     x.e = next;
-    next += rows;
+    if (!alone) next += rows;
     return x;
   };
   auto operand2 = [&](int rows, Seg a, Seg b) {
@@ -897,7 +921,7 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
   for (const Operand* p : {&wA, &tij, &gab, &eA, &eB, &cA, &gx, &dA, &xA, &xB, &v1A, &v1B, &o1A, &x2B, &r2B, &tab, &v2B,
                            &v4B, &o2A, &o2B, &x3B, &ovA, &ooA, &v3A, &v3B, &o3A, &o3B, &yA, &y2A, &yB})
     ops.o[ops.count++] = *p;
-  cudaError_t e = need ? cudaSuccess : fg::row_scales(ops, st);
+  cudaError_t e = need || alone ? cudaSuccess : fg::row_scales(ops, st);
   if (e != cudaSuccess) return e;
 
   fg::Jobs js{};
@@ -905,6 +929,27 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
     if (need) {
       const size_t b = oz::pack_bytes(js);
       *need = b > *need ? b : *need;
+      return cudaSuccess;
+    }
+    if (alone) {
+      // the same products, each after its own operands' scales.  Those of the last two, which have o^2 v
+      // rows, go where E was: its last reader has run.
+      for (int i = 0; i < js.count; ++i) {
+        fg::Jobs one{};
+        one.j[0] = js.j[i];
+        one.count = 1;
+        Job& j = one.j[0];
+        const bool fits = j.a.rows + j.b.rows <= 2 * n2;
+        j.a.e = reinterpret_cast<int*>(fits ? w.ht : E);
+        j.b.e = j.a.e + j.a.rows;
+        fg::Ops both{};
+        both.o[0] = j.a;
+        both.o[1] = j.b;
+        both.count = 2;
+        cudaError_t err = fg::row_scales(both, st);
+        if (err == cudaSuccess) err = fg::run(one, st);
+        if (err != cudaSuccess) return err;
+      }
       return cudaSuccess;
     }
     return w.slices ? oz::run(js, w.slices, st) : fg::run(js, st);
@@ -929,7 +974,7 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
 
   ops.count = 0;
   for (const Operand* p : {&x2A, &r2A, &x3A}) ops.o[ops.count++] = *p;
-  if (!need) e = fg::row_scales(ops, st);
+  if (!need && !alone) e = fg::row_scales(ops, st);
   if (e != cudaSuccess) return e;
   js.count = 0;
   add(x2A, x2B, out(X, v, vv, v, v, ovv, 1, 1));           // (j a)(i b)
@@ -1990,12 +2035,9 @@ cudaError_t launch_dress(const double* h, const double* eri, const double* t1, c
                          float* g32, int ladder_bn) {
   Work w;
   const bool mixed = g32 != nullptr;
-  if (work_bytes < carve(nullptr, n, nocc, &w, mixed)) return cudaErrorInvalidValue;
-  // a caller with less than dress_workspace_bytes (the static scratch), or with a workspace that TMA cannot
-  // read (off 16 bytes), gets the products that pack nothing
-  const bool slices = !mixed && fix_on_tensor_cores(nocc, n - nocc) && (reinterpret_cast<uintptr_t>(work) & 15u) == 0 &&
-                      work_bytes >= carve(nullptr, n, nocc, &w, false, true);
-  carve(work, n, nocc, &w, mixed, slices);
+  if (work_bytes < (mixed ? carve(nullptr, n, nocc, &w, true) : dress_workspace_bytes_min(n, nocc)))
+    return cudaErrorInvalidValue;
+  carve(work, n, nocc, &w, mixed, mixed ? kArrays : room_of(n, nocc, work, work_bytes));
   Dims d{n, nocc, n - nocc};
   const size_t n4 = (size_t)n * n * n * n;
   const size_t o = nocc, v = n - nocc;

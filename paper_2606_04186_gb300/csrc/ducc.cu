@@ -138,7 +138,7 @@ DuccWork ducc_layout(int n, int nocc) {
 
 size_t ducc_workspace_bytes(int n, int nocc) { return ducc_layout(n, nocc).total; }
 
-int ducc_launch_count(int n, int nocc) { return 6 + 8 * (3 + dress_launch_count(n, nocc, false)); }
+int ducc_launch_count(int n, int nocc) { return 6 + 8 * (3 + dress_launch_count(n, nocc, false, dress_workspace_bytes(n, nocc))); }
 
 cudaError_t launch_dress_ducc(const double* h, const double* eri, const double* t1, const double* t2, int n, int nocc,
                               double* e0, double* F, double* W, double* F0, void* work, size_t work_bytes,

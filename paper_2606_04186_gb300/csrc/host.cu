@@ -567,7 +567,7 @@ cudaError_t dress_pool(qflow_ctx* c, const double* t1, const double* t2) {
 
 int dress_pool_launches(const qflow_ctx* c) {
   return (c->opt.form == QFLOW_FORM_DUCC) ? qf::ducc_launch_count(c->n, c->nocc)
-                                          : qf::dress_launch_count(c->n, c->nocc, c->W32 != nullptr);
+                                          : qf::dress_launch_count(c->n, c->nocc, c->W32 != nullptr, c->dwork_bytes);
 }
 
 // Step (a): dressing (+ the FP32 copy of W for the mixed solver).
@@ -1201,7 +1201,7 @@ int qflow_dress_device(const double* h, const double* eri, const double* t1, con
                        int32_t nocc, double* e0, double* F, double* W, void* work, size_t work_bytes, void* stream) {
   if (!h || !eri || !t1 || !t2 || !e0 || !F || !W || !work || n < 2 || n > 128 || nocc < 1 || nocc >= n)
     return QFLOW_ERR_ARG;
-  if (work_bytes < qf::dress_workspace_bytes(n, nocc)) return QFLOW_ERR_ARG;
+  if (work_bytes < qf::dress_workspace_bytes_min(n, nocc)) return QFLOW_ERR_ARG;
   return cuda_status(qf::launch_dress(h, eri, t1, t2, n, nocc, e0, F, W, work, work_bytes, (cudaStream_t)stream));
 }
 

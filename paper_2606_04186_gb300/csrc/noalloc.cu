@@ -81,7 +81,7 @@ extern "C" int qflow_dress_device_static(const double* h, const double* eri, con
   if (!h || !eri || !t1 || !t2 || !e0 || !F || !W || n < 2 || n > 128 || nocc < 1 || nocc >= n)
     return QFLOW_ERR_ARG;
   const size_t scales = qf::dress_scale_bytes(n, nocc);
-  if (qf::dress_workspace_bytes_min(n, nocc) - scales > (size_t)QFLOW_STATIC_SCRATCH_BYTES ||
+  if (qf::dress_workspace_bytes_min(n, nocc) > (size_t)QFLOW_STATIC_SCRATCH_BYTES ||
       scales > kStaticScratchBytes - (size_t)QFLOW_STATIC_SCRATCH_BYTES)
     return QFLOW_ERR_TOO_LARGE;
   void* scratch = nullptr;

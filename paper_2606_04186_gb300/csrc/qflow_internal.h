@@ -91,11 +91,12 @@ cudaError_t launch_to_f32(const double* W, float* W32, size_t count, cudaStream_
 
 // Dressing (step a) on caller-provided device buffers; returns a CUDA error code.
 size_t dress_workspace_bytes(int n, int nocc);
-// The least launch_dress (FP64) runs with: without the packed operands of the tensor-core products.
+// The least launch_dress (FP64) runs with: its arrays, without the products' scale exponents and the
+// packed operands of the tensor-core products.
 size_t dress_workspace_bytes_min(int n, int nocc);
-size_t dress_scale_bytes(int n, int nocc);  // the scale exponents' part of it
+size_t dress_scale_bytes(int n, int nocc);  // the scale exponents' part
 size_t dress_workspace_bytes_mixed(int n, int nocc);  // + FP32 GEMM scratch of the mixed path
-int dress_launch_count(int n, int nocc, bool mixed);  // kernels one launch_dress issues
+int dress_launch_count(int n, int nocc, bool mixed, size_t work_bytes);  // kernels one launch_dress issues
 // g32: NULL for FP64 contractions; else n^4 floats of scratch, and the T2 terms are contracted
 // in FP32 (mixed precision); the mixed form adds the T2 term of the vvvv block only where at most
 // three of its four virtual indices differ (all a (k, k) space with k <= 3 reads), the other
