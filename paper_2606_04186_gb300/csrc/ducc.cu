@@ -104,9 +104,9 @@ __global__ void k_acc_hermitian(const double* __restrict__ e0, const double* __r
   if (blockIdx.x == 0 && threadIdx.x == 0) *oe += c * 2.0 * (*e0);
 }
 
-// Workspace layout (bytes, each part 256-aligned).
+// Workspace layout (bytes, each part 256-aligned); the dressings' own workspace is what follows.
 struct DuccWork {
-  size_t dress, t1s, t2s, e, F, W, hB, gB, total;
+  size_t t1s, t2s, e, F, W, hB, gB, dress;
 };
 DuccWork ducc_layout(int n, int nocc) {
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
@@ -114,8 +114,6 @@ DuccWork ducc_layout(int n, int nocc) {
   const size_t ov = (size_t)nocc * (n - nocc), oovv = ov * ov;
   DuccWork w{};
   size_t off = 0;
-  w.dress = off;
-  off += al(dress_workspace_bytes(n, nocc));
   w.t1s = off;
   off += al(ov * sizeof(double));
   w.t2s = off;
@@ -130,21 +128,23 @@ DuccWork ducc_layout(int n, int nocc) {
   off += al(n2 * sizeof(double));
   w.gB = off;
   off += al(n4 * sizeof(double));
-  w.total = off;
+  w.dress = off;
   return w;
 }
 
 }  // namespace
 
-size_t ducc_workspace_bytes(int n, int nocc) { return ducc_layout(n, nocc).total; }
+size_t ducc_workspace_bytes(int n, int nocc, size_t dress_bytes) { return ducc_layout(n, nocc).dress + dress_bytes; }
 
-int ducc_launch_count(int n, int nocc) { return 6 + 8 * (3 + dress_launch_count(n, nocc, false, dress_workspace_bytes(n, nocc))); }
+int ducc_launch_count(int n, int nocc, size_t work_bytes) {
+  return 6 + 8 * (3 + dress_launch_count(n, nocc, false, work_bytes - ducc_layout(n, nocc).dress));
+}
 
 cudaError_t launch_dress_ducc(const double* h, const double* eri, const double* t1, const double* t2, int n, int nocc,
                               double* e0, double* F, double* W, double* F0, void* work, size_t work_bytes,
                               cudaStream_t st) {
   const DuccWork L = ducc_layout(n, nocc);
-  if (work_bytes < L.total) return cudaErrorInvalidValue;
+  if (work_bytes < L.dress + dress_workspace_bytes_min(n, nocc)) return cudaErrorInvalidValue;
   unsigned char* base = static_cast<unsigned char*>(work);
   double* t1s = reinterpret_cast<double*>(base + L.t1s);
   double* t2s = reinterpret_cast<double*>(base + L.t2s);
@@ -173,7 +173,7 @@ cudaError_t launch_dress_ducc(const double* h, const double* eri, const double* 
     for (int k = 0; k < 4 && e == cudaSuccess; ++k) {
       k_scaled<<<grid_for(ov), TPB, 0, st>>>(t1, lam[k], t1s, ov);
       k_scaled<<<grid_for(oovv), TPB, 0, st>>>(t2, lam[k], t2s, oovv);
-      e = launch_dress(oh, og, t1s, t2s, n, nocc, ek, Fk, Wk, base + L.dress, L.t1s - L.dress, st);
+      e = launch_dress(oh, og, t1s, t2s, n, nocc, ek, Fk, Wk, base + L.dress, work_bytes - L.dress, st);
       if (e == cudaSuccess) {
         k_acc_hermitian<<<grid_for(n4), TPB, 0, st>>>(ek, Fk, Wk, w * cof[k], n, e0, F, W);
         e = cudaGetLastError();

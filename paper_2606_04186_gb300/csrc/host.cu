@@ -14,6 +14,7 @@
 #include <numeric>
 #include <vector>
 
+#include "alloc_largest.h"
 #include "qflow_internal.h"
 
 using qf::SolveArgs;
@@ -414,9 +415,6 @@ int qflow_init(qflow_handle* out, const double* h, const double* eri, int32_t n,
   group_spaces(spaces, nspaces, pl, &grouped, &gidx, c->cls_count, c->cls_off);
   const size_t n1 = n, n4 = n1 * n1 * n1 * n1;
   cudaError_t e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
-  c->dwork_bytes = (c->opt.precision == QFLOW_PREC_MIXED) ? qf::dress_workspace_bytes_mixed(n, nocc)
-                   : (c->opt.form == QFLOW_FORM_DUCC)      ? qf::ducc_workspace_bytes(n, nocc)
-                                                          : qf::dress_workspace_bytes(n, nocc);
   const size_t npool = (size_t)(c->n_t1 + c->n_t2);
   if (e == cudaSuccess) e = dalloc(&c->h, n1 * n1);
   if (e == cudaSuccess) e = dalloc(&c->eri, n4);
@@ -433,7 +431,6 @@ int qflow_init(qflow_handle* out, const double* h, const double* eri, int32_t n,
   if (e == cudaSuccess) e = dalloc(&c->owns, (size_t)std::max<int64_t>(nspaces, 1));
   if (e == cudaSuccess) e = dalloc(&c->spaces, (size_t)std::max<int64_t>(nspaces, 1));
   if (e == cudaSuccess) e = dalloc(&c->sorted_index, (size_t)std::max<int64_t>(nspaces, 1));
-  if (e == cudaSuccess) e = cudaMalloc(&c->dwork, c->dwork_bytes);
   if (e == cudaSuccess) e = cudaMalloc(&c->rwork, qf::mean_maxdiff_workspace(nspaces, (int64_t)npool));
   if (e == cudaSuccess) e = dalloc(&c->red, 4);
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&c->red_host), 4 * sizeof(double));
@@ -467,6 +464,20 @@ int qflow_init(qflow_handle* out, const double* h, const double* eri, int32_t n,
       e = cudaMalloc(&c->guess[k], bytes);
       if (e == cudaSuccess) e = cudaMemsetAsync(c->guess[k], 0, bytes, c->stream);  // zero = start from Phi
     }
+  }
+  if (e == cudaSuccess) {  // last: the FP64 products' packed operands are left out where the rest fills the GPU
+    size_t sizes[3] = {qf::dress_workspace_bytes(n, nocc),
+                       qf::dress_workspace_bytes_min(n, nocc) + qf::dress_scale_bytes(n, nocc),
+                       qf::dress_workspace_bytes_min(n, nocc)};
+    if (c->opt.form == QFLOW_FORM_DUCC)
+      for (size_t& b : sizes) b = qf::ducc_workspace_bytes(n, nocc, b);
+    const bool mixed = c->opt.precision == QFLOW_PREC_MIXED;
+    if (mixed) sizes[0] = qf::dress_workspace_bytes_mixed(n, nocc);
+    e = qf::alloc_largest(sizes, mixed ? 1 : 3, cudaErrorMemoryAllocation, [&](size_t bytes) {
+      const cudaError_t r = cudaMalloc(&c->dwork, bytes);
+      if (r == cudaErrorMemoryAllocation) cudaGetLastError();  // the next size is tried
+      return r;
+    }, &c->dwork_bytes);
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->h, h, sizeof(double) * n1 * n1, cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->eri, eri, sizeof(double) * n4, cudaMemcpyHostToDevice, c->stream);
@@ -566,7 +577,7 @@ cudaError_t dress_pool(qflow_ctx* c, const double* t1, const double* t2) {
 }
 
 int dress_pool_launches(const qflow_ctx* c) {
-  return (c->opt.form == QFLOW_FORM_DUCC) ? qf::ducc_launch_count(c->n, c->nocc)
+  return (c->opt.form == QFLOW_FORM_DUCC) ? qf::ducc_launch_count(c->n, c->nocc, c->dwork_bytes)
                                           : qf::dress_launch_count(c->n, c->nocc, c->W32 != nullptr, c->dwork_bytes);
 }
 

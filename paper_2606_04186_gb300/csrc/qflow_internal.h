@@ -113,8 +113,8 @@ cudaError_t tune_ladder(int n, int nocc, const float* g32, void* work, size_t wo
 
 // Step (a) in the Hermitian (DUCC) form (ducc.cu): e0, F, W of the part G common to every space,
 // and F0 = the bare Fock matrix (the per-space part needs it).  FP64.
-size_t ducc_workspace_bytes(int n, int nocc);
-int ducc_launch_count(int n, int nocc);
+size_t ducc_workspace_bytes(int n, int nocc, size_t dress_bytes);  // with dressings in dress_bytes
+int ducc_launch_count(int n, int nocc, size_t work_bytes);
 cudaError_t launch_dress_ducc(const double* h, const double* eri, const double* t1, const double* t2, int n, int nocc,
                               double* e0, double* F, double* W, double* F0, void* work, size_t work_bytes,
                               cudaStream_t st);
