@@ -279,9 +279,9 @@ int qflow_last_sweep_info(qflow_handle hnd, double* phase_ms, int64_t* kernel_la
 int qflow_schedule(qflow_handle hnd, int32_t* persistent, int32_t* chunk, int32_t* warps_per_cta, int32_t* graph,
                    float* candidate_ms, int32_t* n_candidates);
 
-/* Tile width in use for the mixed dressing's ladder + oooo product (QFLOW_SCHED_AUTO times
- * 32, 64 and 128 columns at the second sweep, beside the solver's candidates) and the times of
- * those three candidates in milliseconds (count 0 when the width was fixed, came from the
+/* Tile width in use for the mixed dressing's launch of the ladder + oooo product and the rings
+ * (QFLOW_SCHED_AUTO times that launch at 32, 64 and 128 columns at the second sweep, beside the
+ * solver's candidates) and the times of those three candidates in milliseconds (count 0 when the width was fixed, came from the
  * per-process cache, or before the calibration).  Any output may be NULL. */
 #define QFLOW_LADDER_TUNE_MAX 3
 int qflow_dress_schedule(qflow_handle hnd, int32_t* ladder_bn, float* candidate_ms, int32_t* n_candidates);

@@ -1828,8 +1828,8 @@ cudaError_t run_jobs(tc::PackedJobs<Store>& jobs, const Arena& ar, int* err, cud
   return tc::gemm_packed<BN>(jobs, err, st);
 }
 
-// The ladder + oooo product's tile width is a run-time choice among kLadderBN (timed by
-// tune_ladder); its B operand is padded to the widest candidate so any of them can run on it.
+// The tile width of the ladder + oooo product and the rings, which share a launch, is a run-time choice among
+// kLadderBN (timed by tune_ladder); their B operands are padded to the widest candidate so any of them can run.
 constexpr int kLadderBN[3] = {32, 64, 128};
 constexpr int kLadderPad = 128;
 constexpr int kLadderDefault = 64;  // one wave of 81 tiles at o = 10 (v^2 = 5184)
@@ -1842,13 +1842,37 @@ cudaError_t run_ladder(tc::PackedJobs<StoreR2>& js, const Arena& ar, int* err, i
   }
 }
 
-// The packed operands of the ladder + oooo product: rows (i, j), cols (a, b), k = (e, f) then
-// (m, n).
-cudaError_t pack_ladder(const TcCtx& c, int o, int v, Arena& ar, Op* a1, Op* b1, cudaStream_t st) {
-  const int oo = o * o, vv = v * v;
-  const auto ja = operand(LR2G1A{c}, oo, vv + oo, kTileM, ar, a1);
-  const auto jb = operand(LR2G1B{c}, vv, vv + oo, kLadderPad, ar, b1);
-  return pack_all(ar, st, ja, jb);
+// The products of the doubles residual, one launch: the ladder + oooo map (rows (i, j), cols (a, b),
+// k = (e, f) then (m, n)) into acc and the rings' four output maps into part, all on packed operands.
+struct R2Launch {
+  tc::PackedJobs<StoreR2> js{};
+  float* part = nullptr;
+};
+cudaError_t prepare_r2(const TcCtx& c, float* acc, Arena& ar, R2Launch* l, cudaStream_t st) {
+  const int o = c.o, v = c.v, ov = o * v, vv = v * v, oo = o * o;
+  ar.reset();
+  Op a1, b1, a3, b3, a4, b4, a5, b5, a6, b6;
+  const auto p0 = operand(LR2G1A{c}, oo, vv + oo, kTileM, ar, &a1);
+  const auto p1 = operand(LR2G1B{c}, vv, vv + oo, kLadderPad, ar, &b1);
+  const auto p2 = operand(LR2G3A{c}, ov, 5 * ov, kTileM, ar, &a3);
+  const auto p3 = operand(LR2G3B{c}, ov, 5 * ov, kLadderPad, ar, &b3);
+  const auto p4 = operand(LR2G4A{c}, ov, 2 * ov, kTileM, ar, &a4);
+  const auto p5 = operand(LR2G4B{c}, ov, 2 * ov, kLadderPad, ar, &b4);
+  const auto p6 = operand(LR2G5A{c}, ov, ov, kTileM, ar, &a5);
+  const auto p7 = operand(LR2G5B{c}, ov, ov, kLadderPad, ar, &b5);
+  const auto p8 = operand(LR2G6A{c}, ov, 2 * ov, kTileM, ar, &a6);
+  const auto p9 = operand(LR2G6B{c}, ov, 2 * ov, kLadderPad, ar, &b6);
+  const cudaError_t e = pack_all(ar, st, p0, p1, p2, p3, p4, p5, p6, p7, p8, p9);
+  const size_t n_r2 = (size_t)oo * vv;
+  l->part = ar.take(4 * n_r2);
+  auto map = [&](int i) { return ar.base ? l->part + i * n_r2 : nullptr; };
+  l->js.j[0] = job(a1, b1, StoreR2{acc, o, v, 4});
+  l->js.j[1] = job(a3, b3, StoreR2{map(0), o, v, 0});
+  l->js.j[2] = job(a4, b4, StoreR2{map(1), o, v, 1});
+  l->js.j[3] = job(a5, b5, StoreR2{map(2), o, v, 2});
+  l->js.j[4] = job(a6, b6, StoreR2{map(3), o, v, 3});
+  l->js.count = 5;
+  return e;
 }
 
 constexpr int kOvoSplit = 6;  // split K of the oovo v^2 product (720 x 100 x v^2)
@@ -1909,29 +1933,11 @@ cudaError_t t2_terms_tc(const Dims& d, double* W, const float* G, const double* 
   }
   // r2: ladder + oooo term, and the rings (four output maps)
   {
-    ar.reset();
-    Op a1, b1, a3, b3, a4, b4, a5, b5, a6, b6;
-    const auto p0 = operand(LR2G1A{c}, oo, vv + oo, kTileM, ar, &a1);
-    const auto p1 = operand(LR2G1B{c}, vv, vv + oo, kLadderPad, ar, &b1);
-    const auto p2 = operand(LR2G3A{c}, ov, 5 * ov, kTileM, ar, &a3);
-    const auto p3 = operand(LR2G3B{c}, ov, 5 * ov, kLadderPad, ar, &b3);
-    const auto p4 = operand(LR2G4A{c}, ov, 2 * ov, kTileM, ar, &a4);
-    const auto p5 = operand(LR2G4B{c}, ov, 2 * ov, kLadderPad, ar, &b4);
-    const auto p6 = operand(LR2G5A{c}, ov, ov, kTileM, ar, &a5);
-    const auto p7 = operand(LR2G5B{c}, ov, ov, kLadderPad, ar, &b5);
-    const auto p8 = operand(LR2G6A{c}, ov, 2 * ov, kTileM, ar, &a6);
-    const auto p9 = operand(LR2G6B{c}, ov, 2 * ov, kLadderPad, ar, &b6);
-    QF_TRY(pack_all(ar, st, p0, p1, p2, p3, p4, p5, p6, p7, p8, p9));
     const size_t n_r2 = (size_t)oo * vv;
-    float* part = ar.take(4 * n_r2);
-    tc::PackedJobs<StoreR2> js{};
-    js.j[0] = job(a1, b1, StoreR2{acc, o, v, 4});
-    js.j[1] = job(a3, b3, StoreR2{part, o, v, 0});
-    js.j[2] = job(a4, b4, StoreR2{run ? part + n_r2 : nullptr, o, v, 1});
-    js.j[3] = job(a5, b5, StoreR2{run ? part + 2 * n_r2 : nullptr, o, v, 2});
-    js.j[4] = job(a6, b6, StoreR2{run ? part + 3 * n_r2 : nullptr, o, v, 3});
-    js.count = 5;
-    QF_TRY(run_ladder(js, ar, err, ladder_bn, st));
+    R2Launch l;
+    QF_TRY(prepare_r2(c, acc, ar, &l, st));
+    const float* part = l.part;
+    QF_TRY(run_ladder(l.js, ar, err, ladder_bn, st));
     if (run && e == cudaSuccess) {
       const float* f32 = w.f32;
       k_fock_f32<<<blocks_for((size_t)d.n * d.n + oo + vv), TPB, 0, st>>>(F, w.foo, w.fvv, w.f32, d);
@@ -2078,9 +2084,9 @@ cudaError_t launch_dress(const double* h, const double* eri, const double* t1, c
   return cudaGetLastError();
 }
 
-// Times the ladder + oooo product with each tile width of kLadderBN on the workspace of a mixed
-// dressing that has run (its packed scratch and FP32 copies are overwritten, its results are
-// not read): each candidate runs twice on the stream, the second run timed with CUDA events.
+// Times the launch of the ladder + oooo product and the rings with each tile width of kLadderBN on the
+// workspace of a mixed dressing that has run (its packed scratch and FP32 results are overwritten, and
+// not read again): each candidate runs twice on the stream, the second run timed with CUDA events.
 // *best = the fastest width; ms[3] = the candidates' times.  Not capturable (it synchronises).
 cudaError_t tune_ladder(int n, int nocc, const float* g32, void* work, size_t work_bytes, cudaStream_t st, int* best,
                         float* ms) {
@@ -2091,13 +2097,11 @@ cudaError_t tune_ladder(int n, int nocc, const float* g32, void* work, size_t wo
   Work w;
   if (work_bytes < carve(nullptr, n, nocc, &w, true)) return cudaErrorInvalidValue;
   carve(work, n, nocc, &w, true);
-  TcCtx c{g32, reinterpret_cast<const float*>(w.t2f), nullptr, nullptr, nullptr, nullptr, w.wo, n, o, v};
+  auto ring = [](const double* p) { return reinterpret_cast<const float*>(p); };
+  TcCtx c{g32, ring(w.t2f), ring(w.A), ring(w.B), ring(w.Cq), ring(w.D), w.wo, n, o, v};
   Arena ar{w.arena};
-  Op a1, b1;
-  cudaError_t e = pack_ladder(c, o, v, ar, &a1, &b1, st);
-  tc::PackedJobs<StoreR2> js{};
-  js.j[0] = job(a1, b1, StoreR2{w.acc, o, v, 4});
-  js.count = 1;
+  R2Launch l;
+  cudaError_t e = prepare_r2(c, w.acc, ar, &l, st);
   cudaEvent_t t0 = nullptr, t1 = nullptr;
   if (e == cudaSuccess) e = cudaEventCreate(&t0);
   if (e == cudaSuccess) e = cudaEventCreate(&t1);
@@ -2105,7 +2109,7 @@ cudaError_t tune_ladder(int n, int nocc, const float* g32, void* work, size_t wo
   for (int i = 0; i < 3 && e == cudaSuccess; ++i) {
     for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
       e = cudaEventRecord(t0, st);
-      if (e == cudaSuccess) e = run_ladder(js, ar, w.err, kLadderBN[i], st);
+      if (e == cudaSuccess) e = run_ladder(l.js, ar, w.err, kLadderBN[i], st);
       if (e == cudaSuccess) e = cudaEventRecord(t1, st);
       if (e == cudaSuccess) e = cudaEventSynchronize(t1);
       if (e == cudaSuccess) e = cudaEventElapsedTime(&ms[i], t0, t1);
