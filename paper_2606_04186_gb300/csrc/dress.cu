@@ -850,20 +850,23 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
                            size_t* need = nullptr) {
   const int o = d.o, v = d.v, n1 = d.n, n2 = n1 * n1, n3 = n2 * n1;
   const int oo = o * o, vv = v * v, ov = o * v, ovv = o * vv;
-  // start of a block of W: V(mask) has bit 8, 4, 2, 1 set where the first .. fourth index is virtual
+  // start of a block of W: V(mask) has bit 8, 4, 2, 1 set where the first .. fourth index is virtual (integer
+  // arithmetic: a dry run has no W)
   auto V = [&](int mask) {
-    return W + (size_t)o * ((mask & 8 ? n3 : 0) + (mask & 4 ? n2 : 0) + (mask & 2 ? n1 : 0) + (mask & 1));
+    return reinterpret_cast<double*>(
+        reinterpret_cast<uintptr_t>(W) +
+        sizeof(double) * (size_t)o * ((mask & 8 ? n3 : 0) + (mask & 4 ? n2 : 0) + (mask & 2 ? n1 : 0) + (mask & 1)));
   };
   double *E = w.A, *C = w.B, *D = w.Cq, *X = w.D, *Y = w.Cq, *Z = w.r2;
   const bool alone = !need && !w.scales;  // one product at a time
-  int* next = w.scales;
+  uintptr_t next = reinterpret_cast<uintptr_t>(w.scales);  // a dry run's only tell operands apart
   auto operand = [&](int rows, Seg a) {
     Operand x{};
     x.seg[0] = a;
     x.nseg = 1;
     x.rows = rows;
-    x.e = next;
-    if (!alone) next += rows;
+    x.e = reinterpret_cast<int*>(next);
+    if (!alone) next += rows * sizeof(int);
     return x;
   };
   auto operand2 = [&](int rows, Seg a, Seg b) {
@@ -1002,13 +1005,10 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
   return launch();
 }
 
-// Bytes of packed operands (a dry run over the same operands; addresses are never used, and the scale
-// slots only tell operands apart).
+// Bytes of packed operands (a dry run over the same operands, without addresses).
 size_t fix_slice_bytes(int n, int o) {
   const Dims d{n, o, n - o};
-  Work w{};
-  static int slots[1];
-  w.scales = slots;
+  const Work w{};
   size_t need = 0;
   t2_terms_fixed(d, nullptr, nullptr, nullptr, w, nullptr, &need);
   return (need + 255) / 256 * 256;
