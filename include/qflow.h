@@ -308,7 +308,11 @@ size_t qflow_dress_workspace(int32_t n, int32_t nocc);
  * arrays alone, n^2 + nocc^2 + nvir^2 + nocc^4 + nocc nvir + 6 nocc^2 nvir^2 + 256 doubles with each of
  * the twelve arrays rounded up to 256 bytes (24 MiB at 82 orbitals): the products then run without
  * packed operands, and one after another where there is no room for their scale exponents (equal
- * up to FP64 rounding, slower: twice as long at 82 orbitals). */
+ * up to FP64 rounding, slower: twice as long at 82 orbitals).
+ * Accuracy: the T2 products sum integers exactly, with elements cut at 2^-56 of their operand row's
+ * norm (FP64 sums cut at 2^-53 of each term): for ordinary integrals nearer to 64 bits than FP64
+ * sums, also where the orbitals are scaled; but an element of F or W that is small only because large
+ * and small factors meet term by term is accurate to the rows' norms, not to its own size. */
 int qflow_dress_device(const double* h, const double* eri, const double* t1, const double* t2, int32_t n,
                        int32_t nocc, double* e0, double* F, double* W, void* work, size_t work_bytes,
                        void* stream);

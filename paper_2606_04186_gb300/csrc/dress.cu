@@ -273,44 +273,67 @@ __global__ void __launch_bounds__(TPB, kT1Blocks - 1) k_t1_annihilator_fast(doub
 // exact to 2^-54 of the triple's largest element and the sums are exact.  The FP64 form of these
 // passes is bound by the FP64 pipe (0.4 G FMAs each at 82 orbitals: 1.15-1.2 ms against 0.11 ms of HBM
 // time); here a term is three mad.wide and an output element two FP64 operations.
+// BAL, where the integrals have a balance (scaled orbitals, see balance_orbitals): t1[i][a] is an integer relative to
+// 2^(row_i + col_a) >= |t1[i][a]| and a triple's values are relative to the largest of them times its orbital's
+// power of two, which keeps a term exact to 2^-54 of the triple's largest term.  A form of its own: the
+// powers cost the passes of 57 orbitals 80 us of the 1,660 that dressing takes.
 constexpr int kT1Bits = 54;
 
-// t1 in shared memory, transposed and padded with zeros: limbs t1s[a][0..16) in units of 2^(st - 54).
-// Returns false (every thread) when t1 has a non-finite element.
-__device__ __forceinline__ bool load_t1_fixed(const double* __restrict__ t1, int2* t1s, const Dims& d, int* st) {
-  __shared__ unsigned top;
-  if (threadIdx.x == 0) top = 0;
+struct T1Scale {
+  int col[128];      // per virtual orbital: exponent of its largest amplitude; [0] alone without BAL: of all
+  int row[kT1Omax];  // per occupied orbital, at most 0: of its largest amplitude relative to 2^col
+};
+__device__ __forceinline__ int expo(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// t1 in shared memory, transposed and padded with zeros: limbs t1s[a][0..16) in units of 2^(row + col - 54).
+// Returns false (every thread), with zero exponents, when t1 has a non-finite element.
+template <bool BAL>
+__device__ __forceinline__ bool load_t1_fixed(const double* __restrict__ t1, int2* t1s, const Dims& d, T1Scale& sc) {
+  constexpr int kNone = -4000;
+  for (int x = threadIdx.x; x < (BAL ? d.v : 1); x += blockDim.x) sc.col[x] = 0;
+  if (threadIdx.x < kT1Omax) sc.row[threadIdx.x] = kNone;
   __syncthreads();
-  unsigned mx = 0;
-  for (int x = threadIdx.x; x < d.o * d.v; x += blockDim.x) mx = max(mx, (unsigned)__double2hiint(t1[x]) & 0x7fffffffu);
-  mx = __reduce_max_sync(0xffffffffu, mx);
-  if ((threadIdx.x & 31) == 0) atomicMax(&top, mx);
+  int top = 0;
+  for (int x = threadIdx.x; x < d.o * d.v; x += blockDim.x) {
+    const int e = expo(t1[x]);
+    top = max(top, e);
+    if (BAL && e > 0) atomicMax(&sc.col[x % d.v], e);
+  }
+  if (!BAL) {
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) atomicMax(&sc.col[0], top);
+  }
+  const bool bad = __syncthreads_or(top == 0x7ff);
+  if (BAL && !bad) {
+    for (int x = threadIdx.x; x < d.o * d.v; x += blockDim.x) {
+      const int e = expo(t1[x]);
+      if (e > 0) atomicMax(&sc.row[x / d.v], e - sc.col[x % d.v]);
+    }
+    __syncthreads();
+  }
+  for (int x = threadIdx.x; x < (BAL ? d.v : 1); x += blockDim.x) sc.col[x] = bad || sc.col[x] == 0 ? 0 : sc.col[x] - 1022;
+  if (threadIdx.x < kT1Omax && (bad || sc.row[threadIdx.x] == kNone)) sc.row[threadIdx.x] = 0;
   __syncthreads();
-  mx = top;
-  const int e = (int)(mx >> 20);
-  *st = e > 0 ? e - 1022 : 0;
-  if (e == 0x7ff) return false;
+  if (bad) return false;
   for (int x = threadIdx.x; x < d.v * kT1Omax; x += blockDim.x) {
     const int a = x / kT1Omax, i = x % kT1Omax;
-    t1s[x] = (i < d.o) ? limbs(to_fix(t1[i * d.v + a], *st, kT1Bits)) : make_int2(0, 0);
+    t1s[x] = (i < d.o) ? limbs(to_fix(t1[i * d.v + a], BAL ? sc.row[i] + sc.col[a] : sc.col[0], kT1Bits)) : make_int2(0, 0);
   }
   __syncthreads();
   return true;
 }
-// 2^(sx + st - 54) within the double range (a scale below it belongs to sums below 1e-290)
-__device__ __forceinline__ double t1_unit(int sx, int st) {
-  const int e = sx + st - kT1Bits;
+// 2^(e - 54) within the double range (a scale below it belongs to sums below 1e-290)
+__device__ __forceinline__ double t1_unit(int e) {
+  e -= kT1Bits;
   return pow2(e < -1021 ? -1021 : e > 1020 ? 1020 : e);
 }
 
 // Creator pass at POS: rows nocc + a get - sum_i t1[i][a] row_i; COPY: read from src, every row written.
-template <int POS, bool COPY>
-__global__ void __launch_bounds__(TPB, 2) k_t1_creator_fixed(const double* __restrict__ src, double* __restrict__ W,
-                                                              const double* __restrict__ t1, Dims d) {
-  extern __shared__ __align__(16) double t1raw[];
-  int2* t1s = reinterpret_cast<int2*>(t1raw);
-  int st;
-  const bool fine = load_t1_fixed(t1, t1s, d, &st);
+template <int POS, bool COPY, bool BAL>
+__device__ __forceinline__ void t1_creator_pass(const double* __restrict__ src, double* __restrict__ W, const double* __restrict__ t1,
+                                                int2* t1s, T1Scale& sc, const Dims& d) {
+  const bool fine = load_t1_fixed<BAL>(t1, t1s, d, sc);
+  const int st = BAL ? 0 : sc.col[0];
   const double* in = COPY ? src : W;
   const size_t m = (size_t)d.n * d.n * d.n;
   const size_t step = t1_index<double, POS>(d, 1, 0);  // distance of neighbouring rows
@@ -321,7 +344,6 @@ __global__ void __launch_bounds__(TPB, 2) k_t1_creator_fixed(const double* __res
     bool ok = fine;
     {
       double x[kT1Omax];
-      unsigned mx = 0;
 #pragma unroll
       for (int i = 0; i < kT1Omax; ++i) {
         x[i] = 0.0;
@@ -330,13 +352,24 @@ __global__ void __launch_bounds__(TPB, 2) k_t1_creator_fixed(const double* __res
           if (COPY) W[base + i * step] = x[i];
         }
       }
+      if constexpr (BAL) {
+        sx = -4000;
 #pragma unroll
-      for (int i = 0; i < kT1Omax; ++i) mx = max(mx, (unsigned)__double2hiint(x[i]) & 0x7fffffffu);
-      const int e = (int)(mx >> 20);
-      sx = e > 0 ? e - 1022 : 0;
-      ok = ok && e < 0x7ff;
+        for (int i = 0; i < kT1Omax; ++i) {
+          const int e = expo(x[i]);
+          ok = ok && e < 0x7ff;
+          if (e > 0) sx = max(sx, e - 1022 + sc.row[i]);
+        }
+      } else {
+        unsigned mx = 0;
 #pragma unroll
-      for (int i = 0; i < kT1Omax; ++i) w[i] = limbs(to_fix(x[i], sx, kT1Bits));
+        for (int i = 0; i < kT1Omax; ++i) mx = max(mx, (unsigned)__double2hiint(x[i]) & 0x7fffffffu);
+        const int e = (int)(mx >> 20);
+        sx = e > 0 ? e - 1022 : 0;
+        ok = ok && e < 0x7ff;
+      }
+#pragma unroll
+      for (int i = 0; i < kT1Omax; ++i) w[i] = limbs(to_fix(x[i], BAL ? sx - sc.row[i] : sx, kT1Bits));
     }
     const size_t vb = base + d.o * step;
     if (!ok) {  // NaN or infinity: plain sums
@@ -347,7 +380,7 @@ __global__ void __launch_bounds__(TPB, 2) k_t1_creator_fixed(const double* __res
       }
       continue;
     }
-    const double unit = t1_unit(sx, st);
+    const double unit = t1_unit(sx + st);
     constexpr int U = 8;  // rows whose loads are in flight
     for (int a0 = 0; a0 < d.v; a0 += U) {
       double x[U];
@@ -370,19 +403,33 @@ __global__ void __launch_bounds__(TPB, 2) k_t1_creator_fixed(const double* __res
             madw(x1, q.w, w[i + 1].x);
           }
         }
-        W[vb + (a0 + u) * step] = fma(-unit, (double)join(hh, x0 + x1), x[u]);
+        W[vb + (a0 + u) * step] = fma(-(BAL ? t1_unit(sx + sc.col[a0 + u]) : unit), (double)join(hh, x0 + x1), x[u]);
       }
     }
   }
 }
+// Calls: inlined, the balanced passes' registers slow the others down (82 orbitals: 424-530 -> 468-656 us a pass).
+template <int POS, bool COPY>
+__device__ __noinline__ void t1_creator_balanced(const double* __restrict__ src, double* __restrict__ W, const double* __restrict__ t1,
+                                                 int2* t1s, T1Scale& sc, const Dims& d) {
+  t1_creator_pass<POS, COPY, true>(src, W, t1, t1s, sc, d);
+}
+template <int POS, bool COPY>
+__global__ void __launch_bounds__(TPB, 2) k_t1_creator_fixed(const double* __restrict__ src, double* __restrict__ W,
+                                                              const double* __restrict__ t1, const int* __restrict__ bal, Dims d) {
+  extern __shared__ __align__(16) double t1raw[];
+  __shared__ T1Scale sc;
+  int2* t1s = reinterpret_cast<int2*>(t1raw);
+  if (!bal[0]) t1_creator_pass<POS, COPY, false>(src, W, t1, t1s, sc, d);
+  else t1_creator_balanced<POS, COPY>(src, W, t1, t1s, sc, d);
+}
 
 // Annihilator pass at POS: rows q < nocc get + sum_a t1[q][a] row_(nocc + a).
-template <int POS>
-__global__ void __launch_bounds__(TPB, 2) k_t1_annihilator_fixed(double* __restrict__ W, const double* __restrict__ t1, Dims d) {
-  extern __shared__ __align__(16) double t1raw[];
-  int2* t1s = reinterpret_cast<int2*>(t1raw);
-  int st;
-  const bool fine = load_t1_fixed(t1, t1s, d, &st);
+template <int POS, bool BAL>
+__device__ __forceinline__ void t1_annihilator_pass(double* __restrict__ W, const double* __restrict__ t1, int2* t1s, T1Scale& sc,
+                                                    const Dims& d) {
+  const bool fine = load_t1_fixed<BAL>(t1, t1s, d, sc);
+  const int st = BAL ? 0 : sc.col[0];
   const size_t m = (size_t)d.n * d.n * d.n;
   const size_t step = t1_index<double, POS>(d, 1, 0);
   constexpr int U = 12;  // rows read at a time; they share a scale
@@ -397,18 +444,30 @@ __global__ void __launch_bounds__(TPB, 2) k_t1_annihilator_fixed(double* __restr
       bool ok = fine;
       {
         double x[U];
-        unsigned mx = 0;
 #pragma unroll
         for (int u = 0; u < U; ++u) x[u] = a0 + u < d.v ? W[vb + (a0 + u) * step] : 0.0;
+        if constexpr (BAL) {
+          sx = -4000;
 #pragma unroll
-        for (int u = 0; u < U; ++u) mx = max(mx, (unsigned)__double2hiint(x[u]) & 0x7fffffffu);
-        const int e = (int)(mx >> 20);
-        sx = e > 0 ? e - 1022 : 0;
-        ok = ok && e < 0x7ff;
+          for (int u = 0; u < U; ++u) {
+            const int e = expo(x[u]);  // zero beyond the last row
+            ok = ok && e < 0x7ff;
+            if (e > 0) sx = max(sx, e - 1022 + sc.col[a0 + u]);
+          }
 #pragma unroll
-        for (int u = 0; u < U; ++u) w[u] = limbs(to_fix(x[u], sx, kT1Bits));
+          for (int u = 0; u < U; ++u) w[u] = limbs(to_fix(x[u], sx - (a0 + u < d.v ? sc.col[a0 + u] : 0), kT1Bits));
+        } else {
+          unsigned mx = 0;
+#pragma unroll
+          for (int u = 0; u < U; ++u) mx = max(mx, (unsigned)__double2hiint(x[u]) & 0x7fffffffu);
+          const int e = (int)(mx >> 20);
+          sx = e > 0 ? e - 1022 : 0;
+          ok = ok && e < 0x7ff;
+#pragma unroll
+          for (int u = 0; u < U; ++u) w[u] = limbs(to_fix(x[u], sx, kT1Bits));
+        }
       }
-      const double unit = t1_unit(sx, st);
+      const double unit = t1_unit(sx + st);  // BAL: the rows' powers of two follow at the end
 #pragma unroll
       for (int q = 0; q < kT1Omax; q += 2) {
         if (q < d.o) {
@@ -439,22 +498,37 @@ __global__ void __launch_bounds__(TPB, 2) k_t1_annihilator_fixed(double* __restr
     }
 #pragma unroll
     for (int q = 0; q < kT1Omax; ++q)
-      if (q < d.o) W[base + q * step] += acc[q];
+      if (q < d.o) W[base + q * step] = BAL ? fma(pow2(max(sc.row[q], -1000)), acc[q], W[base + q * step]) : W[base + q * step] + acc[q];
   }
 }
+template <int POS>
+__device__ __noinline__ void t1_annihilator_balanced(double* __restrict__ W, const double* __restrict__ t1, int2* t1s, T1Scale& sc,
+                                                     const Dims& d) {
+  t1_annihilator_pass<POS, true>(W, t1, t1s, sc, d);
+}
+template <int POS>
+__global__ void __launch_bounds__(TPB, 2) k_t1_annihilator_fixed(double* __restrict__ W, const double* __restrict__ t1,
+                                                                 const int* __restrict__ bal, Dims d) {
+  extern __shared__ __align__(16) double t1raw[];
+  __shared__ T1Scale sc;
+  int2* t1s = reinterpret_cast<int2*>(t1raw);
+  if (!bal[0]) t1_annihilator_pass<POS, false>(W, t1, t1s, sc, d);
+  else t1_annihilator_balanced<POS>(W, t1, t1s, sc, d);
+}
 
+// bal: balance of the FP64 passes (device)
 template <typename A>
-void t1_passes(const double* eri, double* W, const double* t1, const Dims& d, cudaStream_t st) {
+void t1_passes(const double* eri, double* W, const double* t1, const int* bal, const Dims& d, cudaStream_t st) {
   const size_t mc = (size_t)d.v * d.n * d.n * d.n, ma = (size_t)d.o * d.n * d.n * d.n;
   const size_t n3 = (size_t)d.n * d.n * d.n;
   if (d.o <= kT1Omax) {
     const unsigned g = blocks_for(n3) > 152u * 16u ? 152u * 16u : blocks_for(n3);
     if constexpr (sizeof(A) == 8) {
       const size_t fm = sizeof(int2) * kT1Omax * d.v;
-      k_t1_creator_fixed<0, true><<<g, TPB, fm, st>>>(eri, W, t1, d);
-      k_t1_creator_fixed<2, false><<<g, TPB, fm, st>>>(nullptr, W, t1, d);
-      k_t1_annihilator_fixed<1><<<g, TPB, fm, st>>>(W, t1, d);
-      k_t1_annihilator_fixed<3><<<g, TPB, fm, st>>>(W, t1, d);
+      k_t1_creator_fixed<0, true><<<g, TPB, fm, st>>>(eri, W, t1, bal, d);
+      k_t1_creator_fixed<2, false><<<g, TPB, fm, st>>>(nullptr, W, t1, bal, d);
+      k_t1_annihilator_fixed<1><<<g, TPB, fm, st>>>(W, t1, bal, d);
+      k_t1_annihilator_fixed<3><<<g, TPB, fm, st>>>(W, t1, bal, d);
     } else {
       const size_t sm = sizeof(A) * kT1Omax * d.v;
       // up to 53 orbitals blocks of 64: every SM gets some of the n^3 threads
@@ -475,19 +549,73 @@ void t1_passes(const double* eri, double* W, const double* t1, const Dims& d, cu
   }
 }
 
+// Balance of the FP64 form (fix_gemm.cuh) against scaled orbitals (one warp): integrals that carry a factor per
+// orbital, a_p where p is annihilated and b_p where it is created, are summed with amplitudes that carry the
+// inverse.  Integers relative to each operand's row norm would lose what the factors oppose, so the products
+// take g / (a b) and t a b (occupied orbitals are summed as creators, virtual ones as annihilators).  The
+// factors show in integrals that are alike for all orbitals without them: (pp|pp) in a_p^2 b_p^2, and (rp|rp)
+// against (pr|pr), which are one number, in the ratio a_p^2 b_r^2 / (a_r^2 b_p^2) (a factor r has on both sides
+// drops out of a b).  In quarters of a power of two; no balance (zeros) where the factors of a set spread by less
+// than 2^1.5 and those of the two by less than 2^3, which covers ordinary systems ((pp|pp) within 2^6 of
+// each other and 2^-6 .. 2^6), or where (pp|pp) vanishes.
+__device__ void balance_orbitals(const double* __restrict__ eri, const Dims& d, int* __restrict__ bal) {
+  const int lane = threadIdx.x & 31, r = d.n / 2;
+  auto ex = [&](int p, int q, int u, int w) { return (__double2hiint(eri[gi(d, p, q, u, w)]) >> 20) & 0x7ff; };
+  int q[4], lo[2] = {1 << 20, 1 << 20}, hi[2] = {-(1 << 20), -(1 << 20)}, fine = 1;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int p = lane + 32 * k, virt = p >= d.o;
+    q[k] = 0;
+    if (p < d.n) {
+      const int j = ex(p, p, p, p), x = ex(r, p, r, p), y = ex(p, r, p, r);
+      const int ratio = x > 0 && y > 0 && x < 0x7ff && y < 0x7ff ? x - y : 0;
+      fine &= j > 0 && j < 0x7ff;
+      q[k] = j - 1023 + (virt ? ratio : -ratio);
+      lo[0] = virt ? lo[0] : min(lo[0], q[k]);
+      hi[0] = virt ? hi[0] : max(hi[0], q[k]);
+      lo[1] = virt ? min(lo[1], q[k]) : lo[1];
+      hi[1] = virt ? max(hi[1], q[k]) : hi[1];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    lo[k] = __reduce_min_sync(0xffffffffu, lo[k]);
+    hi[k] = __reduce_max_sync(0xffffffffu, hi[k]);
+  }
+  const int mo = (lo[0] + hi[0]) / 2, mv = (lo[1] + hi[1]) / 2;
+  const bool on = __all_sync(0xffffffffu, fine) && (hi[0] - lo[0] > 6 || hi[1] - lo[1] > 6 || mo + mv > 12 || mo + mv < -12);
+  const int shift = (mv - mo) / 8;  // from one set to the other: a b is what counts
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int p = lane + 32 * k;
+    const int b = ((2 - q[k]) >> 2) + (p >= d.o ? shift : -shift);  // 2^b = 1 / factor
+    if (p < d.n) bal[1 + p] = on ? max(-fg::kMaxBalance, min(fg::kMaxBalance, b)) : 0;
+  }
+  if (lane == 0) bal[0] = on;
+}
+
 // h~ = (1 - K) h (1 + K), a block per column s (n <= 128 threads): (h (1+K))_{p s} of every row p once,
 // in shared memory, then the occupied rows' part.  Bound by the latency of the FP64 sums (v terms,
 // then o); with a thread per element and o + 1 sums of v terms in each it took 69 us at 114 orbitals
-// and 11 us at 24; now 15 and 6.
-__global__ void k_h_tilde(const double* __restrict__ h, const double* __restrict__ t1, double* __restrict__ ht, Dims d) {
+// and 11 us at 24; now 15 and 6.  bal (nullable): one more block sets the balance (1 + n ints).
+__global__ void k_h_tilde(const double* __restrict__ h, const double* __restrict__ t1, double* __restrict__ ht,
+                          const double* __restrict__ eri, int* __restrict__ bal, Dims d) {
   extern __shared__ __align__(16) double hks[];  // [n]
   const int s = blockIdx.x, p = threadIdx.x;
+  if (s == d.n) {
+    if (p < 32) balance_orbitals(eri, d, bal);
+    return;
+  }
   // (h (1+K))_{p s} = h_ps + [s occ] sum_a h_{p,nocc+a} t1[s][a]
-  double v = h[p * d.n + s];
-  if (s < d.o)
-    for (int a = 0; a < d.v; ++a) v += h[p * d.n + d.o + a] * t1[s * d.v + a];
-  hks[p] = v;
+  double v = 0.0;
+  if (p < d.n) {
+    v = h[p * d.n + s];
+    if (s < d.o)
+      for (int a = 0; a < d.v; ++a) v += h[p * d.n + d.o + a] * t1[s * d.v + a];
+    hks[p] = v;
+  }
   __syncthreads();
+  if (p >= d.n) return;
   if (p >= d.o)
     for (int i = 0; i < d.o; ++i) v -= t1[i * d.v + (p - d.o)] * hks[i];
   ht[p * d.n + s] = v;
@@ -532,10 +660,12 @@ __global__ void k_energy_part(const double* __restrict__ ht, const double* __res
   if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
 
-__global__ void k_energy_sum(const double* __restrict__ part, double* __restrict__ e0) {
+// bal (nullable, 1 + n ints): kept in the partial sums' place from here on.
+__global__ void k_energy_sum(double* part, double* __restrict__ e0, const int* __restrict__ bal, int n) {
   __shared__ double red[EGRID];
   red[threadIdx.x] = part[threadIdx.x];
   __syncthreads();
+  if (bal && (int)threadIdx.x <= n) reinterpret_cast<int*>(part)[threadIdx.x] = bal[threadIdx.x];
   for (int s = EGRID / 2; s > 0; s >>= 1) {
     if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
     __syncthreads();
@@ -684,6 +814,7 @@ struct Work {
   // FP64: A..D products of t2_terms_fixed, t2f = u, r2 its sum Z; mixed: A..D and t2f hold floats,
   // r2 = u until the residual is formed there
   double *ht, *foo, *fvv, *wo, *r1, *r2, *A, *B, *Cq, *D, *t2f;
+  int* bal;       // FP64 path: balance of the products (fix_gemm.cuh), in epart's place once the energy is summed
   int* scales;    // FP64 path: scale exponents of the products' operand rows (null: kArrays)
   void* slices;   // FP64 path, where its products run on the tensor cores: packed operands (else null)
   double* epart;  // energy partials
@@ -838,9 +969,9 @@ size_t fix_scale_ints(int o, int v) {
   return 5 * (size_t)o * o + 6 * (size_t)v * v + 20 * (size_t)o * v + 2 * (size_t)o * o * v + v;
 }
 
-Seg seg(const double* p, int rd, int rs1, int rs2, int kd, int ks1, int ks2, int K, int neg = 0, int shift = 0) {
-  return Seg{p, rd, rs1, rs2, kd, ks1, ks2, K, neg, shift};
-}
+// What the summed index of a product is: a pair of virtual, occupied and virtual, or occupied orbitals, or one
+// virtual; the balance of a digit stands at its orbital.
+enum Digits { kVV, kOV, kOO, kV };
 Out out(double* p, int rd, int rs1, int rs2, int cd, int cs1, int cs2, int add) {
   return Out{p, rd, rs1, rs2, cd, cs1, cs2, add, nullptr, 0, 0, 0, 0};
 }
@@ -875,59 +1006,75 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
     x.nseg = 2;
     return x;
   };
+  // segments by what they are summed over and by side: integrals (g) and amplitudes (t) take opposite balances
+  auto on = [o](Digits d, int side) {
+    return [=](const double* p, int rd, int rs1, int rs2, int kd, int ks1, int ks2, int K, int neg = 0, int shift = 0) {
+      return Seg{p, rd, rs1, rs2, kd, ks1, ks2, K, neg, shift, side, d == kVV ? o : d == kV ? -1 : 0, d == kOO ? 0 : o};
+    };
+  };
+  const auto gVV = on(kVV, 1);
+  const auto tVV = on(kVV, -1);
+  const auto gOV = on(kOV, 1);
+  const auto tOV = on(kOV, -1);
+  const auto gOO = on(kOO, 1);
+  const auto tOO = on(kOO, -1);
+  const auto gV = on(kV, 1);
+  const auto tV = on(kV, -1);
   // views of t2 / u: rows and k named by their indices
-  auto t_ia_me = [&](const double* t, int neg, int sh) { return seg(t, v, ovv, v, v, vv, 1, ov, neg, sh); };  // t(i m a e)
-  auto t_ja_me = [&](int neg) { return seg(t2, v, ovv, 1, v, vv, v, ov, neg); };                              // t(j m e a)
-  auto g_nf_me = [&](int swap) { return seg(V(5), v, n1, swap ? n2 : 1, v, n3, swap ? 1 : n2, ov); };           // g(m E n F) / g(m F n E)
-  const Operand wA = operand(oo, seg(V(5), o, n3, n1, v, n2, 1, vv));                    // (k l): g(k E l F)
-  const Operand tij = operand(oo, seg(t2, 1, vv, 0, v, v, 1, vv));                       // (i j): t(i j e f)
-  const Operand gab = operand(vv, seg(V(15), v, n3, n1, v, n2, 1, vv));                  // (a b): g(A E B F)
+  auto t_ia_me = [&](const double* t, int neg, int sh) { return tOV(t, v, ovv, v, v, vv, 1, ov, neg, sh); };  // t(i m a e)
+  auto t_ja_me = [&](int neg) { return tOV(t2, v, ovv, 1, v, vv, v, ov, neg); };                              // t(j m e a)
+  auto g_nf_me = [&](int swap) { return gOV(V(5), v, n1, swap ? n2 : 1, v, n3, swap ? 1 : n2, ov); };           // g(m E n F) / g(m F n E)
+  const Operand wA = operand(oo, gVV(V(5), o, n3, n1, v, n2, 1, vv));                    // (k l): g(k E l F)
+  const Operand tij = operand(oo, tVV(t2, 1, vv, 0, v, v, 1, vv));                       // (i j): t(i j e f)
+  const Operand gab = operand(vv, gVV(V(15), v, n3, n1, v, n2, 1, vv));                  // (a b): g(A E B F)
   const Operand eA = operand2(ov, t_ia_me(U, 0, -1), t_ia_me(t2, 1, 0));
   const Operand eB = operand2(ov, g_nf_me(0), g_nf_me(1));
   const Operand cA = operand(ov, t_ia_me(t2, 0, 0));
   const Operand gx = operand(ov, g_nf_me(1));
   const Operand dA = operand(ov, t_ja_me(0));
   const Operand xA = operand2(ov, t_ia_me(U, 0, 0), t_ia_me(t2, 1, 0));
-  const Operand xB = operand2(ov, seg(V(6), v, 1, n1, v, n3, n2, ov),                    // (j b): g(m E B j)
-                              seg(V(3), v, n2, n1, v, n3, 1, ov));                       //        g(m j B E)
-  const Operand v1A = operand2(vv, seg(V(7), v, n1, 1, v, n3, n2, ov),                   // (a e): g(m F A E)
-                               seg(V(7), v, n1, n2, v, n3, 1, ov, 1));                   //       -g(m E A F)
-  const Operand v1B = operand2(ov, seg(U, o, 1, vv, v, ovv, v, ov), seg(t2, o, 1, vv, v, ovv, v, ov));  // (b i): u, t(m i f b)
-  const Operand o1A = operand(ov, seg(V(7), v, n3, n1, v, n2, 1, vv));                   // (m b): g(m E B F)
-  const Operand x2A = operand2(ov, t_ja_me(0), seg(D, 1, ov, 0, ov, 0, 1, ov, 0, -1));   // (j a): t(j m e a), D/2
-  const Operand x2B = operand2(ov, seg(V(3), v, n2, n1, v, n3, 1, ov, 1),                // (i b): -g(m i B E)
-                               seg(t2, v, ovv, 1, v, vv, v, ov));                        //        t(i n f b)
-  const Operand r2A = operand2(oo, seg(W, o, n2, 1, o, n3, n1, oo), seg(w.wo, o, oo, 1, o, oo * o, o, oo));  // (i j): g, wo(m i n j)
-  const Operand r2B = operand2(vv, seg(t2, vv, 0, 1, oo, 0, vv, oo), seg(t2, vv, 0, 1, oo, 0, vv, oo));  // (a b): t(m n a b)
-  const Operand tab = operand(vv, seg(t2, vv, 0, 1, oo, 0, vv, oo));                     // (a b): t(m n a b)
-  const Operand v2B = operand(ov, seg(V(4), o, n2, 1, o, n3, n1, oo));                   // (e i): g(m E n i)
-  const Operand v4B = operand(vv, seg(V(5), v, n2, 1, o, n3, n1, oo));                   // (e f): g(m E n F)
-  const Operand o2A = operand2(oo, seg(V(1), o, n3, n2, v, n1, 1, ov),                   // (m i): g(m i n E)
-                               seg(V(4), o, n3, 1, v, n1, n2, ov, 1));                   //       -g(m E n i)
-  const Operand o2B = operand2(ov, seg(U, o, v, ovv, v, vv, 1, ov), seg(t2, o, v, ovv, v, vv, 1, ov));  // (b j): u, t(j n b e)
-  const Operand x3A = operand2(ov, seg(E, 1, ov, 0, ov, 0, 1, ov), seg(C, 1, ov, 0, ov, 0, 1, ov));     // (i a): E, C
+  const Operand xB = operand2(ov, gOV(V(6), v, 1, n1, v, n3, n2, ov),                    // (j b): g(m E B j)
+                              gOV(V(3), v, n2, n1, v, n3, 1, ov));                       //        g(m j B E)
+  const Operand v1A = operand2(vv, gOV(V(7), v, n1, 1, v, n3, n2, ov),                   // (a e): g(m F A E)
+                               gOV(V(7), v, n1, n2, v, n3, 1, ov, 1));                   //       -g(m E A F)
+  const Operand v1B = operand2(ov, tOV(U, o, 1, vv, v, ovv, v, ov), tOV(t2, o, 1, vv, v, ovv, v, ov));  // (b i): u, t(m i f b)
+  const Operand o1A = operand(ov, gVV(V(7), v, n3, n1, v, n2, 1, vv));                   // (m b): g(m E B F)
+  const Operand x2A = operand2(ov, t_ja_me(0), gOV(D, 1, ov, 0, v, v, 1, ov, 0, -1));   // (j a): t(j m e a), D/2
+  const Operand x2B = operand2(ov, gOV(V(3), v, n2, n1, v, n3, 1, ov, 1),                // (i b): -g(m i B E)
+                               tOV(t2, v, ovv, 1, v, vv, v, ov));                        //        t(i n f b)
+  const Operand r2A = operand2(oo, gOO(W, o, n2, 1, o, n3, n1, oo), gOO(w.wo, o, oo, 1, o, oo * o, o, oo));  // (i j): g, wo(m i n j)
+  const Operand r2B = operand2(vv, tOO(t2, vv, 0, 1, o, o * vv, vv, oo), tOO(t2, vv, 0, 1, o, o * vv, vv, oo));  // (a b): t(m n a b)
+  const Operand tab = operand(vv, tOO(t2, vv, 0, 1, o, o * vv, vv, oo));                     // (a b): t(m n a b)
+  const Operand v2B = operand(ov, gOO(V(4), o, n2, 1, o, n3, n1, oo));                   // (e i): g(m E n i)
+  const Operand v4B = operand(vv, gOO(V(5), v, n2, 1, o, n3, n1, oo));                   // (e f): g(m E n F)
+  const Operand o2A = operand2(oo, gOV(V(1), o, n3, n2, v, n1, 1, ov),                   // (m i): g(m i n E)
+                               gOV(V(4), o, n3, 1, v, n1, n2, ov, 1));                   //       -g(m E n i)
+  const Operand o2B = operand2(ov, tOV(U, o, v, ovv, v, vv, 1, ov), tOV(t2, o, v, ovv, v, vv, 1, ov));  // (b j): u, t(j n b e)
+  const Operand x3A = operand2(ov, gOV(E, 1, ov, 0, v, v, 1, ov), gOV(C, 1, ov, 0, v, v, 1, ov));     // (i a): E, C
   const Operand x3B = operand2(ov, t_ia_me(U, 0, 0), t_ia_me(t2, 0, 0));                 // (j b): u, t(j n b f)
-  const Operand ovA = operand2(ov, seg(V(5), v, n3, n2, v, n1, 1, ov),                   // (m e): g(m E n F)
-                               seg(V(5), v, n3, 1, v, n1, n2, ov, 1));                   //       -g(m F n E)
-  const Operand ooA = operand(ov, seg(V(5), v, n3, 1, v, n1, n2, ov));                   // (i b): g(i F n B)
+  const Operand ovA = operand2(ov, gOV(V(5), v, n3, n2, v, n1, 1, ov),                   // (m e): g(m E n F)
+                               gOV(V(5), v, n3, 1, v, n1, n2, ov, 1));                   //       -g(m F n E)
+  const Operand ooA = operand(ov, gOV(V(5), v, n3, 1, v, n1, n2, ov));                   // (i b): g(i F n B)
   Operand ooB = dA;                                                                      // (j a): -t(j n f a)
   ooB.seg[0].neg = 1;
-  const Operand v3A = operand(vv, seg(V(7), v, n2, n1, v, n3, 1, ov, 1));                // (e b): -g(m E B F)
-  const Operand v3B = operand(ov, seg(t2, o, v, vv, v, ovv, 1, ov));                     // (a i): t(m i a f)
-  const Operand o3A = operand(oo, seg(V(4), o, n3, 1, v, n1, n2, ov, 1));                // (m j): -g(m E n j)
-  const Operand o3B = operand(ov, seg(t2, o, 1, ovv, v, vv, v, ov));                     // (b i): t(i n e b)
-  const Operand yA = operand(oo * v, seg(t2, 1, v, 0, v, 0, 1, v));                      // (i j a): t(i j a e)
-  const Operand y2A = operand(oo * v, seg(t2, v, vv, 1, v, 0, v, v));                    // (i j b): t(i j e b)
-  const Operand yB = operand(v, seg(w.fvv, 1, v, 0, v, 0, 1, v));                        // b: Fvv(b e)
+  const Operand v3A = operand(vv, gOV(V(7), v, n2, n1, v, n3, 1, ov, 1));                // (e b): -g(m E B F)
+  const Operand v3B = operand(ov, tOV(t2, o, v, vv, v, ovv, 1, ov));                     // (a i): t(m i a f)
+  const Operand o3A = operand(oo, gOV(V(4), o, n3, 1, v, n1, n2, ov, 1));                // (m j): -g(m E n j)
+  const Operand o3B = operand(ov, tOV(t2, o, 1, ovv, v, vv, v, ov));                     // (b i): t(i n e b)
+  const Operand yA = operand(oo * v, tV(t2, 1, v, 0, v, 0, 1, v));                      // (i j a): t(i j a e)
+  const Operand y2A = operand(oo * v, tV(t2, v, vv, 1, v, 0, v, v));                    // (i j b): t(i j e b)
+  const Operand yB = operand(v, gV(w.fvv, 1, v, 0, v, 0, 1, v));                        // b: Fvv(b e)
 
   fg::Ops ops{};
   for (const Operand* p : {&wA, &tij, &gab, &eA, &eB, &cA, &gx, &dA, &xA, &xB, &v1A, &v1B, &o1A, &x2B, &r2B, &tab, &v2B,
                            &v4B, &o2A, &o2B, &x3B, &ovA, &ooA, &v3A, &v3B, &o3A, &o3B, &yA, &y2A, &yB})
     ops.o[ops.count++] = *p;
+  ops.bal = w.bal;
   cudaError_t e = need || alone ? cudaSuccess : fg::row_scales(ops, st);
   if (e != cudaSuccess) return e;
 
   fg::Jobs js{};
+  js.bal = w.bal;
   auto launch = [&]() -> cudaError_t {
     if (need) {
       const size_t b = oz::pack_bytes(js);
@@ -941,6 +1088,7 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
         fg::Jobs one{};
         one.j[0] = js.j[i];
         one.count = 1;
+        one.bal = w.bal;
         Job& j = one.j[0];
         const bool fits = j.a.rows + j.b.rows <= 2 * n2;
         j.a.e = reinterpret_cast<int*>(fits ? w.ht : E);
@@ -949,6 +1097,7 @@ cudaError_t t2_terms_fixed(const Dims& d, double* W, const double* t2, const dou
         both.o[0] = j.a;
         both.o[1] = j.b;
         both.count = 2;
+        both.bal = w.bal;
         cudaError_t err = fg::row_scales(both, st);
         if (err == cudaSuccess) err = fg::run(one, st);
         if (err != cudaSuccess) return err;
@@ -2047,16 +2196,21 @@ cudaError_t launch_dress(const double* h, const double* eri, const double* t1, c
   Dims d{n, nocc, n - nocc};
   const size_t n4 = (size_t)n * n * n * n;
   const size_t o = nocc, v = n - nocc;
+  // FP64 form: the orbitals' balance, set beside h~, in r2's place (and what follows it: at least 1.5 KB) until
+  // the energy's partial sums are free
+  const bool fixed = !mixed && v > 0 && o > 0;
+  int* bal = fixed ? reinterpret_cast<int*>(w.r2) : nullptr;
+  k_h_tilde<<<fixed ? n + 1 : n, n < 32 ? 32 : n, n * sizeof(double), st>>>(h, t1, w.ht, eri, bal, d);
   if (v > 0 && o > 0) {  // W = the bare integrals with T1 applied (the first pass copies them)
-    if (mixed) t1_passes<float>(eri, W, t1, d, st);  // FP32 correction sums onto the FP64 elements
-    else t1_passes<double>(eri, W, t1, d, st);
+    if (mixed) t1_passes<float>(eri, W, t1, nullptr, d, st);  // FP32 correction sums onto the FP64 elements
+    else t1_passes<double>(eri, W, t1, bal, d, st);
   } else {
     k_copy<<<blocks_for(n4) > 152u * 64u ? 152u * 64u : blocks_for(n4), TPB, 0, st>>>(eri, W, n4);
   }
-  k_h_tilde<<<n, n, n * sizeof(double), st>>>(h, t1, w.ht, d);
   k_fock<<<(n * n + 31) / 32, 32, 0, st>>>(w.ht, W, F, d);  // a warp per block: all SMs take part
   k_energy_part<<<EGRID, TPB, 0, st>>>(w.ht, W, t2, w.epart, d);
-  k_energy_sum<<<1, EGRID, 0, st>>>(w.epart, e0);
+  k_energy_sum<<<1, EGRID, 0, st>>>(w.epart, e0, bal, n);
+  w.bal = fixed ? reinterpret_cast<int*>(w.epart) : nullptr;
   if (v > 0 && o > 0) {
     // mixed: u lives in the r2 slot until the doubles residual is written there
     double* U = mixed ? w.r2 : w.t2f;

@@ -3,10 +3,17 @@
 //
 // What bounds it: FP64 FMAs run at 2 per clock and SM on GB300, so an FP64 tile kernel cannot pass
 // 1.25 TFLOP/s.  Here an operand row is scaled by a power of two above its norm and held as 55-bit
-// fixed-point limbs (fixed.cuh): three mad.wide per term, 21 terms per clock and SM.  Rounding: an
-// element is off by at most 2^-56 of its row's norm and a sum of K terms by about
-// 2^-57 sqrt(K) max(1, ..) of the product of the norms, no more than FP64 accumulation makes of it;
-// the sums themselves are exact, so the result does not depend on tiles or splits.
+// fixed-point limbs (fixed.cuh): three mad.wide per term, 21 terms per clock and SM.  The sums are exact, so
+// the result does not depend on tiles or splits.
+// Accuracy: an element is off by at most 2^-56 of its row's norm, and the low x low products left out are at
+// most 2^-58 of the norms' product each (K of them: about 2^-59 sqrt(K) where their signs mix, K 2^-58
+// where elements are equal).  So the error is bounded by the product of the two rows' norms, |a| |b|, where that
+// of FP64 sums (up to K 2^-53 of it) is bounded by sum |a_k b_k|: it is smaller where those are of
+// like size, and an output that is small against its rows' norms, because large elements of one row meet
+// small ones of the other, has fewer correct digits.  Scaled orbitals do that systematically and are taken out by
+// the balance (Seg): the ladder of 24 orbitals with amplitudes scaled by d_a d_b and integrals by its inverse,
+// relative to the largest output, for d over 1, 2 and 4 decades: without it 1e-14, 3e-13, 6e-10, with it 1e-15
+// throughout (emulated), FP64 sums 8e-16.
 // Overflow: |hi| <= 2^28 in norm, so the high sum stays below 2^57 and the cross sums below
 // 2 2^28 (2^26 sqrt(K)) < 2^63 for K < 2^16 (a product here has at most 2 n^2 <= 2^15 terms).
 //
@@ -19,20 +26,32 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "fixed.cuh"
 
 namespace qf {
 namespace fg {
 
 // Element (r, k) of a segment: p[(r / rd) rs1 + (r % rd) rs2 + (k / kd) ks1 + (k % kd) ks2], times
-// -1 if neg, times 2^shift.
+// -1 if neg, times 2^shift, times 2^(bs (t[b1 + k / kd] + t[b2 + k % kd])) with the launch's balance t
+// (b1 or b2 negative: that digit has none).  The two operands of a product have the same digits and
+// opposite bs, so the balance leaves their product as it is and only evens out its terms.
 struct Seg {
   const double* p;
   int rd, rs1, rs2;
   int kd, ks1, ks2;
   int K;
   int neg, shift;
+  int bs, b1, b2;
 };
+__host__ __device__ __forceinline__ int balance_of(const Seg& s, const int* t, int k1, int k2) {
+  return s.bs * ((s.b1 < 0 ? 0 : t[s.b1 + k1]) + (s.b2 < 0 ? 0 : t[s.b2 + k2]));
+}
+// A launch's balance (device, written before it): [0] whether there is one, [1..] exponents of at most
+// kMaxBalance in size.  Null: none.
+constexpr int kMaxBalance = 31;
+__device__ __forceinline__ const int* balance_table(const int* bal) { return bal && bal[0] ? bal + 1 : nullptr; }
 constexpr int kSegs = 2;
 struct Operand {
   Seg seg[kSegs];
@@ -63,12 +82,14 @@ constexpr int kMaxJobs = 8;
 struct Jobs {
   Job j[kMaxJobs];
   int count, tiles;
+  const int* bal;
 };
 constexpr int kMaxOps = 32;
 struct Ops {
   Operand o[kMaxOps];
   int block0[kMaxOps + 1];
   int count;
+  const int* bal;
 };
 
 namespace {
@@ -137,40 +158,48 @@ __global__ void __launch_bounds__(kThreads) k_row_scales(const __grid_constant__
   const int r0 = ((int)blockIdx.x - ops.block0[o]) * kScaleRows;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   NormAcc mine;  // of row r0 + lane, this warp's share
-  for (int g = 0; g < op.nseg; ++g) {
-    const Seg& s = op.seg[g];
-    if (row_fast(s)) {  // a lane per row, k dealt to the warps
-      const int r = r0 + lane;
-      if (r < op.rows) {
-        const double* p = s.p + (size_t)(r / s.rd) * s.rs1 + (size_t)(r % s.rd) * s.rs2;
-        int k1 = warp / s.kd, k2 = warp % s.kd;
-        for (int k = warp; k < s.K; k += 8) {
-          mine.add(p[(size_t)k1 * s.ks1 + (size_t)k2 * s.ks2], s.shift);
-          for (k2 += 8; k2 >= s.kd; k2 -= s.kd) ++k1;
-        }
-      }
-    } else {  // four rows per warp, lanes along k
-      for (int x = 0; x < kScaleRows / 8; ++x) {
-        const int rl = warp * (kScaleRows / 8) + x, r = r0 + rl;
-        NormAcc acc;
+  auto scan = [&](auto balanced) {
+    auto exponent = [&](const Seg& s, int k1, int k2) {
+      if constexpr (decltype(balanced)::value) return s.shift + balance_of(s, ops.bal + 1, k1, k2);
+      else return s.shift;
+    };
+    for (int g = 0; g < op.nseg; ++g) {
+      const Seg& s = op.seg[g];
+      if (row_fast(s)) {  // a lane per row, k dealt to the warps
+        const int r = r0 + lane;
         if (r < op.rows) {
           const double* p = s.p + (size_t)(r / s.rd) * s.rs1 + (size_t)(r % s.rd) * s.rs2;
-          int k1 = lane / s.kd, k2 = lane % s.kd;
-          for (int k = lane; k < s.K; k += 32) {
-            acc.add(p[(size_t)k1 * s.ks1 + (size_t)k2 * s.ks2], s.shift);
-            for (k2 += 32; k2 >= s.kd; k2 -= s.kd) ++k1;
+          int k1 = warp / s.kd, k2 = warp % s.kd;
+          for (int k = warp; k < s.K; k += 8) {
+            mine.add(p[(size_t)k1 * s.ks1 + (size_t)k2 * s.ks2], exponent(s, k1, k2));
+            for (k2 += 8; k2 >= s.kd; k2 -= s.kd) ++k1;
           }
         }
+      } else {  // four rows per warp, lanes along k
+        for (int x = 0; x < kScaleRows / 8; ++x) {
+          const int rl = warp * (kScaleRows / 8) + x, r = r0 + rl;
+          NormAcc acc;
+          if (r < op.rows) {
+            const double* p = s.p + (size_t)(r / s.rd) * s.rs1 + (size_t)(r % s.rd) * s.rs2;
+            int k1 = lane / s.kd, k2 = lane % s.kd;
+            for (int k = lane; k < s.K; k += 32) {
+              acc.add(p[(size_t)k1 * s.ks1 + (size_t)k2 * s.ks2], exponent(s, k1, k2));
+              for (k2 += 32; k2 >= s.kd; k2 -= s.kd) ++k1;
+            }
+          }
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) {
-          const int e2 = __shfl_xor_sync(0xffffffffu, acc.e, d);
-          const float s2 = __shfl_xor_sync(0xffffffffu, acc.s, d);
-          acc.merge(e2, s2);
+          for (int d = 16; d > 0; d >>= 1) {
+            const int e2 = __shfl_xor_sync(0xffffffffu, acc.e, d);
+            const float s2 = __shfl_xor_sync(0xffffffffu, acc.s, d);
+            acc.merge(e2, s2);
+          }
+          if (lane == rl) mine.merge(acc.e, acc.s);
         }
-        if (lane == rl) mine.merge(acc.e, acc.s);
       }
     }
-  }
+  };
+  if (balance_table(ops.bal)) scan(std::true_type{});
+  else scan(std::false_type{});
   se[warp][lane] = mine.e;
   ss[warp][lane] = mine.s;
   __syncthreads();
@@ -194,11 +223,13 @@ struct Rows {
 constexpr size_t kStageBytes = sizeof(Stage<64, 16>) > sizeof(Stage<32, 32>) ? sizeof(Stage<64, 16>) : sizeof(Stage<32, 32>);
 constexpr size_t kSmemBytes = 2 * kStageBytes + sizeof(Rows);
 
-// Reads one operand's share of a stage (4 elements per thread) into registers.
-template <int T, int KT>
+// Reads one operand's share of a stage (4 elements per thread) into registers.  BAL: with a balance (a form of
+// its own, since its bytes and table reads spill registers that the other form has).
+template <int T, int KT, bool BAL>
 struct Fetch {
   double v[4];
   int k1, k2, kk;  // thread's first k of the stage
+  int adj;         // the elements' balance, a byte each
   bool rf;
   __device__ __forceinline__ void start(const Seg& s) {
     rf = row_fast(s);
@@ -211,12 +242,16 @@ struct Fetch {
     return rf ? (int)threadIdx.x % T : (int)threadIdx.x / KT + i * (kThreads / KT);
   }
   __device__ __forceinline__ int koff(int i) const { return rf ? i * (kThreads / T) : 0; }
-  __device__ __forceinline__ void load(const Seg& s, const int* off, int rows_left) {
+  __device__ __forceinline__ void load(const Seg& s, const int* off, int rows_left, const int* bt) {
     int c1 = k1, c2 = k2;
+    if constexpr (BAL) adj = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       v[i] = 0.0;
-      if (kk + koff(i) < s.K && row(i) < rows_left) v[i] = s.p[(size_t)off[row(i)] + (size_t)(c1 * s.ks1 + c2 * s.ks2)];
+      if (kk + koff(i) < s.K && row(i) < rows_left) {
+        v[i] = s.p[(size_t)off[row(i)] + (size_t)(c1 * s.ks1 + c2 * s.ks2)];
+        if constexpr (BAL) adj |= (balance_of(s, bt, c1, c2) & 0xff) << (8 * i);
+      }
       if (rf)
         for (c2 += kThreads / T; c2 >= s.kd; c2 -= s.kd) ++c1;
     }
@@ -228,15 +263,15 @@ struct Fetch {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int r = row(i);
-      long long t = to_fix(v[i], e[r] - s.shift, kBits);
+      long long t = to_fix(v[i], e[r] - s.shift - (BAL ? (int)(signed char)(adj >> (8 * i)) : 0), kBits);
       if (s.neg) t = -t;
       dst[k0 + koff(i)][r] = limbs(t);
     }
   }
 };
 
-template <int T, int KG>  // tile T x T, k of a stage in KG groups
-__device__ __forceinline__ void product(const Job& jb, int tile, unsigned char* smem) {
+template <int T, int KG, bool BAL>  // tile T x T, k of a stage in KG groups
+__device__ __forceinline__ void product(const Job& jb, int tile, unsigned char* smem, const int* bt) {
   constexpr int KT = (KG == 1) ? 16 : 32, KS = KT / KG, TX = T / 4, GT = TX * TX;  // GT threads per group
   static_assert(GT * KG == kThreads && KT * T == 4 * kThreads, "tile shape");
   Stage<T, KT>* st = reinterpret_cast<Stage<T, KT>*>(smem);
@@ -255,7 +290,7 @@ __device__ __forceinline__ void product(const Job& jb, int tile, unsigned char* 
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) hh[i][j] = xx[i][j] = 0;
-  Fetch<T, KT> fa, fb;
+  Fetch<T, KT, BAL> fa, fb;
   int buf = 0;
   for (int g = 0; g < jb.a.nseg; ++g) {
     const Seg& sa = jb.a.seg[g];
@@ -270,16 +305,16 @@ __device__ __forceinline__ void product(const Job& jb, int tile, unsigned char* 
     __syncthreads();
     fa.start(sa);
     fb.start(sb);
-    fa.load(sa, rw.off[0], ra);
-    fb.load(sb, rw.off[1], rb);
+    fa.load(sa, rw.off[0], ra, bt);
+    fb.load(sb, rw.off[1], rb, bt);
     fa.store(sa, rw.e[0], st[buf].a);
     fb.store(sb, rw.e[1], st[buf].b);
     __syncthreads();
     for (int k0 = 0; k0 < sa.K; k0 += KT) {
       const bool more = k0 + KT < sa.K;
       if (more) {
-        fa.load(sa, rw.off[0], ra);
-        fb.load(sb, rw.off[1], rb);
+        fa.load(sa, rw.off[0], ra, bt);
+        fb.load(sb, rw.off[1], rb, bt);
       }
       const Stage<T, KT>& cur = st[buf];
 #pragma unroll 4
@@ -350,14 +385,25 @@ __device__ __forceinline__ void product(const Job& jb, int tile, unsigned char* 
   }
 }
 
+// A call, so that its registers stay out of the other form.
+__device__ __noinline__ void balanced_product(const Job& jb, int tile, unsigned char* smem, const int* bt) {
+  if (jb.t32) product<32, 4, true>(jb, tile, smem, bt);
+  else product<64, 1, true>(jb, tile, smem, bt);
+}
+
 __global__ void __launch_bounds__(kThreads, 2) k_fix_gemm(const __grid_constant__ Jobs jobs) {
   extern __shared__ __align__(16) unsigned char smem[];
   int j = 0;
   while (j + 1 < jobs.count && (int)blockIdx.x >= jobs.j[j + 1].tile0) ++j;
   const Job& jb = jobs.j[j];
   const int tile = (int)blockIdx.x - jb.tile0;
-  if (jb.t32) product<32, 4>(jb, tile, smem);
-  else product<64, 1>(jb, tile, smem);
+  const int* bt = balance_table(jobs.bal);
+  if (!bt) {
+    if (jb.t32) product<32, 4, false>(jb, tile, smem, bt);
+    else product<64, 1, false>(jb, tile, smem, bt);
+  } else {
+    balanced_product(jb, tile, smem, bt);
+  }
 }
 
 }  // namespace

@@ -7,8 +7,9 @@
 // balanced base-256 digits, exact in FP16.  A product keeps the digit pairs s + t <= 7 (34 MMAs of the
 // 49), one tensor-memory accumulator per diagonal s + t, all eight with 64 columns each: the whole tensor
 // memory.  Up to 7 pairs x 128 k x 2^14 < 2^24: sums of 128 k are exact in the FP32 accumulators, then
-// the diagonals are added into 64-bit integers in registers.  Left out are the pairs s + t >= 8 (2^-60 of
-// the norms' product for 5,000 terms); an element's own cut is 2^-56 of its row's norm.  The result does
+// the diagonals are added into 64-bit integers in registers.  Left out are the pairs s + t >= 8: at most 2^-61
+// of the norms' product per term, 2^-58 together for 5,000 terms of mixed sign; an element's own cut is
+// 2^-56 of its row's norm (accuracy as fix_gemm.cuh's, with the same balance).  The result does
 // not depend on tiles or launch order.
 //
 // What bounds it: 34 MMAs of 128 x 64 x 16 per K step, whose operands come from shared memory (6 KB per
@@ -57,6 +58,7 @@ struct PackOps {
   PackOp o[kMaxPack];
   int block0[kMaxPack + 1];
   int count;
+  const int* bal;
 };
 struct TcJob {
   CUtensorMap ta, tb;
@@ -78,7 +80,7 @@ constexpr int kPR = 32, kPK = 64;  // rows and k of a block's tile
 
 __global__ void __launch_bounds__(256) k_oz_pack(const __grid_constant__ PackOps ops) {
   __shared__ long long ts[kPR][kPK + 1];
-  __shared__ int roff[fg::kSegs][kPR], koff[kPK], kseg[kPK];  // index splits once per row and k of the tile
+  __shared__ int roff[fg::kSegs][kPR], koff[kPK], kseg[kPK], kexp[kPK];  // index splits and exponents once per row and k of the tile
   int o = 0;
   while (o + 1 < ops.count && (int)blockIdx.x >= ops.block0[o + 1]) ++o;
   const PackOp& po = ops.o[o];
@@ -92,7 +94,13 @@ __global__ void __launch_bounds__(256) k_oz_pack(const __grid_constant__ PackOps
     while (g < op.nseg && k >= pad32(op.seg[g].K)) k -= pad32(op.seg[g++].K);
     const bool in = g < op.nseg && k < op.seg[g < op.nseg ? g : 0].K;
     kseg[tid] = in ? g : -1;
-    if (in) koff[tid] = (k / op.seg[g].kd) * op.seg[g].ks1 + (k % op.seg[g].kd) * op.seg[g].ks2;
+    const int* bt = fg::balance_table(ops.bal);
+    if (in) {
+      const fg::Seg& sg = op.seg[g];
+      const int k1 = k / sg.kd, k2 = k % sg.kd;
+      koff[tid] = k1 * sg.ks1 + k2 * sg.ks2;
+      kexp[tid] = sg.shift + (bt ? fg::balance_of(sg, bt, k1, k2) : 0);
+    }
   } else if (tid < kPK + fg::kSegs * kPR) {
     const int g = (tid - kPK) / kPR, r = (tid - kPK) % kPR;
     if (g < op.nseg) roff[g][r] = ((r0 + r) / op.seg[g].rd) * op.seg[g].rs1 + ((r0 + r) % op.seg[g].rd) * op.seg[g].rs2;
@@ -111,7 +119,7 @@ __global__ void __launch_bounds__(256) k_oz_pack(const __grid_constant__ PackOps
       const int e = op.e[r0 + r];
       const double w = s.p[(size_t)roff[g][r] + (size_t)koff[kk]];
       if (e != fg::kBad) {
-        v = to_fix(w, e - s.shift, fg::kBits);
+        v = to_fix(w, e - kexp[kk], fg::kBits);
         if (s.neg) v = -v;
       }
     }
@@ -438,6 +446,7 @@ inline cudaError_t run(const fg::Jobs& js, void* scratch, cudaStream_t st) {
     b += pk.ops.o[i].rows_p / kPR * ((pk.ops.o[i].kp + kPK - 1) / kPK);
   }
   pk.ops.block0[pk.ops.count] = b;
+  pk.ops.bal = js.bal;
   k_oz_pack<<<b, 256, 0, st>>>(pk.ops);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
