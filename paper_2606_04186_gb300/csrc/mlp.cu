@@ -112,7 +112,7 @@ __global__ void k_colsum(const float* __restrict__ X, int rows, int cols, int ld
 // epsilon into the weights.
 constexpr int ST = 32, SK = 64, STP = ST + 4;
 
-template <bool TB, int EPI>
+template <int EPI>
 __global__ void __launch_bounds__(256) k_gemm_small(int M, int N, int K, const float* __restrict__ A, int lda,
                                                     const float* __restrict__ B, int ldb, StoreEpi<EPI> st) {
   // the slabs, then (after the last one) the warps' partial tiles in the same place
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(256) k_gemm_small(int M, int N, int K, const f
   for (int j = 0; j < 8; ++j)
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[i][j] = 0.f;
-  // element (row, k) of an operand slab for this thread's x-th load: along k where k is contiguous
+  // element (row, k) of an operand slab for this thread's x-th load, along whichever is contiguous
   float ra[8], rb[8];
   auto load = [&](int k0) {
 #pragma unroll
@@ -141,9 +141,9 @@ __global__ void __launch_bounds__(256) k_gemm_small(int M, int N, int K, const f
         ra[x] = in ? A[(size_t)(m0 + r) * lda + k0 + k] : 0.f;
       }
       {
-        const int r = TB ? t / SK : t % ST, k = TB ? t % SK : t / ST;
+        const int r = t % ST, k = t / ST;
         const bool in = n0 + r < N && k0 + k < K;
-        rb[x] = in ? (TB ? B[(size_t)(n0 + r) * ldb + k0 + k] : B[(size_t)(k0 + k) * ldb + n0 + r]) : 0.f;
+        rb[x] = in ? B[(size_t)(k0 + k) * ldb + n0 + r] : 0.f;
       }
     }
   };
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(256) k_gemm_small(int M, int N, int K, const f
     for (int x = 0; x < 8; ++x) {
       const int t = tid + x * 256;
       as[t % SK][t / SK] = ra[x];
-      bs[TB ? t % SK : t / ST][TB ? t / SK : t % ST] = rb[x];
+      bs[t / ST][t % ST] = rb[x];
     }
     __syncthreads();
     if (k0 + SK < K) load(k0 + SK);
@@ -204,10 +204,10 @@ cudaError_t gemm(int M, int N, int K, const float* A, int lda, const float* B, i
                  const float* bias, const float* aux, float* colsum, float* pack, int* err, cudaStream_t st, bool tiles = false) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   const StoreEpi<EPI> sv{C, ldc, bias, aux};
-  if constexpr (!TA) {
+  if constexpr (!TA && !TB && (EPI == kBiasTanh || EPI == kBias)) {  // inference
     if (tiles && M <= kSmallRows) {
       const dim3 g((unsigned)((N + ST - 1) / ST), (unsigned)((M + ST - 1) / ST));
-      k_gemm_small<TB, EPI><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, sv);
+      k_gemm_small<EPI><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, sv);
       return cudaGetLastError();
     }
   }
