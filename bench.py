@@ -669,14 +669,15 @@ def run_ours(args):
                                  if name in TRAFFIC_PER_SPACE and args.precision == "mixed" and not args.spaces_limit
                                  else None),
                      "kernel": ("solve_persistent_kernel" if sched["persistent"] else "solve_class_kernel<K>")
-                     if args.precision == "mixed" else ("solve_kernel<K,double,DUCC>" if args.form == "ducc"
-                                                        else "solve_kernel<K,double>"),
+                     if args.precision == "mixed" else ("solve_fixed_kernel<K,DUCC>" if args.form == "ducc"
+                                                        else "solve_fixed_kernel<K>"),
                      "flops_per_launch": flops, "launch_ms": solve_ms,
                      "flops_note": ("products the steps need (solver_flops): sigma of the first-order "
                                     "vector counts only its 117-determinant support, as the kernel "
                                     "computes it; the kernel is latency- and issue-bound (profiles/)"),
                      "peak_note": ("measured FP32 FMA peak of this GPU" if args.precision == "mixed"
-                                   else "measured FP64 FMA peak of this GPU") + " (" + peaks["method"] + ")",
+                                   else "measured FP64 FMA peak of this GPU; sigma's products run on the integer "
+                                   "pipe, so the fraction can pass 1") + " (" + peaks["method"] + ")",
                      "peaks_measured": {k: v for k, v in peaks.items() if k != "method"}},
         "schedule": sched,
         "dress_tensor": ({"gemm_flops": dress_gemm_flops(no, nv), "phase_ms": float(ph[:, 0].mean()),

@@ -116,7 +116,10 @@ typedef struct {
                                  2 = warm-start network (QFLOW_GUESS_NETWORK below): 6e6o
                                  roots are kept like 1, but sweeps start from Phi except the
                                  first sweep after a model is set or trained, which starts the
-                                 6e6o spaces from the network's guess.                       */
+                                 6e6o spaces from the network's guess.
+                                 FP64: a solve from a start vector takes the general kernel,
+                                 about ten times the time per iteration of one from Phi, so
+                                 Phi is the faster choice unless it needs that many more.    */
   int32_t schedule;           /* qflow_schedule_kind (mixed precision; FP64 uses per-class
                                  launches)                                                   */
   int32_t graph;              /* 1 = once the schedule is fixed (mixed: from the third sweep,
@@ -312,7 +315,8 @@ size_t qflow_dress_workspace(int32_t n, int32_t nocc);
  * Accuracy: the T2 products sum integers exactly, with elements cut at 2^-56 of their operand row's
  * norm (FP64 sums cut at 2^-53 of each term): for ordinary integrals nearer to 64 bits than FP64
  * sums, also where the orbitals are scaled; but an element of F or W that is small only because large
- * and small factors meet term by term is accurate to the rows' norms, not to its own size. */
+ * and small factors meet term by term is accurate to the rows' norms, not to its own size.
+ * With more than 16 occupied orbitals the T1 passes are FP64 sums, bound by the FP64 pipe. */
 int qflow_dress_device(const double* h, const double* eri, const double* t1, const double* t2, int32_t n,
                        int32_t nocc, double* e0, double* F, double* W, void* work, size_t work_bytes,
                        void* stream);
@@ -333,7 +337,8 @@ int qflow_dress_device(const double* h, const double* eri, const double* t1, con
  *             FP64: the solver starts from the guess (an all-zero vector means Phi).  Mixed:
  *             the solver first tests Phi (converged there: done), else starts from the span
  *             of Phi and the guess, whose sigma counts as one iteration.  Receives the
- *             converged root (Phi coefficient 1) when save_root != 0
+ *             converged root (Phi coefficient 1) when save_root != 0.  An FP64 solve with a guess
+ *             takes about ten times the time per iteration of one without
  *   precision qflow_precision; max_iter, tol as in qflow_options.
  * Mixed: the warp solver runs at most min(max_iter, 16) Davidson steps; when max_iter > 16 the
  * spaces it leaves unconverged are then solved by the FP64 solver (start from Phi, max_iter

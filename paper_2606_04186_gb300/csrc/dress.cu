@@ -956,8 +956,7 @@ namespace {
 //   E = 1/2 u g~_menf - t g~_mfne,  C = t g~_mfne,  D_janf = sum_me t_jm^ea g~_mfne
 // (the quadratic rings A u - B t + C t^T + D t with A = u g~_menf, B = u g~_mfne: A u, C t and D t are
 // their own pair transposes).  Three launches, so that a block is overwritten after its last use as
-// an operand and no element has two writers: 64-bit sums are exact, so results do not depend on the
-// tiling.  Before: one thread per output element (FP64 FMA chains), 60.3 ms of the 65.5 ms dressing
+// an operand and no element has two writers, so results do not depend on the order of blocks.  Before: one thread per output element (FP64 FMA chains), 60.3 ms of the 65.5 ms dressing
 // at 82 orbitals.
 using fg::Job;
 using fg::Operand;

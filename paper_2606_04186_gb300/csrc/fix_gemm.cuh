@@ -3,8 +3,9 @@
 //
 // What bounds it: FP64 FMAs run at 2 per clock and SM on GB300, so an FP64 tile kernel cannot pass
 // 1.25 TFLOP/s.  Here an operand row is scaled by a power of two above its norm and held as 55-bit
-// fixed-point limbs (fixed.cuh): three mad.wide per term, 21 terms per clock and SM.  The sums are exact, so
-// the result does not depend on tiles or splits.
+// fixed-point limbs (fixed.cuh): three mad.wide per term, 21 terms per clock and SM.  The sums of limb
+// products are exact; the two are joined once per output, or once per k group of a 32 x 32 tile (a rounding at 2^-57
+// of the norms' product each, which is all that the choice of tiles changes).
 // Accuracy: an element is off by at most 2^-56 of its row's norm, and the low x low products left out are at
 // most 2^-58 of the norms' product each (K of them: about 2^-59 sqrt(K) where their signs mix, K 2^-58
 // where elements are equal).  So the error is bounded by the product of the two rows' norms, |a| |b|, where that

@@ -17,7 +17,8 @@
 // against 21 of fix_gemm's integer pipe, of which its conversions leave about 8.  Slices are packed once per
 // launch (16 B per element); a slab of 32 k is four TMA boxes per operand (rows of 128 B = 32 k of two
 // slices, 128-byte swizzle), two stages of 96 KB; eight warps empty the accumulators.  Every wait is
-// bounded; a timeout makes the tile's outputs NaN.
+// bounded; a timeout makes the tile's outputs NaN.  Measured (57 orbitals, first and second launch): tensor pipe
+// 22 and 11 % busy, L2 6 and 25 % of its rate: one block per SM, whose warps wait for copies and sums in turn.
 #pragma once
 
 #include "fix_gemm.cuh"

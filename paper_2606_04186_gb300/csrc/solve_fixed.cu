@@ -26,9 +26,10 @@
 //     projected matrix) is spread over two warps with fused sums, conversions are field arithmetic,
 //     and six CTAs per SM (168 registers, 37 KB: four of the eight subspace vectors in shared memory,
 //     later ones in local memory) cover each other's latency.
-// Measured (sweep's solve phase): all 9,690 spaces of 24 orbitals 18.2 -> 1.47 ms, a cycle of 35,000
-// spaces of 82 orbitals 49.2 -> 4.5 ms, 35 spaces of 10 orbitals 0.72 -> 0.12 ms; FP64 pipe 42-50 %
-// busy, mad.wide about 25 %.  128 threads per space with three CTAs per SM: 1.85 ms at 24 orbitals (the
+// Measured (sweep's solve phase): all 9,690 spaces of 24 orbitals 18.2 -> 1.40 ms, a cycle of 35,000
+// spaces of 82 orbitals 49.2 -> 4.5-4.9 ms, 35 spaces of 10 orbitals 0.72 -> 0.12 ms.  Counters at 24 orbitals:
+// FP64 pipe 53 % busy, mad.wide's 42 %, issue slots 27 % (912 blocks of two warps, waits led by fixed latencies);
+// 4e4o: FP64 pipe 73 %, mad.wide's 11 %.  128 threads per space with three CTAs per SM: 1.85 ms at 24 orbitals (the
 // warps' sums double), 0.084 ms at 10.
 //
 // Spaces outside what this kernel is exact for leave with status kSpaceDefer and are solved by
